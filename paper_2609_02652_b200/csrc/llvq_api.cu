@@ -71,12 +71,15 @@ int llvq_create(llvq_ctx **out, int device, size_t scratch_bytes) {
     const HostTables &h = ctx->host;
     uint32_t lanes[32][4];
     gemv_lane_table(lanes);
-    struct Part { const void *src; size_t bytes; size_t off; } parts[10] = {
-        {h.base.data(), h.base.size() * 8, 0},          {h.desc.data(), h.desc.size() * sizeof(ClassDesc), 0},
-        {h.golay_by_weight.data(), 4096 * 4, 0},        {h.golay_by_message.data(), 4096 * 4, 0},
+    UnrankTables unrank;
+    if (!build_unrank_tables(h, unrank)) { delete ctx; return LLVQ_EINVAL; }
+    struct Part { const void *src; size_t bytes; size_t off; } parts[] = {
+        {h.desc.data(), h.desc.size() * sizeof(ClassDesc), 0},
         {h.cls_scale.data(), kClassSlots * 4, 0},       {h.cls_parity.data(), kClassSlots * 4, 0},
         {h.cls_value.data(), kClassSlots * 8 * 4, 0},   {h.cls_dist.data(), kClassSlots * 8, 0},
-        {h.cls_block.data(), kClassSlots * 8, 0},       {lanes, sizeof lanes, 0}};
+        {h.cls_block.data(), kClassSlots * 8, 0},       {lanes, sizeof lanes, 0},
+        {unrank.blob.data(), unrank.blob.size(), 0},    {unrank.tail8.data(), unrank.tail8.size() * 4, 0},
+        {unrank.tab_a.data(), unrank.tab_a.size() * 8, 0}, {unrank.tab_b.data(), unrank.tab_b.size() * 4, 0}};
     size_t total = 0;
     for (auto &p : parts) { p.off = total; total += round_up(p.bytes, 256); }
     if (cudaMalloc(&ctx->table_blob, total) != cudaSuccess) { delete ctx; return LLVQ_ECUDA; }
@@ -87,18 +90,17 @@ int llvq_create(llvq_ctx **out, int device, size_t scratch_bytes) {
         }
     char *blob = (char *)ctx->table_blob;
     DeviceTables &d = ctx->dev;
-    d.base = (const uint64_t *)(blob + parts[0].off);
-    d.desc = (const ClassDesc *)(blob + parts[1].off);
-    d.golay_by_weight = (const uint32_t *)(blob + parts[2].off);
-    d.golay_by_message = (const uint32_t *)(blob + parts[3].off);
-    d.cls_scale = (const float *)(blob + parts[4].off);
-    d.cls_parity = (const uint32_t *)(blob + parts[5].off);
-    d.cls_value = (const float *)(blob + parts[6].off);
-    d.cls_dist = (const uint8_t *)(blob + parts[7].off);
-    d.cls_block = (const float2 *)(blob + parts[8].off);
-    d.lane_table = (const uint4 *)(blob + parts[9].off);
-    std::memcpy(d.weight_offset, h.weight_offset, sizeof d.weight_offset);
-    d.num_classes = h.num_classes;
+    d.desc = (const ClassDesc *)(blob + parts[0].off);
+    d.cls_scale = (const float *)(blob + parts[1].off);
+    d.cls_parity = (const uint32_t *)(blob + parts[2].off);
+    d.cls_value = (const float *)(blob + parts[3].off);
+    d.cls_dist = (const uint8_t *)(blob + parts[4].off);
+    d.cls_block = (const float2 *)(blob + parts[5].off);
+    d.lane_table = (const uint4 *)(blob + parts[6].off);
+    ctx->unrank.blob = (const uint8_t *)(blob + parts[7].off);
+    ctx->unrank.tail8 = (const uint32_t *)(blob + parts[8].off);
+    ctx->unrank.tab_a = (const uint64_t *)(blob + parts[9].off);
+    ctx->unrank.tab_b = (const uint32_t *)(blob + parts[10].off);
     d.num_points = h.num_points;
 
     if (scratch_bytes == 0) scratch_bytes = (size_t)8 << 20;
@@ -113,7 +115,7 @@ int llvq_create(llvq_ctx **out, int device, size_t scratch_bytes) {
     ctx->bad_codes = reinterpret_cast<uint32_t *>(ctx->error + 1);
     ctx->overflow = reinterpret_cast<uint32_t *>(ctx->error + 2);
     ctx->counter = reinterpret_cast<unsigned long long *>(ctx->error + 4);
-    if (gemv_configure(ctx) != 0 || rotate_configure() != 0 || cudaDeviceSynchronize() != cudaSuccess) { llvq_destroy(ctx); return LLVQ_ECUDA; }
+    if (gemv_configure(ctx) != 0 || expand_configure() != 0 || rotate_configure() != 0 || cudaDeviceSynchronize() != cudaSuccess) { llvq_destroy(ctx); return LLVQ_ECUDA; }
     *out = ctx;
     return LLVQ_OK;
 }

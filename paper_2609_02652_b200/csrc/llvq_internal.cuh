@@ -7,6 +7,7 @@
 
 #include "../../include/llvq.h"
 #include "llvq_tables.h"
+#include "llvq_unrank.cuh"
 
 namespace llvq {
 
@@ -32,18 +33,13 @@ __host__ __device__ inline size_t overlay_table_offset(int64_t rows, int64_t nb)
 }
 
 struct DeviceTables {
-    const uint64_t *base;            // num_classes + 1
     const ClassDesc *desc;           // num_classes
-    const uint32_t *golay_by_weight; // 4096
-    const uint32_t *golay_by_message;// 4096
     const float *cls_scale;          // 512
     const uint32_t *cls_parity;      // 512
     const float *cls_value;          // 512 x 8
     const uint8_t *cls_dist;         // 512 x 8
     const float2 *cls_block;         // 512 x {1 / (4 sqrt m), parity - 16}
     const uint4 *lane_table;         // 32 x {b0, b1, b2, xs}: a lane's operand offsets in two consecutive x records
-    int weight_offset[25];
-    int num_classes;
     uint64_t num_points;
 };
 
@@ -125,6 +121,7 @@ struct llvq_ctx {
     int device;
     llvq::HostTables host;
     llvq::DeviceTables dev;
+    llvq::UnrankView unrank;     // the expander's tables (device)
     void *table_blob;        // one allocation holding every table
     unsigned long long *accum;   // reduction scratch: one 64-bit accumulator a row of the largest launch
     size_t accum_slots;
@@ -158,6 +155,7 @@ cudaError_t launch_dequant(const llvq_ctx *ctx, int layout, const uint8_t *buf, 
                            __half *W, int64_t rows, int64_t nb, cudaStream_t s);
 cudaError_t launch_decode_i8(const llvq_ctx *ctx, int layout, const uint8_t *buf, int8_t *coords, uint16_t *class_ids,
                              int64_t rows, int64_t nb, cudaStream_t s);
+int expand_configure();                    // sets the expander's shared-memory attributes once a device
 int gemv_configure(const llvq_ctx *ctx);   // sets the kernels' shared-memory attributes once
 
 // activation rotation: blocks of at most 2^14 coordinates (64-bit partial sums in 128 KiB of shared memory)

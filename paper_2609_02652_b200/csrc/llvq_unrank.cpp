@@ -1,0 +1,206 @@
+#include "llvq_unrank.h"
+
+#include <cstring>
+#include <map>
+
+namespace llvq {
+namespace {
+
+// Appends every ordering of the multiset `cnt` (values 0..n-1), lexicographically, `bits` bits a value.
+template <typename T>
+void list_orderings(int *cnt, int n, int left, int at, int bits, uint64_t word, std::vector<T> &out) {
+    if (left == 0) { out.push_back((T)word); return; }
+    for (int v = 0; v < n; v++) {
+        if (cnt[v] == 0) continue;
+        cnt[v]--;
+        list_orderings(cnt, n, left - 1, at + 1, bits, word | (uint64_t)v << (bits * at), out);
+        cnt[v]++;
+    }
+}
+
+// the eight bits of b as the low bits of eight nibbles
+uint32_t spread_bits(uint32_t b) {
+    uint32_t w = 0;
+    for (int i = 0; i < 8; i++) w |= ((b >> i) & 1u) << (4 * i);
+    return w;
+}
+
+// Window of the 10-byte layout (codes u = 8 + floor(x / 2)): a block lacks one if two codes are more than seven apart,
+// or a code is below 3 or above 13.
+int window_of(const ClassDesc &d) {
+    int lo[24], hi[24], n = 0;                           // codes of the negative and of the positive coordinate
+    for (int v = 0; v < (d.odd ? 7 : 8); v++)
+        for (int j = 0; j < d.cnt[v]; j++) {
+            const int a = d.odd ? 1 + 2 * v : (v < 4 ? 2 + 4 * v : 4 * (v - 4));
+            lo[n] = d.odd ? 7 - v : 8 - a / 2;
+            hi[n] = 8 + a / 2;
+            n++;
+        }
+    bool can = false, must = false;
+    for (int i = 0; i < n; i++) {
+        const bool bad_hi = hi[i] > 13, bad_lo = lo[i] < 3;
+        can |= bad_hi || bad_lo;
+        must |= bad_hi && bad_lo;
+        for (int j = 0; j < n; j++) can |= i != j && hi[i] - lo[j] > 7;
+    }
+    return must ? kWindowNever : (can ? kWindowDepends : kWindowAlways);
+}
+
+template <typename T>
+T *part(std::vector<uint8_t> &blob, int offset) { return reinterpret_cast<T *>(blob.data() + offset); }
+
+}  // namespace
+
+bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
+    u.blob.assign(kUnrankBlobBytes, 0);
+    u.tail8.clear(); u.tab_a.clear(); u.tab_b.clear();
+    if (t.num_classes > kUnrankClasses - 2) return false;
+
+    UnrankStep *steps = part<UnrankStep>(u.blob, kUnrankSteps);
+    for (uint32_t n = 1; n < 32; n++) {
+        steps[n].shift = (uint32_t)__builtin_ctz(n);
+        const uint32_t odd = n >> steps[n].shift;
+        uint32_t x = odd;                                // correct to 3 bits, doubled by each Newton step
+        for (int i = 0; i < 4; i++) x *= 2u - odd * x;
+        steps[n].inverse = x;
+    }
+
+    // ---- every ordering of eight odd magnitudes with sum j (j + 1) / 2 <= 21
+    {
+        uint16_t *first = part<uint16_t>(u.blob, kUnrankTailBase);
+        static const int cost[7] = {0, 1, 3, 6, 10, 15, 21};
+        int c[7];
+        for (c[6] = 0; c[6] <= 1; c[6]++)
+        for (c[5] = 0; c[5] <= 1; c[5]++)
+        for (c[4] = 0; c[4] <= 2; c[4]++)
+        for (c[3] = 0; c[3] <= 3; c[3]++)
+        for (c[2] = 0; c[2] <= 7; c[2]++)
+        for (c[1] = 0; c[1] <= 8; c[1]++) {
+            int n = 0, sum = 0;
+            for (int v = 1; v < 7; v++) { n += c[v]; sum += c[v] * cost[v]; }
+            if (n > 8 || sum > 21) continue;
+            c[0] = 8 - n;
+            if (u.tail8.size() > 0xffff) return false;
+            first[c[1] | c[2] << 4 | c[3] << 7 | c[4] << 9 | c[5] << 11 | c[6] << 12] = (uint16_t)u.tail8.size();
+            list_orderings(c, 7, 8, 0, 4, 0, u.tail8);
+        }
+    }
+
+    // ---- supports of 8, 12, 16, 24 coordinates: (w - n1 - n2, n1, n2) copies of k = 0, 1, 2 with 8 n1 + 24 n2 <= 48 - w
+    std::map<int, uint32_t> first_a, first_b;
+    static const int weights[4] = {8, 12, 16, 24};
+    for (int w : weights)
+        for (int n2 = 0; 24 * n2 <= 48 - w; n2++)
+            for (int n1 = 0; 8 * n1 + 24 * n2 <= 48 - w; n1++) {
+                int c[3] = {w - n1 - n2, n1, n2};
+                first_a[w << 16 | n1 << 8 | n2] = (uint32_t)u.tab_a.size();
+                list_orderings(c, 3, w, 0, 2, 0, u.tab_a);
+            }
+    // ---- off-support values of 8, 12, 16 coordinates: n1, n2, n3 copies of k = 1, 2, 3 (and zeros) with
+    // n1 + 4 n2 + 9 n3 <= 8 (w = 16), 12 (the last twelve coordinates of w = 0; w = 12 needs 9), 10 (w = 8)
+    uint32_t *rest12 = part<uint32_t>(u.blob, kUnrankRest12);
+    static const int lengths[3] = {8, 12, 16}, room[3] = {8, 12, 10};
+    for (int l = 0; l < 3; l++)
+        for (int n3 = 0; n3 <= 1; n3++)
+            for (int n2 = 0; n2 <= 3; n2++)
+                for (int n1 = 0; n1 <= 12; n1++) {
+                    if (n1 + 4 * n2 + 9 * n3 > room[l] || n1 + n2 + n3 > lengths[l]) continue;
+                    int c[4] = {lengths[l] - n1 - n2 - n3, n1, n2, n3};
+                    first_b[lengths[l] << 16 | n1 << 8 | n2 << 4 | n3] = (uint32_t)u.tab_b.size();
+                    if (lengths[l] == 12) rest12[n1 | n2 << 4 | n3 << 6] = (uint32_t)u.tab_b.size();
+                    list_orderings(c, 4, lengths[l], 0, 2, 0, u.tab_b);
+                }
+
+    // ---- classes
+    uint64_t *base = part<uint64_t>(u.blob, kUnrankBase);
+    UnrankDesc *desc = part<UnrankDesc>(u.blob, kUnrankDescs);
+    for (int c = 0; c < kUnrankClasses; c++) base[c] = c <= t.num_classes ? t.base[(size_t)c] : ~0ull;
+    for (int c = 0; c < t.num_classes; c++) {
+        const ClassDesc &d = t.desc[(size_t)c];
+        UnrankDesc &e = desc[c];
+        if (d.perm_a >= 0x80000000ull || d.perm_b > 0x1000000ull) return false;
+        e.perm_a = (uint32_t)d.perm_a;
+        e.perm_b = (uint32_t)d.perm_b;
+        e.inv_a = 1.0f / (float)d.perm_a;
+        e.inv_b = 1.0f / (float)d.perm_b;
+        e.flags = (uint32_t)d.odd | (uint32_t)d.w << 1 | (uint32_t)d.sign_bits << 6 | (uint32_t)d.nz_b << 11 | (uint32_t)d.shell << 16 |
+                  (uint32_t)window_of(d) << 20;
+        if (d.odd) {
+            e.a = d.cnt[0] | (uint32_t)d.cnt[1] << 8;
+            e.b = 0;
+            for (int v = 2; v < 7; v++) e.b |= (uint32_t)d.cnt[v] << (4 * (v - 2));
+            continue;
+        }
+        e.golay = (uint32_t)t.weight_offset[d.w];
+        int half_sum = 0;                                // sum |x| / 2
+        for (int k = 0; k < 4; k++) half_sum += d.cnt[k] * (1 + 2 * k) + d.cnt[4 + k] * 2 * k;
+        if (d.w > 0) {
+            if (half_sum & 1) return false;
+            e.flags |= (uint32_t)((half_sum >> 1) & 1) << 15;
+            const auto a = first_a.find(d.w << 16 | d.cnt[1] << 8 | d.cnt[2]);
+            if (a == first_a.end() || d.cnt[3]) return false;
+            e.a = a->second;
+        }
+        if (d.w == 0) {
+            e.b = (uint32_t)d.cnt[4] | (uint32_t)d.cnt[5] << 8 | (uint32_t)d.cnt[6] << 16 | (uint32_t)d.cnt[7] << 24;
+        } else if (d.w < 24) {
+            const auto b = first_b.find((24 - d.w) << 16 | d.cnt[5] << 8 | d.cnt[6] << 4 | d.cnt[7]);
+            if (b == first_b.end()) return false;
+            e.b = b->second;
+        }
+    }
+    // ---- guide: class of the smallest index of every slot (a slot's indices share exponent and leading mantissa bits
+    // of their value rounded to float; rounding is monotonic, so slots are ranges of indices)
+    {
+        uint16_t *guide = part<uint16_t>(u.blob, kUnrankGuide);
+        auto slot_of = [](uint64_t idx) {
+            const float f = (float)idx;
+            uint32_t bits;
+            std::memcpy(&bits, &f, 4);
+            const int s = (int)(bits >> kGuideShift) - kGuideFirst;
+            return s < 0 ? 0 : s;
+        };
+        // guide[s] = last class c whose first index lies in a slot before s, or is the slot's first index: the largest c with
+        // slot_of(base[c]) < s is a lower bound that holds for every index of slot s
+        for (int s = 0; s < kGuideSlots + 8; s++) {
+            int c = 0;
+            while (c + 1 < t.num_classes && slot_of(t.base[(size_t)c + 1]) < s) c++;
+            guide[s] = (uint16_t)c;
+        }
+    }
+    std::memcpy(u.blob.data() + kUnrankGolayMsg, t.golay_by_message.data(), 4096 * 4);
+    std::memcpy(u.blob.data() + kUnrankGolayWt, t.golay_by_weight.data(), 4096 * 4);
+
+    // ---- spreading eight nibbles to the places of a byte mask, and single bits likewise
+    struct Moves { uint32_t m[4]; };
+    Moves *merge = part<Moves>(u.blob, kUnrankMerge);
+    uint16_t *at = part<uint16_t>(u.blob, kUnrankDepositAt);
+    uint32_t *deposit = part<uint32_t>(u.blob, kUnrankDeposit);
+    int n = 0;
+    for (int mask = 0; mask < 256; mask++) {
+        // the nibble of rank r must travel place[r] - r places up; in steps of 4, 2, 1 (each step's targets are
+        // distinct, because ranks travel by non-decreasing distances)
+        int place[8], k = 0;
+        for (int i = 0; i < 8; i++) if ((mask >> i) & 1) place[k++] = i;
+        Moves mv = {{0, 0, 0, 0}};
+        for (int r = 0; r < k; r++) {
+            int pos = r;
+            for (int step = 2; step >= 0; step--)
+                if (((place[r] - r) >> step) & 1) {
+                    pos += 1 << step;
+                    mv.m[2 - step] |= 15u << (4 * pos);
+                }
+            mv.m[3] |= 15u << (4 * place[r]);
+        }
+        merge[mask] = mv;
+        at[mask] = (uint16_t)n;
+        for (int bits = 0; bits < (1 << k); bits++) {
+            uint32_t b = 0;
+            for (int r = 0; r < k; r++) b |= (uint32_t)((bits >> r) & 1) << place[r];
+            deposit[n++] = spread_bits(b);
+        }
+    }
+    return n == 6561;
+}
+
+}  // namespace llvq

@@ -1,0 +1,247 @@
+// From an index of the ball to the 24 four-bit codes u_i = 8 + floor(x_i / 2) (and magnitudes, signs), with the tables of
+// llvq_unrank.h: `blob` in shared memory, the lists of orderings in global memory (1.3 MB, resident in L2).
+//
+// The index splits as the paper states it (Sec. 2.1: classes first, then arrangements and signs inside a class, as a
+// mixed-radix number).  The digit order used here:
+//   even type:  ((codeword rank * perm_a + rank_a) * perm_b + rank_b) << sign_bits | signs
+//   odd type:   arrangement rank * 4096 + message bits of the codeword
+// Arrangement ranks are lexicographic over the distinct orderings, smaller magnitude first; sign bits run over the
+// non-zero off-support coordinates first, then the support coordinates but the last, whose sign restores the sum
+// condition mod 8.
+//
+// Coordinates are worked on eight at a time, a nibble each.  With j = (|x| - 1) / 2 (odd type) a positive coordinate's
+// code is 8 + j and a negative one's 7 - j, the complement; with h = |x| / 2 (even type) they are 8 + h and 8 - h, the
+// two's complement.  So a word of codes is the word of j or h, with bit 3 set, complemented nibble-wise where the
+// sign word says so (and, for the even type, one added there).
+#pragma once
+#include <cstdint>
+
+#include "llvq_unrank.h"
+
+#ifdef __CUDACC__
+#define LLVQ_HD __host__ __device__ __forceinline__
+#else
+#define LLVQ_HD inline
+#endif
+
+namespace llvq {
+
+struct UnrankView {
+    const uint8_t *blob;
+    const uint32_t *tail8;
+    const uint64_t *tab_a;
+    const uint32_t *tab_b;
+};
+
+// Magnitudes (j or h) and signs (1 = negative) of the 24 coordinates, eight nibbles a word.
+struct Point {
+    uint32_t mag[3], neg[3];
+};
+
+LLVQ_HD int popcount32(uint32_t v) {
+#ifdef __CUDA_ARCH__
+    return __popc(v);
+#else
+    return __builtin_popcount(v);
+#endif
+}
+LLVQ_HD float u64_to_float(uint64_t v) { return (float)v; }
+LLVQ_HD uint32_t float_bits(float f) {
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(f);
+#else
+    union { float f; uint32_t u; } c;
+    c.f = f;
+    return c.u;
+#endif
+}
+template <typename T>
+LLVQ_HD const T &blob_at(const UnrankView &v, int offset, uint32_t i) { return reinterpret_cast<const T *>(v.blob + offset)[i]; }
+
+// bits 0..7 of b as the low bits of eight nibbles (the partial products do not overlap)
+LLVQ_HD uint32_t spread8(uint32_t b) {
+    b = ((b & 0xffu) * 0x1001u) & 0x000f000fu;
+    b = (b * 0x41u) & 0x03030303u;
+    return (b * 9u) & 0x11111111u;
+}
+// eight two-bit fields as eight nibbles
+LLVQ_HD uint32_t spread_pairs(uint32_t b) {
+    b &= 0xffffu;
+    b = (b | b << 8) & 0x00ff00ffu;
+    b = (b | b << 4) & 0x0f0f0f0fu;
+    return (b | b << 2) & 0x33333333u;
+}
+// the low bits of eight nibbles as bits 0..7
+LLVQ_HD uint32_t gather8(uint32_t w) {
+    w = (w | w >> 3) & 0x03030303u;
+    w = (w | w >> 6) & 0x000f000fu;
+    return (w | w >> 12) & 0xffu;
+}
+
+// Class of a valid index: the last c with base[c] <= idx, searched between the guide's bounds.
+LLVQ_HD int find_class(const UnrankView &v, uint64_t idx) {
+    int s = (int)(float_bits(u64_to_float(idx)) >> kGuideShift) - kGuideFirst;
+    s = s < 0 ? 0 : s;
+    int lo = blob_at<uint16_t>(v, kUnrankGuide, s), hi = blob_at<uint16_t>(v, kUnrankGuide, s + 1) + 1;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (blob_at<uint64_t>(v, kUnrankBase, mid) <= idx) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+// Of `left` coordinates that have T orderings, T * copies / left begin with a given value.  The quotient is exact and below
+// 2^32: shifted right by left's power of two, the product times the inverse of left's odd part modulo 2^32.
+LLVQ_HD uint32_t portion(uint32_t T, uint32_t copies, const UnrankStep &e) { return (uint32_t)(((uint64_t)T * copies) >> e.shift) * e.inverse; }
+
+// Odd type.  The first sixteen coordinates are found one by one (three in four are the first or the second value tried), the
+// ordering of the last eight is an entry of a list.  Rolled up: the code of a step unrolled sixteen times does not fit the
+// instruction cache beside the rest.
+LLVQ_HD void unrank_odd(const UnrankView &v, const UnrankDesc &d, uint64_t r47, Point &p) {
+    const uint32_t cw = blob_at<uint32_t>(v, kUnrankGolayMsg, (uint32_t)r47 & 4095u);
+    uint32_t r = (uint32_t)(r47 >> 12), T = d.perm_a;
+    uint32_t n0 = d.a & 255u, n1 = d.a >> 8, more = d.b;     // copies of j = 0, 1, and of 2.. a nibble each
+    uint32_t word = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll 1
+#endif
+    for (int i = 0; i < 16; i++) {
+        const UnrankStep e = blob_at<UnrankStep>(v, kUnrankSteps, 24 - i);
+        uint32_t s = portion(T, n0, e), j = 0;
+        if (r < s) {
+            n0--;
+        } else {
+            r -= s;
+            s = portion(T, n1, e);
+            if (r < s) {
+                n1--;
+                j = 1;
+            } else {
+                r -= s;
+                uint32_t sh = 0;
+                s = portion(T, more & 15u, e);
+                while (r >= s && sh < 16u) {
+                    r -= s;
+                    sh += 4;
+                    s = portion(T, (more >> sh) & 15u, e);
+                }
+                more -= 1u << sh;
+                j = 2u + (sh >> 2);
+            }
+        }
+        T = s;
+        word = word >> 4 | j << 28;
+        if (i == 7) p.mag[0] = word;
+    }
+    p.mag[1] = word;
+    const uint32_t key = (n1 | (more & 7u) << 4 | (more & 0x30u) << 3 | (more & 0x300u) << 1 | (more & 0x1000u) >> 1 | (more & 0x10000u) >> 4) & 8191u;
+    p.mag[2] = v.tail8[blob_at<uint16_t>(v, kUnrankTailBase, key) + r];
+    // x_i = 1 + 2 c_i modulo 4: 1 + 2j is of the wrong residue, and so negated, where j's parity differs from c_i
+#pragma unroll
+    for (int w = 0; w < 3; w++) p.neg[w] = (p.mag[w] & 0x11111111u) ^ spread8(cw >> (8 * w));
+}
+
+// Deals the low bits of `bits` to the nibbles of `word` that are not zero (two-bit values), in order; drops them from
+// `bits`.
+LLVQ_HD uint32_t deal_signs(const UnrankView &v, uint32_t word, uint32_t &bits) {
+    const uint32_t mask = gather8((word | word >> 1) & 0x11111111u);
+    const int n = popcount32(mask);
+    const uint32_t dealt = blob_at<uint32_t>(v, kUnrankDeposit, blob_at<uint16_t>(v, kUnrankDepositAt, mask) + (bits & ((1u << n) - 1u)));
+    bits >>= n;
+    return dealt;
+}
+
+// The low nibbles of `word`, as many as `mask` has bits, moved to the mask's places.
+LLVQ_HD uint32_t to_places(const UnrankView &v, uint32_t mask, uint32_t word) {
+    struct alignas(16) Moves { uint32_t m0, m1, m2, all; };
+    const Moves m = blob_at<Moves>(v, kUnrankMerge, mask);
+    word = (word & ~m.m0) | ((word << 16) & m.m0);
+    word = (word & ~m.m1) | ((word << 8) & m.m1);
+    word = (word & ~m.m2) | ((word << 4) & m.m2);
+    return word & m.all;
+}
+
+// quotient and remainder of r / d for r < 2^42, quotient < 2^21, d < 2^24, given 1 / d: the float estimate is off by one at
+// most, and the remainder settles it
+LLVQ_HD uint32_t divide(uint64_t r, uint32_t d, float inv, uint32_t &rem) {
+    uint32_t q = (uint32_t)(u64_to_float(r) * inv);
+    int m = (int)((uint32_t)r - q * d);
+    if (m < 0) { m += (int)d; q--; }
+    if (m >= (int)d) { m -= (int)d; q++; }
+    rem = (uint32_t)m;
+    return q;
+}
+
+LLVQ_HD void unrank_even(const UnrankView &v, const UnrankDesc &d, uint64_t r, Point &p) {
+    const uint32_t w = (d.flags >> 1) & 31u, sign_bits = (d.flags >> 6) & 31u, nz_b = (d.flags >> 11) & 15u;
+    const uint32_t sigma = (uint32_t)r & ((1u << sign_bits) - 1u);
+    uint32_t rank_a, rank_b;
+    const uint32_t cw = blob_at<uint32_t>(v, kUnrankGolayWt, d.golay + divide(divide(r >> sign_bits, d.perm_b, d.inv_b, rank_b), d.perm_a, d.inv_a, rank_a));
+    // signs of the support in order: the free ones, then the one that makes sum |x| / 4 + the number of negative support
+    // coordinates even (an off-support sign does not matter: it changes the sum by a multiple of 8)
+    uint32_t on = sigma >> nz_b, off = sigma & ((1u << nz_b) - 1u);
+    on |= w ? (((d.flags >> 15) ^ (uint32_t)popcount32(on)) & 1u) << (w - 1u) : 0u;
+    if (w == 0) {
+        // all 24 values off the support: the first twelve one by one, the others from the list
+        uint32_t T = d.perm_b, n = d.b;
+        uint64_t words = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll 1
+#endif
+        for (int i = 0; i < 12; i++) {
+            const UnrankStep e = blob_at<UnrankStep>(v, kUnrankSteps, 24 - i);
+            uint32_t sh = 0, s = portion(T, n & 255u, e);
+            while (rank_b >= s && sh < 24u) {
+                rank_b -= s;
+                sh += 8;
+                s = portion(T, (n >> sh) & 255u, e);
+            }
+            n -= 1u << sh;
+            T = s;
+            words |= (uint64_t)(sh >> 3) << (4 * i);
+        }
+        const uint32_t rest = v.tab_b[blob_at<uint32_t>(v, kUnrankRest12, ((n >> 8) & 15u) | ((n >> 16) & 3u) << 4 | ((n >> 24) & 1u) << 6) + rank_b];
+        const uint32_t k[3] = {(uint32_t)words, (uint32_t)(words >> 32) | spread_pairs(rest) << 16, spread_pairs(rest >> 8)};
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            p.mag[j] = 2u * k[j];
+            p.neg[j] = deal_signs(v, k[j], off);
+        }
+        return;
+    }
+    const uint64_t a = v.tab_a[d.a + rank_a];
+    if (w == 24) {
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            p.mag[j] = 2u * spread_pairs((uint32_t)(a >> (16 * j))) + 0x11111111u;
+            p.neg[j] = spread8(on >> (8 * j));
+        }
+        return;
+    }
+    // the two sequences, a nibble a value: k in bits 0, 1, the sign in bit 2
+    uint64_t in, out;
+    {
+        const uint32_t lo = spread_pairs((uint32_t)a) | spread8(on) << 2, hi = spread_pairs((uint32_t)a >> 16) | spread8(on >> 8) << 2;
+        in = (uint64_t)hi << 32 | lo;
+        const uint32_t b = v.tab_b[d.b + rank_b];
+        const uint32_t blo = spread_pairs(b), bhi = spread_pairs(b >> 16);
+        const uint32_t slo = deal_signs(v, blo, off), shi = deal_signs(v, bhi, off);
+        out = (uint64_t)(bhi | shi << 2) << 32 | (blo | slo << 2);
+    }
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        const uint32_t mask = (cw >> (8 * j)) & 255u, n = (uint32_t)popcount32(mask);
+        const uint32_t m = to_places(v, mask, (uint32_t)in) | to_places(v, mask ^ 255u, (uint32_t)out);
+        in >>= 4u * n;
+        out >>= 32u - 4u * n;
+        p.neg[j] = (m >> 2) & 0x11111111u;
+        p.mag[j] = 2u * (m & 0x33333333u) + spread8(mask);
+    }
+}
+
+// codes u of eight coordinates from their magnitudes and signs
+LLVQ_HD uint32_t point_codes(const Point &p, int w, bool odd) {
+    return ((p.mag[w] | 0x88888888u) ^ (p.neg[w] * 15u)) + (odd ? 0u : p.neg[w]);
+}
+
+}  // namespace llvq

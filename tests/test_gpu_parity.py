@@ -88,6 +88,27 @@ def test_expand_whole_first_shell_class_edges_and_bad_codes(B, ctx, oracle, layo
     assert e.value.code == -6
 
 
+@pytest.mark.parametrize("layout,rows,nb", [(0, 33 * 32 - 5, 7), (2, 33 * 32 - 5, 7), (3, 33 * 32 - 5, 7), (1, 33 * 32 - 5, 7), (0, 7, 3), (3, 32, 4),
+                                            (0, 5200 * 32, 3)])
+def test_expand_every_class_mixed(B, ctx, oracle, layout, rows, nb):
+    """Random points of all 301 classes side by side (every table of the un-ranking, both types in one tile), pieces of every
+    kind, and (the last case) more pieces than the grid has warps."""
+    rng = np.random.default_rng(rows + nb)
+    info = [oracle.class_info(c) for c in range(301)]
+    lo, size = np.array([i["base"] for i in info], np.uint64), np.array([i["size"] for i in info], np.uint64)
+    c = rng.permutation(np.arange(rows * nb) % 301)
+    codes = lo[c] + rng.integers(0, 1 << 62, c.size, dtype=np.uint64) % size[c] | (rng.integers(0, 2, c.size, dtype=np.uint64) << np.uint64(47))
+    d = torch.from_numpy(codes.view(np.int64)).cuda()
+    if layout == 3:
+        want, n = oracle.pack_planes10x(codes, rows, nb)
+        assert B.overlay_count(ctx, d, rows, nb) == n
+        got = B.expand(ctx, layout, d, rows, nb, out=torch.empty(B.overlay_bytes(rows, nb * 24, n), dtype=torch.uint8, device="cuda"))
+    else:
+        want = {0: oracle.pack_planes, 1: oracle.pack_onehot, 2: oracle.pack_planes13}[layout](codes, rows, nb)
+        got = B.expand(ctx, layout, d, rows, nb)
+    assert np.array_equal(got.cpu().numpy(), want)
+
+
 @pytest.mark.parametrize("layout", [0, 1])
 @pytest.mark.parametrize("rows,k", [(40, 24 * 7), (257, 24 * 21), (3072, 3072)])
 def test_decode_bit_exact(B, ctx, oracle, layout, rows, k):
