@@ -1371,9 +1371,23 @@ __global__ void __launch_bounds__(256) decode_i8_kernel(int layout, const uint8_
     class_ids[row * nb + b] = (uint16_t)cls;
 }
 
-__global__ void __launch_bounds__(256) dequant_kernel(int layout, const uint8_t *__restrict__ buf, const __half *__restrict__ row_scale,
-                                                       float g0, float g1, __half *__restrict__ W, int64_t rows, int64_t nb,
-                                                       const uint32_t *cls_parity, const uint8_t *cls_dist, const float *cls_scale) {
+// Decoded weights of one block: fp16(scale * x_i), 48 bytes (16-byte aligned) from dst on.
+__device__ __forceinline__ void store_block_fp16(__half *dst, float s, const int x[24]) {
+#pragma unroll
+    for (int v = 0; v < 3; v++) {
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const __half2 h = __floats2half2_rn(s * (float)x[8 * v + 2 * i], s * (float)x[8 * v + 2 * i + 1]);
+            w[i] = *reinterpret_cast<const uint32_t *>(&h);
+        }
+        *reinterpret_cast<uint4 *>(dst + 8 * v) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+__global__ void __launch_bounds__(256) dequant_onehot_kernel(const uint8_t *__restrict__ buf, const __half *__restrict__ row_scale,
+                                                              float g0, float g1, __half *__restrict__ W, int64_t rows, int64_t nb,
+                                                              const uint8_t *cls_dist, const float *cls_scale) {
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = (int)(gid & 31);
     const int64_t cell_id = gid >> 5, groups = (rows + kRowsPerGroup - 1) / kRowsPerGroup;
@@ -1381,11 +1395,86 @@ __global__ void __launch_bounds__(256) dequant_kernel(int layout, const uint8_t 
     const int64_t rg = cell_id / nb, b = cell_id % nb, row = rg * kRowsPerGroup + lane;
     if (row >= rows) return;
     int cls, gain, x[24];
-    record_coords(layout, buf, rows, nb, rg, b, lane, cls_parity, cls_dist, cls, gain, x);
+    record_coords(LLVQ_ONEHOT, buf, rows, nb, rg, b, lane, nullptr, cls_dist, cls, gain, x);
     // r * gain / (4 sqrt m): cls_scale carries 2^21 / (4 sqrt m)
-    const float s = __half2float(row_scale[row]) * ((gain ? g1 : g0) * (cls_scale[cls] * (1.0f / 2097152.0f)));
-    __half *dst = W + (row * nb + b) * 24;
-    for (int i = 0; i < 24; i++) dst[i] = __float2half_rn(s * (float)x[i]);
+    store_block_fp16(W + (row * nb + b) * 24, __half2float(row_scale[row]) * ((gain ? g1 : g0) * (cls_scale[cls] * (1.0f / 2097152.0f))), x);
+}
+
+// 14-byte layout -> FP16.  Bound: HBM, nearly all of it the weights written (48 bytes a block, 14 read).  A warp takes a tile;
+// lane 4g+t's words hold four consecutive coordinates of a row at each of the positions 4t, 16+4t, 32+4t of a half-step,
+// so it stores them as they are decoded, eight bytes at a time, the four lanes of a quad side by side: every store fills
+// whole 32-byte sectors of eight rows (where a row begins on one) and needs no exchange between lanes.  A block of
+// 24 coordinates a lane, stored two bytes at a time, took 490 us for 4096 x 12288 (265 GB/s), its stores throttled; this 25 us
+// (5150 GB/s of the 62 bytes a block, 0.79 of a copy).
+constexpr int kDequantWarps = 8;
+__global__ void __launch_bounds__(kDequantWarps * 32) dequant_planes_kernel(const uint8_t *__restrict__ buf, const __half *__restrict__ row_scale,
+                                                                            float g0, float g1, __half *__restrict__ W, int64_t rows, int64_t nb,
+                                                                            uint32_t total_units, const uint32_t *cls_parity, const uint8_t *cls_dist,
+                                                                            const float2 *__restrict__ cls_block) {
+    // (class | gain << 9) -> {gain / (4 sqrt m), (parity - 16) / 2 - 2^22}
+    __shared__ float2 tab[2 * kClassSlots];
+    for (int c = threadIdx.x; c < kClassSlots; c += blockDim.x) {
+        const float2 k = __ldg(cls_block + c);
+        const float offset = 0.5f * (float)(__float_as_int(k.y) - 8388608);
+        tab[c] = make_float2(g0 * k.x, offset);
+        tab[c + kClassSlots] = make_float2(g1 * k.x, offset);
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const uint32_t tiles = (uint32_t)(nb / kTileCells), left = (uint32_t)(nb % kTileCells), units = tiles + (left ? 1 : 0);
+    for (uint32_t unit = blockIdx.x * kDequantWarps + (threadIdx.x >> 5); unit < total_units; unit += gridDim.x * kDequantWarps) {
+        const uint32_t rg = unit / units, u = unit % units;
+        const int64_t row0 = (int64_t)rg * kRowsPerGroup;
+        if (u == tiles) {
+            // the nb mod 4 last blocks: a lane a row, a block at a time
+            const int64_t row = row0 + lane;
+            if (row >= rows) continue;
+            const float r = __half2float(row_scale[row]);
+            for (int64_t b = (int64_t)tiles * kTileCells; b < nb; b++) {
+                int cls, gain, x[24];
+                record_coords(LLVQ_PLANES, buf, rows, nb, rg, b, lane, cls_parity, cls_dist, cls, gain, x);
+                store_block_fp16(W + (row * nb + b) * 24, r * tab[cls | gain << 9].x, x);
+            }
+            continue;
+        }
+        const uint8_t *tile = buf + (size_t)rg * ((size_t)nb * kCellBytes) + (size_t)u * kTileBytes;
+        const uint4 w0 = __ldcs(reinterpret_cast<const uint4 *>(tile + 16 * lane)), w1 = __ldcs(reinterpret_cast<const uint4 *>(tile + 512 + 16 * lane));
+        const uint4 w2 = __ldcs(reinterpret_cast<const uint4 *>(tile + 1024 + 16 * lane));
+        const uint4 ha = __ldcs(reinterpret_cast<const uint4 *>(tile + 1536 + 32 * g)), hb = __ldcs(reinterpret_cast<const uint4 *>(tile + 1552 + 32 * g));
+        const uint32_t words[12] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w, w2.x, w2.y, w2.z, w2.w};
+        const uint32_t head[2][4] = {{ha.x, ha.y, ha.z, ha.w}, {hb.x, hb.y, hb.z, hb.w}};      // [slot][half-step]
+#pragma unroll
+        for (int m = 0; m < 2; m++) {
+#pragma unroll
+            for (int e = 0; e < 2; e++) {
+                const int64_t row = row0 + 16 * m + 8 * e + g;
+                if (row >= rows) continue;
+                const float r = __half2float(row_scale[row]);
+                // coordinate 4t of the tile's first block of the row
+                __half *dst = W + (row * nb + (int64_t)u * kTileCells) * 24 + 4 * t;
+#pragma unroll
+                for (int s = 0; s < 2; s++) {
+                    const int h = 2 * s + m;
+                    const float2 k0 = tab[(head[0][h] >> (16 * e)) & 1023u], k1 = tab[(head[1][h] >> (16 * e)) & 1023u];
+                    const float s0 = 2.f * (r * k0.x), s1 = 2.f * (r * k1.x);
+                    const uint32_t own = words[3 * h + e], shared = words[3 * h + 2];
+                    // four codes, doubled, a byte each, to four halves: 2^22 + u by its bits, then x / 2 = u + (parity - 16) / 2, exactly,
+                    // and one rounding of the product with twice the scale
+                    auto put = [&](int at, uint32_t codes, float scale, float offset) {
+                        float f[4];
+#pragma unroll
+                        for (int i = 0; i < 4; i++) f[i] = scale * (__uint_as_float(__byte_perm(codes, 0x4a800000u, 0x7650 + i)) + offset);
+                        const __half2 lo = __floats2half2_rn(f[0], f[1]), hi = __floats2half2_rn(f[2], f[3]);
+                        __stcs(reinterpret_cast<uint2 *>(dst + 48 * s + at),
+                               make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi)));
+                    };
+                    put(0, (own << 1) & 0x1e1e1e1eu, s0, k0.y);
+                    put(16, (own >> 3) & 0x1e1e1e1eu, t < 2 ? s0 : s1, t < 2 ? k0.y : k1.y);
+                    put(32, (e ? shared >> 3 : shared << 1) & 0x1e1e1e1eu, s1, k1.y);
+                }
+            }
+        }
+    }
 }
 
 }  // namespace
@@ -1530,9 +1619,15 @@ cudaError_t launch_gemv_fp16(const __half *W, const __half *x, float *y, int64_t
 cudaError_t launch_dequant(const llvq_ctx *ctx, int layout, const uint8_t *buf, const __half *row_scale, float g0, float g1,
                            __half *W, int64_t rows, int64_t nb, cudaStream_t s) {
     const int64_t groups = (rows + kRowsPerGroup - 1) / kRowsPerGroup;
-    const int64_t blocks = (groups * nb * 32 + 255) / 256;
-    dequant_kernel<<<(unsigned)blocks, 256, 0, s>>>(layout, buf, row_scale, g0, g1, W, rows, nb, ctx->dev.cls_parity, ctx->dev.cls_dist,
-                                                   ctx->dev.cls_scale);
+    if (layout == LLVQ_ONEHOT) {
+        const int64_t blocks = (groups * nb * 32 + 255) / 256;
+        dequant_onehot_kernel<<<(unsigned)blocks, 256, 0, s>>>(buf, row_scale, g0, g1, W, rows, nb, ctx->dev.cls_dist, ctx->dev.cls_scale);
+        return cudaGetLastError();
+    }
+    const int64_t units = groups * (nb / kTileCells + (nb % kTileCells ? 1 : 0));
+    const int64_t blocks = (units + kDequantWarps - 1) / kDequantWarps, most = (int64_t)ctx->sm_count * 8;
+    dequant_planes_kernel<<<(unsigned)(blocks < most ? blocks : most), kDequantWarps * 32, 0, s>>>(buf, row_scale, g0, g1, W, rows, nb, (uint32_t)units, ctx->dev.cls_parity,
+                                                                                                  ctx->dev.cls_dist, ctx->dev.cls_block);
     return cudaGetLastError();
 }
 

@@ -200,6 +200,22 @@ def test_fp16_arm_and_dequant(B, ctx, oracle):
     assert (np.abs(y.cpu().numpy() - ref_y) <= 1e-5 * np.maximum(scale, 1e-30)).all()
 
 
+@pytest.mark.parametrize("layout,rows,nb", [(0, 1, 1), (0, 31, 4), (0, 33, 5), (0, 64, 6), (0, 95, 7), (0, 4100, 9), (1, 33, 5)])
+def test_dequant_pieces(B, ctx, rows, nb, layout):
+    """Tiles, every number of leftover blocks, rows that end inside a row group, rows that begin off a 32-byte sector: equal to
+    fp16(f32 scale * integer coordinate) formed from decode_i8, bit for bit."""
+    case = make_case(rows, 24 * nb, seed=rows + nb)
+    buf = B.expand(ctx, layout, case.d_codes, rows, nb)
+    W = B.dequant_fp16(ctx, layout, buf, case.d_scale, GAIN, rows, nb * 24)
+    coords, _ = B.decode_i8(ctx, layout, buf, rows, nb)
+    x = coords.float()
+    shell = (x * x).sum(2) / 16                                  # sum x^2 = 16 m
+    inv_norm = (1.0 / (4.0 * shell.double().sqrt())).float()
+    gain = torch.where((case.d_codes.view(rows, nb) >> 47) != 0, GAIN[1], GAIN[0]).float()
+    scale = case.d_scale.float()[:, None] * (gain * inv_norm)
+    assert torch.equal(W, (scale[:, :, None] * x).half().view(rows, nb * 24))
+
+
 def test_noweights_control_returns_zero(B, ctx):
     case = make_case(4096, 4096, seed=2)
     y = torch.full((case.rows,), float("nan"), dtype=torch.float32, device="cuda")
