@@ -1,14 +1,14 @@
-"""Thin ctypes binding of libllvq.so (declared in include/llvq.h): argument marshalling only.
+"""Thin binding of libllvq.so (declared in include/llvq.h): argument marshalling only.
 
 Every function has the name of the C entry point without its prefix and takes torch CUDA tensors
-where the C call takes device pointers.  Nothing is computed here; if the shared library is
-missing or a call fails, an exception is raised - there is no fallback path.
+where the C call takes device pointers.  The calls that launch work go through _native.so (csrc/llvq_torch.cpp), the
+queries through ctypes.  Nothing is computed here; if a shared library is missing or a call fails, an exception is
+raised - there is no fallback path.
 """
 from __future__ import annotations
 
 import ctypes
 import os
-from typing import Sequence
 
 import torch
 
@@ -20,6 +20,7 @@ MAX_GROUP = 8
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libllvq.so")
 _lib = None
+_native = None     # the extension module with the launching calls, once load() has bound it
 
 SYMBOLS = (
     "llvq_create", "llvq_destroy", "llvq_strerror", "llvq_status", "llvq_selftest_wait_limit", "llvq_set_pdl", "llvq_num_classes", "llvq_class_base", "llvq_layout_bytes",
@@ -47,11 +48,16 @@ class Rotation(ctypes.Structure):
 
 def load() -> ctypes.CDLL:
     """Loads libllvq.so from the package directory; raises if it has not been built."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(f"{LIB_PATH} is missing: build it with `python -m paper_2609_02652_b200.build` "
                                "(nvcc, sm_100a); there is no CPU fallback")
+        try:
+            from . import _native as native
+        except ImportError as e:
+            raise RuntimeError("_native.so cannot be loaded: build it with `python -m paper_2609_02652_b200.build` "
+                               f"(g++, the torch headers); there is no CPU fallback ({e})") from e
         L = ctypes.CDLL(LIB_PATH)
         vp, i64, ci, sz = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, ctypes.c_size_t
         L.llvq_create.argtypes = [ctypes.POINTER(vp), ci, sz]
@@ -87,7 +93,8 @@ def load() -> ctypes.CDLL:
         for name in SYMBOLS:
             if name not in ("llvq_destroy", "llvq_strerror", "llvq_class_base", "llvq_rotate_block"):
                 getattr(L, name).restype = ci
-        _lib = L
+        native.bind(LlvqError, {name: ctypes.cast(getattr(L, name), vp).value for name in SYMBOLS})
+        _lib, _native = L, native
     return _lib
 
 
@@ -102,12 +109,15 @@ def _dev(t: torch.Tensor, dtype, what: str) -> int:
     return t.data_ptr()
 
 
+def _launch():
+    """The extension module with the launching calls."""
+    if _native is None:
+        load()
+    return _native
+
+
 def _stream(stream) -> int:
     return (stream if stream is not None else torch.cuda.current_stream()).cuda_stream
-
-
-def _gain(gain: Sequence[float]):
-    return (ctypes.c_float * 2)(float(gain[0]), float(gain[1]))
 
 
 class Context:
@@ -117,6 +127,7 @@ class Context:
         self._p = ctypes.c_void_p()
         _check(load().llvq_create(ctypes.byref(self._p), int(device), int(scratch_bytes)), "llvq_create")
         self.device = int(device)
+        self.handle = self._p.value          # the same as an integer; 0 once destroyed
 
     @property
     def ptr(self) -> ctypes.c_void_p:
@@ -128,6 +139,7 @@ class Context:
         if self._p:
             load().llvq_destroy(self._p)
             self._p = ctypes.c_void_p()
+            self.handle = 0
 
     def __del__(self):
         try:
@@ -183,46 +195,25 @@ def overlay_bytes(rows: int, k_padded: int, exceptions: int) -> int:
 
 def overlay_count(ctx: Context, codes: torch.Tensor, rows: int, nb: int, stream=None) -> int:
     """Blocks of the matrix that PLANES10X keeps in its exception table (synchronises the stream)."""
-    n = ctypes.c_uint64()
-    _check(load().llvq_overlay_count(ctx.ptr, _dev(codes, torch.int64, "codes"), int(rows), int(nb), ctypes.byref(n), _stream(stream)),
-           "llvq_overlay_count")
-    return int(n.value)
+    return _launch().overlay_count(ctx, codes, rows, nb, stream)
 
 
 def expand(ctx: Context, layout: int, codes: torch.Tensor, rows: int, nb: int, out: torch.Tensor | None = None,
            bad_count: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     """codes: int64 CUDA tensor of rows*nb code words -> uint8 layout buffer (PLANES10X: sized by llvq_layout_bytes,
     i.e. with room for one exception in 32 blocks, unless `out` is given)."""
-    if out is None:
-        out = torch.empty(layout_bytes(layout, rows, nb * 24), dtype=torch.uint8, device=codes.device)
-    bc = _dev(bad_count, torch.int32, "bad_count") if bad_count is not None else None
-    _check(load().llvq_expand(ctx.ptr, int(layout), _dev(codes, torch.int64, "codes"), int(rows), int(nb),
-                              _dev(out, torch.uint8, "out"), out.numel(), bc, _stream(stream)), "llvq_expand")
-    return out
+    return _launch().expand(ctx, layout, codes, rows, nb, out, bad_count, stream)
 
 
 def gemv(ctx: Context, layout: int, layout_buf: torch.Tensor, row_scale: torch.Tensor, gain, x: torch.Tensor,
          rows: int, k_padded: int, y: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-    if y is None:
-        y = torch.empty(rows, dtype=torch.float32, device=x.device)
-    _check(load().llvq_gemv(ctx.ptr, int(layout), _dev(layout_buf, torch.uint8, "layout_buf"),
-                            _dev(row_scale, torch.float16, "row_scale"), _gain(gain), _dev(x, torch.float16, "x"),
-                            _dev(y, torch.float32, "y"), int(rows), int(k_padded), _stream(stream)), "llvq_gemv")
-    return y
+    return _launch().gemv(ctx, layout, layout_buf, row_scale, gain, x, rows, k_padded, y, stream)
 
 
 def gemv_batch(ctx: Context, layout_buf: torch.Tensor, row_scale: torch.Tensor, gain, x: torch.Tensor, rows: int,
                k_padded: int, y: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     """llvq_gemv_batch: x is fp16 [batch, k_padded] (contiguous), the result f32 [batch, rows]."""
-    batch = int(x.shape[0])
-    if x.dim() != 2 or int(x.shape[1]) != int(k_padded) or not x.is_contiguous():
-        raise ValueError("x must be a contiguous [batch, k_padded] tensor")
-    if y is None:
-        y = torch.empty((batch, rows), dtype=torch.float32, device=x.device)
-    _check(load().llvq_gemv_batch(ctx.ptr, _dev(layout_buf, torch.uint8, "layout_buf"), _dev(row_scale, torch.float16, "row_scale"),
-                                  _gain(gain), _dev(x, torch.float16, "x"), _dev(y, torch.float32, "y"), int(rows), int(k_padded),
-                                  batch, _stream(stream)), "llvq_gemv_batch")
-    return y
+    return _launch().gemv_batch(ctx, layout_buf, row_scale, gain, x, rows, k_padded, y, stream)
 
 
 def gemv_plan(sm_count: int, rows, k_padded: int, batch: int = 1) -> dict:
@@ -240,10 +231,7 @@ def gemv_static(layout_buf: torch.Tensor, row_scale: torch.Tensor, gain, x: torc
                 y: torch.Tensor, stream=None) -> torch.Tensor:
     """llvq_gemv_static: no context and no allocation inside the library; the caller supplies y.  Runs on the
     current CUDA device; at most 65536 rows; calls must not overlap on the GPU (they share built-in scratch)."""
-    _check(load().llvq_gemv_static(_dev(layout_buf, torch.uint8, "layout_buf"), _dev(row_scale, torch.float16, "row_scale"),
-                                   _gain(gain), _dev(x, torch.float16, "x"), _dev(y, torch.float32, "y"), int(rows),
-                                   int(k_padded), _stream(stream)), "llvq_gemv_static")
-    return y
+    return _launch().gemv_static(layout_buf, row_scale, gain, x, rows, k_padded, y, stream)
 
 
 def static_status(stream=None) -> None:
@@ -272,25 +260,18 @@ def make_problems(problems) -> ctypes.Array:
 def gemv_grouped(ctx: Context, layout: int, problems, x: torch.Tensor, k_padded: int, stream=None) -> None:
     """problems: a host array from make_problems, or the sequence make_problems takes."""
     arr = problems if isinstance(problems, ctypes.Array) else make_problems(problems)
-    _check(load().llvq_gemv_grouped(ctx.ptr, int(layout), arr, len(arr), _dev(x, torch.float16, "x"), int(k_padded),
-                                    _stream(stream)), "llvq_gemv_grouped")
+    _launch().gemv_grouped(ctx, layout, arr, x, k_padded, stream)
 
 
 def gemv_rotated(ctx: Context, problems, x: torch.Tensor, k_padded: int, n: int, block: int = 0,
                  negate_bits: torch.Tensor | None = None, stream=None) -> None:
     """llvq_gemv_rotated: the grouped 14-byte-layout GEMV on rotate(x[:n]) (the rest of x passes through), one launch."""
     arr = problems if isinstance(problems, ctypes.Array) else make_problems(problems)
-    rot = Rotation(None if negate_bits is None else _dev(negate_bits, torch.int32, "negate_bits"), int(n), int(block))
-    _check(load().llvq_gemv_rotated(ctx.ptr, arr, len(arr), _dev(x, torch.float16, "x"), int(k_padded), ctypes.byref(rot),
-                                    _stream(stream)), "llvq_gemv_rotated")
+    _launch().gemv_rotated(ctx, arr, x, k_padded, n, block, negate_bits, stream)
 
 
 def gemv_fp16(W: torch.Tensor, x: torch.Tensor, rows: int, k: int, y: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-    if y is None:
-        y = torch.empty(rows, dtype=torch.float32, device=x.device)
-    _check(load().llvq_gemv_fp16(_dev(W, torch.float16, "W"), _dev(x, torch.float16, "x"), _dev(y, torch.float32, "y"),
-                                 int(rows), int(k), _stream(stream)), "llvq_gemv_fp16")
-    return y
+    return _launch().gemv_fp16(W, x, rows, k, y, stream)
 
 
 def rotate_block(n: int, block: int = 0) -> int:
@@ -301,32 +282,17 @@ def rotate_block(n: int, block: int = 0) -> int:
 def rotate(ctx: Context, x: torch.Tensor, block: int = 0, negate_bits: torch.Tensor | None = None,
            y: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     """llvq_rotate: block-diagonal Walsh-Hadamard rotation of the fp16 vector x; `negate_bits` int32 words, bit i = flip x_i."""
-    if y is None:
-        y = torch.empty_like(x)
-    _check(load().llvq_rotate(ctx.ptr, _dev(x, torch.float16, "x"), _dev(y, torch.float16, "y"),
-                              None if negate_bits is None else _dev(negate_bits, torch.int32, "negate_bits"),
-                              int(x.numel()), int(block), _stream(stream)), "llvq_rotate")
-    return y
+    return _launch().rotate(ctx, x, block, negate_bits, y, stream)
 
 
 def gemv_noweights(ctx: Context, row_scale: torch.Tensor, x: torch.Tensor, rows: int, k_padded: int,
                    y: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-    if y is None:
-        y = torch.empty(rows, dtype=torch.float32, device=x.device)
-    _check(load().llvq_gemv_noweights(ctx.ptr, _dev(row_scale, torch.float16, "row_scale"), _dev(x, torch.float16, "x"),
-                                      _dev(y, torch.float32, "y"), int(rows), int(k_padded), _stream(stream)),
-           "llvq_gemv_noweights")
-    return y
+    return _launch().gemv_noweights(ctx, row_scale, x, rows, k_padded, y, stream)
 
 
 def dequant_fp16(ctx: Context, layout: int, layout_buf: torch.Tensor, row_scale: torch.Tensor, gain, rows: int,
                  k_padded: int, W: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-    if W is None:
-        W = torch.empty((rows, k_padded), dtype=torch.float16, device=layout_buf.device)
-    _check(load().llvq_dequant_fp16(ctx.ptr, int(layout), _dev(layout_buf, torch.uint8, "layout_buf"),
-                                    _dev(row_scale, torch.float16, "row_scale"), _gain(gain), _dev(W, torch.float16, "W"),
-                                    int(rows), int(k_padded), _stream(stream)), "llvq_dequant_fp16")
-    return W
+    return _launch().dequant_fp16(ctx, layout, layout_buf, row_scale, gain, rows, k_padded, W, stream)
 
 
 def decode_i8(ctx: Context, layout: int, layout_buf: torch.Tensor, rows: int, nb: int, stream=None):

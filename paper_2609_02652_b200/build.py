@@ -1,39 +1,62 @@
-"""Builds the CUDA library in-tree: nvcc for sm_100a -> paper_2609_02652_b200/libllvq.so."""
+"""Builds the native code in-tree: nvcc for sm_100a -> libllvq.so, and the host compiler -> _native.so (the torch
+binding of its calls)."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
+HEADER = os.path.join(HERE, "..", "include", "llvq.h")
 SOURCES = ["llvq_api.cu", "llvq_expand.cu", "llvq_gemv.cu", "llvq_rotate.cu", "llvq_tables.cpp", "llvq_unrank.cpp"]
 LIB = os.path.join(HERE, "libllvq.so")
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared", "-cudart", "shared"]
+BINDING_SOURCE = "llvq_torch.cpp"
+BINDING = os.path.join(HERE, "_native.so")
 
 
-def _nvcc() -> str:
-    exe = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+def _tool(name: str, fallback: str) -> str:
+    exe = shutil.which(name) or fallback
     if not os.path.exists(exe):
-        raise RuntimeError("nvcc not found: the CUDA library cannot be built")
+        raise RuntimeError(f"{name} not found: the native code cannot be built")
     return exe
 
 
-def _stale() -> bool:
-    if not os.path.exists(LIB):
+def _stale(target: str, deps) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "llvq.h")]
+    t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _run(cmd, target: str) -> None:
+    tmp = target + f".tmp{os.getpid()}"
+    subprocess.check_call([*cmd, "-o", tmp])
+    os.replace(tmp, target)
+
+
+def _build_binding() -> None:
+    import torch
+
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.join(os.path.dirname(os.path.dirname(_tool("nvcc", "/usr/local/cuda/bin/nvcc"))), "include")
+    include = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), cuda,
+               sysconfig.get_paths()["include"]]
+    _run([_tool("g++", "/usr/bin/g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+          *["-isystem" + d for d in include], os.path.join(CSRC, BINDING_SOURCE), "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda",
+          "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python"], BINDING)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    if force or _stale():
-        tmp = LIB + f".tmp{os.getpid()}"
-        cmd = [_nvcc(), *NVCC_FLAGS, *(["-Xptxas", "-v"] if verbose else []), "-o", tmp, *[os.path.join(CSRC, s) for s in SOURCES]]
-        subprocess.check_call(cmd)
-        os.replace(tmp, LIB)
+    own = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != BINDING_SOURCE] + [HEADER]
+    if force or _stale(LIB, own):
+        _run([_tool("nvcc", "/usr/local/cuda/bin/nvcc"), *NVCC_FLAGS, *(["-Xptxas", "-v"] if verbose else []),
+              *[os.path.join(CSRC, s) for s in SOURCES]], LIB)
+    if force or _stale(BINDING, [os.path.join(CSRC, BINDING_SOURCE), HEADER]):
+        _build_binding()
     return LIB
 
 

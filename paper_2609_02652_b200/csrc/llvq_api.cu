@@ -11,13 +11,13 @@ using namespace llvq;
 namespace {
 
 struct DeviceGuard {
-    int prev = -1;
+    int prev = -1, dev;
     bool ok = true;
-    explicit DeviceGuard(int dev) {
+    explicit DeviceGuard(int device) : dev(device) {
         if (cudaGetDevice(&prev) != cudaSuccess) { ok = false; return; }
         if (prev != dev && cudaSetDevice(dev) != cudaSuccess) ok = false;
     }
-    ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
+    ~DeviceGuard() { if (prev >= 0 && prev != dev) cudaSetDevice(prev); }
 };
 
 inline bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
@@ -316,8 +316,6 @@ static int run_gemv(llvq_ctx *ctx, int layout, const llvq_problem *problems, int
     p.cls_value = ctx->dev.cls_value;
     p.cls_block = ctx->dev.cls_block;
     p.lane_table = ctx->dev.lane_table;
-    std::memcpy(p.cls_shell_nibbles, ctx->host.cls_shell_nibbles, sizeof p.cls_shell_nibbles);
-    std::memcpy(p.cls_odd_bits, ctx->host.cls_odd_bits, sizeof p.cls_odd_bits);
     std::memcpy(p.shell_inv_norm, ctx->host.shell_inv_norm, sizeof p.shell_inv_norm);
     p.error = ctx->error;
     if (rot) {

@@ -453,10 +453,6 @@ __host__ __device__ inline int fast_div(int n, const FastDiv &f, int d) {
     return n / d;
 #endif
 }
-__host__ __device__ inline int panel_of_unit(const GemvParams &p, int f) {
-    const int j = fast_div(f, p.div_panel_units, p.total_groups * p.panel);
-    return j < p.npanels ? j : p.npanels - 1;
-}
 // steps over n units of the current row group's stretch; true if the row group changed
 __device__ __forceinline__ bool advance(const GemvParams &p, Cursor &c, int n) {
     c.col += n;
@@ -534,7 +530,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
     // the CTA's first unit (the plan names it) or, seldom, in a later one.
     Cursor cc;
     {
-        int panel = me.panel, first = panel * h_panel, w = min(h_panel, h_units - first), r = u0 - me.panel_first;
+        // the CTA's first panel begins with its first block of x
+        int panel = fast_div(blk_lo / kTileCells, h_div_panel, h_panel), first = panel * h_panel, w = min(h_panel, h_units - first);
+        int r = u0 - panel * (h_groups * h_panel);
         while (r >= h_groups * w && panel < h_npanels - 1) {
             r -= h_groups * w;
             panel++;
@@ -1503,7 +1501,6 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
     const int want = (p.units + kPanelColumns / 2) / kPanelColumns > 1 ? (p.units + kPanelColumns / 2) / kPanelColumns : 1;
     p.panel = (p.units + want - 1) / want;
     p.npanels = (p.units + p.panel - 1) / p.panel;
-    p.div_panel_units = make_fastdiv((uint32_t)(p.total_groups * p.panel));
     p.div_panel = make_fastdiv((uint32_t)p.panel);
     p.div_last = make_fastdiv((uint32_t)(p.units - (p.npanels - 1) * p.panel));
     // Shares of the CTAs.  CTAs start in index order as multiprocessors come free, the first ones while the
@@ -1516,31 +1513,37 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
         if (lead > 0.6 * mean) lead = 0.6 * mean;
         const double skew = mean > 0 ? lead / mean : 0.0;
         double acc = 0.0;
+        const double step = g.grid > 1 ? 2.0 * skew / (g.grid - 1) : 0.0, top = g.grid > 1 ? 1.0 + skew : 1.0;
         p.cta[0].first = 0;
         for (int c = 0; c < g.grid; c++) {
-            const double w = g.grid > 1 ? 1.0 + skew * (1.0 - 2.0 * c / (g.grid - 1)) : 1.0;
-            acc += mean * w;
+            acc += mean * (top - step * c);
             int f = (int)(acc + 0.5);
             if (f < p.cta[c].first) f = p.cta[c].first;
             if (f > p.total_units) f = p.total_units;
             p.cta[c + 1].first = f;
         }
         p.cta[g.grid].first = p.total_units;
-        p.cta[g.grid].blk_lo = p.cta[g.grid].blk_hi = p.cta[g.grid].panel = 0;
-        p.cta[g.grid].panel_first = 0;
+        p.cta[g.grid].blk_lo = p.cta[g.grid].blk_hi = 0;
     }
-    // the stretch of x a CTA meets: the whole panels its units lie in (consecutive ones)
+    // the stretch of x a CTA meets: the whole panels its units lie in (consecutive ones); the CTAs' first units ascend, so
+    // the panel they lie in is stepped on from one to the next
     p.xblocks = 0;
     p.rot_span = 0;
+    const int64_t panel_units = (int64_t)p.total_groups * p.panel;
+    int panel = 0;
+    int64_t panel_end = panel_units;                   // the last panel has no end
+    auto step_to = [&](int unit) {
+        while (unit >= panel_end && panel < p.npanels - 1) { panel++; panel_end += panel_units; }
+    };
     for (int c = 0; c < g.grid; c++) {
         const int f0 = p.cta[c].first, f1 = p.cta[c + 1].first;
-        const int lo = panel_of_unit(p, f0) * p.panel * kTileCells;
-        int hi = (panel_of_unit(p, f1 - 1 > f0 ? f1 - 1 : f0) + 1) * p.panel * kTileCells;
+        step_to(f0);
+        const int lo = panel * p.panel * kTileCells;
+        if (f1 - 1 > f0) step_to(f1 - 1);
+        int hi = (panel + 1) * p.panel * kTileCells;
         if (hi > p.nb) hi = p.nb;
         p.cta[c].blk_lo = (uint16_t)lo;
         p.cta[c].blk_hi = (uint16_t)hi;
-        p.cta[c].panel = (uint16_t)panel_of_unit(p, f0);
-        p.cta[c].panel_first = p.cta[c].panel * (p.total_groups * p.panel);
         if (hi - lo > p.xblocks) p.xblocks = hi - lo;
         if (p.rot_log2 > 0) {
             // the whole rotation blocks that meet the CTA's blocks of x (the kernel computes the same)
@@ -1676,8 +1679,7 @@ struct StaticDevice {
     unsigned long long *accum = nullptr;
     float2 *cls_block = nullptr;
     uint4 *lane_table = nullptr;
-    uint32_t cls_shell_nibbles[64], cls_odd_bits[16];      // class constants (host copies, handed to every launch)
-    float shell_inv_norm[16];
+    float shell_inv_norm[16];      // a class constant (a host copy, handed to every launch)
     int *error = nullptr;
     int sm_count = 0, max_smem_optin = 0;
 };
@@ -1691,8 +1693,6 @@ int static_setup(int device, StaticDevice &d) {
     if (cudaGetSymbolAddress((void **)&d.error, g_static_error) != cudaSuccess) return LLVQ_ECUDA;
     llvq::HostTables host;                                   // host memory only
     if (!llvq::build_tables(host)) return LLVQ_EINVAL;
-    memcpy(d.cls_shell_nibbles, host.cls_shell_nibbles, sizeof d.cls_shell_nibbles);
-    memcpy(d.cls_odd_bits, host.cls_odd_bits, sizeof d.cls_odd_bits);
     memcpy(d.shell_inv_norm, host.shell_inv_norm, sizeof d.shell_inv_norm);
     uint32_t lanes[32][4];
     llvq::gemv_lane_table(lanes);
@@ -1762,8 +1762,6 @@ extern "C" int llvq_gemv_static(const void *layout_buf, const void *row_scale, c
     p.total_groups = (int)groups;
     p.total_units = (int)(groups * p.units);
     p.accum = d.accum;
-    memcpy(p.cls_shell_nibbles, d.cls_shell_nibbles, sizeof p.cls_shell_nibbles);
-    memcpy(p.cls_odd_bits, d.cls_odd_bits, sizeof p.cls_odd_bits);
     memcpy(p.shell_inv_norm, d.shell_inv_norm, sizeof p.shell_inv_norm);
     p.error = d.error;
     p.cls_block = d.cls_block;

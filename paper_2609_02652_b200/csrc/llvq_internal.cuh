@@ -70,13 +70,11 @@ struct GemvProblemDev {
     const uint4 *exc_table;      // 10-byte layout: the exact records the short records leave out
 };
 
-// A CTA's share of a launch, planned on the host: its first unit, the panel that unit lies in and the panel's first
-// unit, and the blocks of x [blk_lo, blk_hi) its units touch (the whole panels its range of units meets).
+// A CTA's share of a launch, planned on the host: its first unit, and the blocks of x [blk_lo, blk_hi) its units touch
+// (the whole panels its range of units meets).  Eight bytes, because they are parameters of every launch.
 struct CtaShare {
     int first;
-    int panel_first;
     uint16_t blk_lo, blk_hi;
-    uint16_t panel, pad;
 };
 
 struct GemvParams {
@@ -91,7 +89,7 @@ struct GemvParams {
     int total_units;       // total_groups * units
     int units_base, units_rem;   // total_units divided by the warps of the grid (set by gemv_plan; the one-hot arm's order)
     int panel, npanels;          // unit columns a panel, panels (set by gemv_plan; the 14-byte layout's order of work)
-    FastDiv div_panel_units, div_panel, div_last;   // by total_groups * panel, by panel, by the last panel's width
+    FastDiv div_panel, div_last; // by panel, by the last panel's width
     int xblocks;                 // most blocks of x any CTA needs (set by gemv_plan)
     uint32_t group_bytes;        // bytes of a row group's records (set by gemv_plan)
     CtaShare cta[kMaxGridCtas + 1];    // the share of every CTA of the grid; [grid].first is the total (set by gemv_plan)
@@ -101,10 +99,6 @@ struct GemvParams {
     const float *cls_value;
     const float2 *cls_block;     // 512 x {1 / (4 sqrt m), parity - 16 as an integer's bits}; zeros for an unused class slot
     const uint4 *lane_table;     // 32 x this lane's offsets of its operand words in the x records of a half-step
-    // the class constants the 14-byte GEMV needs, in the parameters themselves (no load from global memory
-    // stands between a CTA's start and its block-constant table)
-    uint32_t cls_shell_nibbles[64];   // nibble c & 7 of word c >> 3: shell of class c, 0 if unused
-    uint32_t cls_odd_bits[16];        // bit c & 31 of word c >> 5: odd type
     float shell_inv_norm[16];         // [m] = 1 / (4 sqrt m)
     int *error;               // set when a bounded wait ran out
     // rotation of x inside the GEMV (llvq_gemv_rotated); rot_log2 = 0 means none
