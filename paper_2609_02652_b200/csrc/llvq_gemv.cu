@@ -37,6 +37,7 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "llvq_internal.cuh"
 #include "llvq_rotate.cuh"
@@ -388,13 +389,86 @@ __device__ __forceinline__ void contract_half(const HalfA &h, const StepX &sx, f
     // sum_i x_i X_i = sum_i u_i (2 X_i) + (parity - 16) sum_i X_i, limb pair by limb pair, in integers
     const int e0 = __float_as_int(h.k0.y) * sx.xsum + (d[0] + 256 * d[1]);
     const int e1 = __float_as_int(h.k1.y) * sx.xsum + (d[2] + 256 * d[3]);
-    if (FIRST) { r0 = (float)e0 * h.k0.x; r1 = (float)e1 * h.k1.x; }
+    if (FIRST) { r0 = __fmul_rn((float)e0, h.k0.x); r1 = __fmul_rn((float)e1, h.k1.x); }
     else { r0 = fmaf((float)e0, h.k0.x, r0); r1 = fmaf((float)e1, h.k1.x, r1); }
 }
 template <bool FIRST>
 __device__ __forceinline__ void half_step(uint32_t wa, uint32_t wb, uint32_t wc, uint32_t hw, const StepX &sx, uint32_t tq,
                                           float &r0, float &r1) {
     contract_half<FIRST>(decode_half(wa, wb, wc, hw, tq), sx, r0, r1);
+}
+
+// ---- several activation vectors.  Two vectors share the eight columns of the contraction - column g = 4 (vector) + limb -
+// and a block slot has an instruction sequence of its own: positions 0..23 of the half-step for slot 0, 24..47 for slot 1,
+// the other slot's positions zero in B.  Against one vector with block-diagonal B that is three instructions instead
+// of four for two vectors and two slots, and a row's sum lies in two lanes instead of four, so half the exchanges.
+// The price is that a lane looks up the headers of both slots; every vector shares that.  Bound: instruction issue.  Four
+// vectors, us a launch, before (a vector at a time, its atomic waited for before the next vector's) and after:
+// 1024 x 2560 6.8 and 5.5, 4096 x 4096 10.7 and 8.8, 8192 x 8192 19.4 and 17.8; two vectors on 8192 x 8192 12.5 and 11.9.
+struct PairA {
+    uint32_t a0, a1, a2, a3, c0, c1;
+    float2 k00, k01, k10, k11;                     // block constants: slot, then row g or g + 8
+};
+__device__ __forceinline__ PairA decode_pair(uint32_t wa, uint32_t wb, uint32_t wc, uint32_t hw0, uint32_t hw1, uint32_t tq) {
+    constexpr uint32_t kNib = 0x0f0f0f0fu;
+    PairA h;
+    h.a0 = wa & kNib; h.a1 = wb & kNib; h.a2 = (wa >> 4) & kNib; h.a3 = (wb >> 4) & kNib;
+    h.c0 = wc & kNib; h.c1 = (wc >> 4) & kNib;
+    h.k00 = lds_f2(and_or(hw0 << 3, 0x1ff8u, tq));
+    h.k01 = lds_f2(and_or(hw0 >> 13, 0x1ff8u, tq));
+    h.k10 = lds_f2(and_or(hw1 << 3, 0x1ff8u, tq));
+    h.k11 = lds_f2(and_or(hw1 >> 13, 0x1ff8u, tq));
+    return h;
+}
+// This lane's addresses in the x records of a block: its words of slot 0's operand (a0 and a1), of slot 1's (a2, and a0
+// again eight bytes on), and its vector's and limb pair's share of the activation sum.  The records of a block's vectors
+// lie side by side.
+struct PairAddr { uint32_t a0, a1, a2, xs; };
+__device__ __forceinline__ PairAddr pair_addr(int lane, uint32_t rec) {
+    const int g = lane >> 2, t = lane & 3;
+    const uint32_t v = rec + kXRecBytes * (g >> 2), plane = v + 24 * (g & 3), zero = v + 96;
+    PairAddr a;
+    a.a0 = plane + 4 * t;
+    a.a1 = t < 2 ? plane + 16 + 4 * t : zero;
+    a.a2 = t >= 2 ? plane + 4 * (t - 2) : zero;
+    a.xs = rec + kXRecBytes * (t >> 1) + 100 + 4 * (t & 1);
+    return a;
+}
+struct PairX { uint32_t b0, b1, b2, b3; int xs0, xs1; };
+// OFF: slot 0's block and the vector pair; OFF1: slot 1's
+template <int OFF, int OFF1>
+__device__ __forceinline__ PairX load_pair(const PairAddr &a) {
+    PairX x;
+    x.b0 = lds32_at<OFF>(a.a0); x.b1 = lds32_at<OFF>(a.a1);
+    x.b2 = lds32_at<OFF1>(a.a2); x.b3 = lds32_at<OFF1 + 8>(a.a0);
+    x.xs0 = (int)lds32_at<OFF>(a.xs); x.xs1 = (int)lds32_at<OFF1>(a.xs);
+    return x;
+}
+// s0, s1: this lane's shares of the sums of rows g and g + 8 over the blocks of slot 0 and of slot 1
+template <bool FIRST>
+__device__ __forceinline__ void contract_pair(const PairA &h, const PairX &x, float *s0, float *s1) {
+    int d[4], f[4];
+    mma_k32(d, h.a0, h.a1, h.a2, h.a3, x.b0, x.b1);
+    mma_k32(f, h.a0, h.a1, h.a2, h.a3, 0u, x.b2);
+    mma_k16(f, h.c0, h.c1, x.b3);
+    const int e00 = __float_as_int(h.k00.y) * x.xs0 + (d[0] + 256 * d[1]), e01 = __float_as_int(h.k01.y) * x.xs0 + (d[2] + 256 * d[3]);
+    const int e10 = __float_as_int(h.k10.y) * x.xs1 + (f[0] + 256 * f[1]), e11 = __float_as_int(h.k11.y) * x.xs1 + (f[2] + 256 * f[3]);
+    if (FIRST) {
+        // rounded products, as where a product goes through a shuffle: no sum below may take them into a multiply-add
+        s0[0] = __fmul_rn((float)e00, h.k00.x); s0[1] = __fmul_rn((float)e01, h.k01.x);
+        s1[0] = __fmul_rn((float)e10, h.k10.x); s1[1] = __fmul_rn((float)e11, h.k11.x);
+    } else {
+        s0[0] = fmaf((float)e00, h.k00.x, s0[0]); s0[1] = fmaf((float)e01, h.k01.x, s0[1]);
+        s1[0] = fmaf((float)e10, h.k10.x, s1[0]); s1[1] = fmaf((float)e11, h.k11.x, s1[1]);
+    }
+}
+// v[2m + e] = this lane's share (its limb pair) of row 16m + 8e + g -> even lanes get the sums of rows g, g + 8, odd lanes
+// those of rows 16 + g, 24 + g.  The additions are those of one vector alone (quad_sum), so the bits are too.
+__device__ __forceinline__ void pair_sum(const float (&v)[4], bool odd, float &r0, float &r1) {
+    const float own = odd ? 65536.f : 1.f, other = odd ? 1.f : 65536.f;
+    const float g0 = __shfl_xor_sync(0xffffffffu, odd ? v[0] : v[2], 1), g1 = __shfl_xor_sync(0xffffffffu, odd ? v[1] : v[3], 1);
+    r0 = fmaf(odd ? v[2] : v[0], own, g0 * other);     // products with powers of two are exact
+    r1 = fmaf(odd ? v[3] : v[1], own, g1 * other);
 }
 
 // x (fp16) -> records.  X_i = rint(x_i * 2^F) with F chosen from the largest |x| so that |X_i| < 2^29; the
@@ -466,8 +540,17 @@ __device__ __forceinline__ bool advance(const GemvParams &p, Cursor &c, int n) {
     c.col = c.panel * p.panel;
     return true;
 }
+// f(0), f(1), ... f(N - 1), the index a compile-time constant
+template <int N, int I = 0, typename F>
+__device__ __forceinline__ void each_pair(F &f) {
+    if constexpr (I < N) {
+        f(std::integral_constant<int, I>{});
+        each_pair<N, I + 1>(f);
+    }
+}
+
 // BATCH activation vectors share one pass over the records: the decode of a half-step and its block constants
-// are computed once, the contraction, the scaling and the reduction once a vector.  x is BATCH vectors of
+// are computed once, the contraction, the scaling and the reduction once a pair of vectors.  x is BATCH vectors of
 // 24 nb halves one after the other, y BATCH vectors of rows floats (p.prob[].y is vector 0's), the accumulators
 // BATCH sets of total_groups * 32.
 // ROTATE: x is rotated on its way into the records (llvq_gemv_rotated): every CTA rotates the Walsh-Hadamard
@@ -489,8 +572,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
     const uint32_t tab_pad = (0u - (smem_addr(smem) + kWarps * kSlots * kTileBytes)) & 8191u;
     float2 *tab = reinterpret_cast<float2 *>(smem + kWarps * kSlots * kTileBytes + tab_pad);
     unsigned char *xrec = smem + kWarps * kSlots * kTileBytes + tab_pad + p.nprob * 8192;
-    const uint32_t xrec_stride = ((p.xblocks * kXRecBytes + 127) / 128) * 128;     // a vector's records
-    uint64_t *bars = reinterpret_cast<uint64_t *>(xrec + BATCH * xrec_stride);
+    constexpr int kXBlock = BATCH * kXRecBytes;                                    // the vectors' records of a block lie side by side
+    uint64_t *bars = reinterpret_cast<uint64_t *>(xrec + ((p.xblocks * kXBlock + 127) / 128) * 128);
     uint32_t *warp_max = reinterpret_cast<uint32_t *>(bars + kWarps * kSlots);     // one slot a warp and vector
     long long *rot = reinterpret_cast<long long *>(warp_max + BATCH * kWarps);     // ROTATE: the exact sums of this CTA's blocks of x
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -524,7 +607,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
     const int u0 = cta_u0 + (warp * cta_n + kWarps - 1) / kWarps;
     const int n_units = cta_u0 + ((warp + 1) * cta_n + kWarps - 1) / kWarps - u0;
     const int blk_lo = me.blk_lo, blk_hi = me.blk_hi;
-    const uint32_t xs0 = smem_addr(xrec) - (uint32_t)blk_lo * kXRecBytes;     // address of block 0's record, were it there
+    const uint32_t xs0 = smem_addr(xrec) - (uint32_t)blk_lo * kXBlock;        // address of block 0's record, were it there
 
     // consume side and issue side walk the same sequence of units.  The warp's first unit lies in the panel of
     // the CTA's first unit (the plan names it) or, seldom, in a later one.
@@ -818,36 +901,45 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
         const bool one_each = e_hi - e_lo <= kThreads;         // then no thread meets two of the pieces wanted
         uint4 mine[BATCH];
         int mine_e = -1;
+        // the loads of every vector are in flight together: four to eight 128-bit loads a thread
+        constexpr int kInFlight = BATCH <= 2 ? 4 : 2;
+        uint32_t m[BATCH];
 #pragma unroll
         for (int j = 0; j < BATCH; j++) {
-            uint32_t m = j == 0 ? settled(warm, warm, warm) : 0u;
-            const uint4 *xg = reinterpret_cast<const uint4 *>(p.x) + (size_t)j * nx;
+            m[j] = j == 0 ? settled(warm, warm, warm) : 0u;
             mine[j] = make_uint4(0u, 0u, 0u, 0u);
-            for (int base = 0; base < nx; base += 4 * kThreads) {
-                uint4 v[4];
+        }
+        const uint4 *xg0 = reinterpret_cast<const uint4 *>(p.x);
+        for (int base = 0; base < nx; base += kInFlight * kThreads) {
+            uint4 v[BATCH][kInFlight];
 #pragma unroll
-                for (int i = 0; i < 4; i++) {
-                    const int e = base + i * kThreads + tid;
-                    v[i] = (e < nx && j < p.batch) ? __ldcg(xg + e) : make_uint4(0u, 0u, 0u, 0u);
-                }
-                if (j == 0 && base == 0) {
-                    // while the first loads are on their way: what the loop needs besides x.
-                    // The zero word and the two sums of every x record this CTA will fill
-                    for (int b = tid; b < BATCH * (blk_hi - blk_lo); b += kThreads) {
-                        const int jj = BATCH == 1 ? 0 : b / (blk_hi - blk_lo), bb = b - jj * (blk_hi - blk_lo);
-                        asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(smem_addr(xrec) + jj * xrec_stride + bb * kXRecBytes + 96), "r"(0) : "memory");
-                    }
-                    build_tables();
-                }
+            for (int j = 0; j < BATCH; j++)
 #pragma unroll
-                for (int i = 0; i < 4; i++) {
+                for (int i = 0; i < kInFlight; i++) {
                     const int e = base + i * kThreads + tid;
-                    m = max_abs_pair(max_abs_pair(max_abs_pair(max_abs_pair(m, v[i].x), v[i].y), v[i].z), v[i].w);
-                    if (e >= e_lo && e < e_hi) { mine[j] = v[i]; mine_e = e; }
+                    v[j][i] = (e < nx && (BATCH == 1 || j < p.batch)) ? __ldcg(xg0 + (size_t)j * nx + e) : make_uint4(0u, 0u, 0u, 0u);
                 }
+            if (base == 0) {
+                // while the first loads are on their way: what the loop needs besides x.
+                // The zero word and the two sums of every x record this CTA will fill
+                for (int b = tid; b < BATCH * (blk_hi - blk_lo); b += kThreads)
+                    asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(smem_addr(xrec) + b * kXRecBytes + 96), "r"(0) : "memory");
+                build_tables();
             }
-            m = __reduce_max_sync(0xffffffffu, max(m & 0xffffu, m >> 16));
-            if (lane == 0) warp_max[j * kWarps + warp] = m;    // plain stores: atomics on one word would serialise the warps
+#pragma unroll
+            for (int j = 0; j < BATCH; j++)
+#pragma unroll
+                for (int i = 0; i < kInFlight; i++) {
+                    const int e = base + i * kThreads + tid;
+                    const uint4 &w = v[j][i];
+                    m[j] = max_abs_pair(max_abs_pair(max_abs_pair(max_abs_pair(m[j], w.x), w.y), w.z), w.w);
+                    if (e >= e_lo && e < e_hi) { mine[j] = w; mine_e = e; }
+                }
+        }
+#pragma unroll
+        for (int j = 0; j < BATCH; j++) {
+            const uint32_t most = __reduce_max_sync(0xffffffffu, max(m[j] & 0xffffu, m[j] >> 16));
+            if (lane == 0) warp_max[j * kWarps + warp] = most; // plain stores: atomics on one word would serialise the warps
         }
         __syncthreads();                               // publishes the maxima, the block constants and the zeroed sums
         // the second copy of records goes out now that the loads of x have returned: ahead of the conversion, whose
@@ -858,16 +950,17 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
         }
 #pragma unroll
         for (int j = 0; j < BATCH; j++) {
-            const uint32_t m = warp_max[j * kWarps + (lane < kWarps ? lane : 0)];
-            xexp[j] = max((int)(__reduce_max_sync(0xffffffffu, m) >> 10), 1) - 14;
+            if (BATCH > 1 && j >= p.batch) break;
+            const uint32_t most = warp_max[j * kWarps + (lane < kWarps ? lane : 0)];
+            xexp[j] = max((int)(__reduce_max_sync(0xffffffffu, most) >> 10), 1) - 14;
             const float scale = pow2f(29 - xexp[j]);
             const uint4 *xg = reinterpret_cast<const uint4 *>(p.x) + (size_t)j * nx;
-            const uint32_t xsj = xs0 + j * xrec_stride;
+            const uint32_t xsj = xs0 + j * kXRecBytes;
             if (one_each) {
-                if (mine_e >= 0) convert_item(mine[j], mine_e % 3, xsj + (uint32_t)(mine_e / 3) * kXRecBytes, scale);
+                if (mine_e >= 0) convert_item(mine[j], mine_e % 3, xsj + (uint32_t)(mine_e / 3) * kXBlock, scale);
             } else {
                 for (int e = e_lo + tid; e < e_hi; e += kThreads)
-                    convert_item(j < p.batch ? __ldcg(xg + e) : make_uint4(0u, 0u, 0u, 0u), e % 3, xsj + (uint32_t)(e / 3) * kXRecBytes, scale);
+                    convert_item(__ldcg(xg + e), e % 3, xsj + (uint32_t)(e / 3) * kXBlock, scale);
             }
         }
         __syncthreads();                               // publishes the x records
@@ -925,8 +1018,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
         const int row = (cc.group - pr.group_begin) * kRowsPerGroup + my_row;
         const float row_scale = n == 0 ? first_row_scale : (row < pr.rows ? __half2float(pr.row_scale[row]) : 0.f);
         // this lane's addresses in the x records of the run's first tile
-        const uint32_t xk = xs0 + (uint32_t)cc.col * (4 * kXRecBytes);
-        LaneOffsets xa = {xk + lo.b0, xk + lo.b1, xk + lo.b2, xk + lo.xs};
+        const uint32_t xk = xs0 + (uint32_t)cc.col * (4 * kXBlock);
+        [[maybe_unused]] LaneOffsets xa = {xk + lo.b0, xk + lo.b1, xk + lo.b2, xk + lo.xs};
+        [[maybe_unused]] PairAddr xp = pair_addr(lane, xk);
+        // several vectors: [2 * pair + e] is row 16 * (lane & 1) + 8 e + g of vector (lane & 3) >> 1 of the pair
         long long sum[BATCH];
 #pragma unroll
         for (int j = 0; j < BATCH; j++) sum[j] = 0;
@@ -943,14 +1038,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
             // headers: four words a lane pair (14-byte layout) or two (one byte a header: hh.x serves half-steps 0, 1, hh.y 2, 3)
             uint4 hh;
             if (COMPACT) { const uint2 h2 = lds64(sbuf + (pair16 >> 1) + (OVERLAY ? 1152 : 1536)); hh = make_uint4(h2.x, h2.y, h2.y, h2.x); }
-            else hh = lds128(sbuf + pair16 + 1536);
+            else hh = lds128(sbuf + (BATCH == 1 ? pair16 : 32 * (lane >> 2)) + 1536);
             // The slot's words are in registers: refill it at once with the unit kSlots ahead, so
             // that every slot but the one just read is in flight while this unit is decoded.  The
             // copy's address is made to depend on the loaded words, which holds the copy back
             // until the four shared-memory reads of the whole warp have completed.
-            issue(bar, sbuf + (settled(a0.w, a1.w, OVERLAY ? a2.x : a2.w) | settled(hh.w, hh.x, a0.x)));
-            float acc[BATCH][4];
+            if (BATCH == 1) issue(bar, sbuf + (settled(a0.w, a1.w, OVERLAY ? a2.x : a2.w) | settled(hh.w, hh.x, a0.x)));
             if constexpr (BATCH == 1) {
+                float acc[4];
                 // one vector: every shared-memory load first, then the eight contractions back to back (four independent
                 // accumulator tiles in the tensor pipe at once), then the eight scale steps
                 const StepX s1 = load_step<0>(xa), s2 = load_step<2 * kXRecBytes>(xa);
@@ -973,42 +1068,39 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
                 mma_k16(d2, h2.c0, h2.c1, s2.b2);
                 mma_k16(d3, h3.c0, h3.c1, s2.b2);
                 auto e = [](const int (&d)[4], float ky, int xsum, int r) { return __float_as_int(ky) * xsum + (d[2 * r] + 256 * d[2 * r + 1]); };
-                acc[0][0] = (float)e(d0, h0.k0.y, s1.xsum, 0) * h0.k0.x;
-                acc[0][1] = (float)e(d0, h0.k1.y, s1.xsum, 1) * h0.k1.x;
-                acc[0][2] = (float)e(d1, h1.k0.y, s1.xsum, 0) * h1.k0.x;
-                acc[0][3] = (float)e(d1, h1.k1.y, s1.xsum, 1) * h1.k1.x;
-                acc[0][0] = fmaf((float)e(d2, h2.k0.y, s2.xsum, 0), h2.k0.x, acc[0][0]);
-                acc[0][1] = fmaf((float)e(d2, h2.k1.y, s2.xsum, 1), h2.k1.x, acc[0][1]);
-                acc[0][2] = fmaf((float)e(d3, h3.k0.y, s2.xsum, 0), h3.k0.x, acc[0][2]);
-                acc[0][3] = fmaf((float)e(d3, h3.k1.y, s2.xsum, 1), h3.k1.x, acc[0][3]);
+                acc[0] = (float)e(d0, h0.k0.y, s1.xsum, 0) * h0.k0.x;
+                acc[1] = (float)e(d0, h0.k1.y, s1.xsum, 1) * h0.k1.x;
+                acc[2] = (float)e(d1, h1.k0.y, s1.xsum, 0) * h1.k0.x;
+                acc[3] = (float)e(d1, h1.k1.y, s1.xsum, 1) * h1.k1.x;
+                acc[0] = fmaf((float)e(d2, h2.k0.y, s2.xsum, 0), h2.k0.x, acc[0]);
+                acc[1] = fmaf((float)e(d2, h2.k1.y, s2.xsum, 1), h2.k1.x, acc[1]);
+                acc[2] = fmaf((float)e(d3, h3.k0.y, s2.xsum, 0), h3.k0.x, acc[2]);
+                acc[3] = fmaf((float)e(d3, h3.k1.y, s2.xsum, 1), h3.k1.x, acc[3]);
+                sum[0] += __float2ll_rn(quad_sum(acc) * inv_q);
+                xa.b0 += 4 * kXBlock; xa.b1 += 4 * kXBlock; xa.b2 += 4 * kXBlock; xa.xs += 4 * kXBlock;
             } else {
-                StepX sx[BATCH];
-#pragma unroll
-                for (int j = 0; j < BATCH; j++) {
-                    const LaneOffsets xj = {xa.b0 + j * xrec_stride, xa.b1 + j * xrec_stride, xa.b2 + j * xrec_stride, xa.xs + j * xrec_stride};
-                    sx[j] = load_step<0>(xj);
-                }
-                const HalfA h0 = decode_half<COMPACT, 0>(a0.x, a0.y, a0.z, hh.x, tq);
-#pragma unroll
-                for (int j = 0; j < BATCH; j++) contract_half<true>(h0, sx[j], acc[j][0], acc[j][1]);
-                const HalfA h1 = decode_half<COMPACT, 16>(a0.w, a1.x, a1.y, COMPACT ? hh.x : hh.y, tq);
-#pragma unroll
-                for (int j = 0; j < BATCH; j++) contract_half<true>(h1, sx[j], acc[j][2], acc[j][3]);
-#pragma unroll
-                for (int j = 0; j < BATCH; j++) {
-                    const LaneOffsets xj = {xa.b0 + j * xrec_stride, xa.b1 + j * xrec_stride, xa.b2 + j * xrec_stride, xa.xs + j * xrec_stride};
-                    sx[j] = load_step<2 * kXRecBytes>(xj);
-                }
-                const HalfA h2 = decode_half<COMPACT, 0>(a1.z, a1.w, a2.x, COMPACT ? hh.y : hh.z, tq);
-#pragma unroll
-                for (int j = 0; j < BATCH; j++) contract_half<false>(h2, sx[j], acc[j][0], acc[j][1]);
-                const HalfA h3 = decode_half<COMPACT, 16>(a2.y, a2.z, a2.w, COMPACT ? hh.y : hh.w, tq);
-#pragma unroll
-                for (int j = 0; j < BATCH; j++) contract_half<false>(h3, sx[j], acc[j][2], acc[j][3]);
+                // the tile is decoded once; then pair by pair of vectors
+                const uint4 hb = lds128(sbuf + 1536 + 32 * (lane >> 2) + 16);      // hh: slot 0's headers, hb: slot 1's
+                issue(bar, sbuf + (settled(a0.w, a1.w, a2.w) | settled(hh.w, hb.w, a0.x)));
+                const PairA h0 = decode_pair(a0.x, a0.y, a0.z, hh.x, hb.x, tq), h1 = decode_pair(a0.w, a1.x, a1.y, hh.y, hb.y, tq);
+                const PairA h2 = decode_pair(a1.z, a1.w, a2.x, hh.z, hb.z, tq), h3 = decode_pair(a2.y, a2.z, a2.w, hh.w, hb.w, tq);
+                auto one_pair = [&](auto index) {
+                    constexpr int J = decltype(index)::value, kPair = J * 2 * kXRecBytes;
+                    const PairX x0 = load_pair<kPair, kPair + kXBlock>(xp), x1 = load_pair<kPair + 2 * kXBlock, kPair + 3 * kXBlock>(xp);
+                    float u[4], w[4];                                      // slot 0 and slot 1, rows [2m + e]
+                    contract_pair<true>(h0, x0, u, w);
+                    contract_pair<true>(h1, x0, u + 2, w + 2);
+                    contract_pair<false>(h2, x1, u, w);
+                    contract_pair<false>(h3, x1, u + 2, w + 2);
+                    const float v[4] = {u[0] + w[0], u[1] + w[1], u[2] + w[2], u[3] + w[3]};
+                    float r0, r1;
+                    pair_sum(v, odd_lane, r0, r1);
+                    sum[2 * J] += __float2ll_rn(r0 * inv_q);
+                    sum[2 * J + 1] += __float2ll_rn(r1 * inv_q);
+                };
+                each_pair<BATCH / 2>(one_pair);
+                xp.a0 += 4 * kXBlock; xp.a1 += 4 * kXBlock; xp.a2 += 4 * kXBlock; xp.xs += 4 * kXBlock;
             }
-#pragma unroll
-            for (int j = 0; j < BATCH; j++) sum[j] += __float2ll_rn(quad_sum(acc[j]) * inv_q);
-            xa.b0 += 4 * kXRecBytes; xa.b1 += 4 * kXRecBytes; xa.b2 += 4 * kXRecBytes; xa.xs += 4 * kXRecBytes;
             bar += 8;
             sbuf += kTileBytes;
             const bool wrap = sbuf == sbuf_end;        // every slot completes once a round
@@ -1021,50 +1113,84 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
             // the run ends with the nb mod 4 last block columns of the row group: a pair, a single, or both
             if (!mbar_wait(bar, parity)) { failed = true; break; }
             uint32_t guard = 0, piece = sbuf;
-            float acc[BATCH][4];
+            if constexpr (BATCH == 1) {
+                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+                if (p.tail_cells >= 2) {
+                    const uint32_t xt = xs0 + (uint32_t)tiles * (4 * kXBlock);
 #pragma unroll
-            for (int j = 0; j < BATCH; j++) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-            const uint32_t xt = xs0 + (uint32_t)tiles * (4 * kXRecBytes);
-            if (p.tail_cells >= 2) {
-#pragma unroll
-                for (int m = 0; m < 2; m++) {
-                    const uint32_t wa = lds32(piece + 128 * (3 * m) + lane4), wb = lds32(piece + 128 * (3 * m + 1) + lane4);
-                    const uint32_t wc = lds32(piece + 128 * (3 * m + 2) + lane4);
-                    const uint32_t hw = COMPACT ? lds32(piece + 768 + 4 * (lane >> 1)) : lds32(piece + 768 + 8 * (lane >> 1) + 4 * m);
-                    guard |= settled(wa, wb, wc) | settled(hw, wa, wb);
-                    const HalfA h = m == 0 ? decode_half<COMPACT, 0>(wa, wb, wc, hw, tq_tail) : decode_half<COMPACT, 16>(wa, wb, wc, hw, tq_tail);
-#pragma unroll
-                    for (int j = 0; j < BATCH; j++) {
-                        const uint32_t xj = xt + j * xrec_stride;
-                        const LaneOffsets ta = {xj + lo.b0, xj + lo.b1, xj + lo.b2, xj + lo.xs};
-                        contract_half<false>(h, load_step<0>(ta), acc[j][2 * m], acc[j][2 * m + 1]);
+                    for (int m = 0; m < 2; m++) {
+                        const uint32_t wa = lds32(piece + 128 * (3 * m) + lane4), wb = lds32(piece + 128 * (3 * m + 1) + lane4);
+                        const uint32_t wc = lds32(piece + 128 * (3 * m + 2) + lane4);
+                        const uint32_t hw = COMPACT ? lds32(piece + 768 + 4 * (lane >> 1)) : lds32(piece + 768 + 8 * (lane >> 1) + 4 * m);
+                        guard |= settled(wa, wb, wc) | settled(hw, wa, wb);
+                        const HalfA h = m == 0 ? decode_half<COMPACT, 0>(wa, wb, wc, hw, tq_tail) : decode_half<COMPACT, 16>(wa, wb, wc, hw, tq_tail);
+                        const LaneOffsets ta = {xt + lo.b0, xt + lo.b1, xt + lo.b2, xt + lo.xs};
+                        contract_half<false>(h, load_step<0>(ta), acc[2 * m], acc[2 * m + 1]);
                     }
+                    piece += 2 * kSrcCell;
                 }
-                piece += 2 * kSrcCell;
-            }
-            if (p.tail_cells & 1) {
-                // one block: the slots of this half-step are the two halves of the row group
-                const uint32_t xl = xs0 + (uint32_t)(p.nb - 1) * kXRecBytes;
-                const LaneOffsets l1 = lane_offsets(lane, true);
-                const uint32_t wa = lds32(piece + lane4), wb = lds32(piece + 128 + lane4);
-                const uint32_t wc = lds32(piece + 256 + lane4);
-                // 13-byte layout: two bytes a lane pair, the pairs two to a word
-                const uint32_t hw = COMPACT ? lds32(piece + 384 + 4 * (lane >> 2)) >> (8 * (lane & 2)) : lds32(piece + 384 + 4 * (lane >> 1));
-                guard |= settled(wa, wb, wc) | settled(hw, wa, wb);
-                const HalfA h = decode_half<COMPACT, 0>(wa, wb, wc, hw, tq_tail);
-#pragma unroll
-                for (int j = 0; j < BATCH; j++) {
-                    const uint32_t xj = xl + j * xrec_stride;
-                    const LaneOffsets ta = {xj + l1.b0, xj + l1.b1, xj + l1.b2, xj + l1.xs};
+                if (p.tail_cells & 1) {
+                    // one block: the slots of this half-step are the two halves of the row group
+                    const uint32_t xl = xs0 + (uint32_t)(p.nb - 1) * kXBlock;
+                    const LaneOffsets l1 = lane_offsets(lane, true);
+                    const uint32_t wa = lds32(piece + lane4), wb = lds32(piece + 128 + lane4);
+                    const uint32_t wc = lds32(piece + 256 + lane4);
+                    // 13-byte layout: two bytes a lane pair, the pairs two to a word
+                    const uint32_t hw = COMPACT ? lds32(piece + 384 + 4 * (lane >> 2)) >> (8 * (lane & 2)) : lds32(piece + 384 + 4 * (lane >> 1));
+                    guard |= settled(wa, wb, wc) | settled(hw, wa, wb);
+                    const HalfA h = decode_half<COMPACT, 0>(wa, wb, wc, hw, tq_tail);
+                    const LaneOffsets ta = {xl + l1.b0, xl + l1.b1, xl + l1.b2, xl + l1.xs};
                     float c0, c1;
                     contract_half<true>(h, load_step<0>(ta), c0, c1);
-                    acc[j][0] += high_lane ? 0.f : c0; acc[j][1] += high_lane ? 0.f : c1;
-                    acc[j][2] += high_lane ? c0 : 0.f; acc[j][3] += high_lane ? c1 : 0.f;
+                    acc[0] += high_lane ? 0.f : c0; acc[1] += high_lane ? 0.f : c1;
+                    acc[2] += high_lane ? c0 : 0.f; acc[3] += high_lane ? c1 : 0.f;
                 }
-            }
-            issue(bar, sbuf + guard);
+                issue(bar, sbuf + guard);
+                sum[0] += __float2ll_rn(quad_sum(acc) * inv_q);
+            } else {
+                const bool two = p.tail_cells >= 2, one = p.tail_cells & 1;
+                uint32_t w[6] = {0, 0, 0, 0, 0, 0}, l[3] = {0, 0, 0};
+                uint4 hp = make_uint4(0u, 0u, 0u, 0u);                     // slot 0's headers of m = 0, 1, then slot 1's
+                uint2 hl = make_uint2(0u, 0u);                             // the headers of the two halves of the row group
+                if (two) {
 #pragma unroll
-            for (int j = 0; j < BATCH; j++) sum[j] += __float2ll_rn(quad_sum(acc[j]) * inv_q);
+                    for (int k = 0; k < 6; k++) w[k] = lds32(piece + 128 * k + lane4);
+                    hp = lds128(piece + 768 + 16 * (lane >> 2));
+                    piece += 2 * kSrcCell;
+                }
+                if (one) {
+#pragma unroll
+                    for (int k = 0; k < 3; k++) l[k] = lds32(piece + 128 * k + lane4);
+                    hl = lds64(piece + 384 + 8 * (lane >> 2));
+                }
+                guard = settled(w[0], w[1], w[2]) | settled(w[3], w[4], w[5]) | settled(hp.x, hp.w, l[0]) | settled(l[1], l[2], hl.y);
+                issue(bar, sbuf + guard);
+                const PairA h0 = decode_pair(w[0], w[1], w[2], hp.x, hp.z, tq_tail), h1 = decode_pair(w[3], w[4], w[5], hp.y, hp.w, tq_tail);
+                const PairA hs = decode_pair(l[0], l[1], l[2], hl.x, hl.y, tq_tail);
+                const PairAddr xt = pair_addr(lane, xs0 + (uint32_t)tiles * (4 * kXBlock)), xl = pair_addr(lane, xs0 + (uint32_t)(p.nb - 1) * kXBlock);
+                auto one_pair = [&](auto index) {
+                    constexpr int J = decltype(index)::value, kPair = J * 2 * kXRecBytes;
+                    float u[4] = {0.f, 0.f, 0.f, 0.f}, v[4] = {0.f, 0.f, 0.f, 0.f};
+                    if (two) {
+                        const PairX x = load_pair<kPair, kPair + kXBlock>(xt);
+                        contract_pair<true>(h0, x, u, v);
+                        contract_pair<true>(h1, x, u + 2, v + 2);
+                    }
+                    if (one) {
+                        // the slots are the two halves of the row group, with the same block of x
+                        float c0[2], c1[2];
+                        contract_pair<true>(hs, load_pair<kPair, kPair>(xl), c0, c1);
+                        u[0] += c0[0]; u[1] += c0[1];
+                        v[2] += c1[0]; v[3] += c1[1];
+                    }
+                    const float z[4] = {u[0] + v[0], u[1] + v[1], u[2] + v[2], u[3] + v[3]};
+                    float r0, r1;
+                    pair_sum(z, odd_lane, r0, r1);
+                    sum[2 * J] += __float2ll_rn(r0 * inv_q);
+                    sum[2 * J + 1] += __float2ll_rn(r1 * inv_q);
+                };
+                each_pair<BATCH / 2>(one_pair);
+            }
             bar += 8;
             sbuf += kTileBytes;
             if (sbuf == sbuf_end) { sbuf = my_ring; bar = my_bar; parity ^= 1u; }
@@ -1101,15 +1227,30 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
         if (BATCH == 1) {
             hand_over(p, pr, p.accum, pr.y, cc.group, my_row, sum[0], run, xexp[0] + pr.qexp_base, row_scale, handed);
         } else {
-            // one hand-over a vector; each waits for its answer (a batched launch has arithmetic to hide behind)
+            // this lane's rows are 16 * (lane & 1) + g and the one eight further on, its vector of a pair (lane & 3) >> 1; all the
+            // atomics are on their way before the first answer is looked at
+            const int in_group = 16 * (lane & 1) + (lane >> 2), row_in = (cc.group - pr.group_begin) * kRowsPerGroup + in_group, of_pair = (lane & 3) >> 1;
+            unsigned long long *slot = p.accum + (size_t)cc.group * 32 + in_group;
+            const size_t stride = (size_t)p.total_groups * 32;
+            const unsigned long long counted = (unsigned long long)((long long)run * kUnitBias) + ((unsigned long long)run << kCountShift);
+            unsigned long long old[BATCH];
+            float scale[2];
+#pragma unroll
+            for (int e = 0; e < 2; e++) scale[e] = row_in + 8 * e < pr.rows ? __half2float(pr.row_scale[row_in + 8 * e]) : 0.f;
 #pragma unroll
             for (int j = 0; j < BATCH; j++) {
-                if (j >= p.batch) break;               // a launch may carry fewer vectors than the kernel is built for
-                Handed hj;
-                hj.slot = nullptr;
-                hand_over(p, pr, p.accum + (size_t)j * p.total_groups * 32, pr.y + (size_t)j * p.y_stride, cc.group, my_row, sum[j], run,
-                          xexp[j] + pr.qexp_base, row_scale, hj);
-                settle(p, hj);
+                const int v = (j & ~1) + of_pair, e = j & 1;
+                if (v < p.batch && row_in + 8 * e < pr.rows) old[j] = atomicAdd(slot + v * stride + 8 * e, (unsigned long long)sum[j] + counted);
+            }
+#pragma unroll
+            for (int j = 0; j < BATCH; j++) {
+                const int v = (j & ~1) + of_pair, e = j & 1;
+                if (v < p.batch && row_in + 8 * e < pr.rows && (int)(old[j] >> kCountShift) + run == p.units) {
+                    const long long total = (long long)((old[j] + ((unsigned long long)sum[j] + counted)) & kSumMask) - (long long)p.units * kUnitBias;
+                    const int xe = of_pair ? xexp[(j & ~1) + 1] : xexp[j & ~1];
+                    pr.y[(size_t)v * p.y_stride + row_in + 8 * e] = (float)total * (pow2f(xe + pr.qexp_base) * scale[e]);
+                    slot[v * stride + 8 * e] = 0ull;       // ready for the next launch on this context
+                }
             }
         }
         if (advance(p, cc, run) && cc.panel < p.npanels) q = find_problem(p, cc.group);
@@ -1555,7 +1696,7 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
         }
     }
     const int vectors = p.batch <= 1 ? 1 : (p.batch == 2 ? 2 : 4);             // the kernel is built for 1, 2 and 4
-    const size_t xbytes = ((size_t)p.xblocks * kXRecBytes + 127) / 128 * 128 * vectors;
+    const size_t xbytes = ((size_t)p.xblocks * kXRecBytes * vectors + 127) / 128 * 128;
     g.smem = (size_t)kWarps * kSlots * kTileBytes + 8192 /* alignment of the tables */ + (size_t)p.nprob * 8192 + xbytes + kWarps * kSlots * 8 + kWarps * 4 * vectors + 16 + (size_t)p.rot_span * 8;
     if (layout == LLVQ_PLANES10X) g.smem += (size_t)kWarps * 32 * 8;        // the warps' slots for the products of exception blocks
     return g;
