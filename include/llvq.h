@@ -251,9 +251,9 @@ int llvq_gemv(llvq_ctx *ctx, int layout, const void *layout_buf, const void *row
 
 /* [Sec. 5 "Batching", the paper's stated boundary: one record decode reused across activations]
  * llvq_gemv on the LLVQ_PLANES layout for batch (1..LLVQ_MAX_BATCH) activation vectors in one pass
- * over the records: x is fp16 [batch][k_padded], y is f32 [batch][rows].  Up to four vectors share
- * one pass (the records are read and decoded once for them); five to eight take two passes.  Each
- * vector has its own fixed-point scale and its own accumulators, and y[j] is bit-identical to what
+ * over the records: x is fp16 [batch][k_padded], y is f32 [batch][rows].  The vectors share
+ * one pass (the records are read and decoded once for them); five to eight take two passes where the
+ * context's scratch or a multiprocessor's shared memory holds those of four only.  Each vector has its own fixed-point scale and its own accumulators, and y[j] is bit-identical to what
  * llvq_gemv returns for x[j].  Needs min(batch, 4) times the scratch of llvq_gemv (LLVQ_ESIZE
  * otherwise). */
 int llvq_gemv_batch(llvq_ctx *ctx, const void *layout_buf, const void *row_scale, const float *gain,

@@ -47,6 +47,9 @@ namespace {
 
 constexpr int kWarps = 16;                 // warps per CTA
 constexpr int kThreads = kWarps * 32;
+// The build for five to eight vectors needs more registers than sixteen warps leave a thread (128): twelve warps with 166 run
+// eight vectors on 4096 x 4096 in 16.4 us, sixteen that spill in 23.6, eight with 201 in 19.6; two passes of four take 17.4.
+__host__ __device__ constexpr int gemv_warps(int batch) { return batch > 4 ? 12 : kWarps; }
 constexpr int kSlots = 2;                  // ring slots per warp
 constexpr int kEarlySlots = 1;             // slots filled before the wait for the previous kernel; the rest once x is being prepared
 
@@ -559,7 +562,8 @@ __device__ __forceinline__ void each_pair(F &f) {
 // LLVQ_PLANES10X (tiles of three-bit codes, leftover blocks as in the 13-byte layout, and after each run the exact
 // records of the run's exception blocks, whose short records are empty and add nothing).
 template <bool NO_WEIGHTS, int BATCH, bool ROTATE = false, int LAYOUT = LLVQ_PLANES>
-__global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_constant__ GemvParams p) {
+__global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(const __grid_constant__ GemvParams p) {
+    constexpr int kWarps = gemv_warps(BATCH), kThreads = 32 * kWarps;
     constexpr bool COMPACT = LAYOUT != LLVQ_PLANES, OVERLAY = LAYOUT == LLVQ_PLANES10X;
     static_assert(!OVERLAY || (BATCH == 1 && !ROTATE && !NO_WEIGHTS), "the 10-byte layout: one vector, as it is");
     constexpr int kSrcCell = COMPACT ? kCell13Bytes : kCellBytes;        // bytes of a leftover block column of a row group
@@ -731,9 +735,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
     // the first run's row scale, the rotation's sign flips; and x on its way into L2 with its translation into
     // this multiprocessor's TLB (its values are read only after the wait, through L2, which is where the previous
     // kernel's writes to x land).
-    static_assert(kThreads == 512, "one thread a class slot");
-    float2 my_class = make_float2(0.f, 0.f);
-    if (!COMPACT) asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(my_class.x), "=f"(my_class.y) : "l"(h_cls_block + tid));
+    constexpr int kClasses = (kClassSlots + kThreads - 1) / kThreads;
+    float2 my_class[kClasses];
+#pragma unroll
+    for (int i = 0; i < kClasses; i++) {
+        my_class[i] = make_float2(0.f, 0.f);
+        if (!COMPACT && (kClassSlots % kThreads == 0 || tid + i * kThreads < kClassSlots))
+            asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(my_class[i].x), "=f"(my_class[i].y) : "l"(h_cls_block + tid + i * kThreads));
+    }
     uint4 lane_consts;
     asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(lane_consts.x), "=r"(lane_consts.y), "=r"(lane_consts.z), "=r"(lane_consts.w) : "l"(h_lane_table + lane));
     const int my_row = (lane >> 2) + 8 * (lane & 3);       // the row of the group this lane ends up with
@@ -806,8 +815,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
             }
         } else {
             for (int m = 0; m < p.nprob; m++) {
-                tab[m * 1024 + tid] = make_float2(my_class.x * p.prob[m].gain0, my_class.y);
-                tab[m * 1024 + 512 + tid] = make_float2(my_class.x * p.prob[m].gain1, my_class.y);
+#pragma unroll
+                for (int i = 0; i < kClasses; i++) {
+                    const int c = tid + i * kThreads;
+                    if (kClassSlots % kThreads != 0 && c >= kClassSlots) break;
+                    tab[m * 1024 + c] = make_float2(my_class[i].x * p.prob[m].gain0, my_class[i].y);
+                    tab[m * 1024 + 512 + c] = make_float2(my_class[i].x * p.prob[m].gain1, my_class[i].y);
+                }
             }
         }
     };
@@ -902,7 +916,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
         uint4 mine[BATCH];
         int mine_e = -1;
         // the loads of every vector are in flight together: four to eight 128-bit loads a thread
-        constexpr int kInFlight = BATCH <= 2 ? 4 : 2;
+        constexpr int kInFlight = BATCH <= 2 ? 4 : (BATCH <= 4 ? 2 : 1);
         uint32_t m[BATCH];
 #pragma unroll
         for (int j = 0; j < BATCH; j++) {
@@ -1086,6 +1100,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
                 const PairA h2 = decode_pair(a1.z, a1.w, a2.x, hh.z, hb.z, tq), h3 = decode_pair(a2.y, a2.z, a2.w, hh.w, hb.w, tq);
                 auto one_pair = [&](auto index) {
                     constexpr int J = decltype(index)::value, kPair = J * 2 * kXRecBytes;
+                    if (J > BATCH / 4 && 2 * J >= p.batch) return;         // a launch may carry fewer vectors than the kernel is built for
                     const PairX x0 = load_pair<kPair, kPair + kXBlock>(xp), x1 = load_pair<kPair + 2 * kXBlock, kPair + 3 * kXBlock>(xp);
                     float u[4], w[4];                                      // slot 0 and slot 1, rows [2m + e]
                     contract_pair<true>(h0, x0, u, w);
@@ -1170,6 +1185,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_planes_kernel(const __grid_c
                 const PairAddr xt = pair_addr(lane, xs0 + (uint32_t)tiles * (4 * kXBlock)), xl = pair_addr(lane, xs0 + (uint32_t)(p.nb - 1) * kXBlock);
                 auto one_pair = [&](auto index) {
                     constexpr int J = decltype(index)::value, kPair = J * 2 * kXRecBytes;
+                    if (J > BATCH / 4 && 2 * J >= p.batch) return;         // a launch may carry fewer vectors than the kernel is built for
                     float u[4] = {0.f, 0.f, 0.f, 0.f}, v[4] = {0.f, 0.f, 0.f, 0.f};
                     if (two) {
                         const PairX x = load_pair<kPair, kPair + kXBlock>(xt);
@@ -1695,9 +1711,10 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
             if (c_hi - c_lo > p.rot_span) p.rot_span = c_hi - c_lo;
         }
     }
-    const int vectors = p.batch <= 1 ? 1 : (p.batch == 2 ? 2 : 4);             // the kernel is built for 1, 2 and 4
+    const int vectors = p.batch <= 2 ? p.batch : (p.batch <= 4 ? 4 : 8);       // the kernel is built for 1, 2, 4 and 8
+    const int warps = gemv_warps(vectors);
     const size_t xbytes = ((size_t)p.xblocks * kXRecBytes * vectors + 127) / 128 * 128;
-    g.smem = (size_t)kWarps * kSlots * kTileBytes + 8192 /* alignment of the tables */ + (size_t)p.nprob * 8192 + xbytes + kWarps * kSlots * 8 + kWarps * 4 * vectors + 16 + (size_t)p.rot_span * 8;
+    g.smem = (size_t)warps * kSlots * kTileBytes + 8192 /* alignment of the tables */ + (size_t)p.nprob * 8192 + xbytes + warps * kSlots * 8 + warps * 4 * vectors + 16 + (size_t)p.rot_span * 8;
     if (layout == LLVQ_PLANES10X) g.smem += (size_t)kWarps * 32 * 8;        // the warps' slots for the products of exception blocks
     return g;
 }
@@ -1718,6 +1735,7 @@ int gemv_configure(const llvq_ctx *ctx) {
     if (allow_max_smem(gemv_planes_kernel<true, 1>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 2>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 4>, bytes)) return -1;
+    if (allow_max_smem(gemv_planes_kernel<false, 8>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 1, true>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 1, false, LLVQ_PLANES13>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 1, false, LLVQ_PLANES10X>, bytes)) return -1;
@@ -1728,7 +1746,7 @@ int gemv_configure(const llvq_ctx *ctx) {
 cudaError_t launch_gemv(int layout, const GemvParams &p, const GemvLaunch &g, bool no_weights, bool pdl, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)g.grid);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(32 * gemv_warps(p.batch));
     cfg.dynamicSmemBytes = g.smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -1743,7 +1761,8 @@ cudaError_t launch_gemv(int layout, const GemvParams &p, const GemvLaunch &g, bo
         if (p.rot_log2 > 0) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 1, true>, p);
         if (p.batch <= 1) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 1>, p);
         if (p.batch == 2) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 2>, p);
-        return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 4>, p);
+        if (p.batch <= 4) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 4>, p);
+        return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 8>, p);
     }
     cfg.numAttrs = 0;
     return cudaLaunchKernelEx(&cfg, gemv_onehot_kernel, p);

@@ -366,6 +366,23 @@ def test_gemv_batch_matches_single_vector_calls_and_oracle(B, ctx, oracle, rows,
     assert torch.equal(Y, Y2)
 
 
+@pytest.mark.parametrize("rows,nb,batch", [(33, 3, 5), (64, 4, 6), (95, 9, 7), (5000, 107, 8), (100, 171, 5)])
+def test_gemv_batch_of_more_than_four(B, ctx, rows, nb, batch):
+    """Five to eight vectors in one pass, and in two where the scratch holds the sums of four only: both the bits of
+    one vector at a time."""
+    case = make_case(rows, 24 * nb, seed=rows + nb + batch)
+    buf = B.expand(ctx, 0, case.d_codes, rows, nb)
+    X = torch.stack([torch.roll(case.d_x, 5 * j) * (0.5 + j) for j in range(batch)]).half().contiguous()
+    ref = torch.stack([B.gemv(ctx, 0, buf, case.d_scale, GAIN, X[j].contiguous(), rows, nb * 24) for j in range(batch)])
+    small = B.create(0, scratch_bytes=4 * 8 * ((rows + 31) // 32 * 32))
+    try:
+        for c in (ctx, small):
+            assert torch.equal(B.gemv_batch(c, buf, case.d_scale, GAIN, X, rows, nb * 24), ref)
+            B.status(c)
+    finally:
+        small.close()
+
+
 def test_gemv_batch_limits(B, ctx):
     case = make_case(64, 96, seed=1)
     buf = B.expand(ctx, 0, case.d_codes, case.rows, case.nb)
