@@ -61,7 +61,7 @@ int llvq_create(llvq_ctx **out, int device, size_t scratch_bytes) {
     llvq_ctx *ctx = new (std::nothrow) llvq_ctx();
     if (!ctx) return LLVQ_ECUDA;
     ctx->device = device;
-    ctx->table_blob = nullptr; ctx->accum = nullptr; ctx->error = nullptr; ctx->bad_codes = nullptr; ctx->use_pdl = 1; ctx->weights_dirty = 0;
+    ctx->table_blob = nullptr; ctx->accum = nullptr; ctx->error = nullptr; ctx->bad_codes = nullptr; ctx->host_counter = nullptr; ctx->use_pdl = 1; ctx->weights_dirty = 0;
     if (!build_tables(ctx->host)) { delete ctx; return LLVQ_EINVAL; }
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) { delete ctx; return LLVQ_ECUDA; }
@@ -79,7 +79,8 @@ int llvq_create(llvq_ctx **out, int device, size_t scratch_bytes) {
         {h.cls_value.data(), kClassSlots * 8 * 4, 0},   {h.cls_dist.data(), kClassSlots * 8, 0},
         {h.cls_block.data(), kClassSlots * 8, 0},       {lanes, sizeof lanes, 0},
         {unrank.blob.data(), unrank.blob.size(), 0},    {unrank.tail8.data(), unrank.tail8.size() * 4, 0},
-        {unrank.tab_a.data(), unrank.tab_a.size() * 8, 0}, {unrank.tab_b.data(), unrank.tab_b.size() * 4, 0}};
+        {unrank.tab_b.data(), unrank.tab_b.size() * 4, 0},
+        {unrank.pairs.data(), unrank.pairs.size() * 8, 0}};
     size_t total = 0;
     for (auto &p : parts) { p.off = total; total += round_up(p.bytes, 256); }
     if (cudaMalloc(&ctx->table_blob, total) != cudaSuccess) { delete ctx; return LLVQ_ECUDA; }
@@ -98,16 +99,18 @@ int llvq_create(llvq_ctx **out, int device, size_t scratch_bytes) {
     d.cls_block = (const float2 *)(blob + parts[5].off);
     d.lane_table = (const uint4 *)(blob + parts[6].off);
     ctx->unrank.blob = (const uint8_t *)(blob + parts[7].off);
+    ctx->unrank.far = ctx->unrank.blob;
     ctx->unrank.tail8 = (const uint32_t *)(blob + parts[8].off);
-    ctx->unrank.tab_a = (const uint64_t *)(blob + parts[9].off);
-    ctx->unrank.tab_b = (const uint32_t *)(blob + parts[10].off);
+    ctx->unrank.tab_b = (const uint32_t *)(blob + parts[9].off);
+    ctx->unrank.pairs = (const uint64_t *)(blob + parts[10].off);
     d.num_points = h.num_points;
 
     if (scratch_bytes == 0) scratch_bytes = (size_t)8 << 20;
     ctx->accum_slots = scratch_bytes / 8;
     if (cudaMalloc(&ctx->accum, ctx->accum_slots * 8) != cudaSuccess ||
         cudaMemset(ctx->accum, 0, ctx->accum_slots * 8) != cudaSuccess ||
-        cudaMalloc(&ctx->error, 32) != cudaSuccess || cudaMemset(ctx->error, 0, 32) != cudaSuccess) {
+        cudaMalloc(&ctx->error, 32) != cudaSuccess || cudaMemset(ctx->error, 0, 32) != cudaSuccess ||
+        cudaHostAlloc((void **)&ctx->host_counter, 8, cudaHostAllocDefault) != cudaSuccess) {
         llvq_destroy(ctx);
         return LLVQ_ECUDA;
     }
@@ -126,6 +129,7 @@ void llvq_destroy(llvq_ctx *ctx) {
     cudaFree(ctx->table_blob);
     cudaFree(ctx->accum);
     cudaFree(ctx->error);
+    cudaFreeHost(ctx->host_counter);
     delete ctx;
 }
 
@@ -185,11 +189,10 @@ int llvq_overlay_count(llvq_ctx *ctx, const uint64_t *codes, int64_t rows, int64
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
     cudaStream_t s = (cudaStream_t)stream;
-    unsigned long long n = 0;
-    if (cudaMemsetAsync(ctx->counter, 0, 8, s) != cudaSuccess || launch_overlay_count(ctx, codes, rows, nb, ctx->counter, s) != cudaSuccess ||
-        cudaMemcpyAsync(&n, ctx->counter, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
-        return LLVQ_ECUDA;
-    *count = n;
+    // the kernel writes the total to page-locked memory of the context: no memset before it and no copy after it
+    *ctx->host_counter = 0;
+    if (launch_overlay_count(ctx, codes, rows, nb, ctx->counter, ctx->host_counter, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return LLVQ_ECUDA;
+    *count = *ctx->host_counter;
     return LLVQ_OK;
 }
 

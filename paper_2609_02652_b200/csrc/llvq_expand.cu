@@ -23,7 +23,7 @@ struct WarpScratch {
     uint32_t nat[4][4][kNatStride];        // [block of the piece][codes of eight coordinates: 0..2, header: 3][row]
     uint32_t exceptions[4];                // 10-byte layout: rows of a block without a window
 };
-constexpr int kExpandSmem = kUnrankBlobBytes + kExpandWarps * (int)sizeof(WarpScratch);
+constexpr int kExpandSmem = kUnrankSharedBytes + kExpandWarps * (int)sizeof(WarpScratch);
 
 __device__ __forceinline__ void copy_blob(uint8_t *to, const uint8_t *from, int bytes) {
     for (int i = threadIdx.x * 16; i < bytes; i += blockDim.x * 16)
@@ -83,11 +83,11 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
     constexpr bool COMPACT = LAYOUT != LLVQ_PLANES, OVERLAY = LAYOUT == LLVQ_PLANES10X;
     constexpr int kCell = COMPACT ? kCell13Bytes : kCellBytes, kTile = OVERLAY ? kTile10Bytes : (COMPACT ? kTile13Bytes : kTileBytes);
     extern __shared__ __align__(16) uint8_t smem[];
-    copy_blob(smem, global.blob, kUnrankBlobBytes);
+    copy_blob(smem, global.blob, kUnrankSharedBytes);
     UnrankView v = global;
     v.blob = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    WarpScratch &s = reinterpret_cast<WarpScratch *>(smem + kUnrankBlobBytes)[warp];
+    WarpScratch &s = reinterpret_cast<WarpScratch *>(smem + kUnrankSharedBytes)[warp];
     __syncthreads();
 
     const uint32_t tiles = (uint32_t)(nb / kTileCells), left = (uint32_t)(nb % kTileCells);
@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(kExpandThreads, 1)
 expand_onehot_kernel(UnrankView global, DeviceTables T, const uint64_t *__restrict__ codes, int64_t rows, int64_t nb, int64_t cells,
                      uint8_t *__restrict__ out, uint32_t *bad_count, uint32_t *ctx_bad) {
     extern __shared__ __align__(16) uint8_t smem[];
-    copy_blob(smem, global.blob, kUnrankBlobBytes);
+    copy_blob(smem, global.blob, kUnrankSharedBytes);
     UnrankView v = global;
     v.blob = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -352,59 +352,97 @@ expand_onehot_kernel(UnrankView global, DeviceTables T, const uint64_t *__restri
 }
 
 // ---- the exception table of the 10-byte layout is filled in a fixed order, so its entries' places are known before
-// they are written.  A warp a tile counts the tile's exceptions (lane = row): the class settles all but one block in
-// some thousands, only those are un-ranked (from the tables in global memory): 15 us for 1.04 M blocks, where un-ranking
-// them all took 450.  INDEX: the count goes to the index
-// entry after the tile's (the running sum over the index then gives every tile's first entry); else the counts are
-// added up in *total.
-constexpr int kCountWarps = 16;
-constexpr int kCountSmem = kUnrankGolayMsg;               // the part of the blob with the classes and the guide
+// they are written.  A warp a tile counts the tile's exceptions (lane = row): a bit of the class guide says of nearly every
+// index (59 in 60 of the synthetic stream) that its classes hold none, the class settles most others, and only one block in
+// some thousands is un-ranked (from the tables in global memory).  So the count streams the codes: bound HBM, 8 bytes a
+// block.  INDEX: the count goes to the index entry after the tile's (the running sum over the index then gives every
+// tile's first entry); else the counts are added up in total[0], and the last CTA (total[1] counts them) writes the sum to
+// `host`, page-locked memory, and leaves both at zero.
+// Blocks to look at wait in a list until there are thirty-two or the warp's tiles are through: a look's chain of dependent
+// reads (3 us) is then paid once a warp, not once a tile.
+constexpr int kCountWarps = 8;
 template <bool INDEX>
 __global__ void __launch_bounds__(kCountWarps * 32)
-overlay_count_kernel(UnrankView global, uint64_t num_points, const uint64_t *__restrict__ codes, int64_t rows, int64_t nb, uint32_t total_tiles,
-                     uint32_t *index, unsigned long long *total) {
-    __shared__ __align__(16) uint8_t blob[kCountSmem];
-    copy_blob(blob, global.blob, kCountSmem);
-    UnrankView v = global;
-    v.blob = blob;
+overlay_count_kernel(UnrankView v, uint64_t num_points, const uint64_t *__restrict__ codes, int64_t rows, int64_t nb, uint32_t total_tiles,
+                     uint32_t *index, unsigned long long *total, volatile unsigned long long *host) {
+    __shared__ uint32_t window[kGuideSlots / 32];
+    __shared__ uint64_t list_all[kCountWarps][160];                // index of a block to look at
+    __shared__ uint32_t tile_all[kCountWarps][160];                // and its tile
+    for (int i = threadIdx.x; i < kGuideSlots / 32; i += blockDim.x) window[i] = __ldg(reinterpret_cast<const uint32_t *>(v.blob + kUnrankWindow) + i);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint64_t *list = list_all[warp];
+    uint32_t *tile_of = tile_all[warp];
     const uint32_t tiles = (uint32_t)(nb / kTileCells);
     __syncthreads();
     uint32_t sum = 0;
-    for (uint32_t tile = (uint32_t)warp * gridDim.x + blockIdx.x; tile < total_tiles; tile += kCountWarps * gridDim.x) {
-        const uint32_t rg = tile / tiles, u = tile % tiles;
-        const int64_t row = (int64_t)rg * kRowsPerGroup + lane;
-        uint64_t code[4];
-#pragma unroll
-        for (int q = 0; q < 4; q++) code[q] = row < rows ? codes[row * nb + (int64_t)u * kTileCells + q] : ~0ull;
-        uint32_t count = 0;
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            if (code_names_point(code[q], num_points)) {
-                const uint64_t idx = code[q] & ((1ull << kIndexBits) - 1);
-                const int c = find_class(v, idx);
-                const uint32_t window = blob_at<UnrankDesc>(v, kUnrankDescs, c).flags >> 20;
-                if (window == kWindowNever) count++;
-                else if (window == kWindowDepends) {
-                    const UnrankDesc d = blob_at<UnrankDesc>(v, kUnrankDescs, c);
-                    Point p;
-                    unrank(global, d, idx - blob_at<uint64_t>(v, kUnrankBase, c), p);
-                    const bool odd = d.flags & 1u;
-                    const uint32_t cw[3] = {point_codes(p, 0, odd), point_codes(p, 1, odd), point_codes(p, 2, odd)};
-                    count += window_base(cw) == 0u;
-                }
+    int listed = 0;
+    // looks at the last (at most 32) blocks of the list
+    auto look = [&]() {
+        __syncwarp();
+        const int n = min(listed, 32);
+        listed -= n;
+        if (lane < n) {
+            const uint64_t idx = list[listed + lane];
+            const int c = find_class(v, idx);
+            const UnrankDesc d = blob_at<UnrankDesc>(v, kUnrankDescs, c);
+            bool exception = d.flags >> 20 == kWindowNever;
+            if (d.flags >> 20 == kWindowDepends) {
+                Point p;
+                unrank(v, d, idx - blob_at<uint64_t>(v, kUnrankBase, c), p);
+                const bool odd = d.flags & 1u;
+                const uint32_t cw[3] = {point_codes(p, 0, odd), point_codes(p, 1, odd), point_codes(p, 2, odd)};
+                exception = window_base(cw) == 0u;
+            }
+            if (exception) {
+                if (INDEX) atomicAdd(index + tile_of[listed + lane] + 1, 1u);
+                else sum++;
             }
         }
-        if (INDEX) {
-            count = __reduce_add_sync(0xffffffffu, count);
-            if (lane == 0) index[(size_t)tile + 1] = count;
-        } else {
-            sum += count;
+        __syncwarp();
+    };
+    uint64_t code[4], next[4];
+    auto load = [&](uint32_t tile, uint64_t (&to)[4]) {
+        const uint32_t rg = tile / tiles, u = tile - rg * tiles;
+        const int64_t row = (int64_t)rg * kRowsPerGroup + lane;
+#pragma unroll
+        for (int q = 0; q < 4; q++) to[q] = (row < rows && tile < total_tiles) ? __ldcs(codes + row * nb + (int64_t)u * kTileCells + q) : ~0ull;
+    };
+    uint32_t tile = blockIdx.x * kCountWarps + warp;
+    const uint32_t stride = kCountWarps * gridDim.x;
+    load(tile, next);
+    for (; tile < total_tiles; tile += stride) {
+#pragma unroll
+        for (int q = 0; q < 4; q++) code[q] = next[q];
+        load(tile + stride, next);
+        if (INDEX && lane == 0) index[(size_t)tile + 1] = 0u;      // before any addition to it, which the look's barrier puts behind
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const uint64_t idx = code[q] & ((1ull << kIndexBits) - 1);
+            const int slot = guide_slot(idx);
+            const bool wanted = code_names_point(code[q], num_points) && ((window[slot >> 5] >> (slot & 31)) & 1u);
+            const uint32_t votes = __ballot_sync(0xffffffffu, wanted);
+            if (wanted) {
+                const int at = listed + __popc(votes & ((1u << lane) - 1u));
+                list[at] = idx;
+                tile_of[at] = tile;
+            }
+            listed += __popc(votes);
         }
+        while (listed >= 32) look();                               // at most 31 stay, and a tile adds at most 128
     }
+    if (listed > 0) look();
     if (!INDEX) {
         sum = __reduce_add_sync(0xffffffffu, sum);
-        if (lane == 0 && sum) atomicAdd(total, (unsigned long long)sum);
+        if (lane == 0 && sum) {
+            atomicAdd(total, (unsigned long long)sum);
+            __threadfence();
+        }
+        __syncthreads();                                           // the CTA's sums are in
+        if (threadIdx.x == 0 && atomicAdd(total + 1, 1ull) == gridDim.x - 1) {
+            __threadfence();
+            *host = atomicExch(total, 0ull);
+            atomicExch(total + 1, 0ull);
+        }
     }
 }
 
@@ -413,19 +451,28 @@ overlay_count_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
 // the entries that will find no room are counted, and the bytes between the parts of the buffer zeroed.
 __global__ void __launch_bounds__(1024) overlay_index_kernel(uint8_t *out, size_t records_end, size_t index_offset, size_t table_offset,
                                                              int64_t n, uint32_t capacity, uint32_t *overflow) {
-    constexpr int kEach = 8;                                       // consecutive entries a thread and round
+    constexpr int kEach = 8, kRound = 1024 * kEach;                // entries a thread and a round
     uint32_t *index = reinterpret_cast<uint32_t *>(out + index_offset);
-    __shared__ uint32_t warp_sum[32];
+    __shared__ uint32_t warp_sum[32], staged[kRound + kRound / kEach];     // a word's pad after eight: consecutive threads' eights start in different banks
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t carry = 0;                                            // the same in every thread
-    for (int64_t base = 0; base < n; base += 1024 * kEach) {
-        const int64_t at = base + (int64_t)tid * kEach;
-        uint32_t c[kEach], mine = 0;
+    uint32_t c[kEach];
+    auto load = [&](int64_t base) {                                // a round's entries, neighbours to neighbours
 #pragma unroll
         for (int j = 0; j < kEach; j++) {
-            c[j] = at + j < n ? index[at + j + 1] : 0u;
-            mine += c[j];
+            const int64_t at = base + j * 1024 + tid;
+            c[j] = at < n ? index[at + 1] : 0u;
         }
+    };
+    load(0);
+    for (int64_t base = 0; base < n; base += kRound) {
+#pragma unroll
+        for (int j = 0; j < kEach; j++) staged[(j * 1024 + tid) + (j * 1024 + tid) / kEach] = c[j];
+        __syncthreads();
+        load(base + kRound);
+        uint32_t mine = 0;
+#pragma unroll
+        for (int j = 0; j < kEach; j++) mine += staged[tid * (kEach + 1) + j];
         uint32_t incl = mine;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -439,10 +486,16 @@ __global__ void __launch_bounds__(1024) overlay_index_kernel(uint8_t *out, size_
         carry += __reduce_add_sync(0xffffffffu, w);
 #pragma unroll
         for (int j = 0; j < kEach; j++) {
-            run += c[j];
-            if (at + j < n) index[at + j + 1] = min(run, capacity);
+            run += staged[tid * (kEach + 1) + j];
+            staged[tid * (kEach + 1) + j] = min(run, capacity);
         }
-        __syncthreads();                                           // warp_sum is free for the next round
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kEach; j++) {
+            const int64_t at = base + j * 1024 + tid;
+            if (at < n) index[at + 1] = staged[(j * 1024 + tid) + (j * 1024 + tid) / kEach];
+        }
+        __syncthreads();                                           // the shared words are free for the next round
     }
     if (tid == 0) {
         index[0] = 0;
@@ -465,15 +518,15 @@ int expand_configure() {
     if (cudaFuncSetAttribute(expand_planes_kernel<LLVQ_PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return -1;
     if (cudaFuncSetAttribute(expand_planes_kernel<LLVQ_PLANES13>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return -1;
     if (cudaFuncSetAttribute(expand_planes_kernel<LLVQ_PLANES10X>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return -1;
-    return cudaFuncSetAttribute(expand_onehot_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUnrankBlobBytes) == cudaSuccess ? 0 : -1;
+    return cudaFuncSetAttribute(expand_onehot_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUnrankSharedBytes) == cudaSuccess ? 0 : -1;
 }
 
 cudaError_t launch_overlay_count(const llvq_ctx *ctx, const uint64_t *codes, int64_t rows, int64_t nb, unsigned long long *counter,
-                                 cudaStream_t s) {
+                                 unsigned long long *host, cudaStream_t s) {
     const int64_t groups = (rows + kRowsPerGroup - 1) / kRowsPerGroup, tiles = nb / kTileCells;
     if (tiles == 0) return cudaSuccess;
-    overlay_count_kernel<false><<<grid_for(ctx, groups * tiles, 4), kCountWarps * 32, 0, s>>>(ctx->unrank, ctx->dev.num_points, codes, rows, nb,
-                                                                                                          (uint32_t)(groups * tiles), nullptr, counter);
+    overlay_count_kernel<false><<<grid_for(ctx, (groups * tiles + kCountWarps - 1) / kCountWarps, 8), kCountWarps * 32, 0, s>>>(ctx->unrank, ctx->dev.num_points, codes, rows, nb,
+                                                                                                          (uint32_t)(groups * tiles), nullptr, counter, host);
     return cudaGetLastError();
 }
 
@@ -484,7 +537,7 @@ cudaError_t launch_expand(const llvq_ctx *ctx, int layout, const uint64_t *codes
     const UnrankView v = ctx->unrank;
     const uint64_t points = ctx->dev.num_points;
     if (layout == LLVQ_ONEHOT) {
-        expand_onehot_kernel<<<grid_for(ctx, groups * nb), kExpandThreads, kUnrankBlobBytes, s>>>(v, ctx->dev, codes, rows, nb, groups * nb, o8, bad_count,
+        expand_onehot_kernel<<<grid_for(ctx, groups * nb), kExpandThreads, kUnrankSharedBytes, s>>>(v, ctx->dev, codes, rows, nb, groups * nb, o8, bad_count,
                                                                                                               ctx->bad_codes);
         return cudaGetLastError();
     }
@@ -499,8 +552,8 @@ cudaError_t launch_expand(const llvq_ctx *ctx, int layout, const uint64_t *codes
         const uint32_t capacity = room > 0xffffffffull ? 0xffffffffu : (uint32_t)room;
         // count the tiles' exceptions into the index, turn the counts into first entries, expand
         if (tiles > 0)
-            overlay_count_kernel<true><<<grid_for(ctx, groups * tiles, 4), kCountWarps * 32, 0, s>>>(v, points, codes, rows, nb, (uint32_t)(groups * tiles), index,
-                                                                                                                 nullptr);
+            overlay_count_kernel<true><<<grid_for(ctx, (groups * tiles + kCountWarps - 1) / kCountWarps, 8), kCountWarps * 32, 0, s>>>(v, points, codes, rows, nb, (uint32_t)(groups * tiles), index,
+                                                                                                                 nullptr, nullptr);
         overlay_index_kernel<<<1, 1024, 0, s>>>(o8, (size_t)groups * overlay_group_bytes(nb), index_offset, table_offset, groups * tiles, capacity, ctx->overflow);
         expand_planes_kernel<LLVQ_PLANES10X><<<grid, kExpandThreads, kExpandSmem, s>>>(v, points, codes, rows, nb, (uint32_t)pieces, o8, bad_count, ctx->bad_codes, index, table,
                                                                                        capacity);

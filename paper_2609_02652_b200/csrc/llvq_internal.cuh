@@ -122,7 +122,8 @@ struct llvq_ctx {
     int *error;              // device flag: a kernel's bounded wait ran out
     uint32_t *bad_codes;     // device count: codes that named no point, over the expansions since the last llvq_status
     uint32_t *overflow;      // device count: exception-table entries that found no room, since the last llvq_status
-    unsigned long long *counter;   // device scratch of llvq_overlay_count
+    unsigned long long *counter;   // device scratch of llvq_overlay_count: two words, zero between calls
+    unsigned long long *host_counter;   // page-locked: its result
     int use_pdl;             // launch the GEMV with programmatic stream serialization
     int weights_dirty;       // an expansion was enqueued since the last GEMV: that GEMV must not read records ahead of it
     int sm_count;
@@ -132,9 +133,10 @@ struct llvq_ctx {
 namespace llvq {
 cudaError_t launch_expand(const llvq_ctx *ctx, int layout, const uint64_t *codes, int64_t rows, int64_t nb,
                           void *out, size_t out_bytes, uint32_t *bad_count, cudaStream_t s);
-// adds the number of blocks the 10-byte layout would keep in its exception table to *counter (device)
+// writes the number of blocks the 10-byte layout would keep in its exception table to *host (page-locked); `counter` is two
+// device words that are zero before and after
 cudaError_t launch_overlay_count(const llvq_ctx *ctx, const uint64_t *codes, int64_t rows, int64_t nb, unsigned long long *counter,
-                                 cudaStream_t s);
+                                 unsigned long long *host, cudaStream_t s);
 struct GemvLaunch {
     int grid;
     size_t smem;

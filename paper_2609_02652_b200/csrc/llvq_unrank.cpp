@@ -1,5 +1,6 @@
 #include "llvq_unrank.h"
 
+#include <array>
 #include <cstring>
 #include <map>
 
@@ -53,7 +54,7 @@ T *part(std::vector<uint8_t> &blob, int offset) { return reinterpret_cast<T *>(b
 
 bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
     u.blob.assign(kUnrankBlobBytes, 0);
-    u.tail8.clear(); u.tab_a.clear(); u.tab_b.clear();
+    u.pairs.clear(); u.tail8.clear(); u.tab_b.clear();
     if (t.num_classes > kUnrankClasses - 2) return false;
 
     UnrankStep *steps = part<UnrankStep>(u.blob, kUnrankSteps);
@@ -65,37 +66,84 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
         steps[n].inverse = x;
     }
 
-    // ---- every ordering of eight odd magnitudes with sum j (j + 1) / 2 <= 21
+    // ---- the multisets of odd magnitudes 1 + 2j, by their copies of j = 1..6 (sum j (j + 1) / 2 <= 21, at most 24 of them)
+    std::map<std::array<int, 7>, int> set_of;            // key: copies of j = 1..6, [0] unused
+    std::vector<std::array<int, 7>> sets;
     {
-        uint16_t *first = part<uint16_t>(u.blob, kUnrankTailBase);
         static const int cost[7] = {0, 1, 3, 6, 10, 15, 21};
-        int c[7];
+        std::array<int, 7> c{};
         for (c[6] = 0; c[6] <= 1; c[6]++)
         for (c[5] = 0; c[5] <= 1; c[5]++)
         for (c[4] = 0; c[4] <= 2; c[4]++)
         for (c[3] = 0; c[3] <= 3; c[3]++)
         for (c[2] = 0; c[2] <= 7; c[2]++)
-        for (c[1] = 0; c[1] <= 8; c[1]++) {
-            int n = 0, sum = 0;
-            for (int v = 1; v < 7; v++) { n += c[v]; sum += c[v] * cost[v]; }
-            if (n > 8 || sum > 21) continue;
-            c[0] = 8 - n;
-            if (u.tail8.size() > 0xffff) return false;
-            first[c[1] | c[2] << 4 | c[3] << 7 | c[4] << 9 | c[5] << 11 | c[6] << 12] = (uint16_t)u.tail8.size();
-            list_orderings(c, 7, 8, 0, 4, 0, u.tail8);
+        for (c[1] = 0; c[1] <= 21; c[1]++) {
+            int sum = 0;
+            for (int v = 1; v < 7; v++) sum += c[v] * cost[v];
+            if (sum > 21) continue;
+            set_of[c] = (int)sets.size();
+            sets.push_back(c);
+        }
+        if ((int)sets.size() != kOddSets) return false;
+    }
+    auto copies_in = [](const std::array<int, 7> &c) { int n = 0; for (int v = 1; v < 7; v++) n += c[v]; return n; };
+    // every ordering of eight
+    uint16_t *tail_first = part<uint16_t>(u.blob, kUnrankTailBase);
+    for (int k = 0; k < kOddSets; k++) {
+        const int n = copies_in(sets[k]);
+        if (n > 8) continue;
+        int c[7];
+        for (int v = 1; v < 7; v++) c[v] = sets[k][v];
+        c[0] = 8 - n;
+        if (u.tail8.size() > 0xffff) return false;
+        tail_first[k] = (uint16_t)u.tail8.size();
+        list_orderings(c, 7, 8, 0, 4, 0, u.tail8);
+    }
+    // the draws of two from L
+    PairStep *pair_steps = part<PairStep>(u.blob, kUnrankPairs);
+    for (int i = 0; i < kPairSteps; i++) {
+        const int L = 24 - 2 * i, draws = L * (L - 1);
+        const uint32_t shift = (uint32_t)__builtin_ctz(draws), odd = (uint32_t)draws >> shift;
+        uint32_t x = odd;
+        for (int k = 0; k < 5; k++) x *= 2u - odd * x;
+        pair_steps[i] = {x, shift, (uint32_t)u.pairs.size(), (uint32_t)draws};
+        u.pairs.resize(u.pairs.size() + (size_t)kOddSets * draws, 0);
+        for (int k = 0; k < kOddSets; k++) {
+            std::array<int, 7> c = sets[k];
+            const int n = copies_in(c);
+            if (n > L) continue;
+            uint64_t *entry = u.pairs.data() + pair_steps[i].first + (size_t)k * draws;
+            int at = 0;
+            for (int va = 0; va < 7; va++)
+                for (int vb = 0; vb < 7; vb++) {
+                    const int na = va ? c[va] : L - n, nb = (vb ? c[vb] : L - n) - (va == vb);
+                    if (na < 1 || nb < 1) continue;
+                    std::array<int, 7> rest = c;
+                    if (va) rest[va]--;
+                    if (vb) rest[vb]--;
+                    const uint64_t e = (uint64_t)at | (uint64_t)(na * nb) << 16 | (uint64_t)(va | vb << 4) << 32 | (uint64_t)set_of[rest] << 40;
+                    for (int j = 0; j < na * nb; j++) entry[at + j] = e;
+                    at += na * nb;
+                }
+            if (at != draws) return false;
         }
     }
 
     // ---- supports of 8, 12, 16, 24 coordinates: (w - n1 - n2, n1, n2) copies of k = 0, 1, 2 with 8 n1 + 24 n2 <= 48 - w
     std::map<int, uint32_t> first_a, first_b;
     static const int weights[4] = {8, 12, 16, 24};
+    std::vector<uint32_t> support;
+    std::vector<uint64_t> support24;
     for (int w : weights)
         for (int n2 = 0; 24 * n2 <= 48 - w; n2++)
             for (int n1 = 0; 8 * n1 + 24 * n2 <= 48 - w; n1++) {
                 int c[3] = {w - n1 - n2, n1, n2};
-                first_a[w << 16 | n1 << 8 | n2] = (uint32_t)u.tab_a.size();
-                list_orderings(c, 3, w, 0, 2, 0, u.tab_a);
+                first_a[w << 16 | n1 << 8 | n2] = (uint32_t)(w < 24 ? support.size() : support24.size());
+                if (w < 24) list_orderings(c, 3, w, 0, 2, 0, support); else list_orderings(c, 3, w, 0, 2, 0, support24);
             }
+    if (support.size() > kSupports || support24.size() > kSupports24) return false;
+    std::memcpy(u.blob.data() + kUnrankSupport, support.data(), support.size() * 4);
+    std::memcpy(u.blob.data() + kUnrankSupport24, support24.data(), support24.size() * 8);
     // ---- off-support values of 8, 12, 16 coordinates: n1, n2, n3 copies of k = 1, 2, 3 (and zeros) with
     // n1 + 4 n2 + 9 n3 <= 8 (w = 16), 12 (the last twelve coordinates of w = 0; w = 12 needs 9), 10 (w = 8)
     uint32_t *rest12 = part<uint32_t>(u.blob, kUnrankRest12);
@@ -126,9 +174,11 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
         e.flags = (uint32_t)d.odd | (uint32_t)d.w << 1 | (uint32_t)d.sign_bits << 6 | (uint32_t)d.nz_b << 11 | (uint32_t)d.shell << 16 |
                   (uint32_t)window_of(d) << 20;
         if (d.odd) {
-            e.a = d.cnt[0] | (uint32_t)d.cnt[1] << 8;
-            e.b = 0;
-            for (int v = 2; v < 7; v++) e.b |= (uint32_t)d.cnt[v] << (4 * (v - 2));
+            std::array<int, 7> c{};
+            for (int v = 1; v < 7; v++) c[v] = d.cnt[v];
+            const auto k = set_of.find(c);
+            if (k == set_of.end()) return false;
+            e.a = (uint32_t)k->second;
             continue;
         }
         e.golay = (uint32_t)t.weight_offset[d.w];
@@ -167,8 +217,13 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
             while (c + 1 < t.num_classes && slot_of(t.base[(size_t)c + 1]) < s) c++;
             guide[s] = (uint16_t)c;
         }
+        uint32_t *window = part<uint32_t>(u.blob, kUnrankWindow);
+        for (int s = 0; s < kGuideSlots; s++)
+            for (int c = guide[s]; c <= guide[s + 1]; c++)
+                if (desc[c].flags >> 20 != kWindowAlways) window[s >> 5] |= 1u << (s & 31);
     }
-    std::memcpy(u.blob.data() + kUnrankGolayMsg, t.golay_by_message.data(), 4096 * 4);
+    uint32_t *message = part<uint32_t>(u.blob, kUnrankGolayMsg);
+    for (int k = 0; k < 64; k++) { message[k] = t.golay_by_message[k]; message[64 + k] = t.golay_by_message[64 * k]; }
     std::memcpy(u.blob.data() + kUnrankGolayWt, t.golay_by_weight.data(), 4096 * 4);
 
     // ---- spreading eight nibbles to the places of a byte mask, and single bits likewise

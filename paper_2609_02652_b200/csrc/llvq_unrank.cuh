@@ -27,9 +27,10 @@
 namespace llvq {
 
 struct UnrankView {
-    const uint8_t *blob;
+    const uint8_t *blob;         // its first kUnrankSharedBytes are read here
+    const uint8_t *far;          // and the others here
+    const uint64_t *pairs;
     const uint32_t *tail8;
-    const uint64_t *tab_a;
     const uint32_t *tab_b;
 };
 
@@ -55,8 +56,18 @@ LLVQ_HD uint32_t float_bits(float f) {
     return c.u;
 #endif
 }
+// an estimate of a / b, a few units of the last place off at most
+LLVQ_HD float quotient(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fdividef(a, b);
+#else
+    return a / b;
+#endif
+}
 template <typename T>
 LLVQ_HD const T &blob_at(const UnrankView &v, int offset, uint32_t i) { return reinterpret_cast<const T *>(v.blob + offset)[i]; }
+template <typename T>
+LLVQ_HD const T &far_at(const UnrankView &v, int offset, uint32_t i) { return reinterpret_cast<const T *>(v.far + offset)[i]; }
 
 // bits 0..7 of b as the low bits of eight nibbles (the partial products do not overlap)
 LLVQ_HD uint32_t spread8(uint32_t b) {
@@ -78,10 +89,15 @@ LLVQ_HD uint32_t gather8(uint32_t w) {
     return (w | w >> 12) & 0xffu;
 }
 
+// slot of the class guide an index (below 2^48) lies in
+LLVQ_HD int guide_slot(uint64_t idx) {
+    const int s = (int)(float_bits(u64_to_float(idx)) >> kGuideShift) - kGuideFirst;
+    return s < 0 ? 0 : s;
+}
+
 // Class of a valid index: the last c with base[c] <= idx, searched between the guide's bounds.
 LLVQ_HD int find_class(const UnrankView &v, uint64_t idx) {
-    int s = (int)(float_bits(u64_to_float(idx)) >> kGuideShift) - kGuideFirst;
-    s = s < 0 ? 0 : s;
+    const int s = guide_slot(idx);
     int lo = blob_at<uint16_t>(v, kUnrankGuide, s), hi = blob_at<uint16_t>(v, kUnrankGuide, s + 1) + 1;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
@@ -94,48 +110,45 @@ LLVQ_HD int find_class(const UnrankView &v, uint64_t idx) {
 // 2^32: shifted right by left's power of two, the product times the inverse of left's odd part modulo 2^32.
 LLVQ_HD uint32_t portion(uint32_t T, uint32_t copies, const UnrankStep &e) { return (uint32_t)(((uint64_t)T * copies) >> e.shift) * e.inverse; }
 
-// Odd type.  The first sixteen coordinates are found one by one (three in four are the first or the second value tried), the
-// ordering of the last eight is an entry of a list.  Rolled up: the code of a step unrolled sixteen times does not fit the
-// instruction cache beside the rest.
+// Odd type.  Sixteen coordinates come two at a time from the table of draws, the ordering of the last eight is an entry of
+// a list.  The position of the draw is a float estimate, which the exact bounds of the pair it names confirm or, in one case
+// in some thousands, move to the pair before or after.  Rolled up: eight steps' code would crowd the instruction cache.
+// Instructions bound this: with the second eight coordinates one at a time from lists in shared memory (fewer gathers,
+// more instructions) 9728 x 2560 takes 46 us instead of 41.
 LLVQ_HD void unrank_odd(const UnrankView &v, const UnrankDesc &d, uint64_t r47, Point &p) {
-    const uint32_t cw = blob_at<uint32_t>(v, kUnrankGolayMsg, (uint32_t)r47 & 4095u);
-    uint32_t r = (uint32_t)(r47 >> 12), T = d.perm_a;
-    uint32_t n0 = d.a & 255u, n1 = d.a >> 8, more = d.b;     // copies of j = 0, 1, and of 2.. a nibble each
-    uint32_t word = 0;
+    const uint32_t message = (uint32_t)r47 & 4095u;
+    const uint32_t cw = blob_at<uint32_t>(v, kUnrankGolayMsg, message & 63u) ^ blob_at<uint32_t>(v, kUnrankGolayMsg, 64 + (message >> 6));
+    uint32_t r = (uint32_t)(r47 >> 12), T = d.perm_a, set = d.a, word = 0;
+    uint32_t begin, orderings;
 #ifdef __CUDA_ARCH__
 #pragma unroll 1
 #endif
-    for (int i = 0; i < 16; i++) {
-        const UnrankStep e = blob_at<UnrankStep>(v, kUnrankSteps, 24 - i);
-        uint32_t s = portion(T, n0, e), j = 0;
-        if (r < s) {
-            n0--;
-        } else {
-            r -= s;
-            s = portion(T, n1, e);
-            if (r < s) {
-                n1--;
-                j = 1;
-            } else {
-                r -= s;
-                uint32_t sh = 0;
-                s = portion(T, more & 15u, e);
-                while (r >= s && sh < 16u) {
-                    r -= s;
-                    sh += 4;
-                    s = portion(T, (more >> sh) & 15u, e);
-                }
-                more -= 1u << sh;
-                j = 2u + (sh >> 2);
-            }
+    for (int i = 0; i < kPairSteps; i++) {
+        const PairStep e = blob_at<PairStep>(v, kUnrankPairs, i);
+        uint32_t at = (uint32_t)quotient((float)r * (float)e.draws, (float)T);
+        at = at < e.draws ? at : e.draws - 1u;
+        uint64_t pair;
+        // 49 pairs at most: whatever the table holds, the loop ends
+#ifdef __CUDA_ARCH__
+#pragma unroll 1
+#endif
+        for (int tries = 0;; tries++) {
+            pair = v.pairs[e.first + set * e.draws + at];
+            const uint32_t first = (uint32_t)pair & 0xffffu, n = (uint32_t)pair >> 16;
+            begin = (uint32_t)(((uint64_t)T * first) >> e.shift) * e.inverse;
+            orderings = (uint32_t)(((uint64_t)T * n) >> e.shift) * e.inverse;
+            if (r - begin < orderings || tries == 49) break;       // r below begin wraps around
+            at = r < begin ? first - 1u : first + n;
+            at = at < e.draws ? at : e.draws - 1u;
         }
-        T = s;
-        word = word >> 4 | j << 28;
-        if (i == 7) p.mag[0] = word;
+        r -= begin;
+        T = orderings;
+        word = word >> 8 | (uint32_t)(pair >> 32) << 24;
+        set = (uint32_t)(pair >> 40);
+        if (i == kPairSteps / 2 - 1) p.mag[0] = word;
     }
     p.mag[1] = word;
-    const uint32_t key = (n1 | (more & 7u) << 4 | (more & 0x30u) << 3 | (more & 0x300u) << 1 | (more & 0x1000u) >> 1 | (more & 0x10000u) >> 4) & 8191u;
-    p.mag[2] = v.tail8[blob_at<uint16_t>(v, kUnrankTailBase, key) + r];
+    p.mag[2] = v.tail8[blob_at<uint16_t>(v, kUnrankTailBase, set & 255u) + r];
     // x_i = 1 + 2 c_i modulo 4: 1 + 2j is of the wrong residue, and so negated, where j's parity differs from c_i
 #pragma unroll
     for (int w = 0; w < 3; w++) p.neg[w] = (p.mag[w] & 0x11111111u) ^ spread8(cw >> (8 * w));
@@ -176,7 +189,7 @@ LLVQ_HD void unrank_even(const UnrankView &v, const UnrankDesc &d, uint64_t r, P
     const uint32_t w = (d.flags >> 1) & 31u, sign_bits = (d.flags >> 6) & 31u, nz_b = (d.flags >> 11) & 15u;
     const uint32_t sigma = (uint32_t)r & ((1u << sign_bits) - 1u);
     uint32_t rank_a, rank_b;
-    const uint32_t cw = blob_at<uint32_t>(v, kUnrankGolayWt, d.golay + divide(divide(r >> sign_bits, d.perm_b, d.inv_b, rank_b), d.perm_a, d.inv_a, rank_a));
+    const uint32_t cw = far_at<uint32_t>(v, kUnrankGolayWt, d.golay + divide(divide(r >> sign_bits, d.perm_b, d.inv_b, rank_b), d.perm_a, d.inv_a, rank_a));
     // signs of the support in order: the free ones, then the one that makes sum |x| / 4 + the number of negative support
     // coordinates even (an off-support sign does not matter: it changes the sum by a multiple of 8)
     uint32_t on = sigma >> nz_b, off = sigma & ((1u << nz_b) - 1u);
@@ -209,8 +222,8 @@ LLVQ_HD void unrank_even(const UnrankView &v, const UnrankDesc &d, uint64_t r, P
         }
         return;
     }
-    const uint64_t a = v.tab_a[d.a + rank_a];
     if (w == 24) {
+        const uint64_t a = far_at<uint64_t>(v, kUnrankSupport24, d.a + rank_a);
 #pragma unroll
         for (int j = 0; j < 3; j++) {
             p.mag[j] = 2u * spread_pairs((uint32_t)(a >> (16 * j))) + 0x11111111u;
@@ -221,7 +234,8 @@ LLVQ_HD void unrank_even(const UnrankView &v, const UnrankDesc &d, uint64_t r, P
     // the two sequences, a nibble a value: k in bits 0, 1, the sign in bit 2
     uint64_t in, out;
     {
-        const uint32_t lo = spread_pairs((uint32_t)a) | spread8(on) << 2, hi = spread_pairs((uint32_t)a >> 16) | spread8(on >> 8) << 2;
+        const uint32_t a = far_at<uint32_t>(v, kUnrankSupport, d.a + rank_a);
+        const uint32_t lo = spread_pairs(a) | spread8(on) << 2, hi = spread_pairs(a >> 16) | spread8(on >> 8) << 2;
         in = (uint64_t)hi << 32 | lo;
         const uint32_t b = v.tab_b[d.b + rank_b];
         const uint32_t blo = spread_pairs(b), bhi = spread_pairs(b >> 16);

@@ -4,9 +4,10 @@
 // An ordering of a multiset is ranked lexicographically.  Inside the ball there are few multisets: writing an odd
 // magnitude as 1 + 2j, sum x^2 <= 192 leaves sum j(j+1)/2 <= 21 over the 24 coordinates, 225 multisets in all; the
 // even type splits into the support (magnitudes 2 + 4k, a few k > 0) and the rest (4k).  So the orderings of what is
-// left after the first coordinates can be listed: 64 952 of eight odd magnitudes, 6511 of a support, 291 000 of
-// the rest of 8, 12 or 16 coordinates.  Those lists are the tables `tail8`, `tab_a` and `tab_b`; the small tables a
-// thread reads at random are one blob that a CTA copies to shared memory.
+// left after the first coordinates can be listed: 64 952 of eight odd magnitudes, 6511 of a support, 288 000 of
+// the rest of 8, 12 or 16 coordinates.  A thread reads its entries at random: what fits is in one
+// blob that a CTA copies to shared memory (a gather from there takes three or four wavefronts a warp, one from global
+// memory thirty-two).
 #pragma once
 #include <cstdint>
 #include <vector>
@@ -19,9 +20,8 @@ namespace llvq {
 struct UnrankDesc {
     uint32_t perm_a;      // odd: orderings of the 24 magnitudes; even: orderings of the support
     uint32_t perm_b;      // even: orderings off the support
-    uint32_t a;           // even: first entry in tab_a; odd: copies of magnitude 1 | copies of magnitude 3 << 8
-    uint32_t b;           // even, w = 8, 12, 16: first entry in tab_b; w = 0: copies of 0, 4, 8, 12 a byte each;
-                          // odd: copies of magnitudes 5, 7, 9, 11, 13, a nibble each
+    uint32_t a;           // even: first entry of the support's orderings; odd: the multiset's number
+    uint32_t b;           // even, w = 8, 12, 16: first entry in tab_b; w = 0: copies of 0, 4, 8, 12 a byte each
     float inv_a, inv_b;   // 1 / perm_a, 1 / perm_b
     uint32_t flags;       // odd | w << 1 | sign_bits << 6 | nz_b << 11 | repair << 15 | shell << 16 | window << 20
     uint32_t golay;       // first entry of weight w in the code sorted by weight
@@ -32,6 +32,17 @@ static_assert(sizeof(UnrankDesc) == 32, "UnrankDesc layout");
 struct UnrankStep {
     uint32_t inverse, shift;
 };
+
+// Two odd magnitudes at a time: with L coordinates left that have T orderings, T n / (L (L - 1)) begin with a given pair of
+// values, n the ways to draw the pair.  So the rank times L (L - 1) / T is a position among the L (L - 1) draws in order, and
+// the table `pairs` tells for every multiset and position the pair, the positions it takes and the multiset left.
+struct PairStep {
+    uint32_t inverse, shift;   // division by L (L - 1)
+    uint32_t first;            // of this L's entries in `pairs`
+    uint32_t draws;            // L (L - 1)
+};
+constexpr int kPairSteps = 8;                                         // L = 24, 22, .. 10
+constexpr int kOddSets = 225;                                         // multisets of non-zero j with sum j (j + 1) / 2 <= 21
 
 // flags >> 20: can a block of the class lack a window of the 10-byte layout, whatever its ordering and signs?
 enum { kWindowAlways = 0, kWindowDepends = 1, kWindowNever = 2 };
@@ -45,21 +56,28 @@ constexpr int kUnrankBase = 0;                                        // uint64[
 constexpr int kUnrankDescs = kUnrankBase + kUnrankClasses * 8;        // UnrankDesc[304]
 constexpr int kUnrankMerge = kUnrankDescs + kUnrankClasses * 32;      // uint4[256]: moves that spread nibbles to a byte mask's places
 constexpr int kUnrankSteps = kUnrankMerge + 256 * 16;                 // UnrankStep[32], by the number of coordinates left
-constexpr int kUnrankGuide = kUnrankSteps + 32 * 8;                   // uint16[kGuideSlots + 8]: first class of a slot
-constexpr int kUnrankGolayMsg = kUnrankGuide + (kGuideSlots + 8) * 2; // uint32[4096]: codeword of a message
-constexpr int kUnrankGolayWt = kUnrankGolayMsg + 4096 * 4;            // uint32[4096]: codewords by weight, then value
-constexpr int kUnrankTailBase = kUnrankGolayWt + 4096 * 4;            // uint16[8192]: first entry in tail8 of the last eight odd magnitudes
-constexpr int kUnrankDepositAt = kUnrankTailBase + 8192 * 2;          // uint16[256]: first entry in the deposit table of a byte mask
+constexpr int kUnrankPairs = kUnrankSteps + 32 * 8;                   // PairStep[8]
+constexpr int kUnrankWindow = kUnrankPairs + kPairSteps * 16;         // uint32[kGuideSlots / 32]: bit = a slot with a class that is not kWindowAlways
+constexpr int kUnrankGuide = kUnrankWindow + kGuideSlots / 8;         // uint16[kGuideSlots + 8]: first class of a slot
+constexpr int kUnrankGolayMsg = kUnrankGuide + (kGuideSlots + 8) * 2; // uint32[128]: codewords of the messages k and, from 64 on, 64 k, k < 64
+constexpr int kUnrankTailBase = kUnrankGolayMsg + 128 * 4;            // uint16[256]: first entry in tail8 of a multiset of eight odd magnitudes
+constexpr int kUnrankDepositAt = kUnrankTailBase + 256 * 2;      // uint16[256]: first entry in the deposit table of a byte mask
 constexpr int kUnrankDeposit = kUnrankDepositAt + 256 * 2;            // uint32[6561 + 15]: bits dealt to a mask's places, a nibble each
 constexpr int kUnrankRest12 = kUnrankDeposit + 6576 * 4;              // uint32[128]: first entry in tab_b of 12 off-support values
-constexpr int kUnrankBlobBytes = kUnrankRest12 + 128 * 4;
-static_assert(kUnrankDescs % 16 == 0 && kUnrankMerge % 16 == 0 && kUnrankGuide % 16 == 0 && kUnrankGolayMsg % 16 == 0 &&
-              kUnrankTailBase % 16 == 0 && kUnrankDeposit % 16 == 0 && kUnrankBlobBytes % 16 == 0, "alignment of the blob's parts");
+constexpr int kUnrankSharedBytes = kUnrankRest12 + 128 * 4;           // what follows stays in global memory
+constexpr int kUnrankSupport = kUnrankSharedBytes;                    // uint32[kSupports]: 8, 12 or 16 support values' k, two bits each
+constexpr int kSupports = 4192;
+constexpr int kUnrankSupport24 = kUnrankSupport + kSupports * 4;      // uint64[kSupports24]: 24 of them
+constexpr int kSupports24 = 2352;
+constexpr int kUnrankGolayWt = kUnrankSupport24 + kSupports24 * 8;
+constexpr int kUnrankBlobBytes = kUnrankGolayWt + 4096 * 4;
+static_assert(kUnrankDescs % 16 == 0 && kUnrankPairs % 16 == 0 && kUnrankWindow % 16 == 0 && kUnrankMerge % 16 == 0 && kUnrankGuide % 16 == 0 && kUnrankGolayMsg % 16 == 0 &&
+              kUnrankTailBase % 16 == 0 && kUnrankDeposit % 16 == 0 && kUnrankSupport24 % 16 == 0 && kUnrankBlobBytes % 16 == 0, "alignment of the blob's parts");
 
 struct UnrankTables {
     std::vector<uint8_t> blob;       // kUnrankBlobBytes
+    std::vector<uint64_t> pairs;     // first position | positions << 16 | pair << 32 (a nibble a value) | multiset left << 40
     std::vector<uint32_t> tail8;     // eight magnitudes' j, a nibble each, first coordinate lowest
-    std::vector<uint64_t> tab_a;     // w support values' k, two bits each
     std::vector<uint32_t> tab_b;     // 8, 12 or 16 off-support values' k, two bits each
 };
 
