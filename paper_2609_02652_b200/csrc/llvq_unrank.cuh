@@ -1,5 +1,5 @@
 // From an index of the ball to the 24 four-bit codes u_i = 8 + floor(x_i / 2) (and magnitudes, signs), with the tables of
-// llvq_unrank.h: `blob` in shared memory, the lists of orderings in global memory (1.3 MB, resident in L2).
+// llvq_unrank.h: the first part of `blob` in shared memory, the lists in global memory (5.6 MB, resident in L2).
 //
 // The index splits as the paper states it (Sec. 2.1: classes first, then arrangements and signs inside a class, as a
 // mixed-radix number).  The digit order used here:
@@ -114,7 +114,7 @@ LLVQ_HD uint32_t portion(uint32_t T, uint32_t copies, const UnrankStep &e) { ret
 // a list.  The position of the draw is a float estimate, which the exact bounds of the pair it names confirm or, in one case
 // in some thousands, move to the pair before or after.  Rolled up: eight steps' code would crowd the instruction cache.
 // Instructions bound this: with the second eight coordinates one at a time from lists in shared memory (fewer gathers,
-// more instructions) 9728 x 2560 takes 46 us instead of 41.
+// more instructions) 9728 x 2560 takes 46 us instead of 39.
 LLVQ_HD void unrank_odd(const UnrankView &v, const UnrankDesc &d, uint64_t r47, Point &p) {
     const uint32_t message = (uint32_t)r47 & 4095u;
     const uint32_t cw = blob_at<uint32_t>(v, kUnrankGolayMsg, message & 63u) ^ blob_at<uint32_t>(v, kUnrankGolayMsg, 64 + (message >> 6));
