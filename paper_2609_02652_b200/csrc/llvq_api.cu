@@ -230,7 +230,7 @@ int llvq_gemv_plan(int sm_count, const int64_t *rows, int n, int64_t k_padded, i
     if (k_padded <= 0 || k_padded % 24 != 0) return LLVQ_EINVAL;
     if (k_padded > LLVQ_MAX_K) return LLVQ_ESIZE;
     GemvParams p;
-    std::memset(&p, 0, sizeof p);
+    std::memset((void *)&p, 0, sizeof p);
     p.nprob = n;
     p.batch = batch;
     p.nb = (int)(k_padded / 24);
@@ -255,6 +255,27 @@ int llvq_gemv_plan(int sm_count, const int64_t *rows, int n, int64_t k_padded, i
     return LLVQ_OK;
 }
 
+// Completes the launch geometry in `p`: from the context's plans if one was made for these shapes, else anew.
+static GemvLaunch planned(llvq_ctx *ctx, int layout, GemvParams &p) {
+    PlanKey key;
+    std::memset(&key, 0, sizeof key);
+    key.layout = layout; key.nb = p.nb; key.batch = p.batch; key.rot_log2 = p.rot_log2; key.rot_n = p.rot_n; key.nprob = p.nprob;
+    for (int i = 0; i < p.nprob; i++) key.rows[i] = p.prob[i].rows;
+    for (int i = 0; i < ctx->plans_used; i++)
+        if (std::memcmp(&ctx->plans[i].key, &key, sizeof key) == 0) {
+            static_cast<GemvPlan &>(p) = ctx->plans[i].plan;
+            return ctx->plans[i].launch;
+        }
+    const GemvLaunch g = gemv_plan(layout, p, ctx->sm_count);
+    PlanEntry &e = ctx->plans[ctx->plans_next];
+    e.key = key;
+    e.plan = p;
+    e.launch = g;
+    if (ctx->plans_used < llvq_ctx::kPlans) ctx->plans_used++;
+    ctx->plans_next = (ctx->plans_next + 1) % llvq_ctx::kPlans;
+    return g;
+}
+
 static int run_gemv(llvq_ctx *ctx, int layout, const llvq_problem *problems, int n, const void *x, int64_t k_padded,
                     bool no_weights, void *stream, int batch = 1, const llvq_rotation *rot = nullptr) {
     if (!ctx || !problems || !x || n < 1 || n > LLVQ_MAX_GROUP) return LLVQ_EINVAL;
@@ -266,7 +287,7 @@ static int run_gemv(llvq_ctx *ctx, int layout, const llvq_problem *problems, int
     if (k_padded > LLVQ_MAX_K) return LLVQ_ESIZE;
     if (!aligned(x, 16)) return LLVQ_EALIGN;
     GemvParams p;
-    std::memset(&p, 0, sizeof p);
+    std::memset((void *)((char *)&p + sizeof(GemvPlan)), 0, sizeof p - sizeof(GemvPlan));     // the plan is written as a whole
     p.nprob = n;
     p.x = (const __half *)x;
     p.batch = batch;
@@ -332,7 +353,7 @@ static int run_gemv(llvq_ctx *ctx, int layout, const llvq_problem *problems, int
         p.rot_negate = rot->negate_bits;
         p.rot_scale = std::ldexp(1.0 / std::sqrt((double)((int64_t)1 << l)), -24);
     }
-    const GemvLaunch g = gemv_plan(layout, p, ctx->sm_count);
+    const GemvLaunch g = planned(ctx, layout, p);
     if (g.smem + 1024 > (size_t)ctx->max_smem_optin) return LLVQ_ESIZE;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;

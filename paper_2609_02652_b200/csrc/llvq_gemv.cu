@@ -1895,7 +1895,7 @@ extern "C" int llvq_gemv_static(const void *layout_buf, const void *row_scale, c
         }
     }
     GemvParams p;
-    memset(&p, 0, sizeof p);
+    memset((void *)&p, 0, sizeof p);
     p.nprob = 1;
     p.batch = 1;
     p.y_stride = (int)rows;

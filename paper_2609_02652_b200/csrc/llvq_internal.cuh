@@ -77,7 +77,18 @@ struct CtaShare {
     uint16_t blk_lo, blk_hi;
 };
 
-struct GemvParams {
+// What gemv_plan works out from the shapes of a launch alone.
+struct GemvPlan {
+    int units_base, units_rem;   // total_units divided by the warps of the grid (the one-hot arm's order)
+    int panel, npanels;          // unit columns a panel, panels (the 14-byte layout's order of work)
+    FastDiv div_panel, div_last; // by panel, by the last panel's width
+    int xblocks;                 // most blocks of x any CTA needs
+    uint32_t group_bytes;        // bytes of a row group's records
+    int rot_span;                // most coordinates any CTA rotates
+    CtaShare cta[kMaxGridCtas + 1];    // the share of every CTA of the grid; [grid].first is the total
+};
+
+struct GemvParams : GemvPlan {
     GemvProblemDev prob[LLVQ_MAX_GROUP];
     int nprob;
     const __half *x;             // batch vectors of 24 nb halves, one after the other
@@ -87,12 +98,6 @@ struct GemvParams {
     int units;             // units a row group: tiles, plus one for the nb mod 4 last columns
     int total_groups;
     int total_units;       // total_groups * units
-    int units_base, units_rem;   // total_units divided by the warps of the grid (set by gemv_plan; the one-hot arm's order)
-    int panel, npanels;          // unit columns a panel, panels (set by gemv_plan; the 14-byte layout's order of work)
-    FastDiv div_panel, div_last; // by panel, by the last panel's width
-    int xblocks;                 // most blocks of x any CTA needs (set by gemv_plan)
-    uint32_t group_bytes;        // bytes of a row group's records (set by gemv_plan)
-    CtaShare cta[kMaxGridCtas + 1];    // the share of every CTA of the grid; [grid].first is the total (set by gemv_plan)
     unsigned long long *accum;   // total_groups x 32 fixed-point row accumulators (context scratch, zero between launches)
     const float *cls_scale;
     const uint32_t *cls_parity;
@@ -104,9 +109,23 @@ struct GemvParams {
     // rotation of x inside the GEMV (llvq_gemv_rotated); rot_log2 = 0 means none
     int rot_log2;             // log2 of the rotation's block length (3..)
     int rot_n;                // coordinates rotated: a multiple of the block length, at most 24 nb
-    int rot_span;             // most coordinates any CTA rotates (set by gemv_plan)
     const uint32_t *rot_negate;   // sign-flip bits, or null
     double rot_scale;         // 2^-24 / sqrt(block length)
+};
+
+struct GemvLaunch {
+    int grid;
+    size_t smem;
+};
+// Everything gemv_plan looks at, and what it made of it.
+struct PlanKey {
+    int layout, nb, batch, rot_log2, rot_n, nprob;
+    int rows[LLVQ_MAX_GROUP];
+};
+struct PlanEntry {
+    PlanKey key;
+    GemvPlan plan;
+    GemvLaunch launch;
 };
 
 }  // namespace llvq
@@ -128,6 +147,10 @@ struct llvq_ctx {
     int weights_dirty;       // an expansion was enqueued since the last GEMV: that GEMV must not read records ahead of it
     int sm_count;
     int max_smem_optin;
+    // The plans of the last kPlans shapes launched (a decoder has four or five): 2 KB and half a microsecond each.
+    static constexpr int kPlans = 8;
+    llvq::PlanEntry plans[kPlans];
+    int plans_used, plans_next;
 };
 
 namespace llvq {
@@ -137,10 +160,6 @@ cudaError_t launch_expand(const llvq_ctx *ctx, int layout, const uint64_t *codes
 // device words that are zero before and after
 cudaError_t launch_overlay_count(const llvq_ctx *ctx, const uint64_t *codes, int64_t rows, int64_t nb, unsigned long long *counter,
                                  unsigned long long *host, cudaStream_t s);
-struct GemvLaunch {
-    int grid;
-    size_t smem;
-};
 // Completes the launch geometry in `p` (order of work, shares of x) and returns grid and dynamic shared memory.
 GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count);
 void gemv_lane_table(uint32_t (*out)[4]);      // fills the 32 entries of DeviceTables::lane_table (host)

@@ -383,6 +383,41 @@ def test_gemv_batch_of_more_than_four(B, ctx, rows, nb, batch):
         small.close()
 
 
+def test_more_shapes_than_kept_plans(B):
+    """A context keeps the plans of a few shapes: shapes that push each other out, grouped, batched and rotated launches of
+    the same rows among them, give the bits of a context that has seen nothing else."""
+    shapes = [(32 + 40 * i, 24 * (3 + 5 * i)) for i in range(7)]
+    cases = [make_case(r, k, seed=r) for r, k in shapes]
+    c0 = B.create(0)
+    bufs = [B.expand(c0, 0, c.d_codes, c.rows, c.nb) for c in cases]
+
+    def launches(c):
+        out = []
+        for case, buf in zip(cases, bufs):
+            kp = case.nb * 24
+            out.append(B.gemv(c, 0, buf, case.d_scale, GAIN, case.d_x, case.rows, kp))
+            out.append(B.gemv_batch(c, buf, case.d_scale, GAIN, torch.stack([case.d_x, -case.d_x]), case.rows, kp))
+            ys = [torch.empty(case.rows, dtype=torch.float32, device="cuda") for _ in range(2)]
+            B.gemv_grouped(c, 0, [(buf, case.d_scale, GAIN, y, case.rows) for y in ys], case.d_x, kp)
+            yr = torch.empty(case.rows, dtype=torch.float32, device="cuda")
+            B.gemv_rotated(c, [(buf, case.d_scale, GAIN, yr, case.rows)], case.d_x, kp, n=kp, block=8)
+            out += [*ys, yr]
+        return out
+
+    first, again = launches(c0), launches(c0)
+    for i, (a, b) in enumerate(zip(first, again)):
+        assert torch.equal(a, b)
+        if i % 5 == 2:
+            assert torch.equal(a, first[i - 2])      # grouped = alone
+    fresh = B.create(0)
+    try:
+        case, buf = cases[3], bufs[3]
+        assert torch.equal(B.gemv(fresh, 0, buf, case.d_scale, GAIN, case.d_x, case.rows, case.nb * 24), first[15])
+    finally:
+        fresh.close()
+        c0.close()
+
+
 def test_gemv_batch_limits(B, ctx):
     case = make_case(64, 96, seed=1)
     buf = B.expand(ctx, 0, case.d_codes, case.rows, case.nb)
