@@ -350,7 +350,8 @@ int llvq_rotate(llvq_ctx *ctx, const void *x, void *y, const uint32_t *negate_bi
 int64_t llvq_rotate_block(int64_t n, int64_t block);
 
 /* Decoded weights as fp16, W[row*k_padded + 24b + i] = fp16(row_scale * gain[g] * x_i / (4 sqrt m))
- * (product formed in f32, rounded once).  Feeds llvq_gemv_fp16. */
+ * (product formed in f32, rounded once).  Feeds llvq_gemv_fp16.  For LLVQ_PLANES the launch is a link of the
+ * programmatic-dependent-launch chain (llvq_set_pdl), one that waits for the kernel before it ahead of all it reads and writes. */
 int llvq_dequant_fp16(llvq_ctx *ctx, int layout, const void *layout_buf, const void *row_scale,
                       const float *gain, void *W, int64_t rows, int64_t k_padded, void *stream);
 

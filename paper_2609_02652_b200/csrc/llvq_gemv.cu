@@ -1555,78 +1555,135 @@ __global__ void __launch_bounds__(256) dequant_onehot_kernel(const uint8_t *__re
     store_block_fp16(W + (row * nb + b) * 24, __half2float(row_scale[row]) * ((gain ? g1 : g0) * (cls_scale[cls] * (1.0f / 2097152.0f))), x);
 }
 
-// 14-byte layout -> FP16.  Bound: HBM, nearly all of it the weights written (48 bytes a block, 14 read).  A warp takes a tile;
-// lane 4g+t's words hold four consecutive coordinates of a row at each of the positions 4t, 16+4t, 32+4t of a half-step,
-// so it stores them as they are decoded, eight bytes at a time, the four lanes of a quad side by side: every store fills
-// whole 32-byte sectors of eight rows (where a row begins on one) and needs no exchange between lanes.  A block of
-// 24 coordinates a lane, stored two bytes at a time, took 490 us for 4096 x 12288 (265 GB/s), its stores throttled; this 25 us
-// (5150 GB/s of the 62 bytes a block, 0.79 of a copy).
-constexpr int kDequantWarps = 8;
+// 14-byte layout -> FP16.  Bound: HBM writes (48 bytes a block written, 14 read): 22.7 us for 4096 x 12288 (5740 GB/s of the
+// 62 bytes a block), where a plain fill of the weights alone takes 30.  A warp takes a tile; lane 4g+t's words hold four
+// consecutive coordinates of a row at each of the positions 4t, 16+4t, 32+4t of a half-step, so it stores them as they are
+// decoded, eight bytes at a time, the four lanes of a quad side by side: a store fills whole 32-byte sectors of eight rows
+// and needs no exchange between lanes.  (A block of 24 coordinates a lane, stored two bytes at a time: 490 us, its stores throttled.)
+// Where a row begins in the middle of a sector (every other row if nb is odd) the quad's first two lanes run one store
+// ahead of the last two, so that the sectors are whole there, too (2022 x 7890: 14.6 us without that, 12.5 with it).  Where every
+// row begins on a sector (WHOLE_SECTORS) that would cost 4 % for nothing, and is left out.
+// A tile a warp and no loop, the class table formed while the previous kernel of the stream ends: 25.3 -> 22.7 us for
+// 4096 x 12288, 45.6 -> 37.1 for 17408 x 5120, 12.5 -> 8.5 for 2022 x 7890.  Four warps a CTA: eight 9.7 us for the last; class
+// constants from global memory instead of a table 10.3.
+constexpr int kDequantWarps = 4;
+// The lane's twelve coordinates of a half-step's row as three groups of four halves.  Four codes, doubled, a byte each:
+// 2^22 + u by its bits, then x / 2 = u + (parity - 16) / 2, exactly, and one rounding of the product with twice the scale.
+__device__ __forceinline__ void dequant_row(uint32_t own, uint32_t shared, int e, float2 k0, float2 k1, float r, bool first_slot, uint2 v[3]) {
+    const float s0 = 2.f * (r * k0.x), s1 = 2.f * (r * k1.x);
+    auto four = [](uint32_t codes, float scale, float offset) {
+        float f[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) f[i] = scale * (__uint_as_float(__byte_perm(codes, 0x4a800000u, 0x7650 + i)) + offset);
+        const __half2 lo = __floats2half2_rn(f[0], f[1]), hi = __floats2half2_rn(f[2], f[3]);
+        return make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+    };
+    v[0] = four((own << 1) & 0x1e1e1e1eu, s0, k0.y);
+    v[1] = four((own >> 3) & 0x1e1e1e1eu, first_slot ? s0 : s1, first_slot ? k0.y : k1.y);
+    v[2] = four((e ? shared >> 3 : shared << 1) & 0x1e1e1e1eu, s1, k1.y);
+}
+// Stores N groups, 32 bytes a quad and group from `dst` (this lane's place in the first) on.
+template <int N>
+__device__ __forceinline__ void store_groups(__half *dst, const uint2 (&v)[N], bool ahead) {
+#pragma unroll
+    for (int j = -1; j < N; j++) {
+        if (j < 0 ? ahead : (j < N - 1 || !ahead)) {
+            const uint2 &behind = v[j < 0 ? 0 : j], &front = v[j + 1 < N ? j + 1 : N - 1];
+            __stcs(reinterpret_cast<uint2 *>(dst + 16 * (j + (ahead ? 1 : 0))), make_uint2(ahead ? front.x : behind.x, ahead ? front.y : behind.y));
+        }
+    }
+}
+template <bool WHOLE_SECTORS>
 __global__ void __launch_bounds__(kDequantWarps * 32) dequant_planes_kernel(const uint8_t *__restrict__ buf, const __half *__restrict__ row_scale,
                                                                             float g0, float g1, __half *__restrict__ W, int64_t rows, int64_t nb,
-                                                                            uint32_t total_units, const uint32_t *cls_parity, const uint8_t *cls_dist,
-                                                                            const float2 *__restrict__ cls_block) {
+                                                                            uint32_t total_units, const float2 *__restrict__ cls_block) {
     // (class | gain << 9) -> {gain / (4 sqrt m), (parity - 16) / 2 - 2^22}
     __shared__ float2 tab[2 * kClassSlots];
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const uint32_t tiles = (uint32_t)(nb / kTileCells), left = (uint32_t)(nb % kTileCells), units = tiles + (left ? 1 : 0);
+    const uint32_t unit = blockIdx.x * kDequantWarps + (threadIdx.x >> 5), rg = unit / units, u = unit % units;
+    const int64_t row0 = (int64_t)rg * kRowsPerGroup;
+    const uint8_t *src = buf + (size_t)rg * ((size_t)nb * kCellBytes) + (size_t)u * kTileBytes;
+    const bool whole = unit < total_units && u < tiles;
     for (int c = threadIdx.x; c < kClassSlots; c += blockDim.x) {
         const float2 k = __ldg(cls_block + c);
         const float offset = 0.5f * (float)(__float_as_int(k.y) - 8388608);
         tab[c] = make_float2(g0 * k.x, offset);
         tab[c + kClassSlots] = make_float2(g1 * k.x, offset);
     }
+    // the table is formed while the previous kernel of the stream finishes; only then may records be read or W written
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    uint4 w0, w1, w2, ha, hb;
+    if (whole) {                
+        w0 = __ldcs(reinterpret_cast<const uint4 *>(src + 16 * lane)); w1 = __ldcs(reinterpret_cast<const uint4 *>(src + 512 + 16 * lane));
+        w2 = __ldcs(reinterpret_cast<const uint4 *>(src + 1024 + 16 * lane));
+        ha = __ldcs(reinterpret_cast<const uint4 *>(src + 1536 + 32 * g)); hb = __ldcs(reinterpret_cast<const uint4 *>(src + 1552 + 32 * g));
+    }
     __syncthreads();
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const uint32_t tiles = (uint32_t)(nb / kTileCells), left = (uint32_t)(nb % kTileCells), units = tiles + (left ? 1 : 0);
-    for (uint32_t unit = blockIdx.x * kDequantWarps + (threadIdx.x >> 5); unit < total_units; unit += gridDim.x * kDequantWarps) {
-        const uint32_t rg = unit / units, u = unit % units;
-        const int64_t row0 = (int64_t)rg * kRowsPerGroup;
-        if (u == tiles) {
-            // the nb mod 4 last blocks: a lane a row, a block at a time
-            const int64_t row = row0 + lane;
-            if (row >= rows) continue;
-            const float r = __half2float(row_scale[row]);
-            for (int64_t b = (int64_t)tiles * kTileCells; b < nb; b++) {
-                int cls, gain, x[24];
-                record_coords(LLVQ_PLANES, buf, rows, nb, rg, b, lane, cls_parity, cls_dist, cls, gain, x);
-                store_block_fp16(W + (row * nb + b) * 24, r * tab[cls | gain << 9].x, x);
-            }
-            continue;
-        }
-        const uint8_t *tile = buf + (size_t)rg * ((size_t)nb * kCellBytes) + (size_t)u * kTileBytes;
-        const uint4 w0 = __ldcs(reinterpret_cast<const uint4 *>(tile + 16 * lane)), w1 = __ldcs(reinterpret_cast<const uint4 *>(tile + 512 + 16 * lane));
-        const uint4 w2 = __ldcs(reinterpret_cast<const uint4 *>(tile + 1024 + 16 * lane));
-        const uint4 ha = __ldcs(reinterpret_cast<const uint4 *>(tile + 1536 + 32 * g)), hb = __ldcs(reinterpret_cast<const uint4 *>(tile + 1552 + 32 * g));
+    if (unit >= total_units) return;
+    // coordinate 4t of the unit's first block in a row, and whether that row begins inside a sector there
+    auto place = [&](int64_t row) { return W + (row * nb + (int64_t)u * kTileCells) * 24 + 4 * t; };
+    auto runs_ahead = [&](const __half *dst) { return !WHOLE_SECTORS && t < 2 && ((reinterpret_cast<uintptr_t>(dst - 4 * t)) & 16) != 0; };
+    auto constants = [&](uint32_t header, int e) { return tab[(header >> (16 * e)) & 1023u]; };
+    if (whole) {
         const uint32_t words[12] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w, w2.x, w2.y, w2.z, w2.w};
-        const uint32_t head[2][4] = {{ha.x, ha.y, ha.z, ha.w}, {hb.x, hb.y, hb.z, hb.w}};      // [slot][half-step]
+        const uint32_t head[2][4] = {{ha.x, ha.y, ha.z, ha.w}, {hb.x, hb.y, hb.z, hb.w}};  // [slot][half-step]
 #pragma unroll
-        for (int m = 0; m < 2; m++) {
+        for (int m = 0; m < 2; m++)
 #pragma unroll
             for (int e = 0; e < 2; e++) {
                 const int64_t row = row0 + 16 * m + 8 * e + g;
                 if (row >= rows) continue;
                 const float r = __half2float(row_scale[row]);
-                // coordinate 4t of the tile's first block of the row
-                __half *dst = W + (row * nb + (int64_t)u * kTileCells) * 24 + 4 * t;
+                uint2 v[6];
 #pragma unroll
                 for (int s = 0; s < 2; s++) {
                     const int h = 2 * s + m;
-                    const float2 k0 = tab[(head[0][h] >> (16 * e)) & 1023u], k1 = tab[(head[1][h] >> (16 * e)) & 1023u];
-                    const float s0 = 2.f * (r * k0.x), s1 = 2.f * (r * k1.x);
-                    const uint32_t own = words[3 * h + e], shared = words[3 * h + 2];
-                    // four codes, doubled, a byte each, to four halves: 2^22 + u by its bits, then x / 2 = u + (parity - 16) / 2, exactly,
-                    // and one rounding of the product with twice the scale
-                    auto put = [&](int at, uint32_t codes, float scale, float offset) {
-                        float f[4];
-#pragma unroll
-                        for (int i = 0; i < 4; i++) f[i] = scale * (__uint_as_float(__byte_perm(codes, 0x4a800000u, 0x7650 + i)) + offset);
-                        const __half2 lo = __floats2half2_rn(f[0], f[1]), hi = __floats2half2_rn(f[2], f[3]);
-                        __stcs(reinterpret_cast<uint2 *>(dst + 48 * s + at),
-                               make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi)));
-                    };
-                    put(0, (own << 1) & 0x1e1e1e1eu, s0, k0.y);
-                    put(16, (own >> 3) & 0x1e1e1e1eu, t < 2 ? s0 : s1, t < 2 ? k0.y : k1.y);
-                    put(32, (e ? shared >> 3 : shared << 1) & 0x1e1e1e1eu, s1, k1.y);
+                    dequant_row(words[3 * h + e], words[3 * h + 2], e, constants(head[0][h], e), constants(head[1][h], e), r, t < 2, v + 3 * s);
                 }
+                __half *dst = place(row);
+                store_groups(dst, v, runs_ahead(dst));
+            }
+        return;
+    }
+    // the nb mod 4 last blocks: a pair, a single, or both
+    const uint32_t *word = reinterpret_cast<const uint32_t *>(src);
+    if (left >= 2) {
+#pragma unroll
+        for (int m = 0; m < 2; m++)
+#pragma unroll
+            for (int e = 0; e < 2; e++) {
+                const int64_t row = row0 + 16 * m + 8 * e + g;
+                if (row >= rows) continue;
+                const float r = __half2float(row_scale[row]);
+                uint2 v[3];
+                // header word m of lane pairs 2g and 2g + 1
+                dequant_row(word[32 * (3 * m + e) + lane], word[32 * (3 * m + 2) + lane], e, constants(word[192 + 4 * g + m], e),
+                            constants(word[192 + 4 * g + 2 + m], e), r, t < 2, v);
+                __half *dst = place(row);
+                store_groups(dst, v, runs_ahead(dst));
+            }
+        word += 2 * kCellBytes / 4;
+    }
+    if (left & 1) {
+        // slot s of the half-step is rows 16 s .. 16 s + 15 of the last block
+#pragma unroll
+        for (int e = 0; e < 2; e++) {
+            const int64_t row = row0 + 8 * e + g;
+            const float r0 = row < rows ? __half2float(row_scale[row]) : 0.f, r1 = row + 16 < rows ? __half2float(row_scale[row + 16]) : 0.f;
+            float2 k0 = constants(word[96 + 2 * g], e), k1 = constants(word[96 + 2 * g + 1], e);
+            k0.x *= r0; k1.x *= r1;
+            uint2 v[3];
+            dequant_row(word[32 * e + lane], word[64 + lane], e, k0, k1, 1.f, t < 2, v);
+            __half *first = W + (row * nb + nb - 1) * 24, *second = W + ((row + 16) * nb + nb - 1) * 24;
+            if (row < rows) {
+                __stcs(reinterpret_cast<uint2 *>(first + 4 * t), v[0]);
+                if (t < 2) __stcs(reinterpret_cast<uint2 *>(first + 16 + 4 * t), v[1]);
+            }
+            if (row + 16 < rows) {
+                if (t >= 2) __stcs(reinterpret_cast<uint2 *>(second + 4 * (t - 2)), v[1]);
+                __stcs(reinterpret_cast<uint2 *>(second + 8 + 4 * t), v[2]);
             }
         }
     }
@@ -1788,10 +1845,18 @@ cudaError_t launch_dequant(const llvq_ctx *ctx, int layout, const uint8_t *buf, 
         return cudaGetLastError();
     }
     const int64_t units = groups * (nb / kTileCells + (nb % kTileCells ? 1 : 0));
-    const int64_t blocks = (units + kDequantWarps - 1) / kDequantWarps, most = (int64_t)ctx->sm_count * 8;
-    dequant_planes_kernel<<<(unsigned)(blocks < most ? blocks : most), kDequantWarps * 32, 0, s>>>(buf, row_scale, g0, g1, W, rows, nb, (uint32_t)units, ctx->dev.cls_parity,
-                                                                                                  ctx->dev.cls_dist, ctx->dev.cls_block);
-    return cudaGetLastError();
+    const bool whole_sectors = nb % 2 == 0 && reinterpret_cast<uintptr_t>(W) % 32 == 0;
+    auto kernel = whole_sectors ? dequant_planes_kernel<true> : dequant_planes_kernel<false>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((units + kDequantWarps - 1) / kDequantWarps));
+    cfg.blockDim = dim3(kDequantWarps * 32);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = ctx->use_pdl ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, buf, row_scale, g0, g1, W, rows, nb, (uint32_t)units, (const float2 *)ctx->dev.cls_block);
 }
 
 cudaError_t launch_decode_i8(const llvq_ctx *ctx, int layout, const uint8_t *buf, int8_t *coords, uint16_t *class_ids,
