@@ -287,7 +287,7 @@ static int run_gemv(llvq_ctx *ctx, int layout, const llvq_problem *problems, int
     if (k_padded > LLVQ_MAX_K) return LLVQ_ESIZE;
     if (!aligned(x, 16)) return LLVQ_EALIGN;
     GemvParams p;
-    std::memset((void *)((char *)&p + sizeof(GemvPlan)), 0, sizeof p - sizeof(GemvPlan));     // the plan is written as a whole
+    std::memset(static_cast<void *>(static_cast<GemvCall *>(&p)), 0, sizeof(GemvCall));     // the plan is written as a whole
     p.nprob = n;
     p.x = (const __half *)x;
     p.batch = batch;
