@@ -351,7 +351,7 @@ static int run_gemv(llvq_ctx *ctx, int layout, const llvq_problem *problems, int
         p.rot_log2 = l;
         p.rot_n = (int)rot->n;
         p.rot_negate = rot->negate_bits;
-        p.rot_scale = std::ldexp(1.0 / std::sqrt((double)((int64_t)1 << l)), -24);
+        p.rot_scale = std::ldexp(1.0 / std::sqrt((double)((int64_t)1 << l)), 1008);
     }
     const GemvLaunch g = planned(ctx, layout, p);
     if (g.smem + 1024 > (size_t)ctx->max_smem_optin) return LLVQ_ESIZE;

@@ -577,9 +577,11 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
     float2 *tab = reinterpret_cast<float2 *>(smem + kWarps * kSlots * kTileBytes + tab_pad);
     unsigned char *xrec = smem + kWarps * kSlots * kTileBytes + tab_pad + p.nprob * 8192;
     constexpr int kXBlock = BATCH * kXRecBytes;                                    // the vectors' records of a block lie side by side
-    uint64_t *bars = reinterpret_cast<uint64_t *>(xrec + ((p.xblocks * kXBlock + 127) / 128) * 128);
+    // ROTATE: the records take the place of the FP16 values that are rotated
+    const int xrec_bytes = ROTATE ? max(p.xblocks * kXBlock, 2 * p.rot_span) : p.xblocks * kXBlock;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(xrec + ((xrec_bytes + 127) / 128) * 128);
     uint32_t *warp_max = reinterpret_cast<uint32_t *>(bars + kWarps * kSlots);     // one slot a warp and vector
-    long long *rot = reinterpret_cast<long long *>(warp_max + BATCH * kWarps);     // ROTATE: the exact sums of this CTA's blocks of x
+    double *rot = reinterpret_cast<double *>(warp_max + BATCH * kWarps);           // ROTATE: the sums of this CTA's part of x
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t my_ring = smem_addr(ring + warp * kSlots * kTileBytes);
     const uint32_t my_bar = smem_addr(bars + warp * kSlots);
@@ -839,9 +841,9 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
         // The rotated vector's largest magnitude is not known before it is rotated, but every rotated coordinate is
         // a unit-norm combination of its block, so |x'_k| <= ||x||_2: the scan sums the squares instead of taking
         // the maximum, and the fixed-point scale follows from that bound (a few bits coarser than the maximum
-        // would give, of 29).  In the same pass the pieces of this CTA's rotation blocks become integers, take
-        // their first three stages in registers and go to shared memory; the later stages follow there; the
-        // rounded FP16 values - bit for bit those of the rotation kernel - become the fixed-point records.
+        // would give, of 29).  In the same pass the pieces of this CTA's rotation blocks go to shared memory, signs flipped;
+        // the stages follow there, three a pass and the last three in registers; the rounded FP16 values - those of
+        // the rotation kernel - become the fixed-point records.
         const int nx = p.nb * 3, e_lo = 3 * blk_lo, e_hi = 3 * blk_hi;
         const bool one_each = e_hi - e_lo <= kThreads;
         const uint4 *xg = reinterpret_cast<const uint4 *>(p.x);
@@ -855,11 +857,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 const int e = base + i * kThreads + tid;
                 v[i] = e < nx ? __ldcg(xg + e) : make_uint4(0u, 0u, 0u, 0u);
             }
-            if (base == 0) {
-                for (int b = tid; b < blk_hi - blk_lo; b += kThreads)
-                    asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(smem_addr(xrec) + b * kXRecBytes + 96), "r"(0) : "memory");
-                build_tables();
-            }
+            if (base == 0) build_tables();
 #pragma unroll
             for (int i = 0; i < 4; i++) {
                 const int e = base + i * kThreads + tid;
@@ -871,11 +869,9 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                     ss = fmaf(f.y, f.y, ss);
                 }
                 if (8 * e >= c_lo && 8 * e < c_hi) {
-                    long long a[8];
-                    const uint32_t flips = p.rot_negate ? (__ldg(p.rot_negate + (e >> 2)) >> (8 * (e & 3))) & 0xffu : 0u;
-                    rot_load8(v[i], flips, a);
-                    rot_butterflies<3>(a);
-                    rot_store8(rot, 8 * e - c_lo, a);
+                    const uint32_t flips = p.rot_negate ? __ldg(p.rot_negate + (e >> 2)) >> (8 * (e & 3)) : 0u;
+                    auto flipped = [&](int k) { return w[k] ^ ((flips >> (2 * k) & 1u) << 15) ^ ((flips >> (2 * k + 1) & 1u) << 31); };
+                    *reinterpret_cast<uint4 *>(xrec + 2 * (8 * e - c_lo)) = make_uint4(flipped(0), flipped(1), flipped(2), flipped(3));
                 } else if (e >= e_lo && e < e_hi) {
                     mine = v[i];
                     mine_e = e;
@@ -885,8 +881,38 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
         if (lane == 0) warp_max[warp] = __float_as_uint(ss);
-        __syncthreads();                               // publishes the sums of squares, the first stages, the block constants
-        rot_later_passes(rot, p.rot_log2, c_hi - c_lo, tid, kThreads);
+        __syncthreads();                               // publishes the sums of squares, the values, the block constants
+        if (!NO_WEIGHTS) {
+#pragma unroll
+            for (int s = kEarlySlots; s < kSlots; s++) issue(my_bar + 8 * s, my_ring + s * kTileBytes);
+        }
+        const int need_lo = min(p.rot_n, 24 * blk_lo), need_hi = min(p.rot_n, 24 * blk_hi);
+        auto down = [&](int s) { return need_lo & ~((1 << s) - 1); };
+        auto up = [&](int s) { return (need_hi + (1 << s) - 1) & ~((1 << s) - 1); };
+        const RotFirst rf = rot_first(p.rot_log2);
+        const int rot0 = down(rf.stride);              // the coordinate in the first place of `rot`
+        {
+            const __half *raw = reinterpret_cast<const __half *>(xrec);
+            if (rf.stages == 3) rot_narrow<3, true>(rot, rot0, raw, c_lo, c_hi, rot0, up(rf.stride), rf.stride, tid, kThreads);
+            else if (rf.stages == 2) rot_narrow<2, true>(rot, rot0, raw, c_lo, c_hi, rot0, up(rf.stride), rf.stride, tid, kThreads);
+            else if (rf.stages == 1) rot_narrow<1, true>(rot, rot0, raw, c_lo, c_hi, rot0, up(rf.stride), rf.stride, tid, kThreads);
+            else rot_narrow<0, true>(rot, rot0, raw, c_lo, c_hi, rot0, up(rf.stride), rf.stride, tid, kThreads);
+        }
+        __syncthreads();
+        // the zero word and the two sums of every record, now that the FP16 values are read
+        for (int b = tid; b < blk_hi - blk_lo; b += kThreads)
+            asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(smem_addr(xrec) + b * kXRecBytes + 96), "r"(0) : "memory");
+        // down to pieces of 64, whose last six stages a group of eight lanes takes by itself (or of 8, for short blocks)
+        const int last = rf.stride >= 6 ? 6 : 3;
+        for (int s = rf.stride; s > last;) {
+            const int wide = s, r = s % 3 ? s % 3 : 3;
+            s -= r;
+            if (r == 3) rot_narrow<3, false>(rot, rot0, nullptr, down(wide), up(wide), down(s), up(s), s, tid, kThreads);
+            else if (r == 2) rot_narrow<2, false>(rot, rot0, nullptr, down(wide), up(wide), down(s), up(s), s, tid, kThreads);
+            else rot_narrow<1, false>(rot, rot0, nullptr, down(wide), up(wide), down(s), up(s), s, tid, kThreads);
+            if (s > last) __syncthreads();
+        }
+        __syncthreads();
         {
             // every thread of every CTA adds the sixteen sums in the same order
             float total = __uint_as_float(warp_max[lane & (kWarps - 1)]);
@@ -900,15 +926,17 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
         const float scale = pow2f(29 - xexp[0]);
         // rotated pieces: from the exact sums; pieces past the rotated length: as they are (the one this thread
         // met in the scan, or read again when the share is too wide for that)
-        for (int e = e_lo + tid; e < e_hi; e += kThreads) {
-            if (8 * e < c_hi) convert_item(rot_round8(rot, 8 * e - c_lo, p.rot_scale), e % 3, xs0 + (uint32_t)(e / 3) * kXRecBytes, scale);
-            else if (!one_each) convert_item(__ldcg(xg + e), e % 3, xs0 + (uint32_t)(e / 3) * kXRecBytes, scale);
+        for (int e0 = (down(last) >> 3) + 32 * warp; 8 * e0 < need_hi; e0 += kThreads) {
+            const int e = e0 + lane;
+            if (last == 6) {
+                if (8 * e < up(6)) rot_middle8(rot, 8 * e - rot0);
+                __syncwarp();
+            }
+            if (e >= e_lo && 8 * e < need_hi) convert_item(rot_finish8(rot, 8 * e - rot0, p.rot_scale), e % 3, xs0 + (uint32_t)(e / 3) * kXRecBytes, scale);
         }
+        if (!one_each)
+            for (int e = max(e_lo, c_hi >> 3) + tid; e < e_hi; e += kThreads) convert_item(__ldcg(xg + e), e % 3, xs0 + (uint32_t)(e / 3) * kXRecBytes, scale);
         if (one_each && mine_e >= 0) convert_item(mine, mine_e % 3, xs0 + (uint32_t)(mine_e / 3) * kXRecBytes, scale);
-        if (!NO_WEIGHTS) {
-#pragma unroll
-            for (int s = kEarlySlots; s < kSlots; s++) issue(my_bar + 8 * s, my_ring + s * kTileBytes);
-        }
         __syncthreads();                               // publishes the x records
     } else {
         const int nx = p.nb * 3, e_lo = 3 * blk_lo, e_hi = 3 * blk_hi;
@@ -1742,7 +1770,7 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
     // the stretch of x a CTA meets: the whole panels its units lie in (consecutive ones); the CTAs' first units ascend, so
     // the panel they lie in is stepped on from one to the next
     p.xblocks = 0;
-    p.rot_span = 0;
+    p.rot_span = p.rot_keep = 0;
     const int64_t panel_units = (int64_t)p.total_groups * p.panel;
     int panel = 0;
     int64_t panel_end = panel_units;                   // the last panel has no end
@@ -1766,12 +1794,19 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
             if (c_lo > p.rot_n) c_lo = p.rot_n;
             if (c_hi > p.rot_n) c_hi = p.rot_n;
             if (c_hi - c_lo > p.rot_span) p.rot_span = c_hi - c_lo;
+            const int piece = (1 << rot_first(p.rot_log2).stride) - 1;
+            const int need_lo = 24 * lo < p.rot_n ? 24 * lo : p.rot_n, need_hi = 24 * hi < p.rot_n ? 24 * hi : p.rot_n;
+            const int keep = ((need_hi + piece) & ~piece) - (need_lo & ~piece);
+            if (keep > p.rot_keep) p.rot_keep = keep;
         }
     }
     const int vectors = p.batch <= 2 ? p.batch : (p.batch <= 4 ? 4 : 8);       // the kernel is built for 1, 2, 4 and 8
     const int warps = gemv_warps(vectors);
-    const size_t xbytes = ((size_t)p.xblocks * kXRecBytes * vectors + 127) / 128 * 128;
-    g.smem = (size_t)warps * kSlots * kTileBytes + 8192 /* alignment of the tables */ + (size_t)p.nprob * 8192 + xbytes + warps * kSlots * 8 + warps * 4 * vectors + 16 + (size_t)p.rot_span * 8;
+    const size_t records = ((size_t)p.xblocks * kXRecBytes * vectors + 127) / 128 * 128, raw = ((size_t)p.rot_span * 2 + 127) / 128 * 128;
+    g.smem = (size_t)warps * kSlots * kTileBytes + 8192 /* alignment of the tables */ + (size_t)p.nprob * 8192 + warps * kSlots * 8 + warps * 4 * vectors + 16;
+    // a rotation counts with eight bytes a coordinate of its whole blocks, the limit llvq_gemv_rotated states, though it needs less
+    const size_t rot_needs = (records > raw ? records : raw) + ((size_t)p.rot_keep + 15) / 16 * 128, rot_stated = records + (size_t)p.rot_span * 8;
+    g.smem += rot_needs > rot_stated ? rot_needs : rot_stated;
     if (layout == LLVQ_PLANES10X) g.smem += (size_t)kWarps * 32 * 8;        // the warps' slots for the products of exception blocks
     return g;
 }

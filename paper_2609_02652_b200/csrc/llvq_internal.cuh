@@ -84,7 +84,8 @@ struct GemvPlan {
     FastDiv div_panel, div_last; // by panel, by the last panel's width
     int xblocks;                 // most blocks of x any CTA needs
     uint32_t group_bytes;        // bytes of a row group's records
-    int rot_span;                // most coordinates any CTA rotates
+    int rot_span;                // most coordinates of the rotation blocks any CTA's blocks of x lie in
+    int rot_keep;                // most of them any CTA keeps after the first stages (rot_first)
     CtaShare cta[kMaxGridCtas + 1];    // the share of every CTA of the grid; [grid].first is the total
 };
 
@@ -111,7 +112,7 @@ struct GemvCall {
     int rot_log2;             // log2 of the rotation's block length (3..)
     int rot_n;                // coordinates rotated: a multiple of the block length, at most 24 nb
     const uint32_t *rot_negate;   // sign-flip bits, or null
-    double rot_scale;         // 2^-24 / sqrt(block length)
+    double rot_scale;         // 1 / sqrt(block length)
     float shell_inv_norm[16];         // [m] = 1 / (4 sqrt m)
 };
 
@@ -121,6 +122,17 @@ struct GemvLaunch {
     int grid;
     size_t smem;
 };
+// The rotation inside the GEMV: the first pass over x runs the widest `stages` strides, 2^stride and more, down to pieces of
+// 2^stride coordinates; of these a CTA keeps the ones that meet its blocks of x.
+struct RotFirst {
+    int stages, stride;
+};
+__host__ __device__ inline RotFirst rot_first(int block_log2) {
+    RotFirst f;
+    f.stages = block_log2 >= 6 ? 3 : block_log2 - 3;
+    f.stride = block_log2 - f.stages;
+    return f;
+}
 // Everything gemv_plan looks at, and what it made of it.
 struct PlanKey {
     int layout, nb, batch, rot_log2, rot_n, nprob;

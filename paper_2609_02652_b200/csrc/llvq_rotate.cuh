@@ -1,5 +1,5 @@
-// Device pieces of the exact Walsh-Hadamard rotation, shared by the rotation kernel and by the GEMV whose
-// prologue rotates x itself: integers in units of 2^-24, butterflies on 64-bit sums, one rounding to FP16.
+// Device pieces of the exact Walsh-Hadamard rotation: for the rotation kernel integers in units of 2^-24, butterflies on
+// 64-bit sums, one rounding to FP16; for the GEMV whose prologue rotates x itself the same sums in f64.
 #pragma once
 #include <cstdint>
 
@@ -14,14 +14,14 @@ __device__ __forceinline__ int rot_at(int i) { return i ^ ((i >> 4) & 15); }
 
 // R stages of the in-place butterfly on 2^R values: (a, b) -> (a + b, a - b) over every pair that differs in
 // one index bit.  With the values taken at stride 2^s these are stages s .. s + R - 1 of the transform.
-template <int R>
-__device__ __forceinline__ void rot_butterflies(long long (&a)[8]) {
+template <int R, typename T>
+__device__ __forceinline__ void rot_butterflies(T (&a)[8]) {
 #pragma unroll
     for (int h = 1; h < (1 << R); h <<= 1) {
 #pragma unroll
         for (int i = 0; i < (1 << R); i++) {
             if ((i & h) == 0) {
-                const long long u = a[i], w = a[i + h];
+                const T u = a[i], w = a[i + h];
                 a[i] = u + w;
                 a[i + h] = u - w;
             }
@@ -98,6 +98,59 @@ __device__ __forceinline__ uint4 rot_round8(const long long *v, int first, doubl
         const __half hi = __double2half((double)v[rot_at(first + 2 * i + 1)] * scale);
         out[i] = (uint32_t)__half_as_ushort(lo) | ((uint32_t)__half_as_ushort(hi) << 16);
     }
+    return make_uint4(out[0], out[1], out[2], out[3]);
+}
+
+// ---- the rotation of a stretch of x inside the GEMV.  A CTA needs the coordinates [need_lo, need_hi) of the rotated vector, a
+// small part of the blocks they lie in, so the stages run from the widest stride down: once the stages of strides 2^s and
+// more are done, only the pieces of 2^s coordinates that meet the part needed go on.  In f64 the sums are those of the
+// integers: every partial sum ahead of a 2^14 block's last stage is a multiple of 2^-24 below 2^29, hence exact, and where
+// the last stage's is not, it is rounded as the integer would be on its way to f64.  One instruction an addition where the
+// 64-bit integers take two, and no conversion at the end.
+
+// Stages S .. S + R - 1 over the coordinates [lo, hi) (multiples of 2^(S+R)); of the results those in [keep_lo, keep_hi)
+// (multiples of 2^S) are stored.  v holds coordinate first + i in place rot_at(i).  RAW: the inputs are FP16, raw[0] = coordinate lo.
+template <int R, bool RAW>
+__device__ __forceinline__ void rot_narrow(double *v, int first, const __half *raw, int lo, int hi, int keep_lo, int keep_hi, int S, int tid, int nthreads) {
+    for (int g = tid; g < ((hi - lo) >> R); g += nthreads) {
+        const int base = ((g >> S) << (S + R)) | (g & ((1 << S) - 1));
+        double a[8];
+#pragma unroll
+        for (int j = 0; j < (1 << R); j++) {
+            if (RAW) a[j] = __hiloint2double((int)(((uint32_t)(int)reinterpret_cast<const short *>(raw)[base + (j << S)] << 10) & 0x81ffffffu), 0);
+            else a[j] = v[rot_at(lo - first + base + (j << S))];
+        }
+        rot_butterflies<R>(a);
+#pragma unroll
+        for (int j = 0; j < (1 << R); j++) {
+            const int c = lo + base + (j << S);
+            if (c >= keep_lo && c < keep_hi) v[rot_at(c - first)] = a[j];
+        }
+    }
+}
+
+// Stages 3 .. 5 of a piece of 64 by eight neighbouring lanes: the lane whose eight values begin at place `at` takes the values
+// eight apart.  A __syncwarp() belongs between this and rot_finish8.
+__device__ __forceinline__ void rot_middle8(double *v, int at) {
+    const int base = (at & ~63) + ((at >> 3) & 7);
+    double a[8];
+#pragma unroll
+    for (int j = 0; j < 8; j++) a[j] = v[rot_at(base + 8 * j)];
+    rot_butterflies<3>(a);
+#pragma unroll
+    for (int j = 0; j < 8; j++) v[rot_at(base + 8 * j)] = a[j];
+}
+
+// The last three stages of the eight values from place `at` on (a multiple of eight), and the one rounding.
+__device__ __forceinline__ uint4 rot_finish8(const double *v, int at, double scale) {
+    double a[8];
+#pragma unroll
+    for (int k = 0; k < 8; k++) a[k] = v[rot_at(at + k)];
+    rot_butterflies<3>(a);
+    uint32_t out[4];
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+        out[i] = (uint32_t)__half_as_ushort(__double2half(a[2 * i] * scale)) | ((uint32_t)__half_as_ushort(__double2half(a[2 * i + 1] * scale)) << 16);
     return make_uint4(out[0], out[1], out[2], out[3]);
 }
 

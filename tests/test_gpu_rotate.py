@@ -173,6 +173,26 @@ def test_gemv_rotated_matches_oracle_chain_and_the_two_launch_form(B, ctx, oracl
     assert torch.equal(case.d_x.cpu(), torch.from_numpy(case.x))      # x itself is left alone
 
 
+@pytest.mark.parametrize("log2", range(3, 15))
+def test_gemv_rotated_every_block_length(B, ctx, oracle, log2):
+    """Every split of the stages into passes, on more columns than a multiprocessor's share of x, with subnormal and zero
+    entries.  Bound: the 29-bit fixed point of the activations, sqrt(block) / 2^28 of ||x|| at the worst, as above."""
+    n, rows = (8192 if log2 < 14 else 16384), 40
+    case = make_case(rows, n + 40, seed=log2)
+    x = case.x.copy()
+    x[:n:7] = 0
+    x[1:n:5] = (x[1:n:5].astype(np.float32) * 2.0 ** -17).astype(np.float16)
+    case = dataclasses.replace(case, x=x)
+    d_x = torch.from_numpy(x).cuda()
+    neg = np.random.default_rng(log2).integers(0, 2, size=n)
+    buf = B.expand(ctx, 0, case.d_codes, case.rows, case.nb)
+    y = torch.full((rows,), float("nan"), dtype=torch.float32, device="cuda")
+    B.gemv_rotated(ctx, [(buf, case.d_scale, GAIN, y, rows)], d_x, case.nb * 24, n=n, block=1 << log2, negate_bits=_bits(neg))
+    torch.cuda.synchronize()
+    err, _ = check_gemv(oracle, _rotated_reference(oracle, case, n, 1 << log2, neg), y)
+    assert err <= 1e-6
+
+
 def test_gemv_rotated_grouped_launch_and_outlier_activation(B, ctx, oracle):
     """q/k/v-like group sharing one x; x with one huge entry (what the rotation is for): the bound on the
     rotated magnitudes is then loosest, and the result must still meet the bar with room."""
