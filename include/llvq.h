@@ -231,7 +231,8 @@ int llvq_overlay_bytes(int64_t rows, int64_t k_padded, uint64_t exceptions, size
  * caller zeroes).  The context counts such codes as well, whether or not bad_count is given: the next
  * llvq_status returns LLVQ_EINDEX if any expansion since the last one met one.  Bit-exact by construction:
  * integer arithmetic only.  The GEMV enqueued next on this context is launched without programmatic dependent
- * launch, so that it cannot read records ahead of this expansion (see llvq_set_pdl). */
+ * launch, so that it cannot read records ahead of this expansion (see llvq_set_pdl).  The expansion itself sets up while
+ * the previous kernel of the stream ends and waits for it before it reads the codes or writes anything. */
 int llvq_expand(llvq_ctx *ctx, int layout, const uint64_t *codes, int64_t rows, int64_t nb,
                 void *layout_out, size_t out_bytes, uint32_t *bad_count, void *stream);
 

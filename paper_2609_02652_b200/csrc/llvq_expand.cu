@@ -93,6 +93,8 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
     v.blob = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     WarpScratch &s = reinterpret_cast<WarpScratch *>(smem + kUnrankSharedBytes)[warp];
+    // the tables are the library's: they are copied while the previous kernel of the stream ends
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
 
     const uint32_t tiles = (uint32_t)(nb / kTileCells), left = (uint32_t)(nb % kTileCells);
@@ -311,6 +313,7 @@ expand_onehot_kernel(UnrankView global, DeviceTables T, const uint64_t *__restri
     UnrankView v = global;
     v.blob = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
     uint32_t bad = 0;
     for (int64_t cell_id = (int64_t)warp * gridDim.x + blockIdx.x; cell_id < cells; cell_id += (int64_t)kExpandWarps * gridDim.x) {
@@ -378,6 +381,8 @@ overlay_count_kernel(UnrankView v, uint64_t num_points, const uint64_t *__restri
     uint64_t *list = list_all[warp];
     uint32_t *tile_of = tile_all[warp];
     const uint32_t tiles = (uint32_t)(nb / kTileCells);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __syncthreads();
     uint32_t sum = 0;
     int listed = 0;
@@ -469,6 +474,8 @@ __global__ void __launch_bounds__(1024) overlay_index_kernel(uint8_t *out, size_
             c[j] = at < n ? index[at + 1] : 0u;
         }
     };
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     load(0);
     for (int64_t base = 0; base < n; base += kRound) {
 #pragma unroll
@@ -516,6 +523,24 @@ unsigned grid_for(const llvq_ctx *ctx, int64_t work, int per_sm = 1) {
     return (unsigned)(work < most ? work : most);
 }
 
+// Launches with programmatic stream serialization, if the context has it switched on.  The kernels wait for their
+// predecessor ahead of all they read but the library's tables.  The expansions let no kernel start before they end: what
+// follows may be a GEMV of another context, which reads records ahead of its own wait.
+template <typename... P, typename... A>
+cudaError_t launch(const llvq_ctx *ctx, void (*kernel)(P...), unsigned grid, int threads, int smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = ctx->use_pdl ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 }  // namespace
 
 int expand_configure() {
@@ -530,9 +555,8 @@ cudaError_t launch_overlay_count(const llvq_ctx *ctx, const uint64_t *codes, int
                                  unsigned long long *host, cudaStream_t s) {
     const int64_t groups = (rows + kRowsPerGroup - 1) / kRowsPerGroup, tiles = nb / kTileCells;
     if (tiles == 0) return cudaSuccess;
-    overlay_count_kernel<false><<<grid_for(ctx, (groups * tiles + kCountWarps - 1) / kCountWarps, 8), kCountWarps * 32, 0, s>>>(ctx->unrank, ctx->dev.num_points, codes, rows, nb,
-                                                                                                          (uint32_t)(groups * tiles), nullptr, counter, host);
-    return cudaGetLastError();
+    return launch(ctx, overlay_count_kernel<false>, grid_for(ctx, (groups * tiles + kCountWarps - 1) / kCountWarps, 8), kCountWarps * 32, 0, s, ctx->unrank,
+                  ctx->dev.num_points, codes, rows, nb, groups * tiles, nullptr, counter, host);
 }
 
 cudaError_t launch_expand(const llvq_ctx *ctx, int layout, const uint64_t *codes, int64_t rows, int64_t nb,
@@ -541,11 +565,9 @@ cudaError_t launch_expand(const llvq_ctx *ctx, int layout, const uint64_t *codes
     uint8_t *o8 = (uint8_t *)out;
     const UnrankView v = ctx->unrank;
     const uint64_t points = ctx->dev.num_points;
-    if (layout == LLVQ_ONEHOT) {
-        expand_onehot_kernel<<<grid_for(ctx, groups * nb), kExpandThreads, kUnrankSharedBytes, s>>>(v, ctx->dev, codes, rows, nb, groups * nb, o8, bad_count,
-                                                                                                              ctx->bad_codes);
-        return cudaGetLastError();
-    }
+    if (layout == LLVQ_ONEHOT)
+        return launch(ctx, expand_onehot_kernel, grid_for(ctx, groups * nb), kExpandThreads, kUnrankSharedBytes, s, v, ctx->dev, codes, rows, nb, groups * nb, o8,
+                      bad_count, ctx->bad_codes);
     const int64_t left = nb % kTileCells, tiles = nb / kTileCells;
     const int64_t pieces = groups * (tiles + (left >= 2 ? 1 : 0) + (left & 1));
     const unsigned grid = grid_for(ctx, pieces);
@@ -556,18 +578,22 @@ cudaError_t launch_expand(const llvq_ctx *ctx, int layout, const uint64_t *codes
         const size_t room = (out_bytes - table_offset) / 16;
         const uint32_t capacity = room > 0xffffffffull ? 0xffffffffu : (uint32_t)room;
         // count the tiles' exceptions into the index, turn the counts into first entries, expand
-        if (tiles > 0)
-            overlay_count_kernel<true><<<grid_for(ctx, (groups * tiles + kCountWarps - 1) / kCountWarps, 8), kCountWarps * 32, 0, s>>>(v, points, codes, rows, nb, (uint32_t)(groups * tiles), index,
-                                                                                                                 nullptr, nullptr);
-        overlay_index_kernel<<<1, 1024, 0, s>>>(o8, (size_t)groups * overlay_group_bytes(nb), index_offset, table_offset, groups * tiles, capacity, ctx->overflow);
-        expand_planes_kernel<LLVQ_PLANES10X><<<grid, kExpandThreads, kExpandSmem, s>>>(v, points, codes, rows, nb, (uint32_t)pieces, o8, bad_count, ctx->bad_codes, index, table,
-                                                                                       capacity);
-    } else if (layout == LLVQ_PLANES13) {
-        expand_planes_kernel<LLVQ_PLANES13><<<grid, kExpandThreads, kExpandSmem, s>>>(v, points, codes, rows, nb, (uint32_t)pieces, o8, bad_count, ctx->bad_codes, nullptr, nullptr, 0);
-    } else {
-        expand_planes_kernel<LLVQ_PLANES><<<grid, kExpandThreads, kExpandSmem, s>>>(v, points, codes, rows, nb, (uint32_t)pieces, o8, bad_count, ctx->bad_codes, nullptr, nullptr, 0);
+        if (tiles > 0) {
+            const cudaError_t r = launch(ctx, overlay_count_kernel<true>, grid_for(ctx, (groups * tiles + kCountWarps - 1) / kCountWarps, 8), kCountWarps * 32, 0, s, v, points,
+                                         codes, rows, nb, groups * tiles, index, nullptr, nullptr);
+            if (r != cudaSuccess) return r;
+        }
+        const cudaError_t r = launch(ctx, overlay_index_kernel, 1u, 1024, 0, s, o8, (size_t)groups * overlay_group_bytes(nb), index_offset, table_offset, groups * tiles,
+                                     capacity, ctx->overflow);
+        if (r != cudaSuccess) return r;
+        return launch(ctx, expand_planes_kernel<LLVQ_PLANES10X>, grid, kExpandThreads, kExpandSmem, s, v, points, codes, rows, nb, pieces, o8, bad_count, ctx->bad_codes, index,
+                      table, capacity);
     }
-    return cudaGetLastError();
+    if (layout == LLVQ_PLANES13)
+        return launch(ctx, expand_planes_kernel<LLVQ_PLANES13>, grid, kExpandThreads, kExpandSmem, s, v, points, codes, rows, nb, pieces, o8, bad_count, ctx->bad_codes, nullptr,
+                      nullptr, 0u);
+    return launch(ctx, expand_planes_kernel<LLVQ_PLANES>, grid, kExpandThreads, kExpandSmem, s, v, points, codes, rows, nb, pieces, o8, bad_count, ctx->bad_codes, nullptr, nullptr,
+                  0u);
 }
 
 }  // namespace llvq
