@@ -6,10 +6,11 @@
 // class take different code, and codes come in random order, so a warp first finds the class of all 128 blocks of a
 // tile (a lane a row), lists them by type in shared memory and then un-ranks 32 blocks of one type at a time, whatever
 // their place; the codes wait in shared memory until the tile's words are gathered from them.  The small look-up tables
-// are copied to shared memory once a CTA, one CTA a multiprocessor walks over the tiles.
-// Measured (9728 x 2560 into the 14-byte layout, 1.04 M blocks): 39 us, 2600 warp instructions a tile of 128 blocks, issue
+// are copied to shared memory once a CTA, while the previous kernel of the stream ends; one CTA a multiprocessor walks over
+// the tiles.
+// Measured (9728 x 2560 into the 14-byte layout, 1.04 M blocks): 38 us, 2600 warp instructions a tile of 128 blocks, issue
 // slots 55 % busy, the load unit's wavefronts 74 %; a lane a row with a 64-bit division a coordinate and candidate took
-// 484 us, one odd coordinate at a time 45.  Counting and expanding 17408 x 5120 into the 10-byte layout: 195 us against
+// 484 us, one odd coordinate at a time 45.  Counting and expanding 17408 x 5120 into the 10-byte layout: 188 us against
 // 4700.  24 or 28 warps a CTA instead of 32: 47 and 50 us.  The shared tables are kept to 51 KB because the rest of a
 // multiprocessor's memory is the L1 cache that the lists are read through: with 104 KB of tables it took 53 us.
 #include "llvq_internal.cuh"
@@ -101,35 +102,59 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
     const uint32_t pieces = tiles + (left >= 2 ? 1 : 0) + (left & 1);
     const int g = lane >> 2, t = lane & 3;
     uint32_t bad = 0;
+    // The CTA's pieces (every gridDim-th), a warp a piece and round.  A piece is a chain of some ten microseconds, however few
+    // run: where the last round has work for half of the warps or a quarter, two or four share a piece, each its blocks
+    // (500 x 1000: 8.3 us, 14.8 without; 17408 x 5120: 117, 121; a last round of 26 pieces, 9728 x 2560: 38.0, 37.9).
+    // `own` = the blocks of the piece that are this warp's, a bit each, and 16 (0: no piece left), `share` = log2 of the warps on it.
+    const uint32_t mine = (total_pieces - blockIdx.x + gridDim.x - 1) / gridDim.x, full = mine / kExpandWarps * kExpandWarps;
+    const int last_share = mine - full <= kExpandWarps / 4 ? 2 : (mine - full <= kExpandWarps / 2 ? 1 : 0);
+    uint32_t base = 0, piece = 0, own = 0;
+    int share = 0;
     // a piece's codes are loaded while the piece before it is un-ranked
     uint64_t code[4];
-    auto load_codes = [&](uint32_t piece) {
+    auto next_piece = [&]() {
+        uint32_t at = base + warp;
+        own = 15u;
+        if (base >= full) {
+            share = last_share;
+            at = base + (warp >> share);
+            own = share == 0 ? 15u : (share == 1 ? 3u << (2 * (warp & 1)) : 1u << (warp & 3));
+        }
+        base += kExpandWarps;
+        piece = at * gridDim.x + blockIdx.x;
         const uint32_t rg = piece / pieces, u = piece % pieces;
         const int64_t row = (int64_t)rg * kRowsPerGroup + lane;
         const int64_t b0 = u < tiles ? (int64_t)u * kTileCells : (left >= 2 && u == tiles ? (int64_t)tiles * kTileCells : nb - 1);
-        const int ncell = u < tiles ? 4 : (left >= 2 && u == tiles ? 2 : 1);
+        own = at < mine ? (own & (u < tiles ? 15u : (left >= 2 && u == tiles ? 3u : 1u))) | 16u : 0u;
+        const uint32_t load = row < rows ? own : 0u;
 #pragma unroll
-        for (int q = 0; q < 4; q++) code[q] = (row < rows && q < ncell && piece < total_pieces) ? __ldg(codes + row * nb + b0 + q) : 0ull;
+        for (int q = 0; q < 4; q++) code[q] = (load >> q & 1u) ? __ldg(codes + row * nb + b0 + q) : 0ull;
     };
-    uint32_t piece = (uint32_t)warp * gridDim.x + blockIdx.x;      // the CTAs' shares differ by one piece at most
-    load_codes(piece);
-    for (; piece < total_pieces; piece += kExpandWarps * gridDim.x) {
+    next_piece();
+    while (own) {                                                  // the same for all warps that share a piece
+        const int now_share = share, part = warp & ((1 << share) - 1);
+        const uint32_t now_own = own;
+        WarpScratch &n = (&s)[-part];                              // where the piece's codes wait
+        auto meet = [&]() {                                        // the warps that share the piece
+            if (now_share == 0) __syncwarp();
+            else asm volatile("bar.sync %0, %1;" ::"r"(warp >> now_share), "r"(32 << now_share) : "memory");
+        };
+        if (now_share) meet();                                     // the first warp's last piece is written
         const uint32_t rg = piece / pieces, u = piece % pieces;
         const bool row_exists = (int64_t)rg * kRowsPerGroup + lane < rows;
         uint8_t *grp = out + (size_t)rg * ((size_t)tiles * kTile + (size_t)left * kCell);
         const bool is_tile = u < tiles;
         const bool is_pair = !is_tile && left >= 2 && u == tiles;
         const bool single = !is_tile && !is_pair;
-        const int ncell = is_tile ? 4 : (is_pair ? 2 : 1);
         uint32_t next_entry = 0;                                   // OVERLAY: where this tile's next exception goes
         if (OVERLAY && is_tile) next_entry = index[(size_t)rg * tiles + u];
 
         // ---- class of every block, listed by type
         int n_odd = 0, n_even = 0;
-        if (OVERLAY && lane < 4) s.exceptions[lane] = 0;
+        if (OVERLAY && lane < 4 && (now_own >> lane & 1u)) n.exceptions[lane] = 0;
 #pragma unroll
         for (int q = 0; q < 4; q++) {
-            if (q >= ncell) break;
+            if (!(now_own >> q & 1u)) continue;
             const bool valid = row_exists && code_names_point(code[q], num_points);
             bool odd = false;
             uint64_t entry = 0;
@@ -142,8 +167,8 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
                 bad += row_exists;
                 // the empty record
                 const uint32_t zero_code = OVERLAY && is_tile ? 0u : 0x88888888u;
-                s.nat[q][0][lane] = zero_code; s.nat[q][1][lane] = zero_code; s.nat[q][2][lane] = zero_code;
-                s.nat[q][3][lane] = COMPACT ? 0u : (uint32_t)kEmptyClass;
+                n.nat[q][0][lane] = zero_code; n.nat[q][1][lane] = zero_code; n.nat[q][2][lane] = zero_code;
+                n.nat[q][3][lane] = COMPACT ? 0u : (uint32_t)kEmptyClass;
             }
             const uint32_t of_odd = __ballot_sync(0xffffffffu, valid && odd), of_even = __ballot_sync(0xffffffffu, valid && !odd);
             const uint32_t before = (1u << lane) - 1u;
@@ -152,7 +177,7 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
             n_even += __popc(of_even);
         }
         __syncwarp();
-        load_codes(piece + kExpandWarps * gridDim.x);
+        next_piece();
 
         // ---- un-rank: 32 blocks of a type at a time
         auto finish = [&](uint64_t entry, const UnrankDesc &d, const Point &p, bool odd) {
@@ -173,11 +198,11 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
                     // the short record's header byte: the shell above, and below it window, parity and gain mixed with the shell
                     hdr = ((o - 3u) | (uint32_t)odd << 2 | gain << 3) ^ shell | shell << 4;
                 } else {
-                    atomicOr(&s.exceptions[q], 1u << row);
+                    atomicOr(&n.exceptions[q], 1u << row);
                 }
             }
-            s.nat[q][0][row] = cw[0]; s.nat[q][1][row] = cw[1]; s.nat[q][2][row] = cw[2];
-            s.nat[q][3][row] = hdr;
+            n.nat[q][0][row] = cw[0]; n.nat[q][1][row] = cw[1]; n.nat[q][2][row] = cw[2];
+            n.nat[q][3][row] = hdr;
         };
 #pragma unroll 1
         for (int i = lane; i < n_odd; i += 32) {
@@ -195,17 +220,18 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
             unrank_even(v, d, entry & ((1ull << 47) - 1), p);
             finish(entry, d, p, false);
         }
-        __syncwarp();
+        meet();
+        if (part) break;                                           // a shared piece is the last
         if (OVERLAY && is_tile) {
             // the tile's exceptions go to the table in the order block, row, and leave an empty short record
 #pragma unroll 1
             for (int q = 0; q < 4; q++) {
-                const uint32_t rows_out = s.exceptions[q];
+                const uint32_t rows_out = n.exceptions[q];
                 if ((rows_out >> lane) & 1u) {
                     const uint32_t at = next_entry + __popc(rows_out & ((1u << lane) - 1u));
                     if (at < capacity)
-                        table[at] = make_uint4(s.nat[q][3][lane] | (uint32_t)lane << 8 | (u * kTileCells + q) << 13, s.nat[q][0][lane], s.nat[q][1][lane], s.nat[q][2][lane]);
-                    s.nat[q][0][lane] = s.nat[q][1][lane] = s.nat[q][2][lane] = s.nat[q][3][lane] = 0u;
+                        table[at] = make_uint4(n.nat[q][3][lane] | (uint32_t)lane << 8 | (u * kTileCells + q) << 13, n.nat[q][0][lane], n.nat[q][1][lane], n.nat[q][2][lane]);
+                    n.nat[q][0][lane] = n.nat[q][1][lane] = n.nat[q][2][lane] = n.nat[q][3][lane] = 0u;
                 }
                 next_entry += __popc(rows_out);
             }
@@ -218,11 +244,11 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
         auto codes_at = [&](int q0, int m, int e, int kappa0) -> uint32_t {
             const int slot = kappa0 / 24, i0 = kappa0 % 24;
             const int r = single ? 16 * slot + 8 * e + g : 16 * m + 8 * e + g;
-            return s.nat[single ? q0 : q0 + slot][i0 >> 3][r];
+            return n.nat[single ? q0 : q0 + slot][i0 >> 3][r];
         };
         auto header = [&](int q0, int m, int e, int slot) -> uint32_t {
             const int r = single ? 16 * slot + 8 * e + g : 16 * m + 8 * e + g;
-            return s.nat[single ? q0 : q0 + slot][3][r];
+            return n.nat[single ? q0 : q0 + slot][3][r];
         };
         const uint32_t half_sel = (t & 1) ? 0x7362u : 0x5140u;
         // the lane's four nibbles of x to the low nibbles of four bytes, those of y to the high nibbles

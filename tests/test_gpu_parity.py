@@ -109,6 +109,24 @@ def test_expand_every_class_mixed(B, ctx, oracle, layout, rows, nb):
     assert np.array_equal(got.cpu().numpy(), want)
 
 
+@pytest.mark.parametrize("layout", [0, 3])
+@pytest.mark.parametrize("each", [5, 12, 36])
+def test_expand_pieces_shared_by_warps(B, ctx, oracle, layout, each):
+    """Last rounds in which four warps, two warps or (after a full round) four again share a tile, the pair or the single at the
+    end: `each` pieces a multiprocessor, seven blocks a row and rows that end inside a row group."""
+    groups, nb = torch.cuda.get_device_properties(0).multi_processor_count * each // 3, 7
+    rows = 32 * groups - 5
+    rng = np.random.default_rng(each)
+    codes = rng.integers(0, N_POINTS, rows * nb, dtype=np.uint64) | (rng.integers(0, 2, rows * nb, dtype=np.uint64) << np.uint64(47))
+    d = torch.from_numpy(codes.view(np.int64)).cuda()
+    if layout == 3:
+        want, n = oracle.pack_planes10x(codes, rows, nb)
+        got = B.expand(ctx, layout, d, rows, nb, out=torch.empty(B.overlay_bytes(rows, nb * 24, n), dtype=torch.uint8, device="cuda"))
+    else:
+        want, got = oracle.pack_planes(codes, rows, nb), B.expand(ctx, layout, d, rows, nb)
+    assert np.array_equal(got.cpu().numpy(), want)
+
+
 @pytest.mark.parametrize("layout", [0, 1])
 @pytest.mark.parametrize("rows,k", [(40, 24 * 7), (257, 24 * 21), (3072, 3072)])
 def test_decode_bit_exact(B, ctx, oracle, layout, rows, k):
