@@ -7,14 +7,16 @@
 namespace llvq {
 namespace {
 
-// Appends every ordering of the multiset `cnt` (values 0..n-1), lexicographically, `bits` bits a value.
-template <typename T>
-void list_orderings(int *cnt, int n, int left, int at, int bits, uint64_t word, std::vector<T> &out) {
-    if (left == 0) { out.push_back((T)word); return; }
-    for (int v = 0; v < n; v++) {
+// Appends every ordering of the `left` values of the multiset `cnt` (values 0..N-1), lexicographically, BITS bits a value.
+template <int N, int BITS, typename T>
+__attribute__((noinline)) void list_orderings(int *cnt, int left, int at, uint64_t word, std::vector<T> &out) {
+    if (cnt[0] == left) { out.push_back((T)word); return; }         // zeros to the end
+    for (int v = 0; v < N; v++) {
         if (cnt[v] == 0) continue;
+        const uint64_t with = word | (uint64_t)v << (BITS * at);
+        if (left == 1) { out.push_back((T)with); return; }
         cnt[v]--;
-        list_orderings(cnt, n, left - 1, at + 1, bits, word | (uint64_t)v << (bits * at), out);
+        list_orderings<N, BITS>(cnt, left - 1, at + 1, with, out);
         cnt[v]++;
     }
 }
@@ -55,6 +57,7 @@ T *part(std::vector<uint8_t> &blob, int offset) { return reinterpret_cast<T *>(b
 bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
     u.blob.assign(kUnrankBlobBytes, 0);
     u.pairs.clear(); u.tail8.clear(); u.tab_b.clear();
+    u.tail8.reserve(1 << 16); u.tab_b.reserve(300000);
     if (t.num_classes > kUnrankClasses - 2) return false;
 
     UnrankStep *steps = part<UnrankStep>(u.blob, kUnrankSteps);
@@ -87,6 +90,13 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
         if ((int)sets.size() != kOddSets) return false;
     }
     auto copies_in = [](const std::array<int, 7> &c) { int n = 0; for (int v = 1; v < 7; v++) n += c[v]; return n; };
+    // the multiset with one copy of v less (itself for v = 0: the copies of 0 are what is left)
+    std::vector<std::array<int, 7>> less(sets.size());
+    for (int k = 0; k < kOddSets; k++)
+        for (int v = 0; v < 7; v++) {
+            std::array<int, 7> c = sets[k];
+            less[k][v] = v == 0 ? k : (c[v] ? (c[v]--, set_of[c]) : -1);
+        }
     // every ordering of eight
     uint16_t *tail_first = part<uint16_t>(u.blob, kUnrankTailBase);
     for (int k = 0; k < kOddSets; k++) {
@@ -97,10 +107,13 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
         c[0] = 8 - n;
         if (u.tail8.size() > 0xffff) return false;
         tail_first[k] = (uint16_t)u.tail8.size();
-        list_orderings(c, 7, 8, 0, 4, 0, u.tail8);
+        list_orderings<7, 4>(c, 8, 0, 0, u.tail8);
     }
     // the draws of two from L
     PairStep *pair_steps = part<PairStep>(u.blob, kUnrankPairs);
+    size_t entries = 0;
+    for (int i = 0; i < kPairSteps; i++) entries += (size_t)kOddSets * (24 - 2 * i) * (23 - 2 * i);
+    u.pairs.reserve(entries);
     for (int i = 0; i < kPairSteps; i++) {
         const int L = 24 - 2 * i, draws = L * (L - 1);
         const uint32_t shift = (uint32_t)__builtin_ctz(draws), odd = (uint32_t)draws >> shift;
@@ -109,7 +122,7 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
         pair_steps[i] = {x, shift, (uint32_t)u.pairs.size(), (uint32_t)draws};
         u.pairs.resize(u.pairs.size() + (size_t)kOddSets * draws, 0);
         for (int k = 0; k < kOddSets; k++) {
-            std::array<int, 7> c = sets[k];
+            const std::array<int, 7> &c = sets[k];
             const int n = copies_in(c);
             if (n > L) continue;
             uint64_t *entry = u.pairs.data() + pair_steps[i].first + (size_t)k * draws;
@@ -118,10 +131,7 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
                 for (int vb = 0; vb < 7; vb++) {
                     const int na = va ? c[va] : L - n, nb = (vb ? c[vb] : L - n) - (va == vb);
                     if (na < 1 || nb < 1) continue;
-                    std::array<int, 7> rest = c;
-                    if (va) rest[va]--;
-                    if (vb) rest[vb]--;
-                    const uint64_t e = (uint64_t)at | (uint64_t)(na * nb) << 16 | (uint64_t)(va | vb << 4) << 32 | (uint64_t)set_of[rest] << 40;
+                    const uint64_t e = (uint64_t)at | (uint64_t)(na * nb) << 16 | (uint64_t)(va | vb << 4) << 32 | (uint64_t)less[less[k][va]][vb] << 40;
                     for (int j = 0; j < na * nb; j++) entry[at + j] = e;
                     at += na * nb;
                 }
@@ -139,7 +149,7 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
             for (int n1 = 0; 8 * n1 + 24 * n2 <= 48 - w; n1++) {
                 int c[3] = {w - n1 - n2, n1, n2};
                 first_a[w << 16 | n1 << 8 | n2] = (uint32_t)(w < 24 ? support.size() : support24.size());
-                if (w < 24) list_orderings(c, 3, w, 0, 2, 0, support); else list_orderings(c, 3, w, 0, 2, 0, support24);
+                if (w < 24) list_orderings<3, 2>(c, w, 0, 0, support); else list_orderings<3, 2>(c, w, 0, 0, support24);
             }
     if (support.size() > kSupports || support24.size() > kSupports24) return false;
     std::memcpy(u.blob.data() + kUnrankSupport, support.data(), support.size() * 4);
@@ -156,7 +166,7 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
                     int c[4] = {lengths[l] - n1 - n2 - n3, n1, n2, n3};
                     first_b[lengths[l] << 16 | n1 << 8 | n2 << 4 | n3] = (uint32_t)u.tab_b.size();
                     if (lengths[l] == 12) rest12[n1 | n2 << 4 | n3 << 6] = (uint32_t)u.tab_b.size();
-                    list_orderings(c, 4, lengths[l], 0, 2, 0, u.tab_b);
+                    list_orderings<4, 2>(c, lengths[l], 0, 0, u.tab_b);
                 }
 
     // ---- classes
@@ -212,8 +222,7 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
         };
         // guide[s] = last class c whose first index lies in a slot before s, or is the slot's first index: the largest c with
         // slot_of(base[c]) < s is a lower bound that holds for every index of slot s
-        for (int s = 0; s < kGuideSlots + 8; s++) {
-            int c = 0;
+        for (int s = 0, c = 0; s < kGuideSlots + 8; s++) {
             while (c + 1 < t.num_classes && slot_of(t.base[(size_t)c + 1]) < s) c++;
             guide[s] = (uint16_t)c;
         }
