@@ -261,19 +261,7 @@ static GemvLaunch planned(llvq_ctx *ctx, int layout, GemvParams &p) {
     std::memset(&key, 0, sizeof key);
     key.layout = layout; key.nb = p.nb; key.batch = p.batch; key.rot_log2 = p.rot_log2; key.rot_n = p.rot_n; key.nprob = p.nprob;
     for (int i = 0; i < p.nprob; i++) key.rows[i] = p.prob[i].rows;
-    for (int i = 0; i < ctx->plans_used; i++)
-        if (std::memcmp(&ctx->plans[i].key, &key, sizeof key) == 0) {
-            static_cast<GemvPlan &>(p) = ctx->plans[i].plan;
-            return ctx->plans[i].launch;
-        }
-    const GemvLaunch g = gemv_plan(layout, p, ctx->sm_count);
-    PlanEntry &e = ctx->plans[ctx->plans_next];
-    e.key = key;
-    e.plan = p;
-    e.launch = g;
-    if (ctx->plans_used < llvq_ctx::kPlans) ctx->plans_used++;
-    ctx->plans_next = (ctx->plans_next + 1) % llvq_ctx::kPlans;
-    return g;
+    return ctx->plans.get(key, p, [&](GemvPlan &) { return gemv_plan(layout, p, ctx->sm_count); });
 }
 
 static int run_gemv(llvq_ctx *ctx, int layout, const llvq_problem *problems, int n, const void *x, int64_t k_padded,

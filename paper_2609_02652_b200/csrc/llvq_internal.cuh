@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <cstring>
+#include <mutex>
 
 #include "../../include/llvq.h"
 #include "llvq_tables.h"
@@ -138,10 +140,38 @@ struct PlanKey {
     int layout, nb, batch, rot_log2, rot_n, nprob;
     int rows[LLVQ_MAX_GROUP];
 };
-struct PlanEntry {
-    PlanKey key;
-    GemvPlan plan;
-    GemvLaunch launch;
+// The plans of the last kKept shapes launched (a decoder has four or five): 2 KB and half a microsecond each.  Host threads
+// that launch on one stream may ask at the same time: a plan is handed out whole, under the lock (20 ns where nobody waits).
+class PlanCache {
+public:
+    // Copies the plan of `key` to `plan` and returns its launch: the kept one, or what make(plan) works out.
+    template <typename F>
+    GemvLaunch get(const PlanKey &key, GemvPlan &plan, F make) {
+        std::lock_guard<std::mutex> lock(mutex_);
+        for (int i = 0; i < used_; i++)
+            if (std::memcmp(&kept_[i].key, &key, sizeof key) == 0) {
+                plan = kept_[i].plan;
+                return kept_[i].launch;
+            }
+        Entry &e = kept_[next_];
+        e.launch = make(plan);
+        e.key = key;
+        e.plan = plan;
+        if (used_ < kKept) used_++;
+        next_ = (next_ + 1) % kKept;
+        return e.launch;
+    }
+
+private:
+    static constexpr int kKept = 8;
+    struct Entry {
+        PlanKey key;
+        GemvPlan plan;
+        GemvLaunch launch;
+    };
+    std::mutex mutex_;
+    Entry kept_[kKept];
+    int used_ = 0, next_ = 0;
 };
 
 }  // namespace llvq
@@ -163,10 +193,7 @@ struct llvq_ctx {
     int weights_dirty;       // an expansion was enqueued since the last GEMV: that GEMV must not read records ahead of it
     int sm_count;
     int max_smem_optin;
-    // The plans of the last kPlans shapes launched (a decoder has four or five): 2 KB and half a microsecond each.
-    static constexpr int kPlans = 8;
-    llvq::PlanEntry plans[kPlans];
-    int plans_used, plans_next;
+    llvq::PlanCache plans;
 };
 
 namespace llvq {

@@ -436,6 +436,34 @@ def test_more_shapes_than_kept_plans(B):
         c0.close()
 
 
+def test_host_threads_that_share_a_context_and_a_stream(B):
+    """Launches ordered on one stream may come from several host threads: more shapes than the context keeps plans of, each
+    thread in an order of its own, give the bits of one thread alone."""
+    import threading
+
+    c = B.create(0)
+    try:
+        cases = [make_case(32 + 40 * i, 24 * (3 + 7 * i), seed=i) for i in range(11)]
+        bufs = [B.expand(c, 0, m.d_codes, m.rows, m.nb) for m in cases]
+        run = lambda i: B.gemv(c, 0, bufs[i], cases[i].d_scale, GAIN, cases[i].d_x, cases[i].rows, cases[i].nb * 24)
+        refs = [run(i) for i in range(len(cases))]
+        wrong = []
+
+        def work(t):
+            order = np.random.default_rng(t).integers(0, len(cases), 300)
+            ys = [run(i) for i in order]
+            torch.cuda.synchronize()
+            wrong.extend(int(i) for i, y in zip(order, ys) if not torch.equal(y, refs[i]))
+
+        threads = [threading.Thread(target=work, args=(t,)) for t in range(4)]
+        [t.start() for t in threads]
+        [t.join() for t in threads]
+        assert wrong == []
+        B.status(c)
+    finally:
+        c.close()
+
+
 def test_gemv_batch_limits(B, ctx):
     case = make_case(64, 96, seed=1)
     buf = B.expand(ctx, 0, case.d_codes, case.rows, case.nb)
