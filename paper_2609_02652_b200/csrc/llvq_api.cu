@@ -189,7 +189,10 @@ int llvq_overlay_count(llvq_ctx *ctx, const uint64_t *codes, int64_t rows, int64
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
     cudaStream_t s = (cudaStream_t)stream;
-    // the kernel writes the total to page-locked memory of the context: no memset before it and no copy after it
+    // the kernel writes the total to page-locked memory of the context: no memset before it and no copy after it.  Its
+    // scratch must be zero when it starts and is zeroed only by its last CTA, so no two counts of a context may overlap:
+    // the call waits for its result anyway, and host threads that count on streams of their own take turns
+    std::lock_guard<std::mutex> lock(ctx->count_mutex);
     *ctx->host_counter = 0;
     if (launch_overlay_count(ctx, codes, rows, nb, ctx->counter, ctx->host_counter, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return LLVQ_ECUDA;
     *count = *ctx->host_counter;

@@ -189,6 +189,7 @@ struct llvq_ctx {
     uint32_t *overflow;      // device count: exception-table entries that found no room, since the last llvq_status
     unsigned long long *counter;   // device scratch of llvq_overlay_count: two words, zero between calls
     unsigned long long *host_counter;   // page-locked: its result
+    std::mutex count_mutex;  // one llvq_overlay_count at a time: the two above are its own from launch to result
     int use_pdl;             // launch the GEMV with programmatic stream serialization
     int weights_dirty;       // an expansion was enqueued since the last GEMV: that GEMV must not read records ahead of it
     int sm_count;

@@ -208,3 +208,24 @@ def test_gemv_random_shapes_grouped(B, ctx, oracle):
         for i, c in enumerate(cases):
             c.x = cases[0].x
             check_gemv(oracle, c, ys[i])
+
+
+def test_count_from_host_threads_on_streams_of_their_own(B, ctx, oracle):
+    """Counts of one context that overlap on the GPU share no scratch: every thread gets its matrix's count, time after time."""
+    import threading
+
+    cases = [make_overlay_case(oracle, rows, 24 * 64, seed=90 + rows, rate=rate) for rows, rate in ((6000, 0.02), (9000, 0.01), (2000, 0.05))]
+    want = [oracle.pack_planes10x(c.codes, c.rows, c.nb)[1] for c in cases]
+    torch.cuda.synchronize()
+    got = [[] for _ in cases]
+
+    def work(i):
+        stream = torch.cuda.Stream()
+        for _ in range(100):
+            got[i].append(B.overlay_count(ctx, cases[i].d_codes, cases[i].rows, cases[i].nb, stream=stream))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(cases))]
+    [t.start() for t in threads]
+    [t.join() for t in threads]
+    assert got == [[n] * 100 for n in want]
+    assert [B.overlay_count(ctx, c.d_codes, c.rows, c.nb) for c in cases] == want
