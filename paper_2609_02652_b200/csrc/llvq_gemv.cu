@@ -1596,13 +1596,13 @@ __global__ void __launch_bounds__(256) dequant_onehot_kernel(const uint8_t *__re
 // constants from global memory instead of a table 10.3.
 constexpr int kDequantWarps = 4;
 // The lane's twelve coordinates of a half-step's row as three groups of four halves.  Four codes, doubled, a byte each:
-// 2^22 + u by its bits, then x / 2 = u + (parity - 16) / 2, exactly, and one rounding of the product with twice the scale.
+// 2^23 + 2 u by its bits, then x = 2 u + (parity - 16), exactly, and one rounding of the product with the scale.
 __device__ __forceinline__ void dequant_row(uint32_t own, uint32_t shared, int e, float2 k0, float2 k1, float r, bool first_slot, uint2 v[3]) {
-    const float s0 = 2.f * (r * k0.x), s1 = 2.f * (r * k1.x);
+    const float s0 = r * k0.x, s1 = r * k1.x;
     auto four = [](uint32_t codes, float scale, float offset) {
         float f[4];
 #pragma unroll
-        for (int i = 0; i < 4; i++) f[i] = scale * (__uint_as_float(__byte_perm(codes, 0x4a800000u, 0x7650 + i)) + offset);
+        for (int i = 0; i < 4; i++) f[i] = scale * (__uint_as_float(__byte_perm(codes, 0x4b000000u, 0x7650 + i)) + offset);
         const __half2 lo = __floats2half2_rn(f[0], f[1]), hi = __floats2half2_rn(f[2], f[3]);
         return make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
     };
@@ -1625,7 +1625,7 @@ template <bool WHOLE_SECTORS>
 __global__ void __launch_bounds__(kDequantWarps * 32) dequant_planes_kernel(const uint8_t *__restrict__ buf, const __half *__restrict__ row_scale,
                                                                             float g0, float g1, __half *__restrict__ W, int64_t rows, int64_t nb,
                                                                             uint32_t total_units, const float2 *__restrict__ cls_block) {
-    // (class | gain << 9) -> {gain / (4 sqrt m), (parity - 16) / 2 - 2^22}
+    // (class | gain << 9) -> {gain / (4 sqrt m), parity - 16 - 2^23}
     __shared__ float2 tab[2 * kClassSlots];
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const uint32_t tiles = (uint32_t)(nb / kTileCells), left = (uint32_t)(nb % kTileCells), units = tiles + (left ? 1 : 0);
@@ -1635,7 +1635,7 @@ __global__ void __launch_bounds__(kDequantWarps * 32) dequant_planes_kernel(cons
     const bool whole = unit < total_units && u < tiles;
     for (int c = threadIdx.x; c < kClassSlots; c += blockDim.x) {
         const float2 k = __ldg(cls_block + c);
-        const float offset = 0.5f * (float)(__float_as_int(k.y) - 8388608);
+        const float offset = (float)(__float_as_int(k.y) - 8388608);
         tab[c] = make_float2(g0 * k.x, offset);
         tab[c + kClassSlots] = make_float2(g1 * k.x, offset);
     }
@@ -1643,7 +1643,7 @@ __global__ void __launch_bounds__(kDequantWarps * 32) dequant_planes_kernel(cons
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     uint4 w0, w1, w2, ha, hb;
-    if (whole) {                
+    if (whole) {
         w0 = __ldcs(reinterpret_cast<const uint4 *>(src + 16 * lane)); w1 = __ldcs(reinterpret_cast<const uint4 *>(src + 512 + 16 * lane));
         w2 = __ldcs(reinterpret_cast<const uint4 *>(src + 1024 + 16 * lane));
         ha = __ldcs(reinterpret_cast<const uint4 *>(src + 1536 + 32 * g)); hb = __ldcs(reinterpret_cast<const uint4 *>(src + 1552 + 32 * g));

@@ -234,6 +234,23 @@ def test_dequant_pieces(B, ctx, rows, nb, layout):
     assert torch.equal(W, (scale[:, :, None] * x).half().view(rows, nb * 24))
 
 
+def test_dequant_of_scales_near_the_largest_float(B, ctx):
+    """A scale between 2^127 and 2^128: the product with a coordinate overflows to infinity, or is zero where the coordinate is
+    zero - the same values that the f32 product of scale and coordinate has."""
+    rows, nb = 40, 7
+    case = make_case(rows, 24 * nb, seed=3)
+    buf = B.expand(ctx, 0, case.d_codes, rows, nb)
+    coords, _ = B.decode_i8(ctx, 0, buf, rows, nb)
+    x = coords.float()
+    inv_norm = (1.0 / (4.0 * ((x * x).sum(2) / 16).double().sqrt())).float()
+    d_scale = torch.full((rows,), 8.0, dtype=torch.float16, device="cuda")
+    gain = (2.0 ** 127.5, -(2.0 ** 127.9))
+    scale = 8.0 * (torch.where((case.d_codes.view(rows, nb) >> 47) != 0, gain[1], gain[0]).float() * inv_norm)
+    assert ((scale.abs() >= 2.0 ** 127) & scale.isfinite()).any() and (x == 0).any()
+    want = (scale[:, :, None] * x).half().view(rows, nb * 24)
+    assert torch.equal(B.dequant_fp16(ctx, 0, buf, d_scale, gain, rows, nb * 24).nan_to_num(nan=7.0), want.nan_to_num(nan=7.0))
+
+
 def test_noweights_control_returns_zero(B, ctx):
     case = make_case(4096, 4096, seed=2)
     y = torch.full((case.rows,), float("nan"), dtype=torch.float32, device="cuda")
