@@ -24,6 +24,7 @@ struct Entry {
 } entry;
 PyObject *error_class = nullptr;
 PyObject *handle_name = nullptr, *cuda_stream_name = nullptr;
+PyObject *gain_index[2] = {nullptr, nullptr};
 
 // ---- arguments
 int64_t integer(PyObject *o) {
@@ -72,16 +73,18 @@ const at::Tensor &tensor(PyObject *o, at::ScalarType dtype, const char *what) {
 template <typename T = void>
 T *device_pointer(PyObject *o, at::ScalarType dtype, const char *what) { return static_cast<T *>(tensor(o, dtype, what).data_ptr()); }
 
+// float(o[0]), float(o[1]), whatever o indexes by 0 and 1: a tuple, an array, a tensor (which is no sequence to Python's C API)
 struct Gain {
     float v[2];
     explicit Gain(PyObject *o) {
         for (int i = 0; i < 2; i++) {
-            PyObject *item = PySequence_GetItem(o, i);
+            PyObject *item = PyObject_GetItem(o, gain_index[i]);
             if (!item) throw python_error();
-            const double d = PyFloat_AsDouble(item);
-            Py_DECREF(item);
-            if (d == -1.0 && PyErr_Occurred()) throw python_error();
-            v[i] = static_cast<float>(d);
+            PyObject *number = PyFloat_CheckExact(item) ? item : PyNumber_Float(item);
+            if (number != item) Py_DECREF(item);
+            if (!number) throw python_error();
+            v[i] = static_cast<float>(PyFloat_AS_DOUBLE(number));
+            Py_DECREF(number);
         }
     }
 };
@@ -330,6 +333,7 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nu
 PyMODINIT_FUNC PyInit__native() {
     handle_name = PyUnicode_InternFromString("handle");
     cuda_stream_name = PyUnicode_InternFromString("cuda_stream");
-    if (!handle_name || !cuda_stream_name) return nullptr;
+    for (int i = 0; i < 2; i++) gain_index[i] = PyLong_FromLong(i);
+    if (!handle_name || !cuda_stream_name || !gain_index[0] || !gain_index[1]) return nullptr;
     return PyModule_Create(&module);
 }

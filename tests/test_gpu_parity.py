@@ -251,6 +251,21 @@ def test_dequant_of_scales_near_the_largest_float(B, ctx):
     assert torch.equal(B.dequant_fp16(ctx, 0, buf, d_scale, gain, rows, nb * 24).nan_to_num(nan=7.0), want.nan_to_num(nan=7.0))
 
 
+def test_gain_in_every_form_that_indexes(B, ctx):
+    """gain is anything whose elements 0 and 1 float() takes."""
+    case = make_case(64, 96, seed=1)
+    buf = B.expand(ctx, 0, case.d_codes, case.rows, case.nb)
+    pair = (0.75, 1.25)
+    args = lambda gain: (ctx, 0, buf, case.d_scale, gain, case.d_x, 64, 96)
+    want = B.gemv(*args(pair))
+    for gain in (list(pair), np.array(pair), np.array(pair, np.float32), torch.tensor(pair), torch.tensor(pair, device="cuda"), dict(enumerate(pair)), ("0.75", 1.25)):
+        assert torch.equal(B.gemv(*args(gain)), want), type(gain)
+    assert torch.equal(B.gemv(*args((1, True))), B.gemv(*args((1.0, 1.0))))
+    for gain, error in ((None, TypeError), (1.0, TypeError), ((1.0,), IndexError), ({0: 1.0}, KeyError), (("x", 1.0), ValueError)):
+        with pytest.raises(error):
+            B.gemv(*args(gain))
+
+
 def test_noweights_control_returns_zero(B, ctx):
     case = make_case(4096, 4096, seed=2)
     y = torch.full((case.rows,), float("nan"), dtype=torch.float32, device="cuda")
