@@ -257,17 +257,25 @@ def make_problems(problems) -> ctypes.Array:
     return arr
 
 
+def _problems(problems) -> ctypes.Array:
+    """The host array itself if it is one of make_problems's type (any other array is refused: it would be read as one), else
+    a new one of the sequence."""
+    if not isinstance(problems, ctypes.Array):
+        return make_problems(problems)
+    if not issubclass(problems._type_, Problem):
+        raise ctypes.ArgumentError(f"problems: expected an array of {Problem.__name__}, got one of {problems._type_.__name__}")
+    return problems
+
+
 def gemv_grouped(ctx: Context, layout: int, problems, x: torch.Tensor, k_padded: int, stream=None) -> None:
     """problems: a host array from make_problems, or the sequence make_problems takes."""
-    arr = problems if isinstance(problems, ctypes.Array) else make_problems(problems)
-    _launch().gemv_grouped(ctx, layout, arr, x, k_padded, stream)
+    _launch().gemv_grouped(ctx, layout, _problems(problems), x, k_padded, stream)
 
 
 def gemv_rotated(ctx: Context, problems, x: torch.Tensor, k_padded: int, n: int, block: int = 0,
                  negate_bits: torch.Tensor | None = None, stream=None) -> None:
     """llvq_gemv_rotated: the grouped 14-byte-layout GEMV on rotate(x[:n]) (the rest of x passes through), one launch."""
-    arr = problems if isinstance(problems, ctypes.Array) else make_problems(problems)
-    _launch().gemv_rotated(ctx, arr, x, k_padded, n, block, negate_bits, stream)
+    _launch().gemv_rotated(ctx, _problems(problems), x, k_padded, n, block, negate_bits, stream)
 
 
 def gemv_fp16(W: torch.Tensor, x: torch.Tensor, rows: int, k: int, y: torch.Tensor | None = None, stream=None) -> torch.Tensor:

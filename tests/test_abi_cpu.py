@@ -86,6 +86,27 @@ def test_missing_library_fails_loudly(monkeypatch):
         binding.load()
 
 
+def test_arrays_of_another_type_are_refused(lib):
+    """A host array whose elements are not llvq_problem would be read as device pointers."""
+    import torch
+
+    from paper_2609_02652_b200 import binding as B
+
+    class Handle:
+        handle = 1              # never reached: the array is looked at first, and x is no CUDA tensor
+
+    x = torch.zeros(24, dtype=torch.float16)
+    for arr in ((ctypes.c_char * 80)(), (ctypes.c_uint64 * 10)(), (B.Rotation * 2)(), (ctypes.POINTER(B.Problem) * 5)(), (B.Problem * 1 * 2)()):
+        with pytest.raises(ctypes.ArgumentError):
+            B.gemv_grouped(Handle, B.PLANES, arr, x, 24)
+        with pytest.raises(ctypes.ArgumentError):
+            B.gemv_rotated(Handle, arr, x, 24, n=8)
+    with pytest.raises(TypeError, match="x: expected"):
+        B.gemv_grouped(Handle, B.PLANES, (B.Problem * 1)(), x, 24)
+    with pytest.raises(TypeError, match="x: expected"):
+        B.gemv_rotated(Handle, (B.Problem * 1)(), x, 24, n=8)
+
+
 def _plan_invariants(plan, sm_count, rows, k_padded, batch, must_fit=True):
     nb = k_padded // 24
     tiles, left = divmod(nb, 4)
