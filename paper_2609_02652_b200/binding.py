@@ -195,25 +195,25 @@ def overlay_bytes(rows: int, k_padded: int, exceptions: int) -> int:
 
 def overlay_count(ctx: Context, codes: torch.Tensor, rows: int, nb: int, stream=None) -> int:
     """Blocks of the matrix that PLANES10X keeps in its exception table (synchronises the stream)."""
-    return _launch().overlay_count(ctx, codes, rows, nb, stream)
+    return (_native or _launch()).overlay_count(ctx, codes, rows, nb, stream)
 
 
 def expand(ctx: Context, layout: int, codes: torch.Tensor, rows: int, nb: int, out: torch.Tensor | None = None,
            bad_count: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     """codes: int64 CUDA tensor of rows*nb code words -> uint8 layout buffer (PLANES10X: sized by llvq_layout_bytes,
     i.e. with room for one exception in 32 blocks, unless `out` is given)."""
-    return _launch().expand(ctx, layout, codes, rows, nb, out, bad_count, stream)
+    return (_native or _launch()).expand(ctx, layout, codes, rows, nb, out, bad_count, stream)
 
 
 def gemv(ctx: Context, layout: int, layout_buf: torch.Tensor, row_scale: torch.Tensor, gain, x: torch.Tensor,
          rows: int, k_padded: int, y: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-    return _launch().gemv(ctx, layout, layout_buf, row_scale, gain, x, rows, k_padded, y, stream)
+    return (_native or _launch()).gemv(ctx, layout, layout_buf, row_scale, gain, x, rows, k_padded, y, stream)
 
 
 def gemv_batch(ctx: Context, layout_buf: torch.Tensor, row_scale: torch.Tensor, gain, x: torch.Tensor, rows: int,
                k_padded: int, y: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     """llvq_gemv_batch: x is fp16 [batch, k_padded] (contiguous), the result f32 [batch, rows]."""
-    return _launch().gemv_batch(ctx, layout_buf, row_scale, gain, x, rows, k_padded, y, stream)
+    return (_native or _launch()).gemv_batch(ctx, layout_buf, row_scale, gain, x, rows, k_padded, y, stream)
 
 
 def gemv_plan(sm_count: int, rows, k_padded: int, batch: int = 1) -> dict:
@@ -231,7 +231,7 @@ def gemv_static(layout_buf: torch.Tensor, row_scale: torch.Tensor, gain, x: torc
                 y: torch.Tensor, stream=None) -> torch.Tensor:
     """llvq_gemv_static: no context and no allocation inside the library; the caller supplies y.  Runs on the
     current CUDA device; at most 65536 rows; calls must not overlap on the GPU (they share built-in scratch)."""
-    return _launch().gemv_static(layout_buf, row_scale, gain, x, rows, k_padded, y, stream)
+    return (_native or _launch()).gemv_static(layout_buf, row_scale, gain, x, rows, k_padded, y, stream)
 
 
 def static_status(stream=None) -> None:
@@ -269,17 +269,17 @@ def _problems(problems) -> ctypes.Array:
 
 def gemv_grouped(ctx: Context, layout: int, problems, x: torch.Tensor, k_padded: int, stream=None) -> None:
     """problems: a host array from make_problems, or the sequence make_problems takes."""
-    _launch().gemv_grouped(ctx, layout, _problems(problems), x, k_padded, stream)
+    (_native or _launch()).gemv_grouped(ctx, layout, _problems(problems), x, k_padded, stream)
 
 
 def gemv_rotated(ctx: Context, problems, x: torch.Tensor, k_padded: int, n: int, block: int = 0,
                  negate_bits: torch.Tensor | None = None, stream=None) -> None:
     """llvq_gemv_rotated: the grouped 14-byte-layout GEMV on rotate(x[:n]) (the rest of x passes through), one launch."""
-    _launch().gemv_rotated(ctx, _problems(problems), x, k_padded, n, block, negate_bits, stream)
+    (_native or _launch()).gemv_rotated(ctx, _problems(problems), x, k_padded, n, block, negate_bits, stream)
 
 
 def gemv_fp16(W: torch.Tensor, x: torch.Tensor, rows: int, k: int, y: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-    return _launch().gemv_fp16(W, x, rows, k, y, stream)
+    return (_native or _launch()).gemv_fp16(W, x, rows, k, y, stream)
 
 
 def rotate_block(n: int, block: int = 0) -> int:
@@ -290,17 +290,17 @@ def rotate_block(n: int, block: int = 0) -> int:
 def rotate(ctx: Context, x: torch.Tensor, block: int = 0, negate_bits: torch.Tensor | None = None,
            y: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     """llvq_rotate: block-diagonal Walsh-Hadamard rotation of the fp16 vector x; `negate_bits` int32 words, bit i = flip x_i."""
-    return _launch().rotate(ctx, x, block, negate_bits, y, stream)
+    return (_native or _launch()).rotate(ctx, x, block, negate_bits, y, stream)
 
 
 def gemv_noweights(ctx: Context, row_scale: torch.Tensor, x: torch.Tensor, rows: int, k_padded: int,
                    y: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-    return _launch().gemv_noweights(ctx, row_scale, x, rows, k_padded, y, stream)
+    return (_native or _launch()).gemv_noweights(ctx, row_scale, x, rows, k_padded, y, stream)
 
 
 def dequant_fp16(ctx: Context, layout: int, layout_buf: torch.Tensor, row_scale: torch.Tensor, gain, rows: int,
                  k_padded: int, W: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-    return _launch().dequant_fp16(ctx, layout, layout_buf, row_scale, gain, rows, k_padded, W, stream)
+    return (_native or _launch()).dequant_fp16(ctx, layout, layout_buf, row_scale, gain, rows, k_padded, W, stream)
 
 
 def decode_i8(ctx: Context, layout: int, layout_buf: torch.Tensor, rows: int, nb: int, stream=None):

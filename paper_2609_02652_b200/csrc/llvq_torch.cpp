@@ -5,8 +5,12 @@
 // Nothing is computed.  The entry points' addresses come from the library that binding.py has loaded (bind()).
 #include <Python.h>
 
+#include <ATen/Context.h>
 #include <ATen/core/Tensor.h>
 #include <ATen/cuda/EmptyTensor.h>
+#include <ATen/ops/empty.h>
+#include <ATen/record_function.h>
+#include <c10/core/impl/LocalDispatchKeySet.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -99,6 +103,15 @@ void *stream(PyObject *o) {
     return p;
 }
 
+// torch.empty.  Where nothing in this thread could act on the call - no dispatch mode, transform, inference mode or profiler,
+// no fill under deterministic algorithms - the allocation alone is made: the dispatcher takes 0.35 us of a call of 4.4 (1024 x 2560,
+// back to back), its CUDA kernel alone still 0.25.
+at::Tensor new_tensor(at::IntArrayRef shape, at::ScalarType dtype, c10::Device device) {
+    const bool plain = c10::impl::tls_local_dispatch_key_set().included_ == c10::default_included_set && !at::hasCallbacks() &&
+                       !at::globalContext().deterministicAlgorithms();
+    return plain ? at::Tensor(at::detail::empty_cuda(shape, dtype, device, std::nullopt)) : at::empty(shape, at::TensorOptions().dtype(dtype).device(device));
+}
+
 // An output: the tensor the caller gave (checked), or a new one on the device of `like`.
 struct Output {
     PyObject *object;        // owned
@@ -109,8 +122,7 @@ struct Output {
             Py_INCREF(given);
             object = given;
         } else {
-            // torch.empty without its dispatcher
-            at::Tensor t = at::Tensor(at::detail::empty_cuda(shape, dtype, like.device(), std::nullopt));
+            at::Tensor t = new_tensor(shape, dtype, like.device());
             data = t.data_ptr();
             object = THPVariable_Wrap(std::move(t));
             if (!object) throw python_error();

@@ -266,6 +266,40 @@ def test_gain_in_every_form_that_indexes(B, ctx):
             B.gemv(*args(gain))
 
 
+def test_new_outputs_are_allocated_as_torch_empty_does(B, ctx):
+    """An output the caller does not give: dispatch modes and the profiler see its allocation, inference mode makes it an
+    inference tensor, and under deterministic algorithms what the call leaves unwritten (the overlay's unused table entries) is filled."""
+    from torch.utils._python_dispatch import TorchDispatchMode
+
+    class Seen(TorchDispatchMode):
+        def __init__(self):
+            super().__init__()
+            self.ops = []
+
+        def __torch_dispatch__(self, func, types, args=(), kwargs=None):
+            self.ops.append(str(func))
+            return func(*args, **(kwargs or {}))
+
+    case = make_case(64, 24 * 32, seed=1)
+    n = B.overlay_count(ctx, case.d_codes, 64, 32)
+    with Seen() as seen:
+        buf = B.expand(ctx, 0, case.d_codes, 64, 32)
+        y = B.gemv(ctx, 0, buf, case.d_scale, GAIN, case.d_x, 64, 24 * 32)
+    assert sum("aten.empty" in op for op in seen.ops) == 2
+    assert torch.isfinite(y).all() and not y.requires_grad and not y.is_inference()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CPU]) as profile:
+        B.gemv(ctx, 0, buf, case.d_scale, GAIN, case.d_x, 64, 24 * 32)
+    assert "aten::empty" in [event.key for event in profile.key_averages()]
+    with torch.inference_mode():
+        assert B.gemv(ctx, 0, buf, case.d_scale, GAIN, case.d_x, 64, 24 * 32).is_inference()
+    torch.use_deterministic_algorithms(True)
+    try:
+        out = B.expand(ctx, 3, case.d_codes, 64, 32)
+    finally:
+        torch.use_deterministic_algorithms(False)
+    assert B.overlay_bytes(64, 24 * 32, n) < out.numel() and (out[B.overlay_bytes(64, 24 * 32, n):] == 255).all()
+
+
 def test_noweights_control_returns_zero(B, ctx):
     case = make_case(4096, 4096, seed=2)
     y = torch.full((case.rows,), float("nan"), dtype=torch.float32, device="cuda")
