@@ -58,6 +58,11 @@ def load() -> ctypes.CDLL:
         except ImportError as e:
             raise RuntimeError("_native.so cannot be loaded: build it with `python -m paper_2609_02652_b200.build` "
                                f"(g++, the torch headers); there is no CPU fallback ({e})") from e
+        from .build import binding_tag
+
+        if native.built_for != binding_tag():
+            raise RuntimeError(f"_native.so was built for {native.built_for}, this is {binding_tag()}: build it again with "
+                               "`python -m paper_2609_02652_b200.build`")
         L = ctypes.CDLL(LIB_PATH)
         vp, i64, ci, sz = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, ctypes.c_size_t
         L.llvq_create.argtypes = [ctypes.POINTER(vp), ci, sz]

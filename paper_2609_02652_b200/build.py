@@ -38,6 +38,19 @@ def _run(cmd, target: str) -> None:
     os.replace(tmp, target)
 
 
+def binding_tag() -> str:
+    """The torch and the Python that _native.so is built for: it holds the layouts of both, so it must run under no other."""
+    import torch
+
+    return f"torch {torch.__version__} {torch.version.git_version}, {sysconfig.get_config_var('SOABI')}"
+
+
+def _built_for_another() -> bool:
+    """Whether _native.so lacks the tag of the torch and the Python that run now."""
+    with open(BINDING, "rb") as f:
+        return binding_tag().encode() + b"\0" not in f.read()
+
+
 def _build_binding() -> None:
     import torch
 
@@ -45,7 +58,7 @@ def _build_binding() -> None:
     cuda = os.path.join(os.path.dirname(os.path.dirname(_tool("nvcc", "/usr/local/cuda/bin/nvcc"))), "include")
     include = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), cuda,
                sysconfig.get_paths()["include"]]
-    _run([_tool("g++", "/usr/bin/g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+    _run([_tool("g++", "/usr/bin/g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f'-DLLVQ_BUILT_FOR="{binding_tag()}"', f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
           *["-isystem" + d for d in include], os.path.join(CSRC, BINDING_SOURCE), "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda",
           "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python"], BINDING)
 
@@ -55,7 +68,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if force or _stale(LIB, own):
         _run([_tool("nvcc", "/usr/local/cuda/bin/nvcc"), *NVCC_FLAGS, *(["-Xptxas", "-v"] if verbose else []),
               *[os.path.join(CSRC, s) for s in SOURCES]], LIB)
-    if force or _stale(BINDING, [os.path.join(CSRC, BINDING_SOURCE), HEADER]):
+    if force or _stale(BINDING, [os.path.join(CSRC, BINDING_SOURCE), HEADER]) or _built_for_another():
         _build_binding()
     return LIB
 

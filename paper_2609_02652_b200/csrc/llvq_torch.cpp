@@ -347,5 +347,7 @@ PyMODINIT_FUNC PyInit__native() {
     cuda_stream_name = PyUnicode_InternFromString("cuda_stream");
     for (int i = 0; i < 2; i++) gain_index[i] = PyLong_FromLong(i);
     if (!handle_name || !cuda_stream_name || !gain_index[0] || !gain_index[1]) return nullptr;
-    return PyModule_Create(&module);
+    PyObject *m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for", LLVQ_BUILT_FOR) != 0) Py_CLEAR(m);
+    return m;
 }

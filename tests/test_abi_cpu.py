@@ -107,6 +107,30 @@ def test_arrays_of_another_type_are_refused(lib):
         B.gemv_rotated(Handle, (B.Problem * 1)(), x, 24, n=8)
 
 
+def test_binding_is_rebuilt_for_another_torch_or_python(lib, monkeypatch):
+    """The binding holds the layouts of one torch and one Python: another one of either makes it stale, and it is not loaded."""
+    import sysconfig
+
+    import torch
+
+    from paper_2609_02652_b200 import _native, binding, build
+
+    built = []
+    monkeypatch.setattr(build, "_build_binding", lambda: built.append(1))
+    build.build()
+    assert built == [] and _native.built_for == build.binding_tag()
+    with monkeypatch.context() as m:
+        m.setattr(torch, "__version__", torch.__version__ + "1")
+        build.build()
+        m.setattr(binding, "_lib", None)
+        with pytest.raises(RuntimeError, match="build it again"):
+            binding.load()
+    with monkeypatch.context() as m:
+        m.setattr(sysconfig, "get_config_var", lambda name: "cpython-313-other")
+        build.build()
+    assert built == [1, 1]
+
+
 def _plan_invariants(plan, sm_count, rows, k_padded, batch, must_fit=True):
     nb = k_padded // 24
     tiles, left = divmod(nb, 4)
