@@ -1738,9 +1738,12 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
         g.smem = ((size_t)p.nb * 48 + 127) / 128 * 128;
         return g;
     }
-    // panels of about sixteen unit columns, as equal as they come
+    // panels of about sixteen unit columns, as equal as they come.  For more than four vectors of sixteen at most: a CTA that
+    // meets two panels then has a piece of x for each of its twelve warps' threads, and none is read again, vector after vector
+    // (five vectors, us with panels of 18 columns and of 15: 500 x 8192 12.3 and 10.0, two passes 10.7; eight on 2560 x 5120 19.2 and 15.0, 17.4).
     constexpr int kPanelColumns = 16;
-    const int want = (p.units + kPanelColumns / 2) / kPanelColumns > 1 ? (p.units + kPanelColumns / 2) / kPanelColumns : 1;
+    static_assert(2 * kPanelColumns * kTileCells * 3 <= 32 * gemv_warps(LLVQ_MAX_BATCH), "two panels' pieces of x, a thread each");
+    const int most = (p.units + (p.batch > 4 ? kPanelColumns - 1 : kPanelColumns / 2)) / kPanelColumns, want = most > 1 ? most : 1;
     p.panel = (p.units + want - 1) / want;
     p.npanels = (p.units + p.panel - 1) / p.panel;
     p.div_panel = make_fastdiv((uint32_t)p.panel);

@@ -23,3 +23,38 @@ def run_native(tmp_path, source, *more, stdin=None):
 
 def test_plan_cache_hands_out_whole_plans_to_threads(tmp_path):
     assert run_native(tmp_path, "plan_cache.cpp").strip() == "0"
+
+
+def test_plan_of_five_to_eight_vectors(tmp_path):
+    """The pass that llvq_gemv_plan does not describe (twelve warps, eight records of x a block): shares, panels, shared memory,
+    and at most two panels' pieces of x a CTA on a full-size part, a thread each, so that none is read twice."""
+    import numpy as np
+
+    from paper_2609_02652_b200 import build
+
+    build.build()
+    rng = np.random.default_rng(12)
+    shapes = [(148, 500, 8208, 5), (148, 2560, 9744, 5), (148, 1024, 17424, 8), (148, 1, 24, 6), (148, 36864, 5136, 7), (8, 4096, 98304, 8)]
+    for _ in range(300):
+        k = 24 * int(rng.integers(1, 4097) if rng.random() < 0.2 else rng.integers(1, 750))
+        shapes.append((int(rng.choice([1, 8, 132, 148, 160, 320])), int(np.exp(rng.uniform(0, np.log(60000)))), k, int(rng.integers(5, 9))))
+    where = os.path.dirname(build.LIB)
+    out = run_native(tmp_path, "batch_plan.cpp", "-L" + where, "-l:libllvq.so", "-Wl,-rpath," + where, stdin="".join("%d %d %d %d\n" % s for s in shapes))
+    lines = out.strip().splitlines()
+    assert len(lines) == len(shapes)
+    beyond = 0
+    for (sm, rows, k, batch), line in zip(shapes, lines):
+        grid, smem, units, panel, npanels, xblocks, groups, *ctas = map(int, line.split())
+        nb, total, first = k // 24, groups * units, ctas[0::3]
+        assert 1 <= grid <= min(sm, 256) and first[0] == 0 and first[-1] == total and all(a <= b for a, b in zip(first, first[1:]))
+        assert 1 <= panel <= 16 and (npanels - 1) * panel < units <= npanels * panel
+        for c in range(grid):
+            f0, f1, lo, hi = first[c], first[c + 1], ctas[3 * c + 1], ctas[3 * c + 2]
+            last = max(f1 - 1, f0)
+            assert lo == min(f0 // (groups * panel), npanels - 1) * panel * 4
+            assert hi == min(nb, (min(last // (groups * panel), npanels - 1) + 1) * panel * 4) and hi - lo <= xblocks
+        assert smem >= 12 * 2 * 1792 + 8192 + 8 * xblocks * 112 + 12 * 2 * 8 + 12 * 4 * 8
+        if sm >= 132:
+            assert 3 * xblocks <= 12 * 32 and smem + 1024 <= 227 * 1024
+        beyond += smem + 1024 > 227 * 1024
+    assert beyond                     # few multiprocessors and a long row: the launch is refused, and llvq_gemv_batch takes two passes
