@@ -557,15 +557,17 @@ __device__ __forceinline__ void each_pair(F &f) {
 // 24 nb halves one after the other, y BATCH vectors of rows floats (p.prob[].y is vector 0's), the accumulators
 // BATCH sets of total_groups * 32.
 // ROTATE: x is rotated on its way into the records (llvq_gemv_rotated): every CTA rotates the Walsh-Hadamard
-// blocks of x that its share of the matrix touches, exactly as the rotation kernel does, and rounds them to FP16.
+// blocks of x that its share of the matrix touches, exactly as the rotation kernel does, and rounds them to FP16.  Short and
+// long blocks (rot_first) have kernels of their own: either's code in the other's way costs a launch 0.1 us.
 // LAYOUT: LLVQ_PLANES; LLVQ_PLANES13 (one header byte a block; the code words are where the 14-byte layout has them);
 // LLVQ_PLANES10X (tiles of three-bit codes, leftover blocks as in the 13-byte layout, and after each run the exact
 // records of the run's exception blocks, whose short records are empty and add nothing).
-template <bool NO_WEIGHTS, int BATCH, bool ROTATE = false, int LAYOUT = LLVQ_PLANES>
+enum Rotate { kNoRotation, kRotateShort, kRotateLong };
+template <bool NO_WEIGHTS, int BATCH, Rotate ROTATE = kNoRotation, int LAYOUT = LLVQ_PLANES>
 __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(const __grid_constant__ GemvParams p) {
     constexpr int kWarps = gemv_warps(BATCH), kThreads = 32 * kWarps;
     constexpr bool COMPACT = LAYOUT != LLVQ_PLANES, OVERLAY = LAYOUT == LLVQ_PLANES10X;
-    static_assert(!OVERLAY || (BATCH == 1 && !ROTATE && !NO_WEIGHTS), "the 10-byte layout: one vector, as it is");
+    static_assert(!OVERLAY || (BATCH == 1 && ROTATE == kNoRotation && !NO_WEIGHTS), "the 10-byte layout: one vector, as it is");
     constexpr int kSrcCell = COMPACT ? kCell13Bytes : kCellBytes;        // bytes of a leftover block column of a row group
     constexpr int kSrcTile = OVERLAY ? kTile10Bytes : (COMPACT ? kTile13Bytes : kTileBytes);   // bytes of a tile in memory (a ring slot always has kTileBytes)
     extern __shared__ __align__(128) unsigned char smem[];
@@ -577,8 +579,8 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
     float2 *tab = reinterpret_cast<float2 *>(smem + kWarps * kSlots * kTileBytes + tab_pad);
     unsigned char *xrec = smem + kWarps * kSlots * kTileBytes + tab_pad + p.nprob * 8192;
     constexpr int kXBlock = BATCH * kXRecBytes;                                    // the vectors' records of a block lie side by side
-    // ROTATE: the records take the place of the FP16 values that are rotated
-    const int xrec_bytes = ROTATE ? max(p.xblocks * kXBlock, 2 * p.rot_span) : p.xblocks * kXBlock;
+    // long blocks: the records take the place of the FP16 values that are rotated
+    const int xrec_bytes = ROTATE == kRotateLong ? max(p.xblocks * kXBlock, 2 * p.rot_span) : p.xblocks * kXBlock;
     uint64_t *bars = reinterpret_cast<uint64_t *>(xrec + ((xrec_bytes + 127) / 128) * 128);
     uint32_t *warp_max = reinterpret_cast<uint32_t *>(bars + kWarps * kSlots);     // one slot a warp and vector
     double *rot = reinterpret_cast<double *>(warp_max + BATCH * kWarps);           // ROTATE: the sums of this CTA's part of x
@@ -782,7 +784,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
     }
     // ROTATE: the coordinates [c_lo, c_hi) this CTA rotates are the whole rotation blocks that meet its blocks of x
     int c_lo = 0, c_hi = 0;
-    if (ROTATE) {
+    if (ROTATE != kNoRotation) {
         const int mask = (1 << p.rot_log2) - 1;
         c_lo = min(p.rot_n, (24 * blk_lo) & ~mask);
         c_hi = min(p.rot_n, (24 * blk_hi + mask) & ~mask);
@@ -837,19 +839,39 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
     // 2^(29 - xexp).
     bool failed = false;
     int xexp[BATCH];
-    if constexpr (ROTATE) {
+    if constexpr (ROTATE != kNoRotation) {
         // The rotated vector's largest magnitude is not known before it is rotated, but every rotated coordinate is
         // a unit-norm combination of its block, so |x'_k| <= ||x||_2: the scan sums the squares instead of taking
         // the maximum, and the fixed-point scale follows from that bound (a few bits coarser than the maximum
-        // would give, of 29).  In the same pass the pieces of this CTA's rotation blocks go to shared memory, signs flipped;
-        // the stages follow there, three a pass and the last three in registers; the rounded FP16 values - those of
-        // the rotation kernel - become the fixed-point records.
+        // would give, of 29).  In the same pass the pieces of this CTA's rotation blocks go to shared memory, signs flipped, short
+        // blocks with their narrowest three stages done (rot_first); the stages follow there, three a pass, the last six of a piece
+        // of 64 by eight lanes; the rounded FP16 values - those of the rotation kernel - become the fixed-point records.
         const int nx = p.nb * 3, e_lo = 3 * blk_lo, e_hi = 3 * blk_hi;
-        const bool one_each = e_hi - e_lo <= kThreads;
+        constexpr bool in_scan = ROTATE == kRotateShort;
+        // the pieces that a thread keeps in registers if it meets no two of them: those of this CTA's share past the rotated
+        // length; of short blocks those to rotate, too
+        const int s_lo = in_scan && c_lo < c_hi ? c_lo >> 3 : e_lo, s_hi = in_scan ? max(e_hi, c_hi >> 3) : e_hi;
+        const bool one_each = s_hi - s_lo <= kThreads;
         const uint4 *xg = reinterpret_cast<const uint4 *>(p.x);
-        uint4 mine = make_uint4(0u, 0u, 0u, 0u);               // a piece of this CTA's share past the rotated length
+        uint4 mine = make_uint4(0u, 0u, 0u, 0u);
         int mine_e = -1;
         float ss = __uint_as_float(settled(warm, warm, warm));
+        const int need_lo = min(p.rot_n, 24 * blk_lo), need_hi = min(p.rot_n, 24 * blk_hi);
+        auto down = [&](int s) { return need_lo & ~((1 << s) - 1); };
+        auto up = [&](int s) { return (need_hi + (1 << s) - 1) & ~((1 << s) - 1); };
+        const RotFirst rf = rot_first(p.rot_log2);
+        const int rot0 = down(rf.stride);              // the coordinate in the first place of `rot`
+        const bool alone = in_scan && one_each && rf.stride == 3;      // a block of eight is one piece: it stays with its thread
+        auto flipped = [&](const uint4 &x, int e) {
+            const uint32_t flips = p.rot_negate ? __ldg(p.rot_negate + (e >> 2)) >> (8 * (e & 3)) : 0u;
+            auto signs = [&](int k) { return ((flips >> (2 * k) & 1u) << 15) ^ ((flips >> (2 * k + 1) & 1u) << 31); };
+            return make_uint4(x.x ^ signs(0), x.y ^ signs(1), x.z ^ signs(2), x.w ^ signs(3));
+        };
+        // the zero word and the two sums of every record
+        auto zero_sums = [&]() {
+            for (int b = tid; b < blk_hi - blk_lo; b += kThreads)
+                asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(smem_addr(xrec) + b * kXRecBytes + 96), "r"(0) : "memory");
+        };
         for (int base = 0; base < nx; base += 4 * kThreads) {
             uint4 v[4];
 #pragma unroll
@@ -857,7 +879,10 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 const int e = base + i * kThreads + tid;
                 v[i] = e < nx ? __ldcg(xg + e) : make_uint4(0u, 0u, 0u, 0u);
             }
-            if (base == 0) build_tables();
+            if (base == 0) {
+                if (in_scan) zero_sums();
+                build_tables();
+            }
 #pragma unroll
             for (int i = 0; i < 4; i++) {
                 const int e = base + i * kThreads + tid;
@@ -868,16 +893,17 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                     ss = fmaf(f.x, f.x, ss);
                     ss = fmaf(f.y, f.y, ss);
                 }
-                if (8 * e >= c_lo && 8 * e < c_hi) {
-                    const uint32_t flips = p.rot_negate ? __ldg(p.rot_negate + (e >> 2)) >> (8 * (e & 3)) : 0u;
-                    auto flipped = [&](int k) { return w[k] ^ ((flips >> (2 * k) & 1u) << 15) ^ ((flips >> (2 * k + 1) & 1u) << 31); };
-                    *reinterpret_cast<uint4 *>(xrec + 2 * (8 * e - c_lo)) = make_uint4(flipped(0), flipped(1), flipped(2), flipped(3));
-                } else if (e >= e_lo && e < e_hi) {
+                if (!in_scan && 8 * e >= c_lo && 8 * e < c_hi) {
+                    *reinterpret_cast<uint4 *>(xrec + 2 * (8 * e - c_lo)) = flipped(v[i], e);
+                } else if (e >= s_lo && e < s_hi) {
                     mine = v[i];
                     mine_e = e;
                 }
             }
         }
+        if (in_scan && !alone)
+            for (int e = one_each ? mine_e : (c_lo >> 3) + tid; e >= 0 && 8 * e < c_hi; e += one_each ? nx : kThreads)
+                rot_start8(rot, 8 * e - rot0, flipped(one_each ? mine : __ldcg(xg + e), e));
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
         if (lane == 0) warp_max[warp] = __float_as_uint(ss);
@@ -886,24 +912,13 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
 #pragma unroll
             for (int s = kEarlySlots; s < kSlots; s++) issue(my_bar + 8 * s, my_ring + s * kTileBytes);
         }
-        const int need_lo = min(p.rot_n, 24 * blk_lo), need_hi = min(p.rot_n, 24 * blk_hi);
-        auto down = [&](int s) { return need_lo & ~((1 << s) - 1); };
-        auto up = [&](int s) { return (need_hi + (1 << s) - 1) & ~((1 << s) - 1); };
-        const RotFirst rf = rot_first(p.rot_log2);
-        const int rot0 = down(rf.stride);              // the coordinate in the first place of `rot`
-        {
-            const __half *raw = reinterpret_cast<const __half *>(xrec);
-            if (rf.stages == 3) rot_narrow<3, true>(rot, rot0, raw, c_lo, c_hi, rot0, up(rf.stride), rf.stride, tid, kThreads);
-            else if (rf.stages == 2) rot_narrow<2, true>(rot, rot0, raw, c_lo, c_hi, rot0, up(rf.stride), rf.stride, tid, kThreads);
-            else if (rf.stages == 1) rot_narrow<1, true>(rot, rot0, raw, c_lo, c_hi, rot0, up(rf.stride), rf.stride, tid, kThreads);
-            else rot_narrow<0, true>(rot, rot0, raw, c_lo, c_hi, rot0, up(rf.stride), rf.stride, tid, kThreads);
+        if (!in_scan) {
+            rot_narrow<3, true>(rot, rot0, reinterpret_cast<const __half *>(xrec), c_lo, c_hi, rot0, up(rf.stride), rf.stride, tid, kThreads);
+            __syncthreads();
+            zero_sums();                               // the FP16 values, which lay there, are read
         }
-        __syncthreads();
-        // the zero word and the two sums of every record, now that the FP16 values are read
-        for (int b = tid; b < blk_hi - blk_lo; b += kThreads)
-            asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(smem_addr(xrec) + b * kXRecBytes + 96), "r"(0) : "memory");
-        // down to pieces of 64, whose last six stages a group of eight lanes takes by itself (or of 8, for short blocks)
-        const int last = rf.stride >= 6 ? 6 : 3;
+        // down to pieces of 64, whose other stages a group of eight lanes takes by itself, or the short block itself
+        const int last = in_scan ? min(rf.stride, 6) : 6;
         for (int s = rf.stride; s > last;) {
             const int wide = s, r = s % 3 ? s % 3 : 3;
             s -= r;
@@ -912,7 +927,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
             else rot_narrow<1, false>(rot, rot0, nullptr, down(wide), up(wide), down(s), up(s), s, tid, kThreads);
             if (s > last) __syncthreads();
         }
-        __syncthreads();
+        if (!in_scan || rf.stride > last) __syncthreads();
         {
             // every thread of every CTA adds the sixteen sums in the same order
             float total = __uint_as_float(warp_max[lane & (kWarps - 1)]);
@@ -926,17 +941,23 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
         const float scale = pow2f(29 - xexp[0]);
         // rotated pieces: from the exact sums; pieces past the rotated length: as they are (the one this thread
         // met in the scan, or read again when the share is too wide for that)
-        for (int e0 = (down(last) >> 3) + 32 * warp; 8 * e0 < need_hi; e0 += kThreads) {
-            const int e = e0 + lane;
-            if (last == 6) {
-                if (8 * e < up(6)) rot_middle8(rot, 8 * e - rot0);
+        if (!alone)
+            for (int e0 = (down(last) >> 3) + 32 * warp; 8 * e0 < need_hi; e0 += kThreads) {
+                const int e = e0 + lane;
+                if (8 * e < up(last)) {
+                    if (!in_scan || last == 6) rot_middle8<3>(rot, 8 * e - rot0);
+                    else if (last == 5) rot_middle8<2>(rot, 8 * e - rot0);
+                    else if (last == 4) rot_middle8<1>(rot, 8 * e - rot0);
+                }
                 __syncwarp();
+                if (e >= e_lo && 8 * e < need_hi) convert_item(rot_finish8(rot, 8 * e - rot0, !in_scan, p.rot_scale), e % 3, xs0 + (uint32_t)(e / 3) * kXRecBytes, scale);
             }
-            if (e >= e_lo && 8 * e < need_hi) convert_item(rot_finish8(rot, 8 * e - rot0, p.rot_scale), e % 3, xs0 + (uint32_t)(e / 3) * kXRecBytes, scale);
-        }
         if (!one_each)
             for (int e = max(e_lo, c_hi >> 3) + tid; e < e_hi; e += kThreads) convert_item(__ldcg(xg + e), e % 3, xs0 + (uint32_t)(e / 3) * kXRecBytes, scale);
-        if (one_each && mine_e >= 0) convert_item(mine, mine_e % 3, xs0 + (uint32_t)(mine_e / 3) * kXRecBytes, scale);
+        if (one_each && mine_e >= (in_scan && !alone ? max(e_lo, c_hi >> 3) : 0)) {
+            if (alone && 8 * mine_e < c_hi) mine = rot_whole8(flipped(mine, mine_e), p.rot_scale);
+            convert_item(mine, mine_e % 3, xs0 + (uint32_t)(mine_e / 3) * kXRecBytes, scale);
+        }
         __syncthreads();                               // publishes the x records
     } else {
         const int nx = p.nb * 3, e_lo = 3 * blk_lo, e_hi = 3 * blk_hi;
@@ -1805,7 +1826,7 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
     }
     const int vectors = p.batch <= 2 ? p.batch : (p.batch <= 4 ? 4 : 8);       // the kernel is built for 1, 2, 4 and 8
     const int warps = gemv_warps(vectors);
-    const size_t records = ((size_t)p.xblocks * kXRecBytes * vectors + 127) / 128 * 128, raw = ((size_t)p.rot_span * 2 + 127) / 128 * 128;
+    const size_t records = ((size_t)p.xblocks * kXRecBytes * vectors + 127) / 128 * 128, raw = rot_first(p.rot_log2).stages ? ((size_t)p.rot_span * 2 + 127) / 128 * 128 : 0;
     g.smem = (size_t)warps * kSlots * kTileBytes + 8192 /* alignment of the tables */ + (size_t)p.nprob * 8192 + warps * kSlots * 8 + warps * 4 * vectors + 16;
     // a rotation counts with eight bytes a coordinate of its whole blocks, the limit llvq_gemv_rotated states, though it needs less
     const size_t rot_needs = (records > raw ? records : raw) + ((size_t)p.rot_keep + 15) / 16 * 128, rot_stated = records + (size_t)p.rot_span * 8;
@@ -1831,9 +1852,10 @@ int gemv_configure(const llvq_ctx *ctx) {
     if (allow_max_smem(gemv_planes_kernel<false, 2>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 4>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 8>, bytes)) return -1;
-    if (allow_max_smem(gemv_planes_kernel<false, 1, true>, bytes)) return -1;
-    if (allow_max_smem(gemv_planes_kernel<false, 1, false, LLVQ_PLANES13>, bytes)) return -1;
-    if (allow_max_smem(gemv_planes_kernel<false, 1, false, LLVQ_PLANES10X>, bytes)) return -1;
+    if (allow_max_smem(gemv_planes_kernel<false, 1, kRotateShort>, bytes)) return -1;
+    if (allow_max_smem(gemv_planes_kernel<false, 1, kRotateLong>, bytes)) return -1;
+    if (allow_max_smem(gemv_planes_kernel<false, 1, kNoRotation, LLVQ_PLANES13>, bytes)) return -1;
+    if (allow_max_smem(gemv_planes_kernel<false, 1, kNoRotation, LLVQ_PLANES10X>, bytes)) return -1;
     if (allow_max_smem(gemv_onehot_kernel, bytes)) return -1;
     return 0;
 }
@@ -1849,11 +1871,11 @@ cudaError_t launch_gemv(int layout, const GemvParams &p, const GemvLaunch &g, bo
     attr[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (layout == LLVQ_PLANES13) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 1, false, LLVQ_PLANES13>, p);
-    if (layout == LLVQ_PLANES10X) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 1, false, LLVQ_PLANES10X>, p);
+    if (layout == LLVQ_PLANES13) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 1, kNoRotation, LLVQ_PLANES13>, p);
+    if (layout == LLVQ_PLANES10X) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 1, kNoRotation, LLVQ_PLANES10X>, p);
     if (layout == LLVQ_PLANES) {
         if (no_weights) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<true, 1>, p);
-        if (p.rot_log2 > 0) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 1, true>, p);
+        if (p.rot_log2 > 0) return cudaLaunchKernelEx(&cfg, rot_first(p.rot_log2).stages ? gemv_planes_kernel<false, 1, kRotateLong> : gemv_planes_kernel<false, 1, kRotateShort>, p);
         if (p.batch <= 1) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 1>, p);
         if (p.batch == 2) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 2>, p);
         if (p.batch <= 4) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 4>, p);

@@ -102,11 +102,14 @@ __device__ __forceinline__ uint4 rot_round8(const long long *v, int first, doubl
 }
 
 // ---- the rotation of a stretch of x inside the GEMV.  A CTA needs the coordinates [need_lo, need_hi) of the rotated vector, a
-// small part of the blocks they lie in, so the stages run from the widest stride down: once the stages of strides 2^s and
-// more are done, only the pieces of 2^s coordinates that meet the part needed go on.  In f64 the sums are those of the
+// small part of long blocks, so the stages run from the widest stride down: once the stages of strides 2^s and
+// more are done, only the pieces of 2^s coordinates that meet the part needed go on (rot_first says which blocks are long).  In f64 the sums are those of the
 // integers: every partial sum ahead of a 2^14 block's last stage is a multiple of 2^-24 below 2^29, hence exact, and where
 // the last stage's is not, it is rounded as the integer would be on its way to f64.  One instruction an addition where the
 // 64-bit integers take two, and no conversion at the end.
+
+// The f64 value of an FP16's bits (in the low half of h), times 2^-1008: its exponent and mantissa, moved up.
+__device__ __forceinline__ double rot_widen(uint32_t h) { return __hiloint2double((int)(((uint32_t)(int)(short)h << 10) & 0x81ffffffu), 0); }
 
 // Stages S .. S + R - 1 over the coordinates [lo, hi) (multiples of 2^(S+R)); of the results those in [keep_lo, keep_hi)
 // (multiples of 2^S) are stored.  v holds coordinate first + i in place rot_at(i).  RAW: the inputs are FP16, raw[0] = coordinate lo.
@@ -117,7 +120,7 @@ __device__ __forceinline__ void rot_narrow(double *v, int first, const __half *r
         double a[8];
 #pragma unroll
         for (int j = 0; j < (1 << R); j++) {
-            if (RAW) a[j] = __hiloint2double((int)(((uint32_t)(int)reinterpret_cast<const short *>(raw)[base + (j << S)] << 10) & 0x81ffffffu), 0);
+            if (RAW) a[j] = rot_widen(reinterpret_cast<const uint16_t *>(raw)[base + (j << S)]);
             else a[j] = v[rot_at(lo - first + base + (j << S))];
         }
         rot_butterflies<R>(a);
@@ -129,29 +132,62 @@ __device__ __forceinline__ void rot_narrow(double *v, int first, const __half *r
     }
 }
 
-// Stages 3 .. 5 of a piece of 64 by eight neighbouring lanes: the lane whose eight values begin at place `at` takes the values
-// eight apart.  A __syncwarp() belongs between this and rot_finish8.
+// Stages 3 .. 2 + R of a piece of 8 * 2^R by 2^R neighbouring lanes: the lane whose eight values begin at place `at` takes its share
+// of the sets of values eight apart.  A __syncwarp() belongs between this and rot_finish8.
+template <int R>
 __device__ __forceinline__ void rot_middle8(double *v, int at) {
-    const int base = (at & ~63) + ((at >> 3) & 7);
-    double a[8];
+    constexpr int kLanes = 1 << R, kSets = 8 >> R;
+    const int base = (at & ~(8 * kLanes - 1)) + ((at >> 3) & (kLanes - 1));
+    double a[kSets][8];
 #pragma unroll
-    for (int j = 0; j < 8; j++) a[j] = v[rot_at(base + 8 * j)];
-    rot_butterflies<3>(a);
+    for (int c = 0; c < kSets; c++) {
 #pragma unroll
-    for (int j = 0; j < 8; j++) v[rot_at(base + 8 * j)] = a[j];
+        for (int j = 0; j < kLanes; j++) a[c][j] = v[rot_at(base + kLanes * c + 8 * j)];
+        rot_butterflies<R>(a[c]);
+#pragma unroll
+        for (int j = 0; j < kLanes; j++) v[rot_at(base + kLanes * c + 8 * j)] = a[c][j];
+    }
 }
 
-// The last three stages of the eight values from place `at` on (a multiple of eight), and the one rounding.
-__device__ __forceinline__ uint4 rot_finish8(const double *v, int at, double scale) {
-    double a[8];
+// Eight consecutive FP16 values (two a word) and their three narrowest stages.
+__device__ __forceinline__ void rot_widen8(const uint4 &x, double (&a)[8]) {
+    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-    for (int k = 0; k < 8; k++) a[k] = v[rot_at(at + k)];
+    for (int k = 0; k < 8; k++) a[k] = rot_widen(w[k >> 1] >> (16 * (k & 1)));
     rot_butterflies<3>(a);
+}
+
+// The same, stored as the values at places at .. at + 7 (at a multiple of eight).
+__device__ __forceinline__ void rot_start8(double *v, int at, const uint4 &x) {
+    double a[8];
+    rot_widen8(x, a);
+#pragma unroll
+    for (int k = 0; k < 8; k++) v[rot_at(at + k)] = a[k];
+}
+
+// The one rounding of eight sums.
+__device__ __forceinline__ uint4 rot_to_half8(const double (&a)[8], double scale) {
     uint32_t out[4];
 #pragma unroll
     for (int i = 0; i < 4; i++)
         out[i] = (uint32_t)__half_as_ushort(__double2half(a[2 * i] * scale)) | ((uint32_t)__half_as_ushort(__double2half(a[2 * i + 1] * scale)) << 16);
     return make_uint4(out[0], out[1], out[2], out[3]);
+}
+
+// The eight values from place `at` on (a multiple of eight), their three narrowest stages if those are still to do, rounded.
+__device__ __forceinline__ uint4 rot_finish8(const double *v, int at, bool stages_left, double scale) {
+    double a[8];
+#pragma unroll
+    for (int k = 0; k < 8; k++) a[k] = v[rot_at(at + k)];
+    if (stages_left) rot_butterflies<3>(a);
+    return rot_to_half8(a, scale);
+}
+
+// A whole block of eight.
+__device__ __forceinline__ uint4 rot_whole8(const uint4 &x, double scale) {
+    double a[8];
+    rot_widen8(x, a);
+    return rot_to_half8(a, scale);
 }
 
 }  // namespace llvq

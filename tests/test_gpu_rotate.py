@@ -193,6 +193,21 @@ def test_gemv_rotated_every_block_length(B, ctx, oracle, log2):
     assert err <= 1e-6
 
 
+@pytest.mark.parametrize("rows", [40, 3000])
+@pytest.mark.parametrize("n,block", [(8, 8), (24, 8), (16, 16), (96, 32), (64, 64), (1152, 128), (256, 256), (768, 256), (512, 512), (1024, 1024)])
+def test_gemv_rotated_of_a_short_part(B, ctx, oracle, rows, n, block):
+    """Most of x passes through: multiprocessors whose part of x holds no rotated entry, the end of the rotated part inside one, and
+    blocks of each way the rotation starts.  Bound as above."""
+    case = make_case(rows, 9728, seed=n + rows)
+    neg = np.random.default_rng(n).integers(0, 2, size=n)
+    buf = B.expand(ctx, 0, case.d_codes, case.rows, case.nb)
+    y = torch.full((rows,), float("nan"), dtype=torch.float32, device="cuda")
+    B.gemv_rotated(ctx, [(buf, case.d_scale, GAIN, y, rows)], case.d_x, case.nb * 24, n=n, block=block, negate_bits=_bits(neg))
+    torch.cuda.synchronize()
+    err, _ = check_gemv(oracle, _rotated_reference(oracle, case, n, block, neg), y)
+    assert err <= 1e-6
+
+
 def test_gemv_rotated_grouped_launch_and_outlier_activation(B, ctx, oracle):
     """q/k/v-like group sharing one x; x with one huge entry (what the rotation is for): the bound on the
     rotated magnitudes is then loosest, and the result must still meet the bar with room."""
