@@ -279,7 +279,7 @@ int llvq_gemv_grouped(llvq_ctx *ctx, int layout, const llvq_problem *problems, i
  * bit for bit the FP16 values llvq_rotate(x, rotation->n, rotation->block, rotation->negate_bits) would store,
  * so y agrees with llvq_rotate followed by llvq_gemv_grouped to within the GEMV's fixed-point quantum (the
  * scale of that quantum comes from ||x||_2, which bounds every rotated entry, instead of from the largest
- * entry).  x itself is not modified.  The blocks a CTA rotates must fit its shared memory beside the GEMV's
+ * entry).  x itself is not modified.  x must be finite; if an entry is not, every entry of y is NaN.  The blocks a CTA rotates must fit its shared memory beside the GEMV's
  * own: block lengths up to 4096 always do; a longer block may return LLVQ_ESIZE (rotate with llvq_rotate then).
  * Errors: those of llvq_gemv_grouped; LLVQ_EINVAL also for a null rotation, n not a positive multiple of 8
  * or above k_padded, a block that is not acceptable or shorter than 8. */

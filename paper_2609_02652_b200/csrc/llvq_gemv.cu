@@ -150,7 +150,7 @@ __device__ __forceinline__ void settle(const GemvParams &p, Handed &h) {
 // `accum` and `y` are the accumulators and the output of the activation vector the sum belongs to (a batched
 // launch has one set a vector)
 __device__ __forceinline__ void hand_over(const GemvParams &p, const GemvProblemDev &pr, unsigned long long *accum, float *y,
-                                          int group, int lane, long long sum, int count, int qexp, float row_scale, Handed &h) {
+                                          int group, int lane, long long sum, int count, float quantum, float row_scale, Handed &h) {
     settle(p, h);
     const int row = (group - pr.group_begin) * kRowsPerGroup + lane;
     if (row >= pr.rows) return;                      // padding rows of the last row group
@@ -158,7 +158,7 @@ __device__ __forceinline__ void hand_over(const GemvParams &p, const GemvProblem
     h.slot = accum + (size_t)group * 32 + lane;
     h.old = atomicAdd(h.slot, h.addend);
     h.y = y + row;
-    h.yscale = pow2f(qexp) * row_scale;
+    h.yscale = quantum * row_scale;
     h.count = count;
 }
 
@@ -839,6 +839,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
     // 2^(29 - xexp).
     bool failed = false;
     int xexp[BATCH];
+    [[maybe_unused]] float x_scale;                    // ROTATE: 2^xexp
     if constexpr (ROTATE != kNoRotation) {
         // The rotated vector's largest magnitude is not known before it is rotated, but every rotated coordinate is
         // a unit-norm combination of its block, so |x'_k| <= ||x||_2: the scan sums the squares instead of taking
@@ -937,6 +938,9 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
             // every |x'| is below 2^ceil(e2 / 2)
             const int e2 = (int)((__float_as_uint(total * 1.0625f) >> 23) & 255u) - 126;
             xexp[0] = max((e2 + 1) >> 1, -13);
+            // with an entry that is infinite or no number, all rotated entries are zero on the scale of their norm: y must not
+            // look like a result, so its scale is NaN
+            x_scale = total - total == 0.f ? pow2f(xexp[0]) : __int_as_float(0x7fffffff);
         }
         const float scale = pow2f(29 - xexp[0]);
         // rotated pieces: from the exact sums; pieces past the rotated length: as they are (the one this thread
@@ -1290,7 +1294,8 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
         // with no records read (the control launch) every unit contributes zero
         n += run;
         if (BATCH == 1) {
-            hand_over(p, pr, p.accum, pr.y, cc.group, my_row, sum[0], run, xexp[0] + pr.qexp_base, row_scale, handed);
+            const float quantum = ROTATE != kNoRotation ? pow2f(pr.qexp_base) * x_scale : pow2f(xexp[0] + pr.qexp_base);
+            hand_over(p, pr, p.accum, pr.y, cc.group, my_row, sum[0], run, quantum, row_scale, handed);
         } else {
             // this lane's rows are 16 * (lane & 1) + g and the one eight further on, its vector of a pair (lane & 3) >> 1; all the
             // atomics are on their way before the first answer is looked at

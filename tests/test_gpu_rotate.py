@@ -208,6 +208,23 @@ def test_gemv_rotated_of_a_short_part(B, ctx, oracle, rows, n, block):
     assert err <= 1e-6
 
 
+@pytest.mark.parametrize("bad", [float("inf"), -float("inf"), float("nan")])
+@pytest.mark.parametrize("block,at", [(8, 3), (64, 700), (512, 2559), (512, 2565)])
+def test_gemv_rotated_of_an_infinite_or_undefined_entry(B, ctx, bad, block, at):
+    """x must be finite; an entry that is not, rotated or passed through, never gives a y that looks like a result."""
+    rows, n = 3000, 2560
+    case = make_case(rows, n + 20, seed=7)
+    buf = B.expand(ctx, 0, case.d_codes, case.rows, case.nb)
+    x = case.d_x.clone()
+    x[at] = bad
+    y = torch.zeros(rows, dtype=torch.float32, device="cuda")
+    B.gemv_rotated(ctx, [(buf, case.d_scale, GAIN, y, rows)], x, case.nb * 24, n=n, block=block)
+    assert torch.isnan(y).all()
+    B.gemv_rotated(ctx, [(buf, case.d_scale, GAIN, y, rows)], case.d_x, case.nb * 24, n=n, block=block)
+    assert torch.isfinite(y).all() and (y != 0).any()
+    B.status(ctx)
+
+
 def test_gemv_rotated_grouped_launch_and_outlier_activation(B, ctx, oracle):
     """q/k/v-like group sharing one x; x with one huge entry (what the rotation is for): the bound on the
     rotated magnitudes is then loosest, and the result must still meet the bar with room."""
