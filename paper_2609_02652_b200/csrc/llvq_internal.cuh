@@ -128,7 +128,7 @@ struct GemvLaunch {
 // first pass over them runs the widest `stages` strides, 2^stride and more, down to pieces of 2^stride coordinates, of which a CTA
 // keeps the ones that meet its blocks of x.  Shorter blocks have little to leave out: the scan runs their three narrowest
 // stages on the eight values a thread holds (`stages` 0) and keeps whole blocks (`stride` the block).  Us a rotating launch of
-// 4096 x 4096 with blocks of 8, 64, 128, 256, 512: FP16 values first 6.21, 6.12, 6.46, 6.41, 6.03; stages first 5.31, 5.92, 6.33, 6.28, -.
+// 4096 x 4096 with blocks of 8, 64, 128, 256, 512: FP16 values first 6.21, 6.12, 6.46, 6.41, 6.03; stages first 5.29, 5.89, 6.22, 6.21, -.
 struct RotFirst {
     int stages, stride;
 };
