@@ -160,7 +160,7 @@ int llvq_selftest_wait_limit(llvq_ctx *ctx, void *stream) {
     if (!ctx) return LLVQ_EINVAL;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
-    return launch_wait_limit_selftest(ctx, (cudaStream_t)stream) == cudaSuccess ? LLVQ_OK : LLVQ_ECUDA;
+    return launched(launch_wait_limit_selftest(ctx, (cudaStream_t)stream));
 }
 
 int llvq_set_pdl(llvq_ctx *ctx, int enabled) {
@@ -194,7 +194,7 @@ int llvq_overlay_count(llvq_ctx *ctx, const uint64_t *codes, int64_t rows, int64
     // the call waits for its result anyway, and host threads that count on streams of their own take turns
     std::lock_guard<std::mutex> lock(ctx->count_mutex);
     *ctx->host_counter = 0;
-    if (launch_overlay_count(ctx, codes, rows, nb, ctx->counter, ctx->host_counter, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return LLVQ_ECUDA;
+    if (launched(launch_overlay_count(ctx, codes, rows, nb, ctx->counter, ctx->host_counter, s)) != LLVQ_OK || cudaStreamSynchronize(s) != cudaSuccess) return LLVQ_ECUDA;
     *count = *ctx->host_counter;
     return LLVQ_OK;
 }
@@ -223,7 +223,7 @@ int llvq_expand(llvq_ctx *ctx, int layout, const uint64_t *codes, int64_t rows, 
     // the GEMV reads records ahead of its wait for the previous kernel of the stream: the next one on this context
     // is launched as an ordinary kernel, so that it cannot overtake this expansion
     ctx->weights_dirty = 1;
-    return launch_expand(ctx, layout, codes, rows, nb, layout_out, out_bytes, bad_count, (cudaStream_t)stream) == cudaSuccess ? LLVQ_OK : LLVQ_ECUDA;
+    return launched(launch_expand(ctx, layout, codes, rows, nb, layout_out, out_bytes, bad_count, (cudaStream_t)stream));
 }
 
 constexpr int kVectorsPerPass = 4;      // activation vectors a pass that llvq_gemv_plan describes carries at most
@@ -350,7 +350,7 @@ static int run_gemv(llvq_ctx *ctx, int layout, const llvq_problem *problems, int
     if (!guard.ok) return LLVQ_ECUDA;
     const bool pdl = ctx->use_pdl != 0 && !ctx->weights_dirty;
     ctx->weights_dirty = 0;
-    return launch_gemv(layout, p, g, no_weights, pdl, (cudaStream_t)stream) == cudaSuccess ? LLVQ_OK : LLVQ_ECUDA;
+    return launched(launch_gemv(layout, p, g, no_weights, pdl, (cudaStream_t)stream));
 }
 
 int llvq_gemv(llvq_ctx *ctx, int layout, const void *layout_buf, const void *row_scale, const float *gain, const void *x,
@@ -404,7 +404,7 @@ int llvq_gemv_fp16(const void *W, const void *x, float *y, int64_t rows, int64_t
     if (!W || !x || !y || rows <= 0 || k <= 0 || k % 8 != 0) return LLVQ_EINVAL;
     if (!aligned(W, 16) || !aligned(x, 16) || !aligned(y, 4)) return LLVQ_EALIGN;
     if ((rows + 7) / 8 > 0x7fffffffll) return LLVQ_ESIZE;
-    return launch_gemv_fp16((const __half *)W, (const __half *)x, y, rows, k, (cudaStream_t)stream) == cudaSuccess ? LLVQ_OK : LLVQ_ECUDA;
+    return launched(launch_gemv_fp16((const __half *)W, (const __half *)x, y, rows, k, (cudaStream_t)stream));
 }
 
 int64_t llvq_rotate_block(int64_t n, int64_t block) {
@@ -420,8 +420,7 @@ int llvq_rotate(llvq_ctx *ctx, const void *x, void *y, const uint32_t *negate_bi
     if (n > ((int64_t)1 << 40)) return LLVQ_ESIZE;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
-    return launch_rotate((const __half *)x, (__half *)y, negate_bits, n, l, ctx->use_pdl != 0, (cudaStream_t)stream) == cudaSuccess
-               ? LLVQ_OK : LLVQ_ECUDA;
+    return launched(launch_rotate((const __half *)x, (__half *)y, negate_bits, n, l, ctx->use_pdl != 0, (cudaStream_t)stream));
 }
 
 int llvq_dequant_fp16(llvq_ctx *ctx, int layout, const void *layout_buf, const void *row_scale, const float *gain, void *W,
@@ -431,8 +430,8 @@ int llvq_dequant_fp16(llvq_ctx *ctx, int layout, const void *layout_buf, const v
     if (!aligned(layout_buf, 128) || !aligned(W, 16) || !aligned(row_scale, 2)) return LLVQ_EALIGN;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
-    return launch_dequant(ctx, layout, (const uint8_t *)layout_buf, (const __half *)row_scale, gain[0], gain[1], (__half *)W, rows,
-                          k_padded / 24, (cudaStream_t)stream) == cudaSuccess ? LLVQ_OK : LLVQ_ECUDA;
+    return launched(launch_dequant(ctx, layout, (const uint8_t *)layout_buf, (const __half *)row_scale, gain[0], gain[1], (__half *)W, rows,
+                          k_padded / 24, (cudaStream_t)stream));
 }
 
 int llvq_decode_i8(llvq_ctx *ctx, int layout, const void *layout_buf, int8_t *coords, uint16_t *class_ids, int64_t rows,
@@ -442,8 +441,7 @@ int llvq_decode_i8(llvq_ctx *ctx, int layout, const void *layout_buf, int8_t *co
     if (!aligned(layout_buf, 128) || !aligned(class_ids, 2)) return LLVQ_EALIGN;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
-    return launch_decode_i8(ctx, layout, (const uint8_t *)layout_buf, coords, class_ids, rows, nb, (cudaStream_t)stream) == cudaSuccess
-               ? LLVQ_OK : LLVQ_ECUDA;
+    return launched(launch_decode_i8(ctx, layout, (const uint8_t *)layout_buf, coords, class_ids, rows, nb, (cudaStream_t)stream));
 }
 
 }  // extern "C"

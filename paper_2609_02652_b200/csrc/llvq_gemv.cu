@@ -2062,7 +2062,7 @@ extern "C" int llvq_gemv_static(const void *layout_buf, const void *row_scale, c
     p.lane_table = d.lane_table;
     const llvq::GemvLaunch g = llvq::gemv_plan(LLVQ_PLANES, p, d.sm_count);
     if (g.smem + 1024 > (size_t)d.max_smem_optin) return LLVQ_ESIZE;
-    return llvq::launch_gemv(LLVQ_PLANES, p, g, false, true, (cudaStream_t)stream) == cudaSuccess ? LLVQ_OK : LLVQ_ECUDA;
+    return llvq::launched(llvq::launch_gemv(LLVQ_PLANES, p, g, false, true, (cudaStream_t)stream));
 }
 
 

@@ -201,6 +201,12 @@ struct llvq_ctx {
 };
 
 namespace llvq {
+// A launch's status.  The runtime keeps a refused launch's error for whoever asks next; it is this call's, which reports it.
+inline int launched(cudaError_t status) {
+    if (status == cudaSuccess) return LLVQ_OK;
+    cudaGetLastError();
+    return LLVQ_ECUDA;
+}
 cudaError_t launch_expand(const llvq_ctx *ctx, int layout, const uint64_t *codes, int64_t rows, int64_t nb,
                           void *out, size_t out_bytes, uint32_t *bad_count, cudaStream_t s);
 // writes the number of blocks the 10-byte layout would keep in its exception table to *host (page-locked); `counter` is two

@@ -300,6 +300,41 @@ def test_new_outputs_are_allocated_as_torch_empty_does(B, ctx):
     assert B.overlay_bytes(64, 24 * 32, n) < out.numel() and (out[B.overlay_bytes(64, 24 * 32, n):] == 255).all()
 
 
+def test_refused_launch_leaves_no_error_behind(B, ctx):
+    """Launches into a stream capture that is already invalid are refused; the error is returned and not left for the next caller of
+    cudaGetLastError, who would take it for its own."""
+    import ctypes
+
+    runtime = ctypes.CDLL("libcudart.so.12")                     # the one that torch and the library have loaded
+    case = make_case(64, 96, seed=1)
+    buf = B.expand(ctx, 0, case.d_codes, case.rows, case.nb)
+    buf10 = torch.zeros(B.layout_bytes(3, 64, 96), dtype=torch.uint8, device="cuda")
+    W = torch.empty((64, 96), dtype=torch.float16, device="cuda")
+    y = torch.empty(64, dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    left = []
+    with torch.cuda.stream(stream):
+        graph.capture_begin()
+        try:
+            with pytest.raises(B.LlvqError):
+                B.status(ctx, stream=stream)                     # waits for the stream, which invalidates the capture
+            runtime.cudaGetLastError()
+            for call in (lambda: B.expand(ctx, 0, case.d_codes, 64, 4, out=buf), lambda: B.expand(ctx, 3, case.d_codes, 64, 4, out=buf10),
+                         lambda: B.dequant_fp16(ctx, 0, buf, case.d_scale, GAIN, 64, 96, W=W), lambda: B.rotate(ctx, case.d_x, y=case.d_x),
+                         lambda: B.gemv(ctx, 0, buf, case.d_scale, GAIN, case.d_x, 64, 96, y=y)):
+                with pytest.raises(B.LlvqError) as e:
+                    call()
+                assert e.value.code == -4
+                left.append(runtime.cudaGetLastError())
+        finally:
+            with pytest.raises(RuntimeError):
+                graph.capture_end()
+            runtime.cudaGetLastError()
+    assert left == [0] * len(left)
+    assert torch.equal(B.gemv(ctx, 0, buf, case.d_scale, GAIN, case.d_x, 64, 96), B.gemv(ctx, 0, buf, case.d_scale, GAIN, case.d_x, 64, 96))
+
+
 def test_noweights_control_returns_zero(B, ctx):
     case = make_case(4096, 4096, seed=2)
     y = torch.full((case.rows,), float("nan"), dtype=torch.float32, device="cuda")
