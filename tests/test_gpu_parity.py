@@ -674,3 +674,60 @@ def test_gain_range(B, ctx):
     assert torch.isfinite(y).all()
     y1 = B.gemv(ctx, B.PLANES, buf, case.d_scale, (1.0, 1.0), case.d_x, case.rows, 96)
     assert torch.allclose(y.double() * 2.0 ** 59, y1.double(), rtol=1e-6, atol=0)
+
+
+def test_loading_inside_a_captured_graph(B, oracle):
+    """Expansion, matvec, dequantisation and rotation captured as one graph, behind a copy and a side stream's join, replayed on other
+    codes: programmatic launches inside a graph read nothing ahead of what writes it."""
+    rows, nb = 1000, 107
+    k = 24 * nb
+    cases = [make_case(rows, k, seed=60 + i) for i in range(3)]
+    c = B.create(0)
+    try:
+        codes, x, scale = cases[0].d_codes.clone(), cases[0].d_x.clone(), cases[0].d_scale.clone()
+        buf = torch.zeros(B.layout_bytes(0, rows, k), dtype=torch.uint8, device="cuda")
+        buf10 = torch.zeros(B.layout_bytes(3, rows, k), dtype=torch.uint8, device="cuda")
+        y, y10, yr = (torch.zeros(rows, device="cuda") for _ in range(3))
+        W, xr = torch.zeros((rows, k), dtype=torch.float16, device="cuda"), torch.zeros(k, dtype=torch.float16, device="cuda")
+        source, xsource = cases[0].d_codes.clone(), cases[0].d_x.clone()
+
+        def steps():
+            codes.copy_(source)
+            side = torch.cuda.Stream()
+            side.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(side):
+                x.copy_(xsource)
+            torch.cuda.current_stream().wait_stream(side)
+            B.expand(c, 0, codes, rows, nb, out=buf)
+            B.gemv(c, 0, buf, scale, GAIN, x, rows, k, y=y)
+            B.expand(c, 3, codes, rows, nb, out=buf10)
+            B.dequant_fp16(c, 0, buf, scale, GAIN, rows, k, W=W)
+            B.gemv(c, 3, buf10, scale, GAIN, x, rows, k, y=y10)
+            B.rotate(c, x, block=8, y=xr)
+            B.gemv(c, 0, buf, scale, GAIN, xr, rows, k, y=yr)
+
+        steps()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            steps()
+        for case in (cases[1], cases[2], cases[1]):
+            source.copy_(case.d_codes)
+            xsource.copy_(case.d_x)
+            scale.copy_(case.d_scale)
+            for t in (y, y10, yr, W):
+                t.zero_()
+            graph.replay()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert np.array_equal(buf.cpu().numpy(), oracle.pack_planes(case.codes, rows, nb))
+            want10, n = oracle.pack_planes10x(case.codes, rows, nb)
+            used = B.overlay_bytes(rows, k, n)
+            assert np.array_equal(buf10[:used].cpu().numpy(), want10[:used])
+            check_gemv(oracle, case, y)
+            check_gemv(oracle, case, y10)
+            assert torch.equal(W, B.dequant_fp16(c, 0, buf, scale, GAIN, rows, k))
+            assert torch.equal(yr, B.gemv(c, 0, buf, scale, GAIN, B.rotate(c, x, block=8), rows, k))
+        B.status(c)
+    finally:
+        c.close()
