@@ -25,7 +25,8 @@
  *   - Every call takes the caller's CUDA stream (a cudaStream_t passed as void*), enqueues its
  *     work there and returns without synchronising, unless stated otherwise.
  *   - A context holds reduction scratch that its GEMV launches share: launches on one context
- *     must be ordered on one stream (or otherwise serialised).  Use one context per stream.
+ *     must be ordered on one stream (or otherwise serialised); host threads may share that stream.
+ *     Use one context per stream.
  *   - Return value: 0 on success, a negative LLVQ_E* code otherwise.  No call aborts, throws or
  *     traps; a failed call enqueues nothing.
  *
@@ -174,8 +175,8 @@ typedef struct llvq_rotation {
     int64_t block;               /* block length, a power of two in 8..16384 that divides n; 0 = the largest */
 } llvq_rotation;
 
-/* Builds the class, index-base and Golay tables on the host, uploads them to `device`, and
- * allocates the context's reduction scratch (scratch_bytes; 0 = default 8 MiB, eight bytes a row
+/* Builds the class, index-base and Golay tables and the lists of orderings that llvq_expand looks points up in (6 MB) on the
+ * host, uploads them to `device`, and allocates the context's reduction scratch (scratch_bytes; 0 = default 8 MiB, eight bytes a row
  * of the largest launch, rows rounded up to 32 per matrix).  Synchronous.  (The third argument is
  * this library's addition to the call the paper's statement of the problem implies: the scratch is
  * the one thing whose size depends on the caller's largest launch.) */
@@ -206,7 +207,9 @@ int llvq_selftest_wait_limit(llvq_ctx *ctx, void *stream);
  * kernel that precedes the GEMV on the stream starts (weights loaded once satisfy this trivially);
  * llvq_expand takes care of it by itself (the next GEMV on the context is launched as an ordinary
  * kernel); a caller whose own kernel writes scales or records right before a GEMV disables the
- * feature.  enabled = 0 launches every GEMV as an ordinary kernel. */
+ * feature.  llvq_rotate, llvq_expand, llvq_overlay_count and llvq_dequant_fp16 (LLVQ_PLANES) are launched the same way, but
+ * wait for the kernel before them ahead of all they read or write but the context's own tables.
+ * enabled = 0 launches every one of them as an ordinary kernel. */
 int llvq_set_pdl(llvq_ctx *ctx, int enabled);
 
 /* Host queries.  Number of classes (301), points in the ball, and first index of class c
@@ -219,7 +222,8 @@ int llvq_layout_bytes(int layout, int64_t rows, int64_t k_padded, size_t *bytes)
 
 /* [Sec. 3.3, the exception table of the sparse overlay] Host queries and a counting pass for LLVQ_PLANES10X.
  * llvq_overlay_count decodes the rows*nb code words and writes to *count (HOST) how many blocks the layout keeps
- * in its exception table; it synchronises `stream`.  llvq_overlay_bytes gives the bytes of a layout buffer with
+ * in its exception table; it synchronises `stream`, and calls on one context from several host threads take turns.
+ * llvq_overlay_bytes gives the bytes of a layout buffer with
  * room for `exceptions` table entries. */
 int llvq_overlay_count(llvq_ctx *ctx, const uint64_t *codes, int64_t rows, int64_t nb, uint64_t *count, void *stream);
 int llvq_overlay_bytes(int64_t rows, int64_t k_padded, uint64_t exceptions, size_t *bytes);
@@ -254,7 +258,8 @@ int llvq_gemv(llvq_ctx *ctx, int layout, const void *layout_buf, const void *row
  * llvq_gemv on the LLVQ_PLANES layout for batch (1..LLVQ_MAX_BATCH) activation vectors in one pass
  * over the records: x is fp16 [batch][k_padded], y is f32 [batch][rows].  The vectors share
  * one pass (the records are read and decoded once for them); five to eight take two passes where the
- * context's scratch or a multiprocessor's shared memory holds those of four only.  Each vector has its own fixed-point scale and its own accumulators, and y[j] is bit-identical to what
+ * context's scratch holds the sums of four only, or on a device of few multiprocessors, whose shared memory may hold the
+ * records of four only.  Each vector has its own fixed-point scale and its own accumulators, and y[j] is bit-identical to what
  * llvq_gemv returns for x[j].  Needs min(batch, 4) times the scratch of llvq_gemv (LLVQ_ESIZE
  * otherwise). */
 int llvq_gemv_batch(llvq_ctx *ctx, const void *layout_buf, const void *row_scale, const float *gain,

@@ -326,8 +326,6 @@ static int run_gemv(llvq_ctx *ctx, int layout, const llvq_problem *problems, int
     p.total_groups = (int)groups;
     p.total_units = (int)(groups * p.units);
     p.accum = ctx->accum;
-    p.cls_scale = ctx->dev.cls_scale;
-    p.cls_parity = ctx->dev.cls_parity;
     p.cls_value = ctx->dev.cls_value;
     p.cls_block = ctx->dev.cls_block;
     p.lane_table = ctx->dev.lane_table;
@@ -368,8 +366,9 @@ int llvq_gemv_batch(llvq_ctx *ctx, const void *layout_buf, const void *row_scale
     q.layout = layout_buf; q.row_scale = row_scale; q.y = y; q.rows = rows;
     q.gain[0] = gain[0]; q.gain[1] = gain[1];
     // One pass over the records serves all the vectors, if the scratch has room for their sums and a multiprocessor for
-    // their records of x (eight vectors, us in one pass and in two: 1024 x 2560 9.6 and 11.0, 8192 x 8192 35.4 and 35.5,
-    // 34816 x 5120 65.8 and 71.5).
+    // their records of x, which only devices of few multiprocessors lack (eight vectors, us in one pass and in two:
+    // 1024 x 2560 9.8 and 11.1, 8192 x 8192 30.7 and 35.5, 34816 x 5120 61.9 and 71.8; five on 1206 x 14707 15.7 and 15.3, the
+    // worst of 57 shapes).
     int rc = run_gemv(ctx, LLVQ_PLANES, &q, 1, x, k_padded, false, stream, batch);
     if (rc != LLVQ_ESIZE || batch <= kVectorsPerPass) return rc;
     // Otherwise passes of up to four, one after the other on the stream (they share the context's scratch).

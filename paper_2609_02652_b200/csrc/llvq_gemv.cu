@@ -287,10 +287,6 @@ __device__ __forceinline__ StepX load_step(const LaneOffsets &a) {
     return s;
 }
 
-// One half-step: 16 rows x 2 block slots.  wa, wb, wc are this lane's three payload words, hw the two
-// headers of its rows for slot (lane & 3) >> 1, sx the step's operand.  Adds to r0 (row g of the 16) and r1
-// (row g + 8) this lane's share of scale * sum_i x_i * X_i, X the fixed-point activations: its share is the
-// limb pair (lane & 1) of slot (lane & 3) >> 1.  FIRST: r0 and r1 are written, not added to.
 // (a & b) | c in one instruction
 __device__ __forceinline__ uint32_t and_or(uint32_t a, uint32_t b, uint32_t c) {
     uint32_t r;
@@ -384,6 +380,10 @@ __device__ __forceinline__ long long exception_value(const uint4 &ent, uint32_t 
     return __float2ll_rn(((float)e_lo * k.x + ((float)e_hi * k.x) * 65536.f) * inv_q);
 }
 
+// One half-step: 16 rows x 2 block slots.  h holds this lane's payload words and the constants of its rows' blocks in slot
+// (lane & 3) >> 1 (decode_half), sx the step's operand.  Adds to r0 (row g of the 16) and r1
+// (row g + 8) this lane's share of scale * sum_i x_i * X_i, X the fixed-point activations: its share is the
+// limb pair (lane & 1) of slot (lane & 3) >> 1.  FIRST: r0 and r1 are written, not added to.
 template <bool FIRST>
 __device__ __forceinline__ void contract_half(const HalfA &h, const StepX &sx, float &r0, float &r1) {
     int d[4];
@@ -395,12 +395,6 @@ __device__ __forceinline__ void contract_half(const HalfA &h, const StepX &sx, f
     if (FIRST) { r0 = __fmul_rn((float)e0, h.k0.x); r1 = __fmul_rn((float)e1, h.k1.x); }
     else { r0 = fmaf((float)e0, h.k0.x, r0); r1 = fmaf((float)e1, h.k1.x, r1); }
 }
-template <bool FIRST>
-__device__ __forceinline__ void half_step(uint32_t wa, uint32_t wb, uint32_t wc, uint32_t hw, const StepX &sx, uint32_t tq,
-                                          float &r0, float &r1) {
-    contract_half<FIRST>(decode_half(wa, wb, wc, hw, tq), sx, r0, r1);
-}
-
 // ---- several activation vectors.  Two vectors share the eight columns of the contraction - column g = 4 (vector) + limb -
 // and a block slot has an instruction sequence of its own: positions 0..23 of the half-step for slot 0, 24..47 for slot 1,
 // the other slot's positions zero in B.  Against one vector with block-diagonal B that is three instructions instead
@@ -574,7 +568,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
     // shared memory: ring | per-matrix block constants (1024 x {gain / (4 sqrt m), parity - 16}) | x records | barriers
     unsigned char *ring = smem;
     // the block constants start on an 8 KiB boundary of the shared window, so that a matrix's table base and
-    // an entry's offset combine by OR (half_step)
+    // an entry's offset combine by OR (decode_half)
     const uint32_t tab_pad = (0u - (smem_addr(smem) + kWarps * kSlots * kTileBytes)) & 8191u;
     float2 *tab = reinterpret_cast<float2 *>(smem + kWarps * kSlots * kTileBytes + tab_pad);
     unsigned char *xrec = smem + kWarps * kSlots * kTileBytes + tab_pad + p.nprob * 8192;

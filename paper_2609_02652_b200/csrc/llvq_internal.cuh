@@ -104,8 +104,6 @@ struct GemvCall {
     int total_groups;
     int total_units;       // total_groups * units
     unsigned long long *accum;   // total_groups x 32 fixed-point row accumulators (context scratch, zero between launches)
-    const float *cls_scale;
-    const uint32_t *cls_parity;
     const float *cls_value;
     const float2 *cls_block;     // 512 x {1 / (4 sqrt m), parity - 16 as an integer's bits}; zeros for an unused class slot
     const uint4 *lane_table;     // 32 x this lane's offsets of its operand words in the x records of a half-step
@@ -114,7 +112,7 @@ struct GemvCall {
     int rot_log2;             // log2 of the rotation's block length (3..)
     int rot_n;                // coordinates rotated: a multiple of the block length, at most 24 nb
     const uint32_t *rot_negate;   // sign-flip bits, or null
-    double rot_scale;         // 1 / sqrt(block length)
+    double rot_scale;         // 2^1008 / sqrt(block length): the sums are those of x times 2^-1008 (rot_widen)
     float shell_inv_norm[16];         // [m] = 1 / (4 sqrt m)
 };
 
