@@ -107,6 +107,42 @@ def test_arrays_of_another_type_are_refused(lib):
         B.gemv_rotated(Handle, (B.Problem * 1)(), x, 24, n=8)
 
 
+def test_launching_calls_check_their_arguments(lib):
+    """The native binding refuses a destroyed context, what is no CUDA tensor and an x of another shape before anything is launched."""
+    import torch
+
+    from paper_2609_02652_b200 import binding as B
+
+    class Open:
+        handle = 1              # never reached: no argument below is a CUDA tensor
+
+    class Destroyed:
+        handle = 0
+
+    h, u, l, w = torch.zeros(24, dtype=torch.float16), torch.zeros(448, dtype=torch.uint8), torch.zeros(1, dtype=torch.int64), torch.zeros((2, 24), dtype=torch.float16)
+    y = torch.zeros(1)
+    with_context = [lambda c: B.gemv(c, 0, u, h, (1.0, 1.0), h, 1, 24), lambda c: B.gemv_batch(c, u, h, (1.0, 1.0), w, 1, 24), lambda c: B.expand(c, 0, l, 1, 1),
+                    lambda c: B.gemv_grouped(c, 0, (B.Problem * 1)(), h, 24), lambda c: B.gemv_rotated(c, (B.Problem * 1)(), h, 24, n=8), lambda c: B.rotate(c, h),
+                    lambda c: B.gemv_noweights(c, h, h, 1, 24), lambda c: B.dequant_fp16(c, 0, u, h, (1.0, 1.0), 1, 24), lambda c: B.overlay_count(c, l, 1, 1)]
+    for call in with_context:
+        with pytest.raises(TypeError, match="expected a contiguous CUDA tensor of dtype torch"):
+            call(Open)
+        with pytest.raises(RuntimeError, match="context already destroyed"):
+            call(Destroyed)
+        with pytest.raises(AttributeError):
+            call(None)
+    for call in (lambda: B.gemv_static(u, h, (1.0, 1.0), h, 1, 24, y), lambda: B.gemv_fp16(h, h, 1, 24)):
+        with pytest.raises(TypeError, match="expected a contiguous CUDA tensor"):
+            call()
+    for what in (None, "tensor", 3):
+        with pytest.raises(TypeError, match="codes: expected"):
+            B.expand(Open, 0, what, 1, 1)
+    with pytest.raises(TypeError):
+        B.overlay_count(Open, l, None, 1)
+    with pytest.raises(TypeError, match="arguments expected"):
+        B._native.gemv(Open)
+
+
 def test_binding_is_rebuilt_for_another_torch_or_python(lib, monkeypatch):
     """The binding holds the layouts of one torch and one Python: another one of either makes it stale, and it is not loaded."""
     import sysconfig

@@ -58,3 +58,21 @@ def test_plan_of_five_to_eight_vectors(tmp_path):
             assert 3 * xblocks <= 12 * 32 and smem + 1024 <= 227 * 1024
         beyond += smem + 1024 > 227 * 1024
     assert beyond                     # few multiprocessors and a long row: the launch is refused, and llvq_gemv_batch takes two passes
+
+
+def test_unranking_against_the_oracle(tmp_path, oracle):
+    """Class, coordinates and window flags of indices at the edges of every class's digits: the tables and their readers, on the host."""
+    import numpy as np
+
+    from helpers import window_base
+    from paper_2609_02652_b200 import build
+
+    out = run_native(tmp_path, "unrank.cpp", *[os.path.join(build.CSRC, f) for f in ("llvq_tables.cpp", "llvq_unrank.cpp")], stdin=b"")
+    r = np.frombuffer(out, np.dtype([("index", "<u8"), ("cls", "<u2"), ("window", "u1"), ("looked_at", "u1"), ("x", "i1", 24), ("pad", "u1", 4)]))
+    assert np.unique(r["cls"]).size == 301 and r.size > 301 * 100
+    x, cls = oracle.decode_batch(r["index"].copy())
+    assert np.array_equal(r["cls"], cls) and np.array_equal(r["x"], x)
+    none = window_base(x) == 0
+    always, depends, never = 0, 1, 2
+    assert not none[r["window"] == always].any() and none[r["window"] == never].all() and r["looked_at"][none].all()
+    assert none[r["window"] == depends].any() and not none[r["window"] == depends].all()
