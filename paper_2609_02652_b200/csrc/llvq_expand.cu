@@ -2,14 +2,14 @@
 // decoded-field record - class id, gain bit, sign mask, per-coordinate level - in one of the layouts of include/llvq.h.
 // Integer arithmetic only (the float estimates in llvq_unrank.cuh are corrected in integers), so the output is bit-exact.
 //
-// Bound: instruction issue and the gathers from the lists, not HBM (8 bytes in, 10 to 20 out a block).  The two types of
+// Bound: the gathers from the lists and instruction issue, not HBM (8 bytes in, 10 to 20 out a block).  The two types of
 // class take different code, and codes come in random order, so a warp first finds the class of all 128 blocks of a
 // tile (a lane a row), lists them by type in shared memory and then un-ranks 32 blocks of one type at a time, whatever
 // their place; the codes wait in shared memory until the tile's words are gathered from them.  The small look-up tables
 // are copied to shared memory once a CTA, while the previous kernel of the stream ends; one CTA a multiprocessor walks over
 // the tiles.
-// Measured (9728 x 2560 into the 14-byte layout, 1.04 M blocks): 38 us, 2600 warp instructions a tile of 128 blocks, issue
-// slots 55 % busy, the load unit's wavefronts 74 %; a lane a row with a 64-bit division a coordinate and candidate took
+// Measured (9728 x 2560 into the 14-byte layout, 1.04 M blocks): 38 us, 2800 warp instructions a tile of 128 blocks, issue
+// slots 54 % busy, the load unit's wavefronts 59 %, half of all stalls waits on the lists; a lane a row with a 64-bit division a coordinate and candidate took
 // 484 us, one odd coordinate at a time 45.  Counting and expanding 17408 x 5120 into the 10-byte layout: 188 us against
 // 4700.  24 or 28 warps a CTA instead of 32: 47 and 50 us.  The shared tables are kept to 51 KB because the rest of a
 // multiprocessor's memory is the L1 cache that the lists are read through: with 104 KB of tables it took 53 us.

@@ -399,7 +399,8 @@ __device__ __forceinline__ void contract_half(const HalfA &h, const StepX &sx, f
 // and a block slot has an instruction sequence of its own: positions 0..23 of the half-step for slot 0, 24..47 for slot 1,
 // the other slot's positions zero in B.  Against one vector with block-diagonal B that is three instructions instead
 // of four for two vectors and two slots, and a row's sum lies in two lanes instead of four, so half the exchanges.
-// The price is that a lane looks up the headers of both slots; every vector shares that.  Bound: instruction issue.  Four
+// The price is that a lane looks up the headers of both slots; every vector shares that.  Bound: latency (4096 x 4096: issue slots
+// 46 % busy with four vectors, 32 % with eight, whose three warps a scheduler also wait for instructions; tensor pipe 10 %).  Four
 // vectors, us a launch, before (a vector at a time, its atomic waited for before the next vector's) and after:
 // 1024 x 2560 6.8 and 5.5, 4096 x 4096 10.7 and 8.8, 8192 x 8192 19.4 and 17.8; two vectors on 8192 x 8192 12.5 and 11.9.
 struct PairA {
