@@ -61,7 +61,7 @@ int llvq_create(llvq_ctx **out, int device, size_t scratch_bytes) {
     llvq_ctx *ctx = new (std::nothrow) llvq_ctx();
     if (!ctx) return LLVQ_ECUDA;
     ctx->device = device;
-    ctx->table_blob = nullptr; ctx->accum = nullptr; ctx->error = nullptr; ctx->bad_codes = nullptr; ctx->host_counter = nullptr; ctx->use_pdl = 1; ctx->weights_dirty = 0;
+    ctx->table_blob = nullptr; ctx->accum = nullptr; ctx->error = nullptr; ctx->bad_codes = nullptr; ctx->host_counter = nullptr; ctx->use_pdl = 1;
     if (!build_tables(ctx->host)) { delete ctx; return LLVQ_EINVAL; }
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) { delete ctx; return LLVQ_ECUDA; }
@@ -220,10 +220,11 @@ int llvq_expand(llvq_ctx *ctx, int layout, const uint64_t *codes, int64_t rows, 
     if (rows * nb > ((int64_t)1 << 36)) return LLVQ_ESIZE;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
+    const int rc = launched(launch_expand(ctx, layout, codes, rows, nb, layout_out, out_bytes, bad_count, (cudaStream_t)stream));
     // the GEMV reads records ahead of its wait for the previous kernel of the stream: the next one on this context
     // is launched as an ordinary kernel, so that it cannot overtake this expansion
-    ctx->weights_dirty = 1;
-    return launched(launch_expand(ctx, layout, codes, rows, nb, layout_out, out_bytes, bad_count, (cudaStream_t)stream));
+    ctx->order.expanded();
+    return rc;
 }
 
 constexpr int kVectorsPerPass = 4;      // activation vectors a pass that llvq_gemv_plan describes carries at most
@@ -346,9 +347,11 @@ static int run_gemv(llvq_ctx *ctx, int layout, const llvq_problem *problems, int
     if (g.smem + 1024 > (size_t)ctx->max_smem_optin) return LLVQ_ESIZE;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
-    const bool pdl = ctx->use_pdl != 0 && !ctx->weights_dirty;
-    ctx->weights_dirty = 0;
-    return launched(launch_gemv(layout, p, g, no_weights, pdl, (cudaStream_t)stream));
+    const uint64_t expansions = ctx->order.expansions();
+    const bool behind = ctx->order.behind(expansions), pdl = ctx->use_pdl != 0 && behind;
+    const int rc = launched(launch_gemv(layout, p, g, no_weights, pdl, (cudaStream_t)stream));
+    if (!behind && rc == LLVQ_OK) ctx->order.ordered(expansions);
+    return rc;
 }
 
 int llvq_gemv(llvq_ctx *ctx, int layout, const void *layout_buf, const void *row_scale, const float *gain, const void *x,

@@ -3,6 +3,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 #include <cstring>
 #include <mutex>
@@ -175,6 +176,24 @@ private:
     int used_ = 0, next_ = 0;
 };
 
+// A GEMV launched right behind an expansion must not read records ahead of its wait; behind a GEMV that was launched as an
+// ordinary kernel after the expansion, it may.  Host threads that share the stream may ask at any point of one another's
+// launches: an expansion counts once it is enqueued, and an ordinary launch, once it is enqueued itself, for the expansions that
+// were counted before it.
+class RecordOrder {
+public:
+    void expanded() { expansions_.fetch_add(1); }
+    uint64_t expansions() const { return expansions_.load(); }
+    bool behind(uint64_t expansions) const { return ordered_.load() >= expansions; }      // an ordinary launch lies behind all of them
+    void ordered(uint64_t expansions) {
+        uint64_t seen = ordered_.load();
+        while (seen < expansions && !ordered_.compare_exchange_weak(seen, expansions)) {}
+    }
+
+private:
+    std::atomic<uint64_t> expansions_{0}, ordered_{0};
+};
+
 }  // namespace llvq
 
 struct llvq_ctx {
@@ -192,7 +211,7 @@ struct llvq_ctx {
     unsigned long long *host_counter;   // page-locked: its result
     std::mutex count_mutex;  // one llvq_overlay_count at a time: the two above are its own from launch to result
     int use_pdl;             // launch the GEMV with programmatic stream serialization
-    int weights_dirty;       // an expansion was enqueued since the last GEMV: that GEMV must not read records ahead of it
+    llvq::RecordOrder order; // whether a GEMV may read records ahead of its wait
     int sm_count;
     int max_smem_optin;
     llvq::PlanCache plans;

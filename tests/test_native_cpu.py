@@ -76,3 +76,10 @@ def test_unranking_against_the_oracle(tmp_path, oracle):
     always, depends, never = 0, 1, 2
     assert not none[r["window"] == always].any() and none[r["window"] == never].all() and r["looked_at"][none].all()
     assert none[r["window"] == depends].any() and not none[r["window"] == depends].all()
+
+
+def test_no_matvec_reads_ahead_of_an_expansion(tmp_path):
+    """Every interleaving of two host threads' launches on one stream: the matvec on new records reads ahead in some of them, and never
+    without an ordinary launch between it and the expansion."""
+    total, ahead, wrong = map(int, run_native(tmp_path, "record_order.cpp").split())
+    assert total == 462 and ahead > 0 and wrong == 0
