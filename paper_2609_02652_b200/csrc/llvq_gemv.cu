@@ -39,24 +39,12 @@
 #include <mutex>
 #include <type_traits>
 
-#include "llvq_internal.cuh"
+#include "llvq_gemv.cuh"
 #include "llvq_rotate.cuh"
 
 namespace llvq {
 namespace {
 
-constexpr int kWarps = 16;                 // warps per CTA
-constexpr int kThreads = kWarps * 32;
-// The build for five to eight vectors needs more registers than sixteen warps leave a thread (128): twelve warps with 166 run
-// eight vectors on 4096 x 4096 in 16.4 us, sixteen that spill in 23.6, eight with 201 in 19.6; two passes of four take 17.4.
-__host__ __device__ constexpr int gemv_warps(int batch) { return batch > 4 ? 12 : kWarps; }
-constexpr int kSlots = 2;                  // ring slots per warp
-constexpr int kEarlySlots = 1;             // slots filled before the wait for the previous kernel; the rest once x is being prepared
-
-// fixed-point accumulator word: bits 53..63 count units, bits 0..52 sum the biased unit values
-constexpr int kCountShift = 53;
-constexpr unsigned long long kSumMask = (1ull << kCountShift) - 1;
-constexpr long long kUnitBias = 1ll << 41;     // a unit's value is below 2^40 quanta in magnitude
 
 __device__ __forceinline__ void fma_pair(float &lo, float &hi, uint32_t w, uint32_t x) {
     asm("{\n\t.reg .f16 wl, wh, xl, xh;\n\t"
@@ -93,17 +81,6 @@ __device__ __forceinline__ int find_problem(const GemvParams &p, int group) {
         if (i < p.nprob && group >= p.prob[i].group_begin) q = i;
     return q;
 }
-
-// running maximum of |fp16| over both halves of a word, kept as two 15-bit patterns.  The magnitude goes into the maximum's
-// instruction, which an AND of the bits did not: sixteen instructions less in the scan of x, which every launch waits for (us a launch in
-// a chain: 1024 x 2560 3.23 -> 3.19, 4096 x 4096 4.89 -> 4.84, 8192 x 8192 9.08 -> 9.01; two vectors on 4096 x 4096 6.37 -> 6.24)
-__device__ __forceinline__ uint32_t max_abs_pair(uint32_t m, uint32_t x2) {
-    const __half2 r = __hmax2(*reinterpret_cast<const __half2 *>(&m), __habs2(*reinterpret_cast<const __half2 *>(&x2)));
-    return *reinterpret_cast<const uint32_t *>(&r);
-}
-
-// exact power of two as a float, |e| < 126
-__device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }
 
 // The contiguous range of units [u0, u0 + n) of this warp; warps are numbered with the CTA index
 // fastest, so the ranges that are one unit longer spread over all multiprocessors.  The host
@@ -163,57 +140,6 @@ __device__ __forceinline__ void hand_over(const GemvParams &p, const GemvProblem
     h.count = count;
 }
 
-// ---- asynchronous copies: global -> shared, completion counted on an mbarrier in shared memory
-__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
-// Every wait is bounded in time: a poll that fails starts a clock, and once kWaitLimitCycles SM cycles
-// (about a second) have passed without the barrier completing, the caller records an error and winds
-// down.  The first poll reads no clock, so a wait that is already satisfied costs one instruction.
-constexpr long long kWaitLimitCycles = 2000000000ll;
-__device__ __forceinline__ bool mbar_wait_for(uint32_t bar, uint32_t parity, long long limit_cycles) {
-    if (mbar_try(bar, parity)) return true;
-    const long long t0 = clock64();
-    do {
-        if (mbar_try(bar, parity)) return true;
-    } while (clock64() - t0 < limit_cycles);
-    return false;
-}
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) { return mbar_wait_for(bar, parity, kWaitLimitCycles); }
-
-// Ring reads through 32-bit shared-memory addresses.  Volatile: they must stay behind the wait on the
-// slot's barrier and ahead of the copy that refills the slot.
-__device__ __forceinline__ uint4 lds128(uint32_t a) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
-    return v;
-}
-__device__ __forceinline__ uint2 lds64(uint32_t a) {
-    uint2 v;
-    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
-    return v;
-}
-__device__ __forceinline__ uint32_t lds32(uint32_t a) {
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
-    return v;
-}
-// Returns zero, but only once its operands are available: an address that adds this zero cannot be
-// formed before the loads that produced them have completed.
-__device__ __forceinline__ uint32_t settled(uint32_t a, uint32_t b, uint32_t c) {
-    uint32_t z;
-    asm volatile("lop3.b32 %0, %1, %2, %3, 0x00;" : "=r"(z) : "r"(a), "r"(b), "r"(c));
-    return z;
-}
-
 // First byte of a row group's records, and the matrix it belongs to.
 __device__ __forceinline__ const uint8_t *group_base(const GemvParams &p, int group, int &q) {
     if (p.nprob == 1) {                              // the common launch: one matrix
@@ -237,8 +163,7 @@ __device__ __forceinline__ void mma_k16(int (&d)[4], uint32_t a0, uint32_t a1, u
 }
 
 // Bytes of x in shared memory, one record a block: four planes of 24 bytes (plane l = limb l of the 24
-// fixed-point activations, doubled), a zero word at 96, and at 100 and 104 the two halves of the block's
-// activation sum (see stage_x).
+// fixed-point activations, doubled), a zero word at 96, and at 100 and 104 the block's sums of 2 X, limb pair by limb pair (see convert_item).
 constexpr int kXRecBytes = 112;
 
 // Offsets of this lane's operand words inside the two x records of a half-step (or, one = true, inside
@@ -262,37 +187,15 @@ __host__ __device__ __forceinline__ LaneOffsets lane_offsets(int lane, bool one)
     return o;
 }
 
-// Shared-memory reads with a constant byte offset folded into the instruction.  Volatile, so that the
-// compiler never moves one out of the branch that guards it: an address formed for a unit this CTA does not
-// own may lie outside its shared memory.
-template <int OFF>
-__device__ __forceinline__ uint32_t lds32_at(uint32_t a) {
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(a), "n"(OFF));
-    return v;
-}
-__device__ __forceinline__ float2 lds_f2(uint32_t a) {
-    float2 v;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
-    return v;
-}
-
 // The B operand of one step (two block slots) for this lane, and its share of the slots' activation sum.
-struct StepX { uint32_t b0, b1, b2; int xsum; };
+struct StepX { uint32_t b0, b1, b2; float xsum; };
 // a.* are this lane's four addresses for the records at the start of a tile; OFF selects the step
 template <int OFF>
 __device__ __forceinline__ StepX load_step(const LaneOffsets &a) {
     StepX s;
     s.b0 = lds32_at<OFF>(a.b0); s.b1 = lds32_at<OFF>(a.b1); s.b2 = lds32_at<OFF>(a.b2);
-    s.xsum = (int)lds32_at<OFF>(a.xs);
+    s.xsum = (float)(int)lds32_at<OFF>(a.xs);
     return s;
-}
-
-// (a & b) | c in one instruction
-__device__ __forceinline__ uint32_t and_or(uint32_t a, uint32_t b, uint32_t c) {
-    uint32_t r;
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
-    return r;
 }
 
 // The A operand of a half-step (the decode proper: one shift and two ANDs a word) and the block constants of
@@ -375,10 +278,9 @@ __device__ __forceinline__ long long exception_value(const uint4 &ent, uint32_t 
         }
         cw = j == 0 ? ent.z : ent.w;
     }
-    const int off = __float_as_int(k.y);
-    const int e_lo = off * (int)lds32(rec + 100) + (d[0] + 256 * d[1]);
-    const int e_hi = off * (int)lds32(rec + 104) + (d[2] + 256 * d[3]);
-    return __float2ll_rn(((float)e_lo * k.x + ((float)e_hi * k.x) * 65536.f) * inv_q);
+    const float e_lo = fmaf(k.y, (float)(int)lds32(rec + 100), (float)(d[0] + 256 * d[1]));
+    const float e_hi = fmaf(k.y, (float)(int)lds32(rec + 104), (float)(d[2] + 256 * d[3]));
+    return __float2ll_rn((e_lo * k.x + (e_hi * k.x) * 65536.f) * inv_q);
 }
 
 // One half-step: 16 rows x 2 block slots.  h holds this lane's payload words and the constants of its rows' blocks in slot
@@ -390,11 +292,11 @@ __device__ __forceinline__ void contract_half(const HalfA &h, const StepX &sx, f
     int d[4];
     mma_k32(d, h.a0, h.a1, h.a2, h.a3, sx.b0, sx.b1);
     mma_k16(d, h.c0, h.c1, sx.b2);
-    // sum_i x_i X_i = sum_i u_i (2 X_i) + (parity - 16) sum_i X_i, limb pair by limb pair, in integers
-    const int e0 = __float_as_int(h.k0.y) * sx.xsum + (d[0] + 256 * d[1]);
-    const int e1 = __float_as_int(h.k1.y) * sx.xsum + (d[2] + 256 * d[3]);
-    if (FIRST) { r0 = __fmul_rn((float)e0, h.k0.x); r1 = __fmul_rn((float)e1, h.k1.x); }
-    else { r0 = fmaf((float)e0, h.k0.x, r0); r1 = fmaf((float)e1, h.k1.x, r1); }
+    // sum_i x_i X_i = sum_i u_i (2 X_i) + (parity - 16) / 2 sum_i 2 X_i, limb pair by limb pair: whole numbers and halves below 2^23,
+    // so the conversion and the multiply-add round nothing
+    const float e0 = fmaf(h.k0.y, sx.xsum, (float)(d[0] + 256 * d[1])), e1 = fmaf(h.k1.y, sx.xsum, (float)(d[2] + 256 * d[3]));
+    if (FIRST) { r0 = __fmul_rn(e0, h.k0.x); r1 = __fmul_rn(e1, h.k1.x); }
+    else { r0 = fmaf(e0, h.k0.x, r0); r1 = fmaf(e1, h.k1.x, r1); }
 }
 // ---- several activation vectors.  Two vectors share the eight columns of the contraction - column g = 4 (vector) + limb -
 // and a block slot has an instruction sequence of its own: positions 0..23 of the half-step for slot 0, 24..47 for slot 1,
@@ -409,10 +311,16 @@ struct PairA {
     float2 k00, k01, k10, k11;                     // block constants: slot, then row g or g + 8
 };
 __device__ __forceinline__ PairA decode_pair(uint32_t wa, uint32_t wb, uint32_t wc, uint32_t hw0, uint32_t hw1, uint32_t tq) {
-    constexpr uint32_t kNib = 0x0f0f0f0fu;
+    // 2 u a byte (doubled by an addition, which has a cycle where a shift takes two)
+    constexpr uint32_t kNib2 = 0x1e1e1e1eu;
+    auto twice = [](uint32_t w) {
+        uint32_t r;
+        asm("add.u32 %0, %1, %1;" : "=r"(r) : "r"(w));
+        return r;
+    };
     PairA h;
-    h.a0 = wa & kNib; h.a1 = wb & kNib; h.a2 = (wa >> 4) & kNib; h.a3 = (wb >> 4) & kNib;
-    h.c0 = wc & kNib; h.c1 = (wc >> 4) & kNib;
+    h.a0 = twice(wa) & kNib2; h.a1 = twice(wb) & kNib2; h.a2 = (wa >> 3) & kNib2; h.a3 = (wb >> 3) & kNib2;
+    h.c0 = twice(wc) & kNib2; h.c1 = (wc >> 3) & kNib2;
     h.k00 = lds_f2(and_or(hw0 << 3, 0x1ff8u, tq));
     h.k01 = lds_f2(and_or(hw0 >> 13, 0x1ff8u, tq));
     h.k10 = lds_f2(and_or(hw1 << 3, 0x1ff8u, tq));
@@ -450,6 +358,7 @@ __device__ __forceinline__ void contract_pair(const PairA &h, const PairX &x, fl
     mma_k32(d, h.a0, h.a1, h.a2, h.a3, x.b0, x.b1);
     mma_k32(f, h.a0, h.a1, h.a2, h.a3, 0u, x.b2);
     mma_k16(f, h.c0, h.c1, x.b3);
+    // twice sum_i x_i X_i, limb pair by limb pair, a whole number below 2^24: 2 u_i against 2 X_i, and (parity - 16) sum_i 2 X_i; the scale is halved
     const int e00 = __float_as_int(h.k00.y) * x.xs0 + (d[0] + 256 * d[1]), e01 = __float_as_int(h.k01.y) * x.xs0 + (d[2] + 256 * d[3]);
     const int e10 = __float_as_int(h.k10.y) * x.xs1 + (f[0] + 256 * f[1]), e11 = __float_as_int(h.k11.y) * x.xs1 + (f[2] + 256 * f[3]);
     if (FIRST) {
@@ -500,12 +409,9 @@ __device__ __forceinline__ void convert_item(const uint4 &v, int third, uint32_t
 #pragma unroll
     for (int l = 0; l < 4; l++)
         asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(rec + 24 * l + 8 * third), "r"(pl[l][0]), "r"(pl[l][1]) : "memory");
-    // this item's sum of 2 X is a0 + 65536 a1; it is even, and so is a0; if a1 is odd one unit of it moves to
-    // a0, and then both halve exactly: the item adds a0 / 2 and a1 / 2 to the block's s0 and s1
-    int a0 = limb_sum[0] + 256 * limb_sum[1], a1 = limb_sum[2] + 256 * limb_sum[3];
-    a0 += (a1 & 1) << 16;
-    asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(rec + 100), "r"(a0 >> 1) : "memory");
-    asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(rec + 104), "r"(a1 >> 1) : "memory");
+    // this item's share of the block's sum of 2 X, limb pair by limb pair
+    asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(rec + 100), "r"(limb_sum[0] + 256 * limb_sum[1]) : "memory");
+    asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(rec + 104), "r"(limb_sum[2] + 256 * limb_sum[3]) : "memory");
 }
 
 // ---- the order of work.  A unit is a tile of a row group or its leftover blocks (column p.tiles).  Units
@@ -517,15 +423,6 @@ __device__ __forceinline__ void convert_item(const uint4 &v, int third, uint32_t
 struct Cursor {
     int panel, group, col, end;      // end = first column past the panel
 };
-__host__ __device__ inline int fast_div(int n, const FastDiv &f, int d) {
-#ifdef __CUDA_ARCH__
-    (void)d;
-    return f.mul ? (int)(__umulhi((uint32_t)n, f.mul) >> f.shift) : n;
-#else
-    (void)f;
-    return n / d;
-#endif
-}
 // steps over n units of the current row group's stretch; true if the row group changed
 __device__ __forceinline__ bool advance(const GemvParams &p, Cursor &c, int n) {
     c.col += n;
@@ -702,15 +599,14 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
         }
     };
     // issue the copy of the next unit onto barrier `b` and buffer `dst`: by one elected lane under a condition that
-    // is the same for the whole warp, or (the four-vector build, where that form costs a register too many) by
-    // lane 0 under its own predicate
+    // is the same for the whole warp, or (several pairs, where that form costs registers too many) by lane 0 under its own predicate
     const int my_issues = lane == 0 ? n_units : 0;
     auto issue = [&](uint32_t b, uint32_t dst) {
         const int done = iw.done;
         const uint8_t *src;
         uint32_t bytes;
         walk_next(iw, src, bytes);
-        if constexpr (BATCH >= 4) {
+        if constexpr (BATCH > 2) {
             asm volatile(
                 "{\n\t.reg .pred p;\n\t"
                 "setp.lt.s32 p, %0, %1;\n\t"
@@ -811,7 +707,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 const int parity = window ? (f >> 2) & 1 : (h >> 4) & 1, gain = window ? (f >> 3) & 1 : (h >> 5) & 1;
                 const int base = window ? 2 * (3 + (f & 3)) : 0;
                 const GemvProblemDev &pe = p.prob[m];
-                tab[m * 1024 + h] = make_float2(p.shell_inv_norm[shell] * (gain ? pe.gain1 : pe.gain0), __int_as_float(shell ? parity - 16 + base : 0));
+                tab[m * 1024 + h] = make_float2(p.shell_inv_norm[shell] * (gain ? pe.gain1 : pe.gain0), shell ? 0.5f * (float)(parity - 16 + base) : 0.f);
             }
         } else {
             for (int m = 0; m < p.nprob; m++) {
@@ -819,8 +715,10 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 for (int i = 0; i < kClasses; i++) {
                     const int c = tid + i * kThreads;
                     if (kClassSlots % kThreads != 0 && c >= kClassSlots) break;
-                    tab[m * 1024 + c] = make_float2(my_class[i].x * p.prob[m].gain0, my_class[i].y);
-                    tab[m * 1024 + 512 + c] = make_float2(my_class[i].x * p.prob[m].gain1, my_class[i].y);
+                    // one vector: {scale, (parity - 16) / 2}; pairs: {scale / 2, parity - 16 as an integer}
+                    const float offset = BATCH == 1 ? 0.5f * (float)__float_as_int(my_class[i].y) : my_class[i].y, factor = BATCH == 1 ? my_class[i].x : 0.5f * my_class[i].x;
+                    tab[m * 1024 + c] = make_float2(factor * p.prob[m].gain0, offset);
+                    tab[m * 1024 + 512 + c] = make_float2(factor * p.prob[m].gain1, offset);
                 }
             }
         }
@@ -969,7 +867,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
         uint4 mine[BATCH];
         int mine_e = -1;
         // the loads of every vector are in flight together: four to eight 128-bit loads a thread
-        constexpr int kInFlight = BATCH <= 2 ? 4 : (BATCH <= 4 ? 2 : 1);
+        constexpr int kInFlight = BATCH <= 2 ? 4 : 1;
         uint32_t m[BATCH];
 #pragma unroll
         for (int j = 0; j < BATCH; j++) {
@@ -984,7 +882,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
 #pragma unroll
                 for (int i = 0; i < kInFlight; i++) {
                     const int e = base + i * kThreads + tid;
-                    v[j][i] = (e < nx && (BATCH == 1 || j < p.batch)) ? __ldcg(xg0 + (size_t)j * nx + e) : make_uint4(0u, 0u, 0u, 0u);
+                    v[j][i] = (e < nx && (BATCH <= 2 || j < p.batch)) ? __ldcg(xg0 + (size_t)j * nx + e) : make_uint4(0u, 0u, 0u, 0u);
                 }
             if (base == 0) {
                 // while the first loads are on their way: what the loop needs besides x.
@@ -1017,7 +915,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
         }
 #pragma unroll
         for (int j = 0; j < BATCH; j++) {
-            if (BATCH > 1 && j >= p.batch) break;
+            if (BATCH > 2 && j >= p.batch) break;
             const uint32_t most = warp_max[j * kWarps + (lane < kWarps ? lane : 0)];
             xexp[j] = max((int)(__reduce_max_sync(0xffffffffu, most) >> 10), 1) - 14;
             const float scale = pow2f(29 - xexp[j]);
@@ -1134,15 +1032,15 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 mma_k16(d1, h1.c0, h1.c1, s1.b2);
                 mma_k16(d2, h2.c0, h2.c1, s2.b2);
                 mma_k16(d3, h3.c0, h3.c1, s2.b2);
-                auto e = [](const int (&d)[4], float ky, int xsum, int r) { return __float_as_int(ky) * xsum + (d[2 * r] + 256 * d[2 * r + 1]); };
-                acc[0] = (float)e(d0, h0.k0.y, s1.xsum, 0) * h0.k0.x;
-                acc[1] = (float)e(d0, h0.k1.y, s1.xsum, 1) * h0.k1.x;
-                acc[2] = (float)e(d1, h1.k0.y, s1.xsum, 0) * h1.k0.x;
-                acc[3] = (float)e(d1, h1.k1.y, s1.xsum, 1) * h1.k1.x;
-                acc[0] = fmaf((float)e(d2, h2.k0.y, s2.xsum, 0), h2.k0.x, acc[0]);
-                acc[1] = fmaf((float)e(d2, h2.k1.y, s2.xsum, 1), h2.k1.x, acc[1]);
-                acc[2] = fmaf((float)e(d3, h3.k0.y, s2.xsum, 0), h3.k0.x, acc[2]);
-                acc[3] = fmaf((float)e(d3, h3.k1.y, s2.xsum, 1), h3.k1.x, acc[3]);
+                auto e = [](const int (&d)[4], float ky, float xsum, int r) { return fmaf(ky, xsum, (float)(d[2 * r] + 256 * d[2 * r + 1])); };
+                acc[0] = e(d0, h0.k0.y, s1.xsum, 0) * h0.k0.x;
+                acc[1] = e(d0, h0.k1.y, s1.xsum, 1) * h0.k1.x;
+                acc[2] = e(d1, h1.k0.y, s1.xsum, 0) * h1.k0.x;
+                acc[3] = e(d1, h1.k1.y, s1.xsum, 1) * h1.k1.x;
+                acc[0] = fmaf(e(d2, h2.k0.y, s2.xsum, 0), h2.k0.x, acc[0]);
+                acc[1] = fmaf(e(d2, h2.k1.y, s2.xsum, 1), h2.k1.x, acc[1]);
+                acc[2] = fmaf(e(d3, h3.k0.y, s2.xsum, 0), h3.k0.x, acc[2]);
+                acc[3] = fmaf(e(d3, h3.k1.y, s2.xsum, 1), h3.k1.x, acc[3]);
                 sum[0] += __float2ll_rn(quad_sum(acc) * inv_q);
                 xa.b0 += 4 * kXBlock; xa.b1 += 4 * kXBlock; xa.b2 += 4 * kXBlock; xa.xs += 4 * kXBlock;
             } else {
@@ -1153,7 +1051,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 const PairA h2 = decode_pair(a1.z, a1.w, a2.x, hh.z, hb.z, tq), h3 = decode_pair(a2.y, a2.z, a2.w, hh.w, hb.w, tq);
                 auto one_pair = [&](auto index) {
                     constexpr int J = decltype(index)::value, kPair = J * 2 * kXRecBytes;
-                    if (J > BATCH / 4 && 2 * J >= p.batch) return;         // a launch may carry fewer vectors than the kernel is built for
+                    if (J > 1 && 2 * J >= p.batch) return;                 // a launch carries fewer vectors than the kernel is built for
                     const PairX x0 = load_pair<kPair, kPair + kXBlock>(xp), x1 = load_pair<kPair + 2 * kXBlock, kPair + 3 * kXBlock>(xp);
                     float u[4], w[4];                                      // slot 0 and slot 1, rows [2m + e]
                     contract_pair<true>(h0, x0, u, w);
@@ -1238,7 +1136,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 const PairAddr xt = pair_addr(lane, xs0 + (uint32_t)tiles * (4 * kXBlock)), xl = pair_addr(lane, xs0 + (uint32_t)(p.nb - 1) * kXBlock);
                 auto one_pair = [&](auto index) {
                     constexpr int J = decltype(index)::value, kPair = J * 2 * kXRecBytes;
-                    if (J > BATCH / 4 && 2 * J >= p.batch) return;         // a launch may carry fewer vectors than the kernel is built for
+                    if (J > 1 && 2 * J >= p.batch) return;                 // a launch carries fewer vectors than the kernel is built for
                     float u[4] = {0.f, 0.f, 0.f, 0.f}, v[4] = {0.f, 0.f, 0.f, 0.f};
                     if (two) {
                         const PairX x = load_pair<kPair, kPair + kXBlock>(xt);
@@ -1764,12 +1662,14 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
         g.smem = ((size_t)p.nb * 48 + 127) / 128 * 128;
         return g;
     }
-    // panels of about sixteen unit columns, as equal as they come.  For more than four vectors of sixteen at most: a CTA that
+    // panels of about sixteen unit columns, as equal as they come.  For five vectors and more of sixteen at most: a CTA that
     // meets two panels then has a piece of x for each of its twelve warps' threads, and none is read again, vector after vector
-    // (five vectors, us with panels of 18 columns and of 15: 500 x 8192 12.3 and 10.0, two passes 10.7; eight on 2560 x 5120 19.2 and 15.0, 17.4).
-    constexpr int kPanelColumns = 16;
-    static_assert(2 * kPanelColumns * kTileCells * 3 <= 32 * gemv_warps(LLVQ_MAX_BATCH), "two panels' pieces of x, a thread each");
-    const int most = (p.units + (p.batch > 4 ? kPanelColumns - 1 : kPanelColumns / 2)) / kPanelColumns, want = most > 1 ? most : 1;
+    // (five vectors, us with panels of 18 columns and of 15: 500 x 8192 12.3 and 10.0, two passes 10.7).  Vectors in sets of
+    // four on a small matrix: of eight at most, for half the blocks of x to convert; the row groups' sums, twice as many, are added up by the CTA
+    // first (us with sixteen and eight: four vectors on 4096 x 4096 8.2 and 8.1, 1024 x 2560 5.7 and 5.2; eight 15.9 and 15.4, 10.2 and 8.7).
+    constexpr int kPanelColumns = 16, kFewColumns = 8;
+    const bool few = batch_in_sets(p.batch) && p.total_units < 64 * sm_count;
+    const int columns = few ? kFewColumns : kPanelColumns, most = (p.units + (p.batch > 4 || few ? columns - 1 : columns / 2)) / columns, want = most > 1 ? most : 1;
     p.panel = (p.units + want - 1) / want;
     p.npanels = (p.units + p.panel - 1) / p.panel;
     p.div_panel = make_fastdiv((uint32_t)p.panel);
@@ -1829,8 +1729,13 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
             if (keep > p.rot_keep) p.rot_keep = keep;
         }
     }
-    const int vectors = p.batch <= 2 ? p.batch : (p.batch <= 4 ? 4 : 8);       // the kernel is built for 1, 2, 4 and 8
-    const int warps = gemv_warps(vectors);
+    if (batch_in_sets(p.batch)) {
+        const int sets = batch_sets(p.batch), warps = batch_warps(sets);
+        g.smem = (size_t)warps * kSlots * kTileBytes + 2 * 8192 /* the table and its alignment */ + ((size_t)p.xblocks * sets * kBatchSetBytes + 127) / 128 * 128 +
+                 warps * kSlots * 8 + 32 + (LLVQ_MAX_BATCH + 1) * 4 + 16;
+        return g;
+    }
+    const int vectors = p.batch > 2 ? 8 : p.batch, warps = gemv_warps(vectors);        // the kernel is built for 1, 2 and 8
     const size_t records = ((size_t)p.xblocks * kXRecBytes * vectors + 127) / 128 * 128, raw = rot_first(p.rot_log2).stages ? ((size_t)p.rot_span * 2 + 127) / 128 * 128 : 0;
     g.smem = (size_t)warps * kSlots * kTileBytes + 8192 /* alignment of the tables */ + (size_t)p.nprob * 8192 + warps * kSlots * 8 + warps * 4 * vectors + 16;
     // a rotation counts with eight bytes a coordinate of its whole blocks, the limit llvq_gemv_rotated states, though it needs less
@@ -1840,23 +1745,13 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
     return g;
 }
 
-template <typename K>
-static int allow_max_smem(K kernel, int optin) {
-    cudaFuncAttributes a;
-    if (cudaFuncGetAttributes(&a, kernel) != cudaSuccess) return -1;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes) != cudaSuccess) return -1;
-    // ask for the largest shared-memory carve-out, so that a CTA of the next kernel of the stream can
-    // settle beside a running one (programmatic dependent launch) whenever two of them fit
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess ? 0 : -1;
-}
-
 int gemv_configure(const llvq_ctx *ctx) {
     const int bytes = ctx->max_smem_optin;
     if (allow_max_smem(gemv_planes_kernel<false, 1>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<true, 1>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 2>, bytes)) return -1;
-    if (allow_max_smem(gemv_planes_kernel<false, 4>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 8>, bytes)) return -1;
+    if (batch_configure(bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 1, kRotateShort>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 1, kRotateLong>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 1, kNoRotation, LLVQ_PLANES13>, bytes)) return -1;
@@ -1866,6 +1761,10 @@ int gemv_configure(const llvq_ctx *ctx) {
 }
 
 cudaError_t launch_gemv(int layout, const GemvParams &p, const GemvLaunch &g, bool no_weights, bool pdl, cudaStream_t s) {
+    // Us a launch in a chain, in pairs of vectors (8-bit limbs) and in sets of four: three vectors on 1024 x 2560 5.27 and 4.96, 4096 x 4096 8.41
+    // and 7.83, 500 x 8192 6.42 and 5.25, 34816 x 5120 35.7 and 32.1; four 5.57 and 5.24, 8.85 and 8.27, 6.93 and 5.96, 36.1 and 32.4; eight 9.65
+    // and 8.82, 16.5 and 15.1, 12.98 and 12.95, 62.1 and 53.9.  Two on 8192 x 8192 11.9 and 15.0; for five and six see batch_in_sets.
+    if (batch_in_sets(p.batch)) return launch_batch(p, g, pdl, s);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)g.grid);
     cfg.blockDim = dim3(32 * gemv_warps(p.batch));
@@ -1883,7 +1782,6 @@ cudaError_t launch_gemv(int layout, const GemvParams &p, const GemvLaunch &g, bo
         if (p.rot_log2 > 0) return cudaLaunchKernelEx(&cfg, rot_first(p.rot_log2).stages ? gemv_planes_kernel<false, 1, kRotateLong> : gemv_planes_kernel<false, 1, kRotateShort>, p);
         if (p.batch <= 1) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 1>, p);
         if (p.batch == 2) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 2>, p);
-        if (p.batch <= 4) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 4>, p);
         return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 8>, p);
     }
     cfg.numAttrs = 0;
@@ -2060,7 +1958,6 @@ extern "C" int llvq_gemv_static(const void *layout_buf, const void *row_scale, c
     if (g.smem + 1024 > (size_t)d.max_smem_optin) return LLVQ_ESIZE;
     return llvq::launched(llvq::launch_gemv(LLVQ_PLANES, p, g, false, true, (cudaStream_t)stream));
 }
-
 
 // Reports and repairs what a llvq_gemv_static launch that gave up on a bounded wait leaves behind.  Without a
 // context there is no llvq_status to do it: the flag such a launch raises and the partial sums it abandons live in
