@@ -4,12 +4,12 @@
 // four-bit code the record stores.  The activations are taken as fixed point, X_i = rint(x_i * 2^F) with F
 // set by the largest |x| of the call, and 2 X_i is split into four balanced 8-bit limbs.  The inner sum then
 // is an integer contraction that the tensor cores do exactly: mma.sync m16n8k32 / m16n8k16, u8 x s8 -> s32.
-// A is 16 rows x 48 positions (two block slots of 24 coordinates) of codes, one byte each once the two nibbles
-// of a payload byte are split (one shift, two ANDs a word: the whole decode); B is block-diagonal, its eight
+// A is 16 rows x 48 positions (two block slots of 24 coordinates) of doubled codes, one byte each once the two nibbles
+// of a payload byte are split (an addition, a shift, two ANDs a word: the whole decode); B is block-diagonal, its eight
 // columns the four limbs of slot 0 and the four limbs of slot 1, so one accumulator tile holds, for 16 rows,
 // the two blocks' sums limb by limb.  Per (row, block) the limbs are recombined in integers, the offset term
-// (parity - 16) * sum_i X_i is added from a per-block sum prepared with x, and one float multiply-add applies
-// gain[g] / (4 sqrt m), looked up by the header.  Every lane runs the same instructions whatever its class.
+// (parity - 16) * sum_i 2 X_i is added from a per-block sum prepared with x (what is added up is twice sum_i x_i X_i: the
+// halves of an odd sum need no care), and one float multiply-add applies half of gain[g] / (4 sqrt m), looked up by the header.  Every lane runs the same instructions whatever its class.
 //
 // Geometry.  A warp works on the 32 rows of a row group, 16 at a time; the records are stored as the
 // instruction's operand fragments (include/llvq.h), so a lane's 128-bit shared-memory reads are its A
@@ -188,17 +188,23 @@ __host__ __device__ __forceinline__ LaneOffsets lane_offsets(int lane, bool one)
 }
 
 // The B operand of one step (two block slots) for this lane, and its share of the slots' activation sum.
-struct StepX { uint32_t b0, b1, b2; float xsum; };
+struct StepX { uint32_t b0, b1, b2; int xsum; };
 // a.* are this lane's four addresses for the records at the start of a tile; OFF selects the step
 template <int OFF>
 __device__ __forceinline__ StepX load_step(const LaneOffsets &a) {
     StepX s;
     s.b0 = lds32_at<OFF>(a.b0); s.b1 = lds32_at<OFF>(a.b1); s.b2 = lds32_at<OFF>(a.b2);
-    s.xsum = (float)(int)lds32_at<OFF>(a.xs);
+    s.xsum = (int)lds32_at<OFF>(a.xs);
     return s;
 }
 
-// The A operand of a half-step (the decode proper: one shift and two ANDs a word) and the block constants of
+// twice a word, by an addition: it has a cycle where a shift takes two
+__device__ __forceinline__ uint32_t twice(uint32_t w) {
+    uint32_t r;
+    asm("add.u32 %0, %1, %1;" : "=r"(r) : "r"(w));
+    return r;
+}
+// The A operand of a half-step (the decode proper, 2 u a byte: one shift, one addition and two ANDs a word) and the block constants of
 // its two rows; both are shared by every activation vector of a batched launch.
 struct HalfA {
     uint32_t a0, a1, a2, a3, c0, c1;
@@ -207,10 +213,10 @@ struct HalfA {
 // COMPACT (13-byte layout): the two headers are the bytes at bit SHIFT and SHIFT + 8 of hw.
 template <bool COMPACT = false, int SHIFT = 0>
 __device__ __forceinline__ HalfA decode_half(uint32_t wa, uint32_t wb, uint32_t wc, uint32_t hw, uint32_t tq) {
-    constexpr uint32_t kNib = 0x0f0f0f0fu;
+    constexpr uint32_t kNib2 = 0x1e1e1e1eu;
     HalfA h;
-    h.a0 = wa & kNib; h.a1 = wb & kNib; h.a2 = (wa >> 4) & kNib; h.a3 = (wb >> 4) & kNib;
-    h.c0 = wc & kNib; h.c1 = (wc >> 4) & kNib;
+    h.a0 = twice(wa) & kNib2; h.a1 = twice(wb) & kNib2; h.a2 = (wa >> 3) & kNib2; h.a3 = (wb >> 3) & kNib2;
+    h.c0 = twice(wc) & kNib2; h.c1 = (wc >> 3) & kNib2;
     if (COMPACT) {
         // one byte a header, eight bytes an entry
         h.k0 = lds_f2(and_or(SHIFT >= 3 ? hw >> (SHIFT - 3) : hw << (3 - SHIFT), 0x7f8u, tq));
@@ -228,8 +234,8 @@ __device__ __forceinline__ HalfA decode_half(uint32_t wa, uint32_t wb, uint32_t 
 // 14-byte layout, four instructions for each of the six.  hb = the eight header bytes of the lane's rows.
 template <int K>
 __device__ __forceinline__ uint32_t overlay_left_over(uint32_t vk, uint32_t vhigh) {
-    // (vk >> 6 & 0x03030303) | (vhigh >> (4 + (K & 1)) & 0x04040404)
-    return and_or(vhigh >> (4 + (K & 1)), 0x04040404u, (vk >> 6) & 0x03030303u);
+    // (vk >> 5 & 0x06060606) | (vhigh >> (3 + (K & 1)) & 0x08080808)
+    return and_or(vhigh >> (3 + (K & 1)), 0x08080808u, (vk >> 5) & 0x06060606u);
 }
 template <int SHIFT>
 __device__ __forceinline__ void header_consts(uint32_t hw, uint32_t tq, float2 &k0, float2 &k1) {
@@ -238,12 +244,12 @@ __device__ __forceinline__ void header_consts(uint32_t hw, uint32_t tq, float2 &
 }
 __device__ __forceinline__ void decode_overlay_tile(const uint4 &va, const uint4 &vb, uint32_t v8, const uint2 &hb, uint32_t tq,
                                                     HalfA &h0, HalfA &h1, HalfA &h2, HalfA &h3) {
-    constexpr uint32_t k7 = 0x07070707u;
-    h0.a0 = va.x & k7; h0.a2 = (va.x >> 3) & k7; h0.a1 = va.y & k7; h0.a3 = (va.y >> 3) & k7;
-    h1.a0 = va.z & k7; h1.a2 = (va.z >> 3) & k7; h1.a1 = va.w & k7; h1.a3 = (va.w >> 3) & k7;
-    h2.a0 = vb.x & k7; h2.a2 = (vb.x >> 3) & k7; h2.a1 = vb.y & k7; h2.a3 = (vb.y >> 3) & k7;
-    h3.a0 = vb.z & k7; h3.a2 = (vb.z >> 3) & k7; h3.a1 = vb.w & k7; h3.a3 = (vb.w >> 3) & k7;
-    h0.c0 = v8 & k7; h1.c0 = (v8 >> 3) & k7;
+    constexpr uint32_t k14 = 0x0e0e0e0eu;                // 2 v a byte
+    h0.a0 = twice(va.x) & k14; h0.a2 = (va.x >> 2) & k14; h0.a1 = twice(va.y) & k14; h0.a3 = (va.y >> 2) & k14;
+    h1.a0 = twice(va.z) & k14; h1.a2 = (va.z >> 2) & k14; h1.a1 = twice(va.w) & k14; h1.a3 = (va.w >> 2) & k14;
+    h2.a0 = twice(vb.x) & k14; h2.a2 = (vb.x >> 2) & k14; h2.a1 = twice(vb.y) & k14; h2.a3 = (vb.y >> 2) & k14;
+    h3.a0 = twice(vb.z) & k14; h3.a2 = (vb.z >> 2) & k14; h3.a1 = twice(vb.w) & k14; h3.a3 = (vb.w >> 2) & k14;
+    h0.c0 = twice(v8) & k14; h1.c0 = (v8 >> 2) & k14;
     h0.c1 = overlay_left_over<0>(va.x, vb.z);            // X0 = Group(0, 1, 2): low bits in V0, third bit in V6
     h1.c1 = overlay_left_over<1>(va.y, vb.z);            // X1 = Group(1, 1, 2)
     h2.c0 = overlay_left_over<2>(va.z, vb.w);            // X2 = Group(2, 0, 2): V2 and V7
@@ -278,9 +284,11 @@ __device__ __forceinline__ long long exception_value(const uint4 &ent, uint32_t 
         }
         cw = j == 0 ? ent.z : ent.w;
     }
-    const float e_lo = fmaf(k.y, (float)(int)lds32(rec + 100), (float)(d[0] + 256 * d[1]));
-    const float e_hi = fmaf(k.y, (float)(int)lds32(rec + 104), (float)(d[2] + 256 * d[3]));
-    return __float2ll_rn((e_lo * k.x + (e_hi * k.x) * 65536.f) * inv_q);
+    // twice the sums, as in the tile path
+    const int off = __float_as_int(k.y);
+    const int e_lo = off * (int)lds32(rec + 100) + 2 * (d[0] + 256 * d[1]);
+    const int e_hi = off * (int)lds32(rec + 104) + 2 * (d[2] + 256 * d[3]);
+    return __float2ll_rn(((float)e_lo * k.x + ((float)e_hi * k.x) * 65536.f) * inv_q);
 }
 
 // One half-step: 16 rows x 2 block slots.  h holds this lane's payload words and the constants of its rows' blocks in slot
@@ -292,11 +300,11 @@ __device__ __forceinline__ void contract_half(const HalfA &h, const StepX &sx, f
     int d[4];
     mma_k32(d, h.a0, h.a1, h.a2, h.a3, sx.b0, sx.b1);
     mma_k16(d, h.c0, h.c1, sx.b2);
-    // sum_i x_i X_i = sum_i u_i (2 X_i) + (parity - 16) / 2 sum_i 2 X_i, limb pair by limb pair: whole numbers and halves below 2^23,
-    // so the conversion and the multiply-add round nothing
-    const float e0 = fmaf(h.k0.y, sx.xsum, (float)(d[0] + 256 * d[1])), e1 = fmaf(h.k1.y, sx.xsum, (float)(d[2] + 256 * d[3]));
-    if (FIRST) { r0 = __fmul_rn(e0, h.k0.x); r1 = __fmul_rn(e1, h.k1.x); }
-    else { r0 = fmaf(e0, h.k0.x, r0); r1 = fmaf(e1, h.k1.x, r1); }
+    // twice sum_i x_i X_i = sum_i 2 u_i (2 X_i) + (parity - 16) sum_i 2 X_i, limb pair by limb pair, in integers below 2^24; the scale is halved
+    const int e0 = __float_as_int(h.k0.y) * sx.xsum + (d[0] + 256 * d[1]);
+    const int e1 = __float_as_int(h.k1.y) * sx.xsum + (d[2] + 256 * d[3]);
+    if (FIRST) { r0 = __fmul_rn((float)e0, h.k0.x); r1 = __fmul_rn((float)e1, h.k1.x); }
+    else { r0 = fmaf((float)e0, h.k0.x, r0); r1 = fmaf((float)e1, h.k1.x, r1); }
 }
 // ---- several activation vectors.  Two vectors share the eight columns of the contraction - column g = 4 (vector) + limb -
 // and a block slot has an instruction sequence of its own: positions 0..23 of the half-step for slot 0, 24..47 for slot 1,
@@ -311,13 +319,7 @@ struct PairA {
     float2 k00, k01, k10, k11;                     // block constants: slot, then row g or g + 8
 };
 __device__ __forceinline__ PairA decode_pair(uint32_t wa, uint32_t wb, uint32_t wc, uint32_t hw0, uint32_t hw1, uint32_t tq) {
-    // 2 u a byte (doubled by an addition, which has a cycle where a shift takes two)
     constexpr uint32_t kNib2 = 0x1e1e1e1eu;
-    auto twice = [](uint32_t w) {
-        uint32_t r;
-        asm("add.u32 %0, %1, %1;" : "=r"(r) : "r"(w));
-        return r;
-    };
     PairA h;
     h.a0 = twice(wa) & kNib2; h.a1 = twice(wb) & kNib2; h.a2 = (wa >> 3) & kNib2; h.a3 = (wb >> 3) & kNib2;
     h.c0 = twice(wc) & kNib2; h.c1 = (wc >> 3) & kNib2;
@@ -381,8 +383,8 @@ __device__ __forceinline__ void pair_sum(const float (&v)[4], bool odd, float &r
 
 // x (fp16) -> records.  X_i = rint(x_i * 2^F) with F chosen from the largest |x| so that |X_i| < 2^29; the
 // record of a block stores the four balanced limbs of 2 X_i (2 X_i = sum_l limb_l 256^l, limbs in -128..127)
-// plane by plane, and the block's sum of the X_i split in two, sum = s0 + 65536 s1.  An item is eight coordinates (one 128-bit piece of x): item e belongs to block e / 3.
-// The three items of a block add their shares of s0 and s1 with shared-memory atomics; the words were zeroed
+// plane by plane, and the block's sums of 2 X, one a limb pair (limbs 0 and 1 at 100, 2 and 3 at 104).  An item is eight coordinates (one 128-bit piece of x): item e belongs to block e / 3.
+// The three items of a block add their shares of the sums with shared-memory atomics; the words were zeroed
 // before.  `rec` is the shared-memory address of the block's record.
 __device__ __forceinline__ void convert_item(const uint4 &v, int third, uint32_t rec, float scale) {
     const uint32_t hv[4] = {v.x, v.y, v.z, v.w};
@@ -464,7 +466,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
     constexpr int kSrcCell = COMPACT ? kCell13Bytes : kCellBytes;        // bytes of a leftover block column of a row group
     constexpr int kSrcTile = OVERLAY ? kTile10Bytes : (COMPACT ? kTile13Bytes : kTileBytes);   // bytes of a tile in memory (a ring slot always has kTileBytes)
     extern __shared__ __align__(128) unsigned char smem[];
-    // shared memory: ring | per-matrix block constants (1024 x {gain / (4 sqrt m), parity - 16}) | x records | barriers
+    // shared memory: ring | per-matrix block constants (1024 x {gain / (8 sqrt m), parity - 16}) | x records | barriers
     unsigned char *ring = smem;
     // the block constants start on an 8 KiB boundary of the shared window, so that a matrix's table base and
     // an entry's offset combine by OR (decode_half)
@@ -692,7 +694,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
     const bool odd_lane = lane & 1, high_lane = lane & 2;
     const float limb_scale = odd_lane ? 65536.f : 1.f;     // this lane's limb pair: 256^0,1 or 256^2,3
     const uint32_t tab0 = smem_addr(tab);
-    // the block constants of every matrix of the launch: (class | gain << 9) -> {gain / (4 sqrt m), parity - 16}
+    // the block constants of every matrix of the launch: (class | gain << 9) -> {gain / (8 sqrt m), parity - 16}
     // (13-byte layout: the header byte is shell | parity << 4 | gain << 5 - 64 entries a matrix)
     auto build_tables = [&]() {
         if (COMPACT) {
@@ -707,7 +709,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 const int parity = window ? (f >> 2) & 1 : (h >> 4) & 1, gain = window ? (f >> 3) & 1 : (h >> 5) & 1;
                 const int base = window ? 2 * (3 + (f & 3)) : 0;
                 const GemvProblemDev &pe = p.prob[m];
-                tab[m * 1024 + h] = make_float2(p.shell_inv_norm[shell] * (gain ? pe.gain1 : pe.gain0), shell ? 0.5f * (float)(parity - 16 + base) : 0.f);
+                tab[m * 1024 + h] = make_float2(0.5f * p.shell_inv_norm[shell] * (gain ? pe.gain1 : pe.gain0), __int_as_float(shell ? parity - 16 + base : 0));
             }
         } else {
             for (int m = 0; m < p.nprob; m++) {
@@ -715,10 +717,8 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 for (int i = 0; i < kClasses; i++) {
                     const int c = tid + i * kThreads;
                     if (kClassSlots % kThreads != 0 && c >= kClassSlots) break;
-                    // one vector: {scale, (parity - 16) / 2}; pairs: {scale / 2, parity - 16 as an integer}
-                    const float offset = BATCH == 1 ? 0.5f * (float)__float_as_int(my_class[i].y) : my_class[i].y, factor = BATCH == 1 ? my_class[i].x : 0.5f * my_class[i].x;
-                    tab[m * 1024 + c] = make_float2(factor * p.prob[m].gain0, offset);
-                    tab[m * 1024 + 512 + c] = make_float2(factor * p.prob[m].gain1, offset);
+                    tab[m * 1024 + c] = make_float2(0.5f * my_class[i].x * p.prob[m].gain0, my_class[i].y);
+                    tab[m * 1024 + 512 + c] = make_float2(0.5f * my_class[i].x * p.prob[m].gain1, my_class[i].y);
                 }
             }
         }
@@ -1032,7 +1032,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 mma_k16(d1, h1.c0, h1.c1, s1.b2);
                 mma_k16(d2, h2.c0, h2.c1, s2.b2);
                 mma_k16(d3, h3.c0, h3.c1, s2.b2);
-                auto e = [](const int (&d)[4], float ky, float xsum, int r) { return fmaf(ky, xsum, (float)(d[2 * r] + 256 * d[2 * r + 1])); };
+                auto e = [](const int (&d)[4], float ky, int xsum, int r) { return (float)(__float_as_int(ky) * xsum + (d[2 * r] + 256 * d[2 * r + 1])); };
                 acc[0] = e(d0, h0.k0.y, s1.xsum, 0) * h0.k0.x;
                 acc[1] = e(d0, h0.k1.y, s1.xsum, 1) * h0.k1.x;
                 acc[2] = e(d1, h1.k0.y, s1.xsum, 0) * h1.k0.x;
