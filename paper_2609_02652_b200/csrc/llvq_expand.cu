@@ -8,11 +8,12 @@
 // their place; the codes wait in shared memory until the tile's words are gathered from them.  The small look-up tables
 // are copied to shared memory once a CTA, while the previous kernel of the stream ends; one CTA a multiprocessor walks over
 // the tiles.
-// Measured (9728 x 2560 into the 14-byte layout, 1.04 M blocks): 38 us, 2800 warp instructions a tile of 128 blocks, issue
-// slots 54 % busy, the load unit's wavefronts 59 %, half of all stalls waits on the lists; a lane a row with a 64-bit division a coordinate and candidate took
-// 484 us, one odd coordinate at a time 45.  Counting and expanding 17408 x 5120 into the 10-byte layout: 188 us against
-// 4700.  24 or 28 warps a CTA instead of 32: 47 and 50 us.  The shared tables are kept to 51 KB because the rest of a
-// multiprocessor's memory is the L1 cache that the lists are read through: with 104 KB of tables it took 53 us.
+// Measured (9728 x 2560 into the 14-byte layout, 1.04 M blocks): 36.2 us, 2500 warp instructions a tile of 128 blocks, issue
+// slots 50 % busy, the load unit's wavefronts 64 %, half of all stalls waits on the lists (33 % of their sectors come from the
+// L1 cache); a lane a row with a 64-bit division a coordinate and candidate took 484 us, one odd coordinate at a time 45.
+// Counting and expanding 17408 x 5120 into the 10-byte layout: 184 us against 4700.  24 or 28 warps a CTA instead of 32: 47 and
+// 50 us.  The shared tables are kept to 33 KB because the rest of a multiprocessor's memory is the L1 cache that the lists
+// are read through: with 51 KB 38 us, with 104 KB 53.
 #include "llvq_internal.cuh"
 #include "llvq_unrank.cuh"
 
@@ -104,7 +105,8 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
     uint32_t bad = 0;
     // The CTA's pieces (every gridDim-th), a warp a piece and round.  A piece is a chain of some ten microseconds, however few
     // run: where the last round has work for half of the warps or a quarter, two or four share a piece, each its blocks
-    // (500 x 1000: 8.3 us, 14.8 without; 17408 x 5120: 117, 121; a last round of 26 pieces, 9728 x 2560: 38.0, 37.9).
+    // (500 x 1000: 7.5 us; before the tables were made smaller 8.3, 14.8 without; 17408 x 5120: 117, 121; a last round of 26 pieces,
+    // 9728 x 2560: 38.0, 37.9).
     // `own` = the blocks of the piece that are this warp's, a bit each, and 16 (0: no piece left), `share` = log2 of the warps on it.
     const uint32_t mine = (total_pieces - blockIdx.x + gridDim.x - 1) / gridDim.x, full = mine / kExpandWarps * kExpandWarps;
     const int last_share = mine - full <= kExpandWarps / 4 ? 2 : (mine - full <= kExpandWarps / 2 ? 1 : 0);

@@ -21,13 +21,6 @@ __attribute__((noinline)) void list_orderings(int *cnt, int left, int at, uint64
     }
 }
 
-// the eight bits of b as the low bits of eight nibbles
-uint32_t spread_bits(uint32_t b) {
-    uint32_t w = 0;
-    for (int i = 0; i < 8; i++) w |= ((b >> i) & 1u) << (4 * i);
-    return w;
-}
-
 // Window of the 10-byte layout (codes u = 8 + floor(x / 2)): a block lacks one if two codes are more than seven apart,
 // or a code is below 3 or above 13.
 int window_of(const ClassDesc &d) {
@@ -111,27 +104,31 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
     }
     // the draws of two from L
     PairStep *pair_steps = part<PairStep>(u.blob, kUnrankPairs);
+    float *ratios = part<float>(u.blob, kUnrankRatios);
     size_t entries = 0;
     for (int i = 0; i < kPairSteps; i++) entries += (size_t)kOddSets * (24 - 2 * i) * (23 - 2 * i);
     u.pairs.reserve(entries);
     for (int i = 0; i < kPairSteps; i++) {
         const int L = 24 - 2 * i, draws = L * (L - 1);
-        const uint32_t shift = (uint32_t)__builtin_ctz(draws), odd = (uint32_t)draws >> shift;
-        uint32_t x = odd;
-        for (int k = 0; k < 5; k++) x *= 2u - odd * x;
-        pair_steps[i] = {x, shift, (uint32_t)u.pairs.size(), (uint32_t)draws};
+        pair_steps[i] = {(uint32_t)u.pairs.size(), (uint32_t)draws};
         u.pairs.resize(u.pairs.size() + (size_t)kOddSets * draws, 0);
         for (int k = 0; k < kOddSets; k++) {
             const std::array<int, 7> &c = sets[k];
             const int n = copies_in(c);
             if (n > L) continue;
             uint64_t *entry = u.pairs.data() + pair_steps[i].first + (size_t)k * draws;
+            // L! / (the copies' factorials): L over the copies of each value in turn, whole numbers all along
+            uint64_t orderings = 1;
+            for (int v = 1, left = L; v < 7; v++)
+                for (int j = 1; j <= c[v]; j++) orderings = orderings * (uint64_t)left-- / (uint64_t)j;
+            if (orderings >= 0x80000000ull) return false;
+            ratios[256 * i + k] = (float)(draws / (double)orderings * kRatioExcess);
             int at = 0;
             for (int va = 0; va < 7; va++)
                 for (int vb = 0; vb < 7; vb++) {
                     const int na = va ? c[va] : L - n, nb = (vb ? c[vb] : L - n) - (va == vb);
                     if (na < 1 || nb < 1) continue;
-                    const uint64_t e = (uint64_t)at | (uint64_t)(na * nb) << 16 | (uint64_t)(va | vb << 4) << 32 | (uint64_t)less[less[k][va]][vb] << 40;
+                    const uint64_t e = orderings * (uint64_t)at / (uint64_t)draws | (uint64_t)(va | vb << 4) << 32 | (uint64_t)less[less[k][va]][vb] << 40;
                     for (int j = 0; j < na * nb; j++) entry[at + j] = e;
                     at += na * nb;
                 }
@@ -235,12 +232,9 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
     for (int k = 0; k < 64; k++) { message[k] = t.golay_by_message[k]; message[64 + k] = t.golay_by_message[64 * k]; }
     std::memcpy(u.blob.data() + kUnrankGolayWt, t.golay_by_weight.data(), 4096 * 4);
 
-    // ---- spreading eight nibbles to the places of a byte mask, and single bits likewise
+    // ---- spreading eight nibbles to the places of a byte mask
     struct Moves { uint32_t m[4]; };
     Moves *merge = part<Moves>(u.blob, kUnrankMerge);
-    uint16_t *at = part<uint16_t>(u.blob, kUnrankDepositAt);
-    uint32_t *deposit = part<uint32_t>(u.blob, kUnrankDeposit);
-    int n = 0;
     for (int mask = 0; mask < 256; mask++) {
         // the nibble of rank r must travel place[r] - r places up; in steps of 4, 2, 1 (each step's targets are
         // distinct, because ranks travel by non-decreasing distances)
@@ -257,14 +251,8 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
             mv.m[3] |= 15u << (4 * place[r]);
         }
         merge[mask] = mv;
-        at[mask] = (uint16_t)n;
-        for (int bits = 0; bits < (1 << k); bits++) {
-            uint32_t b = 0;
-            for (int r = 0; r < k; r++) b |= (uint32_t)((bits >> r) & 1) << place[r];
-            deposit[n++] = spread_bits(b);
-        }
     }
-    return n == 6561;
+    return true;
 }
 
 }  // namespace llvq

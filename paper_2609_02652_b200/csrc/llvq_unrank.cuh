@@ -56,12 +56,12 @@ LLVQ_HD uint32_t float_bits(float f) {
     return c.u;
 #endif
 }
-// an estimate of a / b, a few units of the last place off at most
-LLVQ_HD float quotient(float a, float b) {
+// floor(a * b), a * b below 2^23
+LLVQ_HD uint32_t floor_product(float a, float b) {
 #ifdef __CUDA_ARCH__
-    return __fdividef(a, b);
+    return __float_as_uint(__fmaf_rd(a, b, 8388608.f)) - 0x4b000000u;       // whole numbers from 2^23 on, rounded down
 #else
-    return a / b;
+    return (uint32_t)((double)a * (double)b);
 #endif
 }
 template <typename T>
@@ -111,57 +111,39 @@ LLVQ_HD int find_class(const UnrankView &v, uint64_t idx) {
 LLVQ_HD uint32_t portion(uint32_t T, uint32_t copies, const UnrankStep &e) { return (uint32_t)(((uint64_t)T * copies) >> e.shift) * e.inverse; }
 
 // Odd type.  Sixteen coordinates come two at a time from the table of draws, the ordering of the last eight is an entry of
-// a list.  The position of the draw is a float estimate, which the exact bounds of the pair it names confirm or, in one case
-// in some thousands, move to the pair before or after.  Rolled up: eight steps' code would crowd the instruction cache.
-// Instructions bound this: with the second eight coordinates one at a time from lists in shared memory (fewer gathers,
-// more instructions) 9728 x 2560 takes 46 us instead of 39.
+// a list.  The position of the draw is a float estimate that is right or one too large, which the first rank of the pair it names
+// tells.  Rolled up: eight steps' code would crowd the instruction cache.  The gathers and their cache bound this: with the bounds
+// of a pair worked out from the number of orderings (four multiplications to 64 bits and a reciprocal a step) instead of the
+// 8 KB of ratios, 9728 x 2560 takes 39 us instead of 36, and so it does with the ratios beside a table of dealt signs of
+// 26 KB; with the second eight coordinates one at a time from lists in shared memory 46.
 LLVQ_HD void unrank_odd(const UnrankView &v, const UnrankDesc &d, uint64_t r47, Point &p) {
     const uint32_t message = (uint32_t)r47 & 4095u;
     const uint32_t cw = blob_at<uint32_t>(v, kUnrankGolayMsg, message & 63u) ^ blob_at<uint32_t>(v, kUnrankGolayMsg, 64 + (message >> 6));
-    uint32_t r = (uint32_t)(r47 >> 12), T = d.perm_a, set = d.a, word = 0;
-    uint32_t begin, orderings;
+    uint32_t r = (uint32_t)(r47 >> 12), set = d.a, word = 0;
 #ifdef __CUDA_ARCH__
 #pragma unroll 1
 #endif
     for (int i = 0; i < kPairSteps; i++) {
         const PairStep e = blob_at<PairStep>(v, kUnrankPairs, i);
-        uint32_t at = (uint32_t)quotient((float)r * (float)e.draws, (float)T);
+        uint32_t at = floor_product((float)r, blob_at<float>(v, kUnrankRatios, 256 * i + set));
         at = at < e.draws ? at : e.draws - 1u;
-        uint64_t pair;
-        // 49 pairs at most: whatever the table holds, the loop ends
+        const uint64_t *entry = v.pairs + (e.first + set * e.draws + at);
+        uint64_t pair = *entry;
+        // position 0 begins with rank 0, so this ends; after one step, at that
 #ifdef __CUDA_ARCH__
 #pragma unroll 1
 #endif
-        for (int tries = 0;; tries++) {
-            pair = v.pairs[e.first + set * e.draws + at];
-            const uint32_t first = (uint32_t)pair & 0xffffu, n = (uint32_t)pair >> 16;
-            begin = (uint32_t)(((uint64_t)T * first) >> e.shift) * e.inverse;
-            orderings = (uint32_t)(((uint64_t)T * n) >> e.shift) * e.inverse;
-            if (r - begin < orderings || tries == 49) break;       // r below begin wraps around
-            at = r < begin ? first - 1u : first + n;
-            at = at < e.draws ? at : e.draws - 1u;
-        }
-        r -= begin;
-        T = orderings;
+        while (r < (uint32_t)pair) pair = *--entry;
+        r -= (uint32_t)pair;
         word = word >> 8 | (uint32_t)(pair >> 32) << 24;
         set = (uint32_t)(pair >> 40);
         if (i == kPairSteps / 2 - 1) p.mag[0] = word;
     }
     p.mag[1] = word;
-    p.mag[2] = v.tail8[blob_at<uint16_t>(v, kUnrankTailBase, set & 255u) + r];
+    p.mag[2] = v.tail8[blob_at<uint16_t>(v, kUnrankTailBase, set) + r];
     // x_i = 1 + 2 c_i modulo 4: 1 + 2j is of the wrong residue, and so negated, where j's parity differs from c_i
 #pragma unroll
     for (int w = 0; w < 3; w++) p.neg[w] = (p.mag[w] & 0x11111111u) ^ spread8(cw >> (8 * w));
-}
-
-// Deals the low bits of `bits` to the nibbles of `word` that are not zero (two-bit values), in order; drops them from
-// `bits`.
-LLVQ_HD uint32_t deal_signs(const UnrankView &v, uint32_t word, uint32_t &bits) {
-    const uint32_t mask = gather8((word | word >> 1) & 0x11111111u);
-    const int n = popcount32(mask);
-    const uint32_t dealt = blob_at<uint32_t>(v, kUnrankDeposit, blob_at<uint16_t>(v, kUnrankDepositAt, mask) + (bits & ((1u << n) - 1u)));
-    bits >>= n;
-    return dealt;
 }
 
 // The low nibbles of `word`, as many as `mask` has bits, moved to the mask's places.
@@ -172,6 +154,16 @@ LLVQ_HD uint32_t to_places(const UnrankView &v, uint32_t mask, uint32_t word) {
     word = (word & ~m.m1) | ((word << 8) & m.m1);
     word = (word & ~m.m2) | ((word << 4) & m.m2);
     return word & m.all;
+}
+
+// Deals the low bits of `bits` to the nibbles of `word` that are not zero (two-bit values), in order; drops them from
+// `bits`.
+LLVQ_HD uint32_t deal_signs(const UnrankView &v, uint32_t word, uint32_t &bits) {
+    const uint32_t mask = gather8((word | word >> 1) & 0x11111111u);
+    const int n = popcount32(mask);
+    const uint32_t dealt = to_places(v, mask, spread8(bits & ((1u << n) - 1u)));
+    bits >>= n;
+    return dealt;
 }
 
 // quotient and remainder of r / d for r < 2^42, quotient < 2^21, d < 2^24, given 1 / d: the float estimate is off by one at

@@ -18,7 +18,7 @@ namespace llvq {
 
 // One class, as the un-ranking reads it.  32 bytes.
 struct UnrankDesc {
-    uint32_t perm_a;      // odd: orderings of the 24 magnitudes; even: orderings of the support
+    uint32_t perm_a;      // odd: orderings of the 24 magnitudes (the un-ranking has no use for it); even: orderings of the support
     uint32_t perm_b;      // even: orderings off the support
     uint32_t a;           // even: first entry of the support's orderings; odd: the multiset's number
     uint32_t b;           // even, w = 8, 12, 16: first entry in tab_b; w = 0: copies of 0, 4, 8, 12 a byte each
@@ -35,12 +35,14 @@ struct UnrankStep {
 
 // Two odd magnitudes at a time: with L coordinates left that have T orderings, T n / (L (L - 1)) begin with a given pair of
 // values, n the ways to draw the pair.  So the rank times L (L - 1) / T is a position among the L (L - 1) draws in order, and
-// the table `pairs` tells for every multiset and position the pair, the positions it takes and the multiset left.
+// the table `pairs` tells for every multiset and position the first rank that begins with the pair drawn there, the pair and the
+// multiset left.  The multiset tells T, so the ratio is a table's, too, kept a little larger than it is: the position that comes of it
+// in f32 is the one wanted or the next (the product's and the factors' roundings are below 2^-22 of it, and it is below 2^10).
 struct PairStep {
-    uint32_t inverse, shift;   // division by L (L - 1)
     uint32_t first;            // of this L's entries in `pairs`
     uint32_t draws;            // L (L - 1)
 };
+constexpr double kRatioExcess = 1.0 + 1.0 / (1 << 20);
 constexpr int kPairSteps = 8;                                         // L = 24, 22, .. 10
 constexpr int kOddSets = 225;                                         // multisets of non-zero j with sum j (j + 1) / 2 <= 21
 
@@ -57,13 +59,12 @@ constexpr int kUnrankDescs = kUnrankBase + kUnrankClasses * 8;        // UnrankD
 constexpr int kUnrankMerge = kUnrankDescs + kUnrankClasses * 32;      // uint4[256]: moves that spread nibbles to a byte mask's places
 constexpr int kUnrankSteps = kUnrankMerge + 256 * 16;                 // UnrankStep[32], by the number of coordinates left
 constexpr int kUnrankPairs = kUnrankSteps + 32 * 8;                   // PairStep[8]
-constexpr int kUnrankWindow = kUnrankPairs + kPairSteps * 16;         // uint32[kGuideSlots / 32]: bit = a slot with a class that is not kWindowAlways
+constexpr int kUnrankRatios = kUnrankPairs + kPairSteps * 8;          // float[8][256]: draws / orderings of a step and multiset
+constexpr int kUnrankWindow = kUnrankRatios + kPairSteps * 256 * 4;   // uint32[kGuideSlots / 32]: bit = a slot with a class that is not kWindowAlways
 constexpr int kUnrankGuide = kUnrankWindow + kGuideSlots / 8;         // uint16[kGuideSlots + 8]: first class of a slot
 constexpr int kUnrankGolayMsg = kUnrankGuide + (kGuideSlots + 8) * 2; // uint32[128]: codewords of the messages k and, from 64 on, 64 k, k < 64
 constexpr int kUnrankTailBase = kUnrankGolayMsg + 128 * 4;            // uint16[256]: first entry in tail8 of a multiset of eight odd magnitudes
-constexpr int kUnrankDepositAt = kUnrankTailBase + 256 * 2;      // uint16[256]: first entry in the deposit table of a byte mask
-constexpr int kUnrankDeposit = kUnrankDepositAt + 256 * 2;            // uint32[6561 + 15]: bits dealt to a mask's places, a nibble each
-constexpr int kUnrankRest12 = kUnrankDeposit + 6576 * 4;              // uint32[128]: first entry in tab_b of 12 off-support values
+constexpr int kUnrankRest12 = kUnrankTailBase + 256 * 2;              // uint32[128]: first entry in tab_b of 12 off-support values
 constexpr int kUnrankSharedBytes = kUnrankRest12 + 128 * 4;           // what follows stays in global memory
 constexpr int kUnrankSupport = kUnrankSharedBytes;                    // uint32[kSupports]: 8, 12 or 16 support values' k, two bits each
 constexpr int kSupports = 4192;
@@ -71,12 +72,12 @@ constexpr int kUnrankSupport24 = kUnrankSupport + kSupports * 4;      // uint64[
 constexpr int kSupports24 = 2352;
 constexpr int kUnrankGolayWt = kUnrankSupport24 + kSupports24 * 8;
 constexpr int kUnrankBlobBytes = kUnrankGolayWt + 4096 * 4;
-static_assert(kUnrankDescs % 16 == 0 && kUnrankPairs % 16 == 0 && kUnrankWindow % 16 == 0 && kUnrankMerge % 16 == 0 && kUnrankGuide % 16 == 0 && kUnrankGolayMsg % 16 == 0 &&
-              kUnrankTailBase % 16 == 0 && kUnrankDeposit % 16 == 0 && kUnrankSupport24 % 16 == 0 && kUnrankBlobBytes % 16 == 0, "alignment of the blob's parts");
+static_assert(kUnrankDescs % 16 == 0 && kUnrankPairs % 16 == 0 && kUnrankRatios % 16 == 0 && kUnrankWindow % 16 == 0 && kUnrankMerge % 16 == 0 && kUnrankGuide % 16 == 0 && kUnrankGolayMsg % 16 == 0 &&
+              kUnrankTailBase % 16 == 0 && kUnrankSupport24 % 16 == 0 && kUnrankBlobBytes % 16 == 0, "alignment of the blob's parts");
 
 struct UnrankTables {
     std::vector<uint8_t> blob;       // kUnrankBlobBytes
-    std::vector<uint64_t> pairs;     // first position | positions << 16 | pair << 32 (a nibble a value) | multiset left << 40
+    std::vector<uint64_t> pairs;     // first rank | pair << 32 (a nibble a value) | multiset left << 40
     std::vector<uint32_t> tail8;     // eight magnitudes' j, a nibble each, first coordinate lowest
     std::vector<uint32_t> tab_b;     // 8, 12 or 16 off-support values' k, two bits each
 };
