@@ -8,12 +8,12 @@
 // their place; the codes wait in shared memory until the tile's words are gathered from them.  The small look-up tables
 // are copied to shared memory once a CTA, while the previous kernel of the stream ends; one CTA a multiprocessor walks over
 // the tiles.
-// Measured (9728 x 2560 into the 14-byte layout, 1.04 M blocks): 36.2 us, 2500 warp instructions a tile of 128 blocks, issue
-// slots 50 % busy, the load unit's wavefronts 64 %, half of all stalls waits on the lists (33 % of their sectors come from the
-// L1 cache); a lane a row with a 64-bit division a coordinate and candidate took 484 us, one odd coordinate at a time 45.
-// Counting and expanding 17408 x 5120 into the 10-byte layout: 184 us against 4700.  24 or 28 warps a CTA instead of 32: 47 and
-// 50 us.  The shared tables are kept to 33 KB because the rest of a multiprocessor's memory is the L1 cache that the lists
-// are read through: with 51 KB 38 us, with 104 KB 53.
+// Measured (9728 x 2560 into the 14-byte layout, 1.04 M blocks): 35.2 us; 17408 x 5120 106 us, counted and expanded into the
+// 10-byte layout 171.  A lane a row with a 64-bit division a coordinate and candidate took 484 and 4700 (10-byte layout) us, one odd
+// coordinate at a time 45.  24 or 28 warps a CTA instead of 32: 47 and 50 us against 38.  A multiprocessor's memory that is not shared is the
+// L1 cache the lists are read through, so the shared tables are kept to 20 KB and a warp's scratch to 2 KB (with 51 and 3.6 KB
+// 33 % of the lists' sectors come from the cache, and 38 % now; with 104 KB of tables 53 us).  The gathers were 85 % of the
+// load unit's time: the parts of a class stand in tables of their own, where 32-byte records lay in one of four banks.
 #include "llvq_internal.cuh"
 #include "llvq_unrank.cuh"
 
@@ -22,13 +22,15 @@ namespace {
 
 constexpr int kExpandWarps = 32;
 constexpr int kExpandThreads = kExpandWarps * 32;
-// a row of 32 words of the tile under construction: 40 apart, so that the two words of a block the four lanes of a quad read
-// lie eight banks apart
-constexpr int kNatStride = 40;
+// A tile under construction.  Until a block is un-ranked, its first two words of codes hold the rank in its class (47 bits),
+// the class << 47 and the gain << 56, the third the class's flags.
 struct WarpScratch {
-    uint64_t list[128];                    // rank in class | class << 47 | gain << 56 | place << 57: odd type from the front, even from the back
-    uint32_t nat[4][4][kNatStride];        // [block of the piece][codes of eight coordinates: 0..2, header: 3][row]
+    uint32_t nat[4][3][32];                // [block of the piece][codes of eight coordinates][row, see `cell`]
+    uint16_t hdr[4][32];                   // its header
     uint32_t exceptions[4];                // 10-byte layout: rows of a block without a window
+    uint8_t place[128];                    // 32 * block + row: odd type from the front, even from the back
+    // neighbouring words' rows lie eight banks apart: the four lanes of a quad read two words of a block, or of two
+    __device__ __forceinline__ uint32_t &cell(int q, int j, int row) { return nat[q][j][row ^ ((q + j) & 1) << 3]; }
 };
 constexpr int kExpandSmem = kUnrankSharedBytes + kExpandWarps * (int)sizeof(WarpScratch);
 
@@ -159,22 +161,26 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
             if (!(now_own >> q & 1u)) continue;
             const bool valid = row_exists && code_names_point(code[q], num_points);
             bool odd = false;
-            uint64_t entry = 0;
             if (valid) {
                 const uint64_t idx = code[q] & ((1ull << kIndexBits) - 1);
                 const int c = find_class(v, idx);
-                odd = blob_at<UnrankDesc>(v, kUnrankDescs, c).flags & 1u;
-                entry = (idx - blob_at<uint64_t>(v, kUnrankBase, c)) | (uint64_t)c << 47 | ((code[q] >> kIndexBits) & 1) << 56 | (uint64_t)(32 * q + lane) << 57;
+                const uint32_t flags = blob_at<uint32_t>(v, kUnrankFlags, c);
+                odd = flags & 1u;
+                const uint64_t entry = (idx - blob_at<uint64_t>(v, kUnrankBase, c)) | (uint64_t)c << 47 | ((code[q] >> kIndexBits) & 1) << 56;
+                n.cell(q, 0, lane) = (uint32_t)entry;
+                n.cell(q, 1, lane) = (uint32_t)(entry >> 32);
+                n.cell(q, 2, lane) = flags;
             } else {
                 bad += row_exists;
                 // the empty record
                 const uint32_t zero_code = OVERLAY && is_tile ? 0u : 0x88888888u;
-                n.nat[q][0][lane] = zero_code; n.nat[q][1][lane] = zero_code; n.nat[q][2][lane] = zero_code;
-                n.nat[q][3][lane] = COMPACT ? 0u : (uint32_t)kEmptyClass;
+#pragma unroll
+                for (int j = 0; j < 3; j++) n.cell(q, j, lane) = zero_code;
+                n.hdr[q][lane] = COMPACT ? 0u : (uint16_t)kEmptyClass;
             }
             const uint32_t of_odd = __ballot_sync(0xffffffffu, valid && odd), of_even = __ballot_sync(0xffffffffu, valid && !odd);
             const uint32_t before = (1u << lane) - 1u;
-            if (valid) s.list[odd ? n_odd + __popc(of_odd & before) : 127 - n_even - __popc(of_even & before)] = entry;
+            if (valid) s.place[odd ? n_odd + __popc(of_odd & before) : 127 - n_even - __popc(of_even & before)] = (uint8_t)(32 * q + lane);
             n_odd += __popc(of_odd);
             n_even += __popc(of_even);
         }
@@ -182,8 +188,8 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
         next_piece();
 
         // ---- un-rank: 32 blocks of a type at a time
-        auto finish = [&](uint64_t entry, const UnrankDesc &d, const Point &p, bool odd) {
-            const uint32_t place = (uint32_t)(entry >> 57), q = place >> 5, row = place & 31u;
+        auto finish = [&](uint32_t place, uint64_t entry, const UnrankDesc &d, const Point &p, bool odd) {
+            const uint32_t q = place >> 5, row = place & 31u;
             const uint32_t cls = (uint32_t)(entry >> 47) & 511u, gain = (uint32_t)(entry >> 56) & 1u;
             uint32_t cw[3];
 #pragma unroll
@@ -203,24 +209,33 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
                     atomicOr(&n.exceptions[q], 1u << row);
                 }
             }
-            n.nat[q][0][row] = cw[0]; n.nat[q][1][row] = cw[1]; n.nat[q][2][row] = cw[2];
-            n.nat[q][3][row] = hdr;
+#pragma unroll
+            for (int j = 0; j < 3; j++) n.cell(q, j, row) = cw[j];
+            n.hdr[q][row] = (uint16_t)hdr;
         };
+        auto waiting = [&](uint32_t place) -> uint64_t { return n.cell(place >> 5, 0, place & 31u) | (uint64_t)n.cell(place >> 5, 1, place & 31u) << 32; };
 #pragma unroll 1
         for (int i = lane; i < n_odd; i += 32) {
-            const uint64_t entry = s.list[i];
-            const UnrankDesc d = blob_at<UnrankDesc>(v, kUnrankDescs, (uint32_t)(entry >> 47) & 511u);
+            const uint32_t place = s.place[i];
+            const uint64_t entry = waiting(place);
+            UnrankDesc d;                                          // nothing else of it is read
+            d.flags = n.cell(place >> 5, 2, place & 31u);
             Point p;
             unrank_odd(v, d, entry & ((1ull << 47) - 1), p);
-            finish(entry, d, p, true);
+            finish(place, entry, d, p, true);
         }
 #pragma unroll 1
         for (int i = lane; i < n_even; i += 32) {
-            const uint64_t entry = s.list[127 - i];
-            const UnrankDesc d = blob_at<UnrankDesc>(v, kUnrankDescs, (uint32_t)(entry >> 47) & 511u);
+            const uint32_t place = s.place[127 - i];
+            const uint64_t entry = waiting(place);
+            const uint32_t cls = (uint32_t)(entry >> 47) & 511u;
+            const UnrankPerms perms = blob_at<UnrankPerms>(v, kUnrankPerms, cls);
+            const UnrankFirsts firsts = blob_at<UnrankFirsts>(v, kUnrankFirsts, cls);
+            const UnrankDesc d = {n.cell(place >> 5, 2, place & 31u), perms.perm_a, perms.perm_b, perms.inv_a, perms.inv_b,
+                                  firsts.a_golay & 0xffffu, firsts.b, firsts.a_golay >> 16};
             Point p;
             unrank_even(v, d, entry & ((1ull << 47) - 1), p);
-            finish(entry, d, p, false);
+            finish(place, entry, d, p, false);
         }
         meet();
         if (part) break;                                           // a shared piece is the last
@@ -232,8 +247,9 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
                 if ((rows_out >> lane) & 1u) {
                     const uint32_t at = next_entry + __popc(rows_out & ((1u << lane) - 1u));
                     if (at < capacity)
-                        table[at] = make_uint4(n.nat[q][3][lane] | (uint32_t)lane << 8 | (u * kTileCells + q) << 13, n.nat[q][0][lane], n.nat[q][1][lane], n.nat[q][2][lane]);
-                    n.nat[q][0][lane] = n.nat[q][1][lane] = n.nat[q][2][lane] = n.nat[q][3][lane] = 0u;
+                        table[at] = make_uint4(n.hdr[q][lane] | (uint32_t)lane << 8 | (u * kTileCells + q) << 13, n.cell(q, 0, lane), n.cell(q, 1, lane), n.cell(q, 2, lane));
+                    n.cell(q, 0, lane) = n.cell(q, 1, lane) = n.cell(q, 2, lane) = 0u;
+                    n.hdr[q][lane] = 0;
                 }
                 next_entry += __popc(rows_out);
             }
@@ -246,11 +262,11 @@ expand_planes_kernel(UnrankView global, uint64_t num_points, const uint64_t *__r
         auto codes_at = [&](int q0, int m, int e, int kappa0) -> uint32_t {
             const int slot = kappa0 / 24, i0 = kappa0 % 24;
             const int r = single ? 16 * slot + 8 * e + g : 16 * m + 8 * e + g;
-            return n.nat[single ? q0 : q0 + slot][i0 >> 3][r];
+            return n.cell(single ? q0 : q0 + slot, i0 >> 3, r);
         };
         auto header = [&](int q0, int m, int e, int slot) -> uint32_t {
             const int r = single ? 16 * slot + 8 * e + g : 16 * m + 8 * e + g;
-            return n.nat[single ? q0 : q0 + slot][3][r];
+            return n.hdr[single ? q0 : q0 + slot][r];
         };
         const uint32_t half_sel = (t & 1) ? 0x7362u : 0x5140u;
         // the lane's four nibbles of x to the low nibbles of four bytes, those of y to the high nibbles
@@ -352,7 +368,7 @@ expand_onehot_kernel(UnrankView global, DeviceTables T, const uint64_t *__restri
             if (code_names_point(code, T.num_points)) {
                 cls = (uint32_t)find_class(v, idx);
                 gain = (uint32_t)(code >> kIndexBits) & 1u;
-                const UnrankDesc d = blob_at<UnrankDesc>(v, kUnrankDescs, cls);
+                const UnrankDesc d = far_at<UnrankDesc>(v, kUnrankDescs, cls);
                 const uint32_t odd = d.flags & 1u;
                 Point p;
                 unrank(v, d, idx - blob_at<uint64_t>(v, kUnrankBase, cls), p);

@@ -91,7 +91,7 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
             less[k][v] = v == 0 ? k : (c[v] ? (c[v]--, set_of[c]) : -1);
         }
     // every ordering of eight
-    uint16_t *tail_first = part<uint16_t>(u.blob, kUnrankTailBase);
+    std::vector<uint32_t> tail_first(sets.size(), 0);
     for (int k = 0; k < kOddSets; k++) {
         const int n = copies_in(sets[k]);
         if (n > 8) continue;
@@ -99,36 +99,56 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
         for (int v = 1; v < 7; v++) c[v] = sets[k][v];
         c[0] = 8 - n;
         if (u.tail8.size() > 0xffff) return false;
-        tail_first[k] = (uint16_t)u.tail8.size();
+        tail_first[k] = (uint32_t)u.tail8.size();
         list_orderings<7, 4>(c, 8, 0, 0, u.tail8);
     }
     // the draws of two from L
-    PairStep *pair_steps = part<PairStep>(u.blob, kUnrankPairs);
-    float *ratios = part<float>(u.blob, kUnrankRatios);
+    // L! / (the copies' factorials): L over the copies of each value in turn, whole numbers all along
+    auto orderings_of = [&](int k, int L) {
+        uint64_t n = 1;
+        for (int v = 1, left = L; v < 7; v++)
+            for (int j = 1; j <= sets[k][v]; j++) n = n * (uint64_t)left-- / (uint64_t)j;
+        return n;
+    };
+    auto ratio_bits = [&](int k, int L) {                // as a float's bits
+        const float f = (float)(L * (L - 1) / (double)orderings_of(k, L) * kRatioExcess);
+        uint32_t bits;
+        std::memcpy(&bits, &f, 4);
+        return bits;
+    };
+    uint32_t *first_ratio = part<uint32_t>(u.blob, kUnrankRatio);
     size_t entries = 0;
     for (int i = 0; i < kPairSteps; i++) entries += (size_t)kOddSets * (24 - 2 * i) * (23 - 2 * i);
     u.pairs.reserve(entries);
     for (int i = 0; i < kPairSteps; i++) {
         const int L = 24 - 2 * i, draws = L * (L - 1);
-        pair_steps[i] = {(uint32_t)u.pairs.size(), (uint32_t)draws};
-        u.pairs.resize(u.pairs.size() + (size_t)kOddSets * draws, 0);
+        const size_t first = u.pairs.size();
+        u.pairs.resize(first + (size_t)kOddSets * draws, 0);
         for (int k = 0; k < kOddSets; k++) {
             const std::array<int, 7> &c = sets[k];
             const int n = copies_in(c);
             if (n > L) continue;
-            uint64_t *entry = u.pairs.data() + pair_steps[i].first + (size_t)k * draws;
-            // L! / (the copies' factorials): L over the copies of each value in turn, whole numbers all along
-            uint64_t orderings = 1;
-            for (int v = 1, left = L; v < 7; v++)
-                for (int j = 1; j <= c[v]; j++) orderings = orderings * (uint64_t)left-- / (uint64_t)j;
+            uint64_t *entry = u.pairs.data() + first + (size_t)k * draws;
+            const uint64_t orderings = orderings_of(k, L);
             if (orderings >= 0x80000000ull) return false;
-            ratios[256 * i + k] = (float)(draws / (double)orderings * kRatioExcess);
+            if (i == 0) first_ratio[k] = ratio_bits(k, L);
             int at = 0;
             for (int va = 0; va < 7; va++)
                 for (int vb = 0; vb < 7; vb++) {
                     const int na = va ? c[va] : L - n, nb = (vb ? c[vb] : L - n) - (va == vb);
                     if (na < 1 || nb < 1) continue;
-                    const uint64_t e = orderings * (uint64_t)at / (uint64_t)draws | (uint64_t)(va | vb << 4) << 32 | (uint64_t)less[less[k][va]][vb] << 40;
+                    const int left = less[less[k][va]][vb];
+                    uint32_t high = (uint32_t)left | (uint32_t)(va | vb << 4) << 8;
+                    if (i == kPairSteps - 1) {
+                        high |= tail_first[left] << 16;
+                    } else {
+                        const uint32_t wanted = ratio_bits(left, L - 2), below = high >> 4;
+                        uint32_t bits = (wanted & ~0xfffu) | below;
+                        if (bits < wanted) bits += 0x1000u;
+                        if (bits - kRatioBase >= 1u << 28) return false;
+                        high |= (bits - kRatioBase - below) << 4;
+                    }
+                    const uint64_t e = orderings * (uint64_t)at / (uint64_t)draws | (uint64_t)high << 32;
                     for (int j = 0; j < na * nb; j++) entry[at + j] = e;
                     at += na * nb;
                 }
@@ -174,20 +194,20 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
         const ClassDesc &d = t.desc[(size_t)c];
         UnrankDesc &e = desc[c];
         if (d.perm_a >= 0x80000000ull || d.perm_b > 0x1000000ull) return false;
-        e.perm_a = (uint32_t)d.perm_a;
-        e.perm_b = (uint32_t)d.perm_b;
-        e.inv_a = 1.0f / (float)d.perm_a;
-        e.inv_b = 1.0f / (float)d.perm_b;
-        e.flags = (uint32_t)d.odd | (uint32_t)d.w << 1 | (uint32_t)d.sign_bits << 6 | (uint32_t)d.nz_b << 11 | (uint32_t)d.shell << 16 |
-                  (uint32_t)window_of(d) << 20;
+        e.flags = (uint32_t)d.shell << 16 | (uint32_t)window_of(d) << 20;
         if (d.odd) {
             std::array<int, 7> c{};
             for (int v = 1; v < 7; v++) c[v] = d.cnt[v];
             const auto k = set_of.find(c);
             if (k == set_of.end()) return false;
-            e.a = (uint32_t)k->second;
+            e.flags |= 1u | (uint32_t)k->second << 1;
             continue;
         }
+        e.flags |= (uint32_t)d.w << 1 | (uint32_t)d.sign_bits << 6 | (uint32_t)d.nz_b << 11;
+        e.perm_a = (uint32_t)d.perm_a;
+        e.perm_b = (uint32_t)d.perm_b;
+        e.inv_a = 1.0f / (float)d.perm_a;
+        e.inv_b = 1.0f / (float)d.perm_b;
         e.golay = (uint32_t)t.weight_offset[d.w];
         int half_sum = 0;                                // sum |x| / 2
         for (int k = 0; k < 4; k++) half_sum += d.cnt[k] * (1 + 2 * k) + d.cnt[4 + k] * 2 * k;
@@ -205,6 +225,16 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
             if (b == first_b.end()) return false;
             e.b = b->second;
         }
+    }
+    uint32_t *flags = part<uint32_t>(u.blob, kUnrankFlags);
+    UnrankPerms *perms = part<UnrankPerms>(u.blob, kUnrankPerms);
+    UnrankFirsts *firsts = part<UnrankFirsts>(u.blob, kUnrankFirsts);
+    for (int c = 0; c < t.num_classes; c++) {
+        const UnrankDesc &e = desc[c];
+        if (e.a >= 0x10000u || e.golay >= 0x10000u) return false;
+        flags[c] = e.flags;
+        perms[c] = {e.perm_a, e.perm_b, e.inv_a, e.inv_b};
+        firsts[c] = {e.a | e.golay << 16, e.b};
     }
     // ---- guide: class of the smallest index of every slot (a slot's indices share exponent and leading mantissa bits
     // of their value rounded to float; rounding is monotonic, so slots are ranges of indices)
@@ -232,25 +262,15 @@ bool build_unrank_tables(const HostTables &t, UnrankTables &u) {
     for (int k = 0; k < 64; k++) { message[k] = t.golay_by_message[k]; message[64 + k] = t.golay_by_message[64 * k]; }
     std::memcpy(u.blob.data() + kUnrankGolayWt, t.golay_by_weight.data(), 4096 * 4);
 
-    // ---- spreading eight nibbles to the places of a byte mask
-    struct Moves { uint32_t m[4]; };
-    Moves *merge = part<Moves>(u.blob, kUnrankMerge);
+    // ---- eight nibbles, as many as a byte mask has bits for its places in order and then the others for the others: where
+    // the bytes of the even places come from, and those of the odd places (nibble r is byte r / 2 of the even or the odd nibbles)
+    uint32_t *merge = part<uint32_t>(u.blob, kUnrankMerge);
     for (int mask = 0; mask < 256; mask++) {
-        // the nibble of rank r must travel place[r] - r places up; in steps of 4, 2, 1 (each step's targets are
-        // distinct, because ranks travel by non-decreasing distances)
-        int place[8], k = 0;
-        for (int i = 0; i < 8; i++) if ((mask >> i) & 1) place[k++] = i;
-        Moves mv = {{0, 0, 0, 0}};
-        for (int r = 0; r < k; r++) {
-            int pos = r;
-            for (int step = 2; step >= 0; step--)
-                if (((place[r] - r) >> step) & 1) {
-                    pos += 1 << step;
-                    mv.m[2 - step] |= 15u << (4 * pos);
-                }
-            mv.m[3] |= 15u << (4 * place[r]);
+        uint32_t in = 0, out = (uint32_t)__builtin_popcount((unsigned)mask);
+        for (int i = 0; i < 8; i++) {
+            const uint32_t r = (mask >> i & 1) ? in++ : out++;
+            merge[mask] |= ((r >> 1) | (r & 1u) << 2) << (4 * (i >> 1) + 16 * (i & 1));
         }
-        merge[mask] = mv;
     }
     return true;
 }

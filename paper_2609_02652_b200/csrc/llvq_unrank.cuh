@@ -46,6 +46,26 @@ LLVQ_HD int popcount32(uint32_t v) {
     return __builtin_popcount(v);
 #endif
 }
+LLVQ_HD uint32_t byte_perm(uint32_t a, uint32_t b, uint32_t select) {
+#ifdef __CUDA_ARCH__
+    return __byte_perm(a, b, select);
+#else
+    uint32_t r = 0;
+    for (int i = 0; i < 32; i += 8) {
+        const uint32_t from = select >> (i / 2) & 7u;
+        r |= ((from < 4u ? a >> (8u * from) : b >> (8u * (from - 4u))) & 0xffu) << i;
+    }
+    return r;
+#endif
+}
+// the low `bits` bits of `low`, and above them the low ones of `high`
+LLVQ_HD uint32_t join(uint32_t low, uint32_t high, uint32_t bits) {
+#ifdef __CUDA_ARCH__
+    return __funnelshift_rc(__funnelshift_lc(0u, low, 32u - bits), high, 32u - bits);
+#else
+    return (uint32_t)((low & ((1ull << bits) - 1)) | (uint64_t)high << bits);
+#endif
+}
 LLVQ_HD float u64_to_float(uint64_t v) { return (float)v; }
 LLVQ_HD uint32_t float_bits(float f) {
 #ifdef __CUDA_ARCH__
@@ -54,6 +74,15 @@ LLVQ_HD uint32_t float_bits(float f) {
     union { float f; uint32_t u; } c;
     c.f = f;
     return c.u;
+#endif
+}
+LLVQ_HD float bits_float(uint32_t u) {
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(u);
+#else
+    union { uint32_t u; float f; } c;
+    c.u = u;
+    return c.f;
 #endif
 }
 // floor(a * b), a * b below 2^23
@@ -112,22 +141,23 @@ LLVQ_HD uint32_t portion(uint32_t T, uint32_t copies, const UnrankStep &e) { ret
 
 // Odd type.  Sixteen coordinates come two at a time from the table of draws, the ordering of the last eight is an entry of
 // a list.  The position of the draw is a float estimate that is right or one too large, which the first rank of the pair it names
-// tells.  Rolled up: eight steps' code would crowd the instruction cache.  The gathers and their cache bound this: with the bounds
-// of a pair worked out from the number of orderings (four multiplications to 64 bits and a reciprocal a step) instead of the
-// 8 KB of ratios, 9728 x 2560 takes 39 us instead of 36, and so it does with the ratios beside a table of dealt signs of
-// 26 KB; with the second eight coordinates one at a time from lists in shared memory 46.
+// tells.  Rolled up: eight steps' code would crowd the instruction cache.  The load unit and its latency bound this, so a step
+// reads one table only, at random (9728 x 2560: 35.2 us, 17408 x 5120: 106).  With the ratios in a table of their own in shared memory
+// it takes 36.2 and 112, with the bounds of a pair worked out from the number of orderings (four multiplications to 64 bits and a
+// reciprocal a step) 39 and 125, with the second eight coordinates one at a time from lists in shared memory 46.
 LLVQ_HD void unrank_odd(const UnrankView &v, const UnrankDesc &d, uint64_t r47, Point &p) {
     const uint32_t message = (uint32_t)r47 & 4095u;
     const uint32_t cw = blob_at<uint32_t>(v, kUnrankGolayMsg, message & 63u) ^ blob_at<uint32_t>(v, kUnrankGolayMsg, 64 + (message >> 6));
-    uint32_t r = (uint32_t)(r47 >> 12), set = d.a, word = 0;
+    uint32_t r = (uint32_t)(r47 >> 12), set = (d.flags >> 1) & 255u, word = 0, left = 24, first = 0, high;
+    float ratio = blob_at<float>(v, kUnrankRatio, set);
 #ifdef __CUDA_ARCH__
 #pragma unroll 1
 #endif
-    for (int i = 0; i < kPairSteps; i++) {
-        const PairStep e = blob_at<PairStep>(v, kUnrankPairs, i);
-        uint32_t at = floor_product((float)r, blob_at<float>(v, kUnrankRatios, 256 * i + set));
-        at = at < e.draws ? at : e.draws - 1u;
-        const uint64_t *entry = v.pairs + (e.first + set * e.draws + at);
+    while (true) {
+        const uint32_t draws = left * (left - 1u);
+        uint32_t at = floor_product((float)r, ratio);
+        at = at < draws ? at : draws - 1u;
+        const uint64_t *entry = v.pairs + (first + set * draws + at);
         uint64_t pair = *entry;
         // position 0 begins with rank 0, so this ends; after one step, at that
 #ifdef __CUDA_ARCH__
@@ -135,25 +165,28 @@ LLVQ_HD void unrank_odd(const UnrankView &v, const UnrankDesc &d, uint64_t r47, 
 #endif
         while (r < (uint32_t)pair) pair = *--entry;
         r -= (uint32_t)pair;
-        word = word >> 8 | (uint32_t)(pair >> 32) << 24;
-        set = (uint32_t)(pair >> 40);
-        if (i == kPairSteps / 2 - 1) p.mag[0] = word;
+        high = (uint32_t)(pair >> 32);
+        word = byte_perm(word, high, 0x5321u);
+        left -= 2u;
+        if (left == 8u) break;
+        first += kOddSets * draws;
+        set = high & 255u;
+        ratio = bits_float((high >> 4) + kRatioBase);
+        if (left == 16u) p.mag[0] = word;
     }
     p.mag[1] = word;
-    p.mag[2] = v.tail8[blob_at<uint16_t>(v, kUnrankTailBase, set) + r];
+    p.mag[2] = v.tail8[(high >> 16) + r];
     // x_i = 1 + 2 c_i modulo 4: 1 + 2j is of the wrong residue, and so negated, where j's parity differs from c_i
 #pragma unroll
     for (int w = 0; w < 3; w++) p.neg[w] = (p.mag[w] & 0x11111111u) ^ spread8(cw >> (8 * w));
 }
 
-// The low nibbles of `word`, as many as `mask` has bits, moved to the mask's places.
+// The nibbles of `word`: as many as `mask` has bits to the mask's places, in order, the others to the other places.  One selector
+// for two byte permutations: masked shifts by 4, 2 and 1 places read 16 bytes for the mask's nibbles and again for the others.
 LLVQ_HD uint32_t to_places(const UnrankView &v, uint32_t mask, uint32_t word) {
-    struct alignas(16) Moves { uint32_t m0, m1, m2, all; };
-    const Moves m = blob_at<Moves>(v, kUnrankMerge, mask);
-    word = (word & ~m.m0) | ((word << 16) & m.m0);
-    word = (word & ~m.m1) | ((word << 8) & m.m1);
-    word = (word & ~m.m2) | ((word << 4) & m.m2);
-    return word & m.all;
+    const uint32_t select = blob_at<uint32_t>(v, kUnrankMerge, mask);
+    const uint32_t even = word & 0x0f0f0f0fu, odd = (word >> 4) & 0x0f0f0f0fu;
+    return byte_perm(even, odd, select) | byte_perm(even, odd, select >> 16) << 4;
 }
 
 // Deals the low bits of `bits` to the nibbles of `word` that are not zero (two-bit values), in order; drops them from
@@ -237,7 +270,7 @@ LLVQ_HD void unrank_even(const UnrankView &v, const UnrankDesc &d, uint64_t r, P
 #pragma unroll
     for (int j = 0; j < 3; j++) {
         const uint32_t mask = (cw >> (8 * j)) & 255u, n = (uint32_t)popcount32(mask);
-        const uint32_t m = to_places(v, mask, (uint32_t)in) | to_places(v, mask ^ 255u, (uint32_t)out);
+        const uint32_t m = to_places(v, mask, join((uint32_t)in, (uint32_t)out, 4u * n));
         in >>= 4u * n;
         out >>= 32u - 4u * n;
         p.neg[j] = (m >> 2) & 0x11111111u;
