@@ -259,7 +259,7 @@ int llvq_gemv(llvq_ctx *ctx, int layout, const void *layout_buf, const void *row
  * over the records: x is fp16 [batch][k_padded], y is f32 [batch][rows].  The vectors share
  * one pass (the records are read and decoded once for them); five to eight take two passes where the
  * context's scratch holds the sums of four only, or on a device of few multiprocessors, whose shared memory may hold the
- * records of four only.  Each vector has its own fixed-point scale and its own accumulators, and y[j] is bit-identical to what
+ * records of four, or of two, only.  Each vector has its own fixed-point scale and its own accumulators, and y[j] is bit-identical to what
  * llvq_gemv returns for x[j].  Needs min(batch, 4) times the scratch of llvq_gemv (LLVQ_ESIZE
  * otherwise). */
 int llvq_gemv_batch(llvq_ctx *ctx, const void *layout_buf, const void *row_scale, const float *gain,
