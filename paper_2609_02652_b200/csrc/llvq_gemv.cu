@@ -310,10 +310,10 @@ __device__ __forceinline__ void contract_half(const HalfA &h, const StepX &sx, f
 // and a block slot has an instruction sequence of its own: positions 0..23 of the half-step for slot 0, 24..47 for slot 1,
 // the other slot's positions zero in B.  Against one vector with block-diagonal B that is three instructions instead
 // of four for two vectors and two slots, and a row's sum lies in two lanes instead of four, so half the exchanges.
-// The price is that a lane looks up the headers of both slots; every vector shares that.  Bound: latency (4096 x 4096: issue slots
-// 46 % busy with four vectors, 32 % with eight, whose three warps a scheduler also wait for instructions; tensor pipe 10 %).  Four
-// vectors, us a launch, before (a vector at a time, its atomic waited for before the next vector's) and after:
-// 1024 x 2560 6.8 and 5.5, 4096 x 4096 10.7 and 8.8, 8192 x 8192 19.4 and 17.8; two vectors on 8192 x 8192 12.5 and 11.9.
+// The price is that a lane looks up the headers of both slots; every vector shares that.  Two, five and six vectors go this way
+// (three, four, seven and eight: llvq_batch.cu).  Bound: latency (the build for eight on 4096 x 4096: issue slots
+// 32 % busy, three warps a scheduler that also wait for instructions; tensor pipe 10 %).  Two vectors on 8192 x 8192: 11.9 us a launch, 12.5 a vector at
+// a time, its atomic waited for before the next vector's.
 struct PairA {
     uint32_t a0, a1, a2, a3, c0, c1;
     float2 k00, k01, k10, k11;                     // block constants: slot, then row g or g + 8
@@ -447,7 +447,7 @@ __device__ __forceinline__ void each_pair(F &f) {
     }
 }
 
-// BATCH activation vectors share one pass over the records: the decode of a half-step and its block constants
+// BATCH (1, 2, or 8 for five and six) activation vectors share one pass over the records: the decode of a half-step and its block constants
 // are computed once, the contraction, the scaling and the reduction once a pair of vectors.  x is BATCH vectors of
 // 24 nb halves one after the other, y BATCH vectors of rows floats (p.prob[].y is vector 0's), the accumulators
 // BATCH sets of total_groups * 32.
