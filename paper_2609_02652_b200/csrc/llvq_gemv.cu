@@ -8,7 +8,7 @@
 // of a payload byte are split (an addition, a shift, two ANDs a word: the whole decode); B is block-diagonal, its eight
 // columns the four limbs of slot 0 and the four limbs of slot 1, so one accumulator tile holds, for 16 rows,
 // the two blocks' sums limb by limb.  Per (row, block) the limbs are recombined in integers, the offset term
-// (parity - 16) * sum_i 2 X_i is added from a per-block sum prepared with x (what is added up is twice sum_i x_i X_i: the
+// (parity - 16) * sum_i 2 X_i is added from a per-block sum prepared with x (what is added up is twice sum_i x_i X_i, in the 14-byte layout: the
 // halves of an odd sum need no care), and one float multiply-add applies half of gain[g] / (4 sqrt m), looked up by the header.  Every lane runs the same instructions whatever its class.
 //
 // Geometry.  A warp works on the 32 rows of a row group, 16 at a time; the records are stored as the
@@ -213,15 +213,18 @@ struct HalfA {
 // COMPACT (13-byte layout): the two headers are the bytes at bit SHIFT and SHIFT + 8 of hw.
 template <bool COMPACT = false, int SHIFT = 0>
 __device__ __forceinline__ HalfA decode_half(uint32_t wa, uint32_t wb, uint32_t wc, uint32_t hw, uint32_t tq) {
-    constexpr uint32_t kNib2 = 0x1e1e1e1eu;
     HalfA h;
-    h.a0 = twice(wa) & kNib2; h.a1 = twice(wb) & kNib2; h.a2 = (wa >> 3) & kNib2; h.a3 = (wb >> 3) & kNib2;
-    h.c0 = twice(wc) & kNib2; h.c1 = (wc >> 3) & kNib2;
     if (COMPACT) {
+        constexpr uint32_t kNib = 0x0f0f0f0fu;
+        h.a0 = wa & kNib; h.a1 = wb & kNib; h.a2 = (wa >> 4) & kNib; h.a3 = (wb >> 4) & kNib;
+        h.c0 = wc & kNib; h.c1 = (wc >> 4) & kNib;
         // one byte a header, eight bytes an entry
         h.k0 = lds_f2(and_or(SHIFT >= 3 ? hw >> (SHIFT - 3) : hw << (3 - SHIFT), 0x7f8u, tq));
         h.k1 = lds_f2(and_or(hw >> (SHIFT + 5), 0x7f8u, tq));
     } else {
+        constexpr uint32_t kNib2 = 0x1e1e1e1eu;
+        h.a0 = twice(wa) & kNib2; h.a1 = twice(wb) & kNib2; h.a2 = (wa >> 3) & kNib2; h.a3 = (wb >> 3) & kNib2;
+        h.c0 = twice(wc) & kNib2; h.c1 = (wc >> 3) & kNib2;
         // the headers of rows g (low half of hw) and g + 8 (high half), eight bytes an entry; tq is 8 KiB-aligned
         h.k0 = lds_f2(and_or(hw << 3, 0x1ff8u, tq));
         h.k1 = lds_f2(and_or(hw >> 13, 0x1ff8u, tq));
@@ -234,8 +237,8 @@ __device__ __forceinline__ HalfA decode_half(uint32_t wa, uint32_t wb, uint32_t 
 // 14-byte layout, four instructions for each of the six.  hb = the eight header bytes of the lane's rows.
 template <int K>
 __device__ __forceinline__ uint32_t overlay_left_over(uint32_t vk, uint32_t vhigh) {
-    // (vk >> 5 & 0x06060606) | (vhigh >> (3 + (K & 1)) & 0x08080808)
-    return and_or(vhigh >> (3 + (K & 1)), 0x08080808u, (vk >> 5) & 0x06060606u);
+    // (vk >> 6 & 0x03030303) | (vhigh >> (4 + (K & 1)) & 0x04040404)
+    return and_or(vhigh >> (4 + (K & 1)), 0x04040404u, (vk >> 6) & 0x03030303u);
 }
 template <int SHIFT>
 __device__ __forceinline__ void header_consts(uint32_t hw, uint32_t tq, float2 &k0, float2 &k1) {
@@ -244,12 +247,12 @@ __device__ __forceinline__ void header_consts(uint32_t hw, uint32_t tq, float2 &
 }
 __device__ __forceinline__ void decode_overlay_tile(const uint4 &va, const uint4 &vb, uint32_t v8, const uint2 &hb, uint32_t tq,
                                                     HalfA &h0, HalfA &h1, HalfA &h2, HalfA &h3) {
-    constexpr uint32_t k14 = 0x0e0e0e0eu;                // 2 v a byte
-    h0.a0 = twice(va.x) & k14; h0.a2 = (va.x >> 2) & k14; h0.a1 = twice(va.y) & k14; h0.a3 = (va.y >> 2) & k14;
-    h1.a0 = twice(va.z) & k14; h1.a2 = (va.z >> 2) & k14; h1.a1 = twice(va.w) & k14; h1.a3 = (va.w >> 2) & k14;
-    h2.a0 = twice(vb.x) & k14; h2.a2 = (vb.x >> 2) & k14; h2.a1 = twice(vb.y) & k14; h2.a3 = (vb.y >> 2) & k14;
-    h3.a0 = twice(vb.z) & k14; h3.a2 = (vb.z >> 2) & k14; h3.a1 = twice(vb.w) & k14; h3.a3 = (vb.w >> 2) & k14;
-    h0.c0 = twice(v8) & k14; h1.c0 = (v8 >> 2) & k14;
+    constexpr uint32_t k7 = 0x07070707u;
+    h0.a0 = va.x & k7; h0.a2 = (va.x >> 3) & k7; h0.a1 = va.y & k7; h0.a3 = (va.y >> 3) & k7;
+    h1.a0 = va.z & k7; h1.a2 = (va.z >> 3) & k7; h1.a1 = va.w & k7; h1.a3 = (va.w >> 3) & k7;
+    h2.a0 = vb.x & k7; h2.a2 = (vb.x >> 3) & k7; h2.a1 = vb.y & k7; h2.a3 = (vb.y >> 3) & k7;
+    h3.a0 = vb.z & k7; h3.a2 = (vb.z >> 3) & k7; h3.a1 = vb.w & k7; h3.a3 = (vb.w >> 3) & k7;
+    h0.c0 = v8 & k7; h1.c0 = (v8 >> 3) & k7;
     h0.c1 = overlay_left_over<0>(va.x, vb.z);            // X0 = Group(0, 1, 2): low bits in V0, third bit in V6
     h1.c1 = overlay_left_over<1>(va.y, vb.z);            // X1 = Group(1, 1, 2)
     h2.c0 = overlay_left_over<2>(va.z, vb.w);            // X2 = Group(2, 0, 2): V2 and V7
@@ -284,27 +287,32 @@ __device__ __forceinline__ long long exception_value(const uint4 &ent, uint32_t 
         }
         cw = j == 0 ? ent.z : ent.w;
     }
-    // twice the sums, as in the tile path
-    const int off = __float_as_int(k.y);
-    const int e_lo = off * (int)lds32(rec + 100) + 2 * (d[0] + 256 * d[1]);
-    const int e_hi = off * (int)lds32(rec + 104) + 2 * (d[2] + 256 * d[3]);
-    return __float2ll_rn(((float)e_lo * k.x + ((float)e_hi * k.x) * 65536.f) * inv_q);
+    const float e_lo = fmaf(k.y, (float)(int)lds32(rec + 100), (float)(d[0] + 256 * d[1]));
+    const float e_hi = fmaf(k.y, (float)(int)lds32(rec + 104), (float)(d[2] + 256 * d[3]));
+    return __float2ll_rn((e_lo * k.x + (e_hi * k.x) * 65536.f) * inv_q);
+}
+
+// The sum of a row and a limb pair with its offset: twice sum_i x_i X_i = sum_i 2 u_i (2 X_i) + (parity - 16) sum_i 2 X_i, in integers
+// below 2^24; the scale is halved.  COMPACT: sum_i x_i X_i itself, the codes as they are and half the offset as a float, whole
+// numbers and halves below 2^23, so that nothing is rounded.  The same to the bit; which is the faster depends on what else the
+// loop does (us, doubled and whole: 14-byte 8192 x 8192 9.49 and 9.56; 13-byte 3071 x 3083 4.47 and 4.37; 10-byte decode layer 28.8 and 28.7).
+template <bool COMPACT>
+__device__ __forceinline__ float offset_sum(float offset, int xsum, int sum) {
+    return COMPACT ? fmaf(offset, (float)xsum, (float)sum) : (float)(__float_as_int(offset) * xsum + sum);
 }
 
 // One half-step: 16 rows x 2 block slots.  h holds this lane's payload words and the constants of its rows' blocks in slot
 // (lane & 3) >> 1 (decode_half), sx the step's operand.  Adds to r0 (row g of the 16) and r1
 // (row g + 8) this lane's share of scale * sum_i x_i * X_i, X the fixed-point activations: its share is the
 // limb pair (lane & 1) of slot (lane & 3) >> 1.  FIRST: r0 and r1 are written, not added to.
-template <bool FIRST>
+template <bool FIRST, bool COMPACT>
 __device__ __forceinline__ void contract_half(const HalfA &h, const StepX &sx, float &r0, float &r1) {
     int d[4];
     mma_k32(d, h.a0, h.a1, h.a2, h.a3, sx.b0, sx.b1);
     mma_k16(d, h.c0, h.c1, sx.b2);
-    // twice sum_i x_i X_i = sum_i 2 u_i (2 X_i) + (parity - 16) sum_i 2 X_i, limb pair by limb pair, in integers below 2^24; the scale is halved
-    const int e0 = __float_as_int(h.k0.y) * sx.xsum + (d[0] + 256 * d[1]);
-    const int e1 = __float_as_int(h.k1.y) * sx.xsum + (d[2] + 256 * d[3]);
-    if (FIRST) { r0 = __fmul_rn((float)e0, h.k0.x); r1 = __fmul_rn((float)e1, h.k1.x); }
-    else { r0 = fmaf((float)e0, h.k0.x, r0); r1 = fmaf((float)e1, h.k1.x, r1); }
+    const float e0 = offset_sum<COMPACT>(h.k0.y, sx.xsum, d[0] + 256 * d[1]), e1 = offset_sum<COMPACT>(h.k1.y, sx.xsum, d[2] + 256 * d[3]);
+    if (FIRST) { r0 = __fmul_rn(e0, h.k0.x); r1 = __fmul_rn(e1, h.k1.x); }
+    else { r0 = fmaf(e0, h.k0.x, r0); r1 = fmaf(e1, h.k1.x, r1); }
 }
 // ---- several activation vectors.  Two vectors share the eight columns of the contraction - column g = 4 (vector) + limb -
 // and a block slot has an instruction sequence of its own: positions 0..23 of the half-step for slot 0, 24..47 for slot 1,
@@ -466,7 +474,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
     constexpr int kSrcCell = COMPACT ? kCell13Bytes : kCellBytes;        // bytes of a leftover block column of a row group
     constexpr int kSrcTile = OVERLAY ? kTile10Bytes : (COMPACT ? kTile13Bytes : kTileBytes);   // bytes of a tile in memory (a ring slot always has kTileBytes)
     extern __shared__ __align__(128) unsigned char smem[];
-    // shared memory: ring | per-matrix block constants (1024 x {gain / (8 sqrt m), parity - 16}) | x records | barriers
+    // shared memory: ring | per-matrix block constants (1024 x {gain / (8 sqrt m), parity - 16}, COMPACT {gain / (4 sqrt m), (parity - 16) / 2}) | x records | barriers
     unsigned char *ring = smem;
     // the block constants start on an 8 KiB boundary of the shared window, so that a matrix's table base and
     // an entry's offset combine by OR (decode_half)
@@ -709,7 +717,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 const int parity = window ? (f >> 2) & 1 : (h >> 4) & 1, gain = window ? (f >> 3) & 1 : (h >> 5) & 1;
                 const int base = window ? 2 * (3 + (f & 3)) : 0;
                 const GemvProblemDev &pe = p.prob[m];
-                tab[m * 1024 + h] = make_float2(0.5f * p.shell_inv_norm[shell] * (gain ? pe.gain1 : pe.gain0), __int_as_float(shell ? parity - 16 + base : 0));
+                tab[m * 1024 + h] = make_float2(p.shell_inv_norm[shell] * (gain ? pe.gain1 : pe.gain0), shell ? 0.5f * (float)(parity - 16 + base) : 0.f);
             }
         } else {
             for (int m = 0; m < p.nprob; m++) {
@@ -1032,7 +1040,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 mma_k16(d1, h1.c0, h1.c1, s1.b2);
                 mma_k16(d2, h2.c0, h2.c1, s2.b2);
                 mma_k16(d3, h3.c0, h3.c1, s2.b2);
-                auto e = [](const int (&d)[4], float ky, int xsum, int r) { return (float)(__float_as_int(ky) * xsum + (d[2 * r] + 256 * d[2 * r + 1])); };
+                auto e = [](const int (&d)[4], float ky, int xsum, int r) { return offset_sum<COMPACT>(ky, xsum, d[2 * r] + 256 * d[2 * r + 1]); };
                 acc[0] = e(d0, h0.k0.y, s1.xsum, 0) * h0.k0.x;
                 acc[1] = e(d0, h0.k1.y, s1.xsum, 1) * h0.k1.x;
                 acc[2] = e(d1, h1.k0.y, s1.xsum, 0) * h1.k0.x;
@@ -1091,7 +1099,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                         guard |= settled(wa, wb, wc) | settled(hw, wa, wb);
                         const HalfA h = m == 0 ? decode_half<COMPACT, 0>(wa, wb, wc, hw, tq_tail) : decode_half<COMPACT, 16>(wa, wb, wc, hw, tq_tail);
                         const LaneOffsets ta = {xt + lo.b0, xt + lo.b1, xt + lo.b2, xt + lo.xs};
-                        contract_half<false>(h, load_step<0>(ta), acc[2 * m], acc[2 * m + 1]);
+                        contract_half<false, COMPACT>(h, load_step<0>(ta), acc[2 * m], acc[2 * m + 1]);
                     }
                     piece += 2 * kSrcCell;
                 }
@@ -1107,7 +1115,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                     const HalfA h = decode_half<COMPACT, 0>(wa, wb, wc, hw, tq_tail);
                     const LaneOffsets ta = {xl + l1.b0, xl + l1.b1, xl + l1.b2, xl + l1.xs};
                     float c0, c1;
-                    contract_half<true>(h, load_step<0>(ta), c0, c1);
+                    contract_half<true, COMPACT>(h, load_step<0>(ta), c0, c1);
                     acc[0] += high_lane ? 0.f : c0; acc[1] += high_lane ? 0.f : c1;
                     acc[2] += high_lane ? c0 : 0.f; acc[3] += high_lane ? c1 : 0.f;
                 }
