@@ -242,8 +242,8 @@ __global__ void __launch_bounds__(32 * batch_warps(SETS), 1) gemv_batch_kernel(c
     const uint32_t ring = smem_addr(smem), tab_pad = (0u - (ring + kWarps * kSlots * kTileBytes)) & 8191u, tab = ring + kWarps * kSlots * kTileBytes + tab_pad;
     float2 *tab_at = reinterpret_cast<float2 *>(smem + kWarps * kSlots * kTileBytes + tab_pad);
     const uint32_t xrec = tab + 8192, bars = xrec + (p.xblocks * kXBlock + 127) / 128 * 128;
-    int4 *cut_at = reinterpret_cast<int4 *>(smem + (bars - ring) + kWarps * kSlots * 8);
-    uint32_t *most_at = reinterpret_cast<uint32_t *>(cut_at + 2);  // largest |x| of every vector, as FP16 bits; then whether an L is kept as L'
+    Cut *cut_at = reinterpret_cast<Cut *>(smem + (bars - ring) + kWarps * kSlots * 8);
+    uint32_t *most_at = reinterpret_cast<uint32_t *>(cut_at + 1);  // largest |x| of every vector, as FP16 bits; then whether an L is kept as L'
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t my_ring = ring + warp * kSlots * kTileBytes, my_bar = bars + 8 * warp * kSlots;
     const GemvProblemDev &pr = p.prob[0];
@@ -267,7 +267,6 @@ __global__ void __launch_bounds__(32 * batch_warps(SETS), 1) gemv_batch_kernel(c
     const int panel_u0 = panel * (p.total_groups * p.panel);
     int u0 = me.first + (warp * cta_n + kWarps - 1) / kWarps, n_units = me.first + ((warp + 1) * cta_n + kWarps - 1) / kWarps - u0;
     bool cut = false;
-    auto ratio = [](int a, int b) { return (int)__fdividef((float)a + 0.5f, (float)b); };           // a / b, a below 2^20
     const int fewest = (cta_n + kWarps - 1) / kWarps;
     if (fewest <= width && cta_n > 0 && me.first + cta_n - panel_u0 <= p.total_groups * width) {
         const FastDiv by_width = panel == p.npanels - 1 ? p.div_last : p.div_panel;
@@ -275,26 +274,13 @@ __global__ void __launch_bounds__(32 * batch_warps(SETS), 1) gemv_batch_kernel(c
         const int head = min(width - (in_panel - width * group0), cta_n), rows = fast_div(cta_n - head, by_width, width), rest = cta_n - head - rows * width;
 #pragma unroll 1
         for (int most = fewest; most <= fewest + 1 && !cut; most++) {
-            const float inverse = __fdividef(1.f, (float)most);
-            auto ranges = [&](int n) { return (int)(((float)(n + most) - 0.5f) * inverse); };      // ranges of `most` units that n units make
-            const int in_head = ranges(head), in_row = ranges(width), in_rest = ranges(rest);
-            if (in_head + rows * in_row + in_rest > kWarps) continue;
+            Cut c;
+            if (!cut_share(group0, head, rows, rest, width, most, kWarps, c)) continue;
             cut = true;
-            int at, end;
-            if (warp < in_head) {
-                at = warp * most;
-                end = min(at + most, head);
-            } else {
-                const int row = ratio(warp - in_head, in_row), begin = head + row * width;
-                at = begin + (warp - in_head - row * in_row) * most;
-                end = min(min(at + most, begin + width), cta_n);
-            }
-            u0 = me.first + min(at, cta_n);
-            n_units = max(end - at, 0);
-            if (tid == 0) {
-                cut_at[0] = make_int4(group0, 1 + rows + (rest > 0 ? 1 : 0), head, rest);
-                cut_at[1] = make_int4(in_head, in_row, in_rest, width);
-            }
+            int at;
+            n_units = cut_range(c, cta_n, most, warp, at);
+            u0 = me.first + at;
+            if (tid == 0) *cut_at = c;
         }
     }
     int r = u0 - panel_u0;
@@ -630,11 +616,11 @@ __global__ void __launch_bounds__(32 * batch_warps(SETS), 1) gemv_batch_kernel(c
         }
     }
     if (cut) {
-        __syncthreads();                               // the warps' sums
+        const bool lost = __syncthreads_or(failed);    // the warps' sums, and whether one has none
         // a thread a row, vector and row group at a time; all the atomics are on their way before the first answer is looked at
         constexpr int kMost = 4 * SETS;                // kWarps row groups at most, of 32 rows and 4 SETS vectors
-        const int4 c0 = cut_at[0], c1 = cut_at[1];
-        const int outputs = c0.y * 32 * p.batch;
+        const Cut c = *cut_at;
+        const int outputs = cut_outputs(c, p.batch, lost);
         unsigned long long old[kMost], word[kMost];
         __half scale[kMost];
         int units[kMost], row[kMost], v[kMost];
@@ -643,17 +629,16 @@ __global__ void __launch_bounds__(32 * batch_warps(SETS), 1) gemv_batch_kernel(c
             const int o = tid + i * kThreads;
             row[i] = -1;
             if (o >= outputs) continue;
-            const int k = o >> 5, s = ratio(k, p.batch);
+            const int k = o >> 5, s = cut_ratio(k, p.batch);
             v[i] = k - s * p.batch;
-            const int r0 = (c0.x + s) * kRowsPerGroup + (o & 31), w0 = s == 0 ? 0 : c1.x + (s - 1) * c1.y;
-            const bool last = s == c0.y - 1 && c0.w > 0;
-            const int w1 = w0 + (s == 0 ? c1.x : (last ? c1.z : c1.y));
-            units[i] = s == 0 ? c0.z : (last ? c0.w : c1.w);
+            const int r0 = (c.first_group + s) * kRowsPerGroup + (o & 31);
+            const CutWarps of = cut_warps(c, s);
+            units[i] = cut_units(c, s);
             if (r0 >= pr.rows) continue;
             row[i] = r0;
             scale[i] = pr.row_scale[r0];
             word[i] = 0ull;
-            for (int w = w0; w < w1; w++) word[i] += *reinterpret_cast<const unsigned long long *>(smem + w * kSlots * kTileBytes + 8 * (kCutStride * v[i] + (o & 31)));
+            for (int w = of.first; w < of.end; w++) word[i] += *reinterpret_cast<const unsigned long long *>(smem + w * kSlots * kTileBytes + 8 * (kCutStride * v[i] + (o & 31)));
             old[i] = atomicAdd(p.accum + (size_t)v[i] * ((size_t)p.total_groups * 32) + r0, word[i]);
         }
 #pragma unroll

@@ -1740,7 +1740,7 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
     if (batch_in_sets(p.batch)) {
         const int sets = batch_sets(p.batch), warps = batch_warps(sets);
         g.smem = (size_t)warps * kSlots * kTileBytes + 2 * 8192 /* the table and its alignment */ + ((size_t)p.xblocks * sets * kBatchSetBytes + 127) / 128 * 128 +
-                 warps * kSlots * 8 + 32 + (LLVQ_MAX_BATCH + 1) * 4 + 16;
+                 warps * kSlots * 8 + kBatchSharedWords * 4;
         return g;
     }
     const int vectors = p.batch > 2 ? 8 : p.batch, warps = gemv_warps(vectors);        // the kernel is built for 1, 2 and 8

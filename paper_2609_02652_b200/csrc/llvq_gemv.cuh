@@ -1,5 +1,6 @@
 // What the matrix-vector kernels share: the accumulator word, the ring of record slots and its bounded waits, shared-memory reads.
 #pragma once
+#include "llvq_cut.h"
 #include "llvq_internal.cuh"
 
 namespace llvq {
@@ -14,6 +15,7 @@ constexpr int kEarlySlots = 1;             // slots filled before the wait for t
 // per CTA.  Two sets need more registers than sixteen warps leave a thread (128): sixteen that spill take twice the time of twelve with 168.
 // Five and six would leave half of the second set idle (34816 x 5120, five: 51.7 us that way, 49.6 in pairs; 500 x 8192 10.9 and 9.9).
 constexpr int kBatchSetBytes = 480;
+constexpr int kBatchSharedWords = sizeof(Cut) / 4 + LLVQ_MAX_BATCH + 1;        // what the CTA of such a launch shares besides: see gemv_batch_kernel
 __host__ __device__ constexpr bool batch_in_sets(int batch) { return batch == 3 || batch == 4 || batch >= 7; }
 __host__ __device__ constexpr int batch_sets(int batch) { return batch > 4 ? 2 : 1; }
 __host__ __device__ constexpr int batch_warps(int sets) { return sets > 1 ? 12 : kWarps; }

@@ -83,3 +83,10 @@ def test_no_matvec_reads_ahead_of_an_expansion(tmp_path):
     without an ordinary launch between it and the expansion."""
     total, ahead, wrong = map(int, run_native(tmp_path, "record_order.cpp").split())
     assert total == 462 and ahead > 0 and wrong == 0
+
+
+def test_shares_cut_at_row_groups(tmp_path):
+    """Every unit of a share is one warp's, a row group's sums are its own warps', and a CTA with a warp that ran into the wait limit hands nothing
+    over: what lies in the place of that warp's sums is a record."""
+    cuts, uncut, wrong = map(int, run_native(tmp_path, "cut.cpp").split())
+    assert cuts > 10000 and uncut > 10000 and wrong == 0
