@@ -228,9 +228,6 @@ int llvq_expand(llvq_ctx *ctx, int layout, const uint64_t *codes, int64_t rows, 
     return rc;
 }
 
-constexpr int kVectorsPerPass = 4;      // activation vectors a pass that llvq_gemv_plan describes carries at most
-constexpr int kTwoByTwo = 1;            // run_gemv's answer where three or four vectors have to go in passes of two
-
 int llvq_gemv_plan(int sm_count, const int64_t *rows, int n, int64_t k_padded, int batch, int32_t *out, int out_len) {
     if (!rows || !out || n < 1 || n > LLVQ_MAX_GROUP || sm_count < 1 || batch < 1 || batch > kVectorsPerPass) return LLVQ_EINVAL;
     if (k_padded <= 0 || k_padded % 24 != 0) return LLVQ_EINVAL;
@@ -346,11 +343,7 @@ static int run_gemv(llvq_ctx *ctx, int layout, const llvq_problem *problems, int
         p.rot_scale = std::ldexp(1.0 / std::sqrt((double)((int64_t)1 << l)), 1008);
     }
     const GemvLaunch g = planned(ctx, layout, p);
-    if (g.smem + 1024 > (size_t)ctx->max_smem_optin) {
-        // three and four vectors: the records of the pairs' build took 32 bytes less a block
-        const bool two_by_two = batch_in_sets(batch) && batch <= kVectorsPerPass && g.smem - 32 * (size_t)p.xblocks + 1024 <= (size_t)ctx->max_smem_optin;
-        return two_by_two ? kTwoByTwo : LLVQ_ESIZE;
-    }
+    if (const int refusal = pass_refusal(batch, g.smem, p.xblocks, (size_t)ctx->max_smem_optin)) return refusal;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
     const uint64_t expansions = ctx->order.expansions();
@@ -378,19 +371,7 @@ int llvq_gemv_batch(llvq_ctx *ctx, const void *layout_buf, const void *row_scale
         q.y = y + (size_t)first * (size_t)rows;
         return run_gemv(ctx, LLVQ_PLANES, &q, 1, (const __half *)x + (size_t)first * (size_t)k_padded, k_padded, false, stream, n);
     };
-    // One pass over the records serves all the vectors, if the scratch has room for their sums and a multiprocessor for
-    // their records of x, which only devices of few multiprocessors lack (eight vectors, us in one pass and in two:
-    // 1024 x 2560 8.8 and 10.5, 4096 x 4096 15.1 and 16.5, 34816 x 5120 53.9 and 64.8).
-    int rc = pass(0, batch);
-    if (rc != kTwoByTwo && (rc != LLVQ_ESIZE || batch <= kVectorsPerPass)) return rc;
-    // Otherwise passes of up to four, or of two, one after the other on the stream (they share the context's scratch).
-    for (int first = 0, n; first < batch; first += n) {
-        n = batch - first < kVectorsPerPass ? batch - first : kVectorsPerPass;
-        rc = pass(first, n);
-        if (rc == kTwoByTwo) rc = pass(first, n = 2);
-        if (rc != LLVQ_OK) return rc;
-    }
-    return LLVQ_OK;
+    return batch_passes(batch, pass);
 }
 
 int llvq_gemv_grouped(llvq_ctx *ctx, int layout, const llvq_problem *problems, int n, const void *x, int64_t k_padded,

@@ -11,12 +11,10 @@ constexpr int kThreads = kWarps * 32;
 constexpr int kSlots = 2;                  // ring slots per warp
 constexpr int kEarlySlots = 1;             // slots filled before the wait for the previous kernel; the rest once x is being prepared
 
-// Three, four, seven and eight vectors have a kernel of their own (llvq_batch.cu): sets of four, the bytes of a block's record of x a set, warps
-// per CTA.  Two sets need more registers than sixteen warps leave a thread (128): sixteen that spill take twice the time of twelve with 168.
-// Five and six would leave half of the second set idle (34816 x 5120, five: 51.7 us that way, 49.6 in pairs; 500 x 8192 10.9 and 9.9).
+// Vectors in sets of four (batch_in_sets): the bytes of a block's record of x a set, warps per CTA.  Two sets need more registers than
+// sixteen warps leave a thread (128): sixteen that spill take twice the time of twelve with 168.
 constexpr int kBatchSetBytes = 480;
 constexpr int kBatchSharedWords = sizeof(Cut) / 4 + LLVQ_MAX_BATCH + 1;        // what the CTA of such a launch shares besides: see gemv_batch_kernel
-__host__ __device__ constexpr bool batch_in_sets(int batch) { return batch == 3 || batch == 4 || batch >= 7; }
 __host__ __device__ constexpr int batch_sets(int batch) { return batch > 4 ? 2 : 1; }
 __host__ __device__ constexpr int batch_warps(int sets) { return sets > 1 ? 12 : kWarps; }
 // the kernel for one vector, for two and, in pairs, for five and six

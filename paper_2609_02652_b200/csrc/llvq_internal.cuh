@@ -176,6 +176,36 @@ private:
     int used_ = 0, next_ = 0;
 };
 
+// Three, four, seven and eight vectors have a kernel of their own, which takes them in sets of four (llvq_batch.cu).
+// Five and six would leave half of the second set idle (34816 x 5120, five: 51.7 us that way, 49.6 in pairs; 500 x 8192 10.9 and 9.9).
+__host__ __device__ constexpr bool batch_in_sets(int batch) { return batch == 3 || batch == 4 || batch >= 7; }
+
+constexpr int kVectorsPerPass = 4;      // activation vectors a pass that llvq_gemv_plan describes carries at most
+constexpr int kTwoByTwo = 1;            // a pass's answer where three or four vectors have to go in passes of two
+// Whether a pass fits a multiprocessor that grants `most` bytes of shared memory: LLVQ_OK or the pass's answer.  Three and four vectors that
+// do not fit as a set go two by two where four did in pairs, whose records of x are 32 bytes a block less.
+inline int pass_refusal(int batch, size_t smem, int xblocks, size_t most) {
+    if (smem + 1024 <= most) return LLVQ_OK;
+    return batch_in_sets(batch) && batch <= kVectorsPerPass && smem - 32 * (size_t)xblocks + 1024 <= most ? kTwoByTwo : LLVQ_ESIZE;
+}
+// The passes over the records that `batch` activation vectors take; pass(first, n) launches vectors [first, first + n) or says why not.
+// One pass serves all of them, if the scratch has room for their sums and a multiprocessor for their records of x, which
+// only devices of few multiprocessors lack (eight vectors, us in one pass and in two: 1024 x 2560 8.8 and 10.5, 4096 x 4096
+// 15.1 and 16.5, 34816 x 5120 53.9 and 64.8).
+template <typename Pass>
+int batch_passes(int batch, Pass pass) {
+    int rc = pass(0, batch);
+    if (rc != kTwoByTwo && (rc != LLVQ_ESIZE || batch <= kVectorsPerPass)) return rc;
+    // Otherwise passes of up to four, or of two, one after the other on the stream (they share the context's scratch).
+    for (int first = 0, n; first < batch; first += n) {
+        n = batch - first < kVectorsPerPass ? batch - first : kVectorsPerPass;
+        rc = pass(first, n);
+        if (rc == kTwoByTwo) rc = pass(first, n = 2);
+        if (rc != LLVQ_OK) return rc;
+    }
+    return LLVQ_OK;
+}
+
 // A GEMV launched right behind an expansion must not read records ahead of its wait; behind a GEMV that was launched as an
 // ordinary kernel after the expansion, it may.  Host threads that share the stream may ask at any point of one another's
 // launches: an expansion counts once it is enqueued, and an ordinary launch, once it is enqueued itself, for the expansions that

@@ -90,3 +90,25 @@ def test_shares_cut_at_row_groups(tmp_path):
     over: what lies in the place of that warp's sums is a record."""
     cuts, uncut, wrong = map(int, run_native(tmp_path, "cut.cpp").split())
     assert cuts > 10000 and uncut > 10000 and wrong == 0
+
+
+def test_passes_of_a_batch(tmp_path):
+    """A batch that one pass cannot carry goes in passes of four or of two, every vector in one of them and in order; what no pass can carry is
+    refused with the size error, and another error ends it.  The plans of a device of few multiprocessors take every such way, those of a full-size one
+    never more than one pass."""
+    from paper_2609_02652_b200 import build
+
+    build.build()
+    where = os.path.dirname(build.LIB)
+    shapes = [(sm, rows, 24 * nb, batch) for sm, rows in ((8, 4096), (8, 500), (1, 64), (148, 4096), (148, 33)) for nb in (70, 340, 355, 380, 500, 700, 4094) for batch in range(1, 9)]
+    out = run_native(tmp_path, "passes.cpp", "-L" + where, "-l:libllvq.so", "-Wl,-rpath," + where, stdin="".join("%d %d %d %d\n" % s for s in shapes))
+    counts, *lines = out.strip().splitlines()
+    launched, refused, wrong = map(int, counts.split())
+    assert launched > 100 and refused > 50 and wrong == 0 and len(lines) == len(shapes)
+    seen = set()
+    for (sm, _, _, batch), line in zip(shapes, lines):
+        *passes, rc = map(int, line.split())
+        assert rc == -3 or sum(passes) == batch
+        assert sm < 148 or passes == [batch]
+        seen.add(tuple(passes))
+    assert {(4,), (2, 2), (2, 1), (8,), (4, 4), (2, 2, 2, 2)} <= seen
