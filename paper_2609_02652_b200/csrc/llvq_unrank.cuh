@@ -139,6 +139,23 @@ LLVQ_HD int find_class(const UnrankView &v, uint64_t idx) {
 // 2^32: shifted right by left's power of two, the product times the inverse of left's odd part modulo 2^32.
 LLVQ_HD uint32_t portion(uint32_t T, uint32_t copies, const UnrankStep &e) { return (uint32_t)(((uint64_t)T * copies) >> e.shift) * e.inverse; }
 
+// The position of rank r among the draws of two from a multiset, given their ratio to its orderings: right, or one too large.
+LLVQ_HD uint32_t draw_position(uint32_t r, float ratio, uint32_t draws) {
+    const uint32_t at = floor_product((float)r, ratio);
+    return at < draws ? at : draws - 1u;
+}
+// The pair of rank r, from the entry at that position: the first rank of the pair there tells whether it was one too large.  Position 0 begins with
+// rank 0, so the loop ends; after one step, at that (a host test runs all the tables).  An `if` in its place: 17408 x 5120 into the
+// 10-byte layout 139.5 -> 140.2 us, 9728 x 2560 into the 14-byte layout 34.8 -> 34.6.
+LLVQ_HD uint64_t pair_drawn(const uint64_t *entry, uint32_t r) {
+    uint64_t pair = *entry;
+#ifdef __CUDA_ARCH__
+#pragma unroll 1
+#endif
+    while (r < (uint32_t)pair) pair = *--entry;
+    return pair;
+}
+
 // Odd type.  Sixteen coordinates come two at a time from the table of draws, the ordering of the last eight is an entry of
 // a list.  The position of the draw is a float estimate that is right or one too large, which the first rank of the pair it names
 // tells.  Rolled up: eight steps' code would crowd the instruction cache.  The load unit and its latency bound this, so a step
@@ -155,15 +172,7 @@ LLVQ_HD void unrank_odd(const UnrankView &v, const UnrankDesc &d, uint64_t r47, 
 #endif
     while (true) {
         const uint32_t draws = left * (left - 1u);
-        uint32_t at = floor_product((float)r, ratio);
-        at = at < draws ? at : draws - 1u;
-        const uint64_t *entry = v.pairs + (first + set * draws + at);
-        uint64_t pair = *entry;
-        // position 0 begins with rank 0, so this ends; after one step, at that
-#ifdef __CUDA_ARCH__
-#pragma unroll 1
-#endif
-        while (r < (uint32_t)pair) pair = *--entry;
+        const uint64_t pair = pair_drawn(v.pairs + (first + set * draws + draw_position(r, ratio, draws)), r);
         r -= (uint32_t)pair;
         high = (uint32_t)(pair >> 32);
         word = byte_perm(word, high, 0x5321u);

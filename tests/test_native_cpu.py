@@ -92,6 +92,15 @@ def test_shares_cut_at_row_groups(tmp_path):
     assert cuts > 10000 and uncut > 10000 and wrong == 0
 
 
+def test_positions_of_pair_draws(tmp_path):
+    """For every multiset, step and ratio the expander can meet, the position estimated for a pair's first and last rank is one of the pair's own or the
+    next, never one before: the reader looks one entry back and no further."""
+    from paper_2609_02652_b200 import build
+
+    pairs, above, wrong = map(int, run_native(tmp_path, "pairs.cpp", *[os.path.join(build.CSRC, f) for f in ("llvq_tables.cpp", "llvq_unrank.cpp")]).split())
+    assert pairs > 10000 and above > 0 and wrong == 0
+
+
 def test_passes_of_a_batch(tmp_path):
     """A batch that one pass cannot carry goes in passes of four or of two, every vector in one of them and in order; what no pass can carry is
     refused with the size error, and another error ends it.  The plans of a device of few multiprocessors take every such way, those of a full-size one
