@@ -319,9 +319,8 @@ __device__ __forceinline__ void contract_half(const HalfA &h, const StepX &sx, f
 // the other slot's positions zero in B.  Against one vector with block-diagonal B that is three instructions instead
 // of four for two vectors and two slots, and a row's sum lies in two lanes instead of four, so half the exchanges.
 // The price is that a lane looks up the headers of both slots; every vector shares that.  Two, five and six vectors go this way
-// (three, four, seven and eight: llvq_batch.cu).  Bound: latency (the build for eight on 4096 x 4096: issue slots
-// 32 % busy, three warps a scheduler that also wait for instructions; tensor pipe 10 %).  Two vectors on 8192 x 8192: 11.9 us a launch, 12.5 a vector at
-// a time, its atomic waited for before the next vector's.
+// (three, four, seven and eight: llvq_batch.cu).  Bound: latency, twelve warps for five and six.  Two vectors on 8192 x 8192: 11.9 us a launch, 12.5 a
+// vector at a time, its atomic waited for before the next vector's.
 struct PairA {
     uint32_t a0, a1, a2, a3, c0, c1;
     float2 k00, k01, k10, k11;                     // block constants: slot, then row g or g + 8
@@ -455,7 +454,7 @@ __device__ __forceinline__ void each_pair(F &f) {
     }
 }
 
-// BATCH (1, 2, or 8 for five and six) activation vectors share one pass over the records: the decode of a half-step and its block constants
+// BATCH (1, 2, or 6 for five and six) activation vectors share one pass over the records: the decode of a half-step and its block constants
 // are computed once, the contraction, the scaling and the reduction once a pair of vectors.  x is BATCH vectors of
 // 24 nb halves one after the other, y BATCH vectors of rows floats (p.prob[].y is vector 0's), the accumulators
 // BATCH sets of total_groups * 32.
@@ -1059,7 +1058,6 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 const PairA h2 = decode_pair(a1.z, a1.w, a2.x, hh.z, hb.z, tq), h3 = decode_pair(a2.y, a2.z, a2.w, hh.w, hb.w, tq);
                 auto one_pair = [&](auto index) {
                     constexpr int J = decltype(index)::value, kPair = J * 2 * kXRecBytes;
-                    if (J > 1 && 2 * J >= p.batch) return;                 // a launch carries fewer vectors than the kernel is built for
                     const PairX x0 = load_pair<kPair, kPair + kXBlock>(xp), x1 = load_pair<kPair + 2 * kXBlock, kPair + 3 * kXBlock>(xp);
                     float u[4], w[4];                                      // slot 0 and slot 1, rows [2m + e]
                     contract_pair<true>(h0, x0, u, w);
@@ -1144,7 +1142,6 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 const PairAddr xt = pair_addr(lane, xs0 + (uint32_t)tiles * (4 * kXBlock)), xl = pair_addr(lane, xs0 + (uint32_t)(p.nb - 1) * kXBlock);
                 auto one_pair = [&](auto index) {
                     constexpr int J = decltype(index)::value, kPair = J * 2 * kXRecBytes;
-                    if (J > 1 && 2 * J >= p.batch) return;                 // a launch carries fewer vectors than the kernel is built for
                     float u[4] = {0.f, 0.f, 0.f, 0.f}, v[4] = {0.f, 0.f, 0.f, 0.f};
                     if (two) {
                         const PairX x = load_pair<kPair, kPair + kXBlock>(xt);
@@ -1743,7 +1740,9 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
                  warps * kSlots * 8 + kBatchSharedWords * 4;
         return g;
     }
-    const int vectors = p.batch > 2 ? 8 : p.batch, warps = gemv_warps(vectors);        // the kernel is built for 1, 2 and 8
+    // the kernel is built for 1, 2 and 6 (us, five vectors, against a build for eight whose fourth pair is skipped: 1024 x 2560 5.7 and 7.3,
+    // 8192 x 8192 22.3 and 24.9, 34816 x 5120 47.8 and 51.3); the room for x is asked for as for eight, and with it the line between one pass and two
+    const int vectors = p.batch > 2 ? 8 : p.batch, warps = gemv_warps(vectors);
     const size_t records = ((size_t)p.xblocks * kXRecBytes * vectors + 127) / 128 * 128, raw = rot_first(p.rot_log2).stages ? ((size_t)p.rot_span * 2 + 127) / 128 * 128 : 0;
     g.smem = (size_t)warps * kSlots * kTileBytes + 8192 /* alignment of the tables */ + (size_t)p.nprob * 8192 + warps * kSlots * 8 + warps * 4 * vectors + 16;
     // a rotation counts with eight bytes a coordinate of its whole blocks, the limit llvq_gemv_rotated states, though it needs less
@@ -1758,7 +1757,7 @@ int gemv_configure(const llvq_ctx *ctx) {
     if (allow_max_smem(gemv_planes_kernel<false, 1>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<true, 1>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 2>, bytes)) return -1;
-    if (allow_max_smem(gemv_planes_kernel<false, 8>, bytes)) return -1;
+    if (allow_max_smem(gemv_planes_kernel<false, 6>, bytes)) return -1;
     if (batch_configure(bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 1, kRotateShort>, bytes)) return -1;
     if (allow_max_smem(gemv_planes_kernel<false, 1, kRotateLong>, bytes)) return -1;
@@ -1790,7 +1789,7 @@ cudaError_t launch_gemv(int layout, const GemvParams &p, const GemvLaunch &g, bo
         if (p.rot_log2 > 0) return cudaLaunchKernelEx(&cfg, rot_first(p.rot_log2).stages ? gemv_planes_kernel<false, 1, kRotateLong> : gemv_planes_kernel<false, 1, kRotateShort>, p);
         if (p.batch <= 1) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 1>, p);
         if (p.batch == 2) return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 2>, p);
-        return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 8>, p);
+        return cudaLaunchKernelEx(&cfg, gemv_planes_kernel<false, 6>, p);
     }
     cfg.numAttrs = 0;
     return cudaLaunchKernelEx(&cfg, gemv_onehot_kernel, p);

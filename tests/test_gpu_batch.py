@@ -40,6 +40,13 @@ def test_every_vector_as_alone(B, ctx, rows, nb, batch):
     B.status(ctx)
 
 
+# the builds for six and for eight, filled and with a vector to spare: one launch whose rows end in a tile of one, two and three blocks
+@pytest.mark.parametrize("rows,nb", [(33, 7), (500, 341), (4096, 170), (20000, 70)])
+@pytest.mark.parametrize("batch", [2, 6, 7])
+def test_every_vector_of_the_other_builds(B, ctx, rows, nb, batch):
+    test_every_vector_as_alone(B, ctx, rows, nb, batch)
+
+
 # Twice the fixed-point activation, given a largest |x| in [2, 4): x = units / 2^28.  The halves of 32656, 32688, 32720 and 32752 are kept in another
 # form; 32640 and 32768 are the numbers beside them; 32624 everywhere is the largest sum of low halves, -32896 the least
 @pytest.mark.parametrize("units", [(32656, 32688, 32720, 32752), (32640, 32656, 32768, -32656), (32624,), (32640,), (65536 + 32640, 98304 - 64, 131072 - 64)])
