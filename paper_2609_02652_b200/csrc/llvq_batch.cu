@@ -6,11 +6,11 @@
 // -32896 <= L_i < 32640.  An FP16 activation has eleven significant bits, so X_i has, and both halves are FP16
 // numbers exactly: a vector needs two columns of the contraction where 8-bit limbs need four, mma.sync m16n8k16
 // f16 x f16 -> f32 serves four vectors, and an accumulator is the integer that limbs are recombined to - nothing is recombined or
-// converted.  A code is taken as 16 + u: its four bits moved to bits 6..9 of an FP16 word with the exponent of 16.  So
-//     e = sum x_i L_i / 2 = sum (16 + u_i) L_i + ((parity - 16) / 2 - 16) sum L_i
-// and one multiply-add a half and block takes the offset off, one more applies the scale.  All of it is exact up to
-// there: the operands are whole numbers, a partial sum is an even number below 2^25 (L_i is even) or a whole number
-// below 2^24 (|H_i| <= 2^14), and e is a whole number or a half below 2^23.
+// converted.  A code is taken as u 2^-18: its four bits moved to bits 6..9 of an FP16 word are that number, a subnormal one, which the
+// instruction takes exactly.  So
+//     2^-18 e = sum x_i L_i / 2^19 = sum (u_i 2^-18) L_i + (parity - 16) / 2^19 sum L_i,
+// and one multiply-add a half and block adds the offset, one more applies the scale.  All of it is exact up to there: in units of
+// 2^-18 the partial sums are whole numbers below 2^24 (|L_i| <= 32896, |H_i| <= 2^14), and e is a whole number below 2^23.
 // One octave breaks the rule on L: 2 X = 32656, 32688, 32720 or 32752 (eleven bits and the sign) leave L = 2 X - 65536, which has
 // twelve.  Such an activation is kept as L' = 2 X, H' = 0 - no other L is that large - and a CTA that meets one takes tiles
 // through a second build of their code, which counts L' back: the contraction of the marks [L' >= 32640] takes 65536 times itself from L
@@ -29,7 +29,8 @@ namespace {
 // x in shared memory, a record a block and set of four vectors.  Column 2v + h of the contraction is half h (L, H) of vector v.
 // Chunk c (0..5) of a column holds coordinates 4c, 4c+2, 4c+1, 4c+3, the order in which a payload byte pair is split; chunk 6 zeros.
 // Chunk c of column n lies at 224 (n >> 2) + 32 c + 8 (n & 3): a half-warp's 64-bit reads are 128 consecutive bytes.  At 448,
-// {sum L, sum H} of each vector.
+// each vector's sum of 2 X in two parts (convert_third).
+constexpr float kCodeUnit = 1.f / (1 << 18);      // what a code's bits count as FP16
 constexpr int kSetBytes = kBatchSetBytes, kHalfBytes = 224, kSumsAt = 448;
 
 __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint2 b) {
@@ -71,24 +72,22 @@ __device__ __forceinline__ uint2 lds64_at(uint32_t a) {
 }
 
 // What the decode needs in registers.  Left shifts are multiplications (by factors the compiler cannot see, or they would become shifts
-// again): the logic unit takes two cycles an instruction, as the multiplier does, and has more to do; with two immediates, mask and exponent would
-// be two instructions.
-struct Factors { uint32_t by4, by8, by16, by64, bits, sixteen; };
+// again): the logic unit takes two cycles an instruction, as the multiplier does, and has more to do.
+struct Factors { uint32_t by4, by8, by16, by64; };
 __device__ __forceinline__ Factors factors() {
     Factors f;
-    asm volatile("mov.u32 %0, 4;\n\tmov.u32 %1, 16;\n\tmov.u32 %2, 64;\n\tmov.u32 %3, 0x03c003c0;\n\tmov.u32 %4, 0x4c004c00;\n\tmov.u32 %5, 8;"
-                 : "=r"(f.by4), "=r"(f.by16), "=r"(f.by64), "=r"(f.bits), "=r"(f.sixteen), "=r"(f.by8));
+    asm volatile("mov.u32 %0, 4;\n\tmov.u32 %1, 16;\n\tmov.u32 %2, 64;\n\tmov.u32 %3, 8;" : "=r"(f.by4), "=r"(f.by16), "=r"(f.by64), "=r"(f.by8));
     return f;
 }
 // The A operand of a half-step (16 rows x two block slots).  Positions 0..15, 16..31, 32..47 of the half-step are an
 // operand each; of the middle one the first two lanes of a quad hold slot 0's last eight coordinates and the other two slot 1's
-// first eight.  k[s][e] = {scale gain / (4 sqrt m), offset (parity - 16) / 2 - 16} of slot s, row g + 8e.
+// first eight.  k[s][e] = {2^18 gain / (4 sqrt m), (parity - 16) / 2^19} of slot s, row g + 8e.
 struct Half {
     uint32_t first[4], middle[4], last[4];
     float2 k[2][2];
 };
 __device__ __forceinline__ Half decode_half16(uint32_t wa, uint32_t wb, uint32_t wc, uint32_t hw0, uint32_t hw1, uint32_t tab, const Factors &f) {
-    auto code = [&](uint32_t w) { return and_or(w, f.bits, f.sixteen); };
+    auto code = [](uint32_t w) { return w & 0x03c003c0u; };
     Half h;
     // low nibbles of bytes 0 and 2, of bytes 1 and 3, then the high nibbles
     const uint32_t sa = wa >> 6, sb = wb >> 6, sc = wc >> 6;
@@ -181,8 +180,8 @@ __device__ __forceinline__ uint32_t max_abs_or_nan(uint32_t m, uint32_t x2) {
     const __half2 r = __hmax2_nan(*reinterpret_cast<const __half2 *>(&m), __habs2(*reinterpret_cast<const __half2 *>(&x2)));
     return *reinterpret_cast<const uint32_t *>(&r);
 }
-// x (FP16, eight coordinates: a third of a block) -> its two chunks of the record, the first of them at `at`.  Returns
-// {sum L, sum H} of the third.  2 rint(x scale) and the nearest multiple of 65536 come from additions of
+// x (FP16, eight coordinates: a third of a block) -> its two chunks of the record, the first of them at `at`.  Returns the third's share of the block's
+// activation sum, {sum L, sum H} but for a unit between the two.  2 rint(x scale) and the nearest multiple of 65536 come from additions of
 // 1.5 * 2^23: x scale is a whole number of eleven significant bits, which such an addition leaves as it is, or below 2^11.  H is
 // floor((z + 32896) / 65536) of the even z = 2 X, the nearest whole number to (z + 129) / 65536, which is never halfway between two.
 // `wide` is set if an L had to be kept as L'.
@@ -229,7 +228,14 @@ __device__ __forceinline__ float2 convert_third(uint4 v, uint32_t at, float scal
     for (int c = 0; c < 2; c++)
         asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at + 32 * c), "r"(lo[2 * c]), "r"(lo[2 * c + 1]), "r"(hi[2 * c]), "r"(hi[2 * c + 1]) : "memory");
     const float2 sl = halves(sum_lo), sh = halves(sum_hi);
-    return make_float2(sl.x + sl.y, sh.x + sh.y);
+    // an odd sum of H passes a unit on to the sum of L, as in the kernels for pairs and for one vector, whose records hold the halves of both
+    // as whole numbers
+    float sum_l = sl.x + sl.y, sum_h = sh.x + sh.y;
+    if (__float_as_uint(sum_h + kRound) & 1u) {
+        sum_l += 65536.f;
+        sum_h -= 1.f;
+    }
+    return make_float2(sum_l, sum_h);
 }
 
 // SETS = 1: three or four vectors; 2: seven or eight.  The launch is one matrix (p.prob[0]).
@@ -346,9 +352,9 @@ __global__ void __launch_bounds__(32 * batch_warps(SETS), 1) gemv_batch_kernel(c
         for (int i = 0; i < kClasses; i++) {
             const int c = tid + i * kThreads;
             if (kClassSlots % kThreads != 0 && c >= kClassSlots) break;
-            const float offset = 0.5f * (float)__float_as_int(my_class[i].y) - 16.f;
-            tab_at[c] = make_float2(my_class[i].x * pr.gain0, offset);
-            tab_at[512 + c] = make_float2(my_class[i].x * pr.gain1, offset);
+            const float offset = (float)__float_as_int(my_class[i].y) * (0.5f * kCodeUnit);
+            tab_at[c] = make_float2(my_class[i].x * (pr.gain0 / kCodeUnit), offset);
+            tab_at[512 + c] = make_float2(my_class[i].x * (pr.gain1 / kCodeUnit), offset);
         }
     };
     // The preparation of x: a vector is shared by `each` warps, ten blocks a warp at a time, three lanes a block.  More vectors than
@@ -357,6 +363,9 @@ __global__ void __launch_bounds__(32 * batch_warps(SETS), 1) gemv_batch_kernel(c
     const int each = (p.batch > kWarps / 2 ? 2 * kWarps : kWarps) / (unsigned)p.batch, work = each * p.batch;
     const int blocks = blk_hi - blk_lo, my_block = lane / 3, third = lane - 3 * my_block;
     const uint32_t xs0 = xrec - (uint32_t)blk_lo * kXBlock;                   // address of block 0's record, were it there
+    // in the shadow of the previous kernel: between the loads of x and their use, its wait for the class constants is a wait for x as well
+    // (us, eight vectors: 1024 x 2560 8.83 -> 8.68, 34816 x 5120 54.0 -> 53.6)
+    build_table();
     __syncthreads();                                   // the maxima are zero
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -377,7 +386,6 @@ __global__ void __launch_bounds__(32 * batch_warps(SETS), 1) gemv_batch_kernel(c
         own1 = load_piece(first_share, 10 * (first_share.part + each) + my_block);
     }
     // every vector's largest |x|
-    if (warp >= work) build_table();
 #pragma unroll 1
     for (int w = warp; w < work; w += kWarps) {
         const Share q = w == warp ? first_share : share_of(w);
@@ -392,7 +400,6 @@ __global__ void __launch_bounds__(32 * batch_warps(SETS), 1) gemv_batch_kernel(c
             e += kInFlight * step;
         };
         load();
-        if (w == warp) build_table();                  // while the first loads are on their way
         for (;;) {
 #pragma unroll
             for (int i = 0; i < kInFlight; i++) m = max_abs_or_nan(max_abs_or_nan(max_abs_or_nan(max_abs_or_nan(m, v[i].x), v[i].y), v[i].z), v[i].w);

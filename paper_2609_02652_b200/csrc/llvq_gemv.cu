@@ -4,12 +4,12 @@
 // four-bit code the record stores.  The activations are taken as fixed point, X_i = rint(x_i * 2^F) with F
 // set by the largest |x| of the call, and 2 X_i is split into four balanced 8-bit limbs.  The inner sum then
 // is an integer contraction that the tensor cores do exactly: mma.sync m16n8k32 / m16n8k16, u8 x s8 -> s32.
-// A is 16 rows x 48 positions (two block slots of 24 coordinates) of doubled codes, one byte each once the two nibbles
-// of a payload byte are split (an addition, a shift, two ANDs a word: the whole decode); B is block-diagonal, its eight
+// A is 16 rows x 48 positions (two block slots of 24 coordinates) of codes, one byte each once the two nibbles
+// of a payload byte are split (one shift, two ANDs a word: the whole decode); B is block-diagonal, its eight
 // columns the four limbs of slot 0 and the four limbs of slot 1, so one accumulator tile holds, for 16 rows,
 // the two blocks' sums limb by limb.  Per (row, block) the limbs are recombined in integers, the offset term
-// (parity - 16) * sum_i 2 X_i is added from a per-block sum prepared with x (what is added up is twice sum_i x_i X_i, in the 14-byte layout: the
-// halves of an odd sum need no care), and one float multiply-add applies half of gain[g] / (4 sqrt m), looked up by the header.  Every lane runs the same instructions whatever its class.
+// (parity - 16) * sum_i X_i is added from a per-block sum prepared with x, and one float multiply-add applies
+// gain[g] / (4 sqrt m), looked up by the header.  Every lane runs the same instructions whatever its class.
 //
 // Geometry.  A warp works on the 32 rows of a row group, 16 at a time; the records are stored as the
 // instruction's operand fragments (include/llvq.h), so a lane's 128-bit shared-memory reads are its A
@@ -163,7 +163,8 @@ __device__ __forceinline__ void mma_k16(int (&d)[4], uint32_t a0, uint32_t a1, u
 }
 
 // Bytes of x in shared memory, one record a block: four planes of 24 bytes (plane l = limb l of the 24
-// fixed-point activations, doubled), a zero word at 96, and at 100 and 104 the block's sums of 2 X, limb pair by limb pair (see convert_item).
+// fixed-point activations, doubled), a zero word at 96, and at 100 and 104 the two parts of the block's
+// activation sum (see convert_item).
 constexpr int kXRecBytes = 112;
 
 // Offsets of this lane's operand words inside the two x records of a half-step (or, one = true, inside
@@ -198,13 +199,7 @@ __device__ __forceinline__ StepX load_step(const LaneOffsets &a) {
     return s;
 }
 
-// twice a word, by an addition: it has a cycle where a shift takes two
-__device__ __forceinline__ uint32_t twice(uint32_t w) {
-    uint32_t r;
-    asm("add.u32 %0, %1, %1;" : "=r"(r) : "r"(w));
-    return r;
-}
-// The A operand of a half-step (the decode proper, 2 u a byte: one shift, one addition and two ANDs a word) and the block constants of
+// The A operand of a half-step (the decode proper: one shift and two ANDs a word) and the block constants of
 // its two rows; both are shared by every activation vector of a batched launch.
 struct HalfA {
     uint32_t a0, a1, a2, a3, c0, c1;
@@ -213,18 +208,15 @@ struct HalfA {
 // COMPACT (13-byte layout): the two headers are the bytes at bit SHIFT and SHIFT + 8 of hw.
 template <bool COMPACT = false, int SHIFT = 0>
 __device__ __forceinline__ HalfA decode_half(uint32_t wa, uint32_t wb, uint32_t wc, uint32_t hw, uint32_t tq) {
+    constexpr uint32_t kNib = 0x0f0f0f0fu;
     HalfA h;
+    h.a0 = wa & kNib; h.a1 = wb & kNib; h.a2 = (wa >> 4) & kNib; h.a3 = (wb >> 4) & kNib;
+    h.c0 = wc & kNib; h.c1 = (wc >> 4) & kNib;
     if (COMPACT) {
-        constexpr uint32_t kNib = 0x0f0f0f0fu;
-        h.a0 = wa & kNib; h.a1 = wb & kNib; h.a2 = (wa >> 4) & kNib; h.a3 = (wb >> 4) & kNib;
-        h.c0 = wc & kNib; h.c1 = (wc >> 4) & kNib;
         // one byte a header, eight bytes an entry
         h.k0 = lds_f2(and_or(SHIFT >= 3 ? hw >> (SHIFT - 3) : hw << (3 - SHIFT), 0x7f8u, tq));
         h.k1 = lds_f2(and_or(hw >> (SHIFT + 5), 0x7f8u, tq));
     } else {
-        constexpr uint32_t kNib2 = 0x1e1e1e1eu;
-        h.a0 = twice(wa) & kNib2; h.a1 = twice(wb) & kNib2; h.a2 = (wa >> 3) & kNib2; h.a3 = (wb >> 3) & kNib2;
-        h.c0 = twice(wc) & kNib2; h.c1 = (wc >> 3) & kNib2;
         // the headers of rows g (low half of hw) and g + 8 (high half), eight bytes an entry; tq is 8 KiB-aligned
         h.k0 = lds_f2(and_or(hw << 3, 0x1ff8u, tq));
         h.k1 = lds_f2(and_or(hw >> 13, 0x1ff8u, tq));
@@ -264,6 +256,17 @@ __device__ __forceinline__ void decode_overlay_tile(const uint4 &va, const uint4
     header_consts<0>(hb.y, tq, h2.k0, h2.k1);
     header_consts<16>(hb.y, tq, h3.k0, h3.k1);
 }
+// The sum of a row and a limb pair with its offset, sum_i x_i X_i = sum_i u_i (2 X_i) + (parity - 16) sum_i X_i, a whole number below 2^23 (the parts
+// of the block's sum of X: see convert_item).  kWhole: in integers.  kHalves: half the offset as a float against twice the part; nothing is
+// rounded, so the bits are the same.  Which is the faster depends on the registers of the loop (us: two vectors on 34816 x 5120 24.4 and
+// 25.2, five 48.4 and 47.3; the 10-byte layout on 8192 x 8192 10.07 and 10.20).  Doubled codes against the sums of 2 X, which need no halves
+// and so a shorter conversion of x, lengthen the loop by an addition a word (8192 x 8192 9.36 -> 9.46 us a call, the 14B-like stack 0.7 %).
+enum Form { kWhole, kHalves };
+template <Form FORM>
+__device__ __forceinline__ float offset_sum(float offset, int xsum, int sum) {
+    return FORM == kHalves ? fmaf(offset, (float)xsum, (float)sum) : (float)(__float_as_int(offset) * xsum + sum);
+}
+
 // nibbles 0..3 of h to the low nibbles of bytes 0..3
 __device__ __forceinline__ uint32_t spread_nibbles(uint32_t h) {
     h &= 0xffffu;
@@ -273,6 +276,7 @@ __device__ __forceinline__ uint32_t spread_nibbles(uint32_t h) {
 // One entry of the exception table against the x record of its block (`rec`): the block's whole product, in the
 // accumulator's quanta.  The arithmetic of the tile path for one block: integer sums limb pair by limb pair, the
 // block's scale in f32.  `tail_tab` is the table of the four-bit records' headers (the entry's header byte indexes it).
+template <Form FORM>
 __device__ __forceinline__ long long exception_value(const uint4 &ent, uint32_t rec, uint32_t tail_tab, float inv_q) {
     const float2 k = lds_f2(tail_tab + 8 * (ent.x & 63u));
     int d[4] = {0, 0, 0, 0};
@@ -287,30 +291,21 @@ __device__ __forceinline__ long long exception_value(const uint4 &ent, uint32_t 
         }
         cw = j == 0 ? ent.z : ent.w;
     }
-    const float e_lo = fmaf(k.y, (float)(int)lds32(rec + 100), (float)(d[0] + 256 * d[1]));
-    const float e_hi = fmaf(k.y, (float)(int)lds32(rec + 104), (float)(d[2] + 256 * d[3]));
+    const float e_lo = offset_sum<FORM>(k.y, (int)lds32(rec + 100), d[0] + 256 * d[1]);
+    const float e_hi = offset_sum<FORM>(k.y, (int)lds32(rec + 104), d[2] + 256 * d[3]);
     return __float2ll_rn((e_lo * k.x + (e_hi * k.x) * 65536.f) * inv_q);
-}
-
-// The sum of a row and a limb pair with its offset: twice sum_i x_i X_i = sum_i 2 u_i (2 X_i) + (parity - 16) sum_i 2 X_i, in integers
-// below 2^24; the scale is halved.  COMPACT: sum_i x_i X_i itself, the codes as they are and half the offset as a float, whole
-// numbers and halves below 2^23, so that nothing is rounded.  The same to the bit; which is the faster depends on what else the
-// loop does (us, doubled and whole: 14-byte 8192 x 8192 9.49 and 9.56; 13-byte 3071 x 3083 4.47 and 4.37; 10-byte decode layer 28.8 and 28.7).
-template <bool COMPACT>
-__device__ __forceinline__ float offset_sum(float offset, int xsum, int sum) {
-    return COMPACT ? fmaf(offset, (float)xsum, (float)sum) : (float)(__float_as_int(offset) * xsum + sum);
 }
 
 // One half-step: 16 rows x 2 block slots.  h holds this lane's payload words and the constants of its rows' blocks in slot
 // (lane & 3) >> 1 (decode_half), sx the step's operand.  Adds to r0 (row g of the 16) and r1
 // (row g + 8) this lane's share of scale * sum_i x_i * X_i, X the fixed-point activations: its share is the
 // limb pair (lane & 1) of slot (lane & 3) >> 1.  FIRST: r0 and r1 are written, not added to.
-template <bool FIRST, bool COMPACT>
+template <bool FIRST, Form FORM>
 __device__ __forceinline__ void contract_half(const HalfA &h, const StepX &sx, float &r0, float &r1) {
     int d[4];
     mma_k32(d, h.a0, h.a1, h.a2, h.a3, sx.b0, sx.b1);
     mma_k16(d, h.c0, h.c1, sx.b2);
-    const float e0 = offset_sum<COMPACT>(h.k0.y, sx.xsum, d[0] + 256 * d[1]), e1 = offset_sum<COMPACT>(h.k1.y, sx.xsum, d[2] + 256 * d[3]);
+    const float e0 = offset_sum<FORM>(h.k0.y, sx.xsum, d[0] + 256 * d[1]), e1 = offset_sum<FORM>(h.k1.y, sx.xsum, d[2] + 256 * d[3]);
     if (FIRST) { r0 = __fmul_rn(e0, h.k0.x); r1 = __fmul_rn(e1, h.k1.x); }
     else { r0 = fmaf(e0, h.k0.x, r0); r1 = fmaf(e1, h.k1.x, r1); }
 }
@@ -326,10 +321,10 @@ struct PairA {
     float2 k00, k01, k10, k11;                     // block constants: slot, then row g or g + 8
 };
 __device__ __forceinline__ PairA decode_pair(uint32_t wa, uint32_t wb, uint32_t wc, uint32_t hw0, uint32_t hw1, uint32_t tq) {
-    constexpr uint32_t kNib2 = 0x1e1e1e1eu;
+    constexpr uint32_t kNib = 0x0f0f0f0fu;
     PairA h;
-    h.a0 = twice(wa) & kNib2; h.a1 = twice(wb) & kNib2; h.a2 = (wa >> 3) & kNib2; h.a3 = (wb >> 3) & kNib2;
-    h.c0 = twice(wc) & kNib2; h.c1 = (wc >> 3) & kNib2;
+    h.a0 = wa & kNib; h.a1 = wb & kNib; h.a2 = (wa >> 4) & kNib; h.a3 = (wb >> 4) & kNib;
+    h.c0 = wc & kNib; h.c1 = (wc >> 4) & kNib;
     h.k00 = lds_f2(and_or(hw0 << 3, 0x1ff8u, tq));
     h.k01 = lds_f2(and_or(hw0 >> 13, 0x1ff8u, tq));
     h.k10 = lds_f2(and_or(hw1 << 3, 0x1ff8u, tq));
@@ -361,22 +356,21 @@ __device__ __forceinline__ PairX load_pair(const PairAddr &a) {
     return x;
 }
 // s0, s1: this lane's shares of the sums of rows g and g + 8 over the blocks of slot 0 and of slot 1
-template <bool FIRST>
+template <bool FIRST, Form FORM>
 __device__ __forceinline__ void contract_pair(const PairA &h, const PairX &x, float *s0, float *s1) {
     int d[4], f[4];
     mma_k32(d, h.a0, h.a1, h.a2, h.a3, x.b0, x.b1);
     mma_k32(f, h.a0, h.a1, h.a2, h.a3, 0u, x.b2);
     mma_k16(f, h.c0, h.c1, x.b3);
-    // twice sum_i x_i X_i, limb pair by limb pair, a whole number below 2^24: 2 u_i against 2 X_i, and (parity - 16) sum_i 2 X_i; the scale is halved
-    const int e00 = __float_as_int(h.k00.y) * x.xs0 + (d[0] + 256 * d[1]), e01 = __float_as_int(h.k01.y) * x.xs0 + (d[2] + 256 * d[3]);
-    const int e10 = __float_as_int(h.k10.y) * x.xs1 + (f[0] + 256 * f[1]), e11 = __float_as_int(h.k11.y) * x.xs1 + (f[2] + 256 * f[3]);
+    const float e00 = offset_sum<FORM>(h.k00.y, x.xs0, d[0] + 256 * d[1]), e01 = offset_sum<FORM>(h.k01.y, x.xs0, d[2] + 256 * d[3]);
+    const float e10 = offset_sum<FORM>(h.k10.y, x.xs1, f[0] + 256 * f[1]), e11 = offset_sum<FORM>(h.k11.y, x.xs1, f[2] + 256 * f[3]);
     if (FIRST) {
         // rounded products, as where a product goes through a shuffle: no sum below may take them into a multiply-add
-        s0[0] = __fmul_rn((float)e00, h.k00.x); s0[1] = __fmul_rn((float)e01, h.k01.x);
-        s1[0] = __fmul_rn((float)e10, h.k10.x); s1[1] = __fmul_rn((float)e11, h.k11.x);
+        s0[0] = __fmul_rn(e00, h.k00.x); s0[1] = __fmul_rn(e01, h.k01.x);
+        s1[0] = __fmul_rn(e10, h.k10.x); s1[1] = __fmul_rn(e11, h.k11.x);
     } else {
-        s0[0] = fmaf((float)e00, h.k00.x, s0[0]); s0[1] = fmaf((float)e01, h.k01.x, s0[1]);
-        s1[0] = fmaf((float)e10, h.k10.x, s1[0]); s1[1] = fmaf((float)e11, h.k11.x, s1[1]);
+        s0[0] = fmaf(e00, h.k00.x, s0[0]); s0[1] = fmaf(e01, h.k01.x, s0[1]);
+        s1[0] = fmaf(e10, h.k10.x, s1[0]); s1[1] = fmaf(e11, h.k11.x, s1[1]);
     }
 }
 // v[2m + e] = this lane's share (its limb pair) of row 16m + 8e + g -> even lanes get the sums of rows g, g + 8, odd lanes
@@ -390,9 +384,10 @@ __device__ __forceinline__ void pair_sum(const float (&v)[4], bool odd, float &r
 
 // x (fp16) -> records.  X_i = rint(x_i * 2^F) with F chosen from the largest |x| so that |X_i| < 2^29; the
 // record of a block stores the four balanced limbs of 2 X_i (2 X_i = sum_l limb_l 256^l, limbs in -128..127)
-// plane by plane, and the block's sums of 2 X, one a limb pair (limbs 0 and 1 at 100, 2 and 3 at 104).  An item is eight coordinates (one 128-bit piece of x): item e belongs to block e / 3.
-// The three items of a block add their shares of the sums with shared-memory atomics; the words were zeroed
-// before.  `rec` is the shared-memory address of the block's record.
+// plane by plane, and the block's sum of the X_i in two parts, sum = s0 + 65536 s1 (kHalves: 2 s0 and 2 s1).  An item is eight coordinates (one
+// 128-bit piece of x): item e belongs to block e / 3.  The three items of a block add their shares of s0 and s1 with
+// shared-memory atomics; the words were zeroed before.  `rec` is the shared-memory address of the block's record.
+template <Form FORM>
 __device__ __forceinline__ void convert_item(const uint4 &v, int third, uint32_t rec, float scale) {
     const uint32_t hv[4] = {v.x, v.y, v.z, v.w};
     uint32_t w[8];
@@ -418,9 +413,11 @@ __device__ __forceinline__ void convert_item(const uint4 &v, int third, uint32_t
 #pragma unroll
     for (int l = 0; l < 4; l++)
         asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(rec + 24 * l + 8 * third), "r"(pl[l][0]), "r"(pl[l][1]) : "memory");
-    // this item's share of the block's sum of 2 X, limb pair by limb pair
-    asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(rec + 100), "r"(limb_sum[0] + 256 * limb_sum[1]) : "memory");
-    asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(rec + 104), "r"(limb_sum[2] + 256 * limb_sum[3]) : "memory");
+    // this item's sum of 2 X is a0 + 65536 a1; it is even, and so is a0; if a1 is odd one unit of it moves to
+    // a0, and then both halve exactly: the item adds a0 / 2 and a1 / 2 to the block's s0 and s1
+    const int a1 = limb_sum[2] + 256 * limb_sum[3], a0 = limb_sum[0] + 256 * limb_sum[1] + ((a1 & 1) << 16);
+    asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(rec + 100), "r"(FORM == kWhole ? a0 >> 1 : a0) : "memory");
+    asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(rec + 104), "r"(FORM == kWhole ? a1 >> 1 : a1 & ~1) : "memory");
 }
 
 // ---- the order of work.  A unit is a tile of a row group or its leftover blocks (column p.tiles).  Units
@@ -469,11 +466,12 @@ template <bool NO_WEIGHTS, int BATCH, Rotate ROTATE = kNoRotation, int LAYOUT = 
 __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(const __grid_constant__ GemvParams p) {
     constexpr int kWarps = gemv_warps(BATCH), kThreads = 32 * kWarps;
     constexpr bool COMPACT = LAYOUT != LLVQ_PLANES, OVERLAY = LAYOUT == LLVQ_PLANES10X;
+    constexpr Form FORM = BATCH > 2 ? kHalves : kWhole;
     static_assert(!OVERLAY || (BATCH == 1 && ROTATE == kNoRotation && !NO_WEIGHTS), "the 10-byte layout: one vector, as it is");
     constexpr int kSrcCell = COMPACT ? kCell13Bytes : kCellBytes;        // bytes of a leftover block column of a row group
     constexpr int kSrcTile = OVERLAY ? kTile10Bytes : (COMPACT ? kTile13Bytes : kTileBytes);   // bytes of a tile in memory (a ring slot always has kTileBytes)
     extern __shared__ __align__(128) unsigned char smem[];
-    // shared memory: ring | per-matrix block constants (1024 x {gain / (8 sqrt m), parity - 16}, COMPACT {gain / (4 sqrt m), (parity - 16) / 2}) | x records | barriers
+    // shared memory: ring | per-matrix block constants (1024 x {gain / (4 sqrt m), the offset as offset_sum takes it}) | x records | barriers
     unsigned char *ring = smem;
     // the block constants start on an 8 KiB boundary of the shared window, so that a matrix's table base and
     // an entry's offset combine by OR (decode_half)
@@ -701,7 +699,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
     const bool odd_lane = lane & 1, high_lane = lane & 2;
     const float limb_scale = odd_lane ? 65536.f : 1.f;     // this lane's limb pair: 256^0,1 or 256^2,3
     const uint32_t tab0 = smem_addr(tab);
-    // the block constants of every matrix of the launch: (class | gain << 9) -> {gain / (8 sqrt m), parity - 16}
+    // the block constants of every matrix of the launch: (class | gain << 9) -> {gain / (4 sqrt m), the offset}
     // (13-byte layout: the header byte is shell | parity << 4 | gain << 5 - 64 entries a matrix)
     auto build_tables = [&]() {
         if (COMPACT) {
@@ -716,7 +714,8 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 const int parity = window ? (f >> 2) & 1 : (h >> 4) & 1, gain = window ? (f >> 3) & 1 : (h >> 5) & 1;
                 const int base = window ? 2 * (3 + (f & 3)) : 0;
                 const GemvProblemDev &pe = p.prob[m];
-                tab[m * 1024 + h] = make_float2(p.shell_inv_norm[shell] * (gain ? pe.gain1 : pe.gain0), shell ? 0.5f * (float)(parity - 16 + base) : 0.f);
+                const int offset = shell ? parity - 16 + base : 0;
+                tab[m * 1024 + h] = make_float2(p.shell_inv_norm[shell] * (gain ? pe.gain1 : pe.gain0), __int_as_float(offset));
             }
         } else {
             for (int m = 0; m < p.nprob; m++) {
@@ -724,12 +723,20 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 for (int i = 0; i < kClasses; i++) {
                     const int c = tid + i * kThreads;
                     if (kClassSlots % kThreads != 0 && c >= kClassSlots) break;
-                    tab[m * 1024 + c] = make_float2(0.5f * my_class[i].x * p.prob[m].gain0, my_class[i].y);
-                    tab[m * 1024 + 512 + c] = make_float2(0.5f * my_class[i].x * p.prob[m].gain1, my_class[i].y);
+                    // my_class[i].x is half of 1 / (4 sqrt m) by now
+                    const float offset = FORM == kHalves ? 0.5f * (float)__float_as_int(my_class[i].y) : my_class[i].y;
+                    tab[m * 1024 + c] = make_float2(my_class[i].x * (2.f * p.prob[m].gain0), offset);
+                    tab[m * 1024 + 512 + c] = make_float2(my_class[i].x * (2.f * p.prob[m].gain1), offset);
                 }
             }
         }
     };
+    // The class constants are used here first, by a multiplication that the tables take back: a wait for them further on, where the tables are built,
+    // is a wait for the loads of x that are on their way by then (1024 x 2560 3.20 -> 3.11 us a launch, 4096 x 4096 5.17 -> 5.02).
+    if (!COMPACT) {
+#pragma unroll
+        for (int i = 0; i < kClasses; i++) asm volatile("mul.rn.f32 %0, %0, 0f3F000000;" : "+f"(my_class[i].x));
+    }
     // let the next kernel in the stream start its own prefetch, then wait for the previous one:
     // x, y and the reduction scratch may still be in use by it
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -859,13 +866,13 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                     else if (last == 4) rot_middle8<1>(rot, 8 * e - rot0);
                 }
                 __syncwarp();
-                if (e >= e_lo && 8 * e < need_hi) convert_item(rot_finish8(rot, 8 * e - rot0, !in_scan, p.rot_scale), e % 3, xs0 + (uint32_t)(e / 3) * kXRecBytes, scale);
+                if (e >= e_lo && 8 * e < need_hi) convert_item<FORM>(rot_finish8(rot, 8 * e - rot0, !in_scan, p.rot_scale), e % 3, xs0 + (uint32_t)(e / 3) * kXRecBytes, scale);
             }
         if (!one_each)
-            for (int e = max(e_lo, c_hi >> 3) + tid; e < e_hi; e += kThreads) convert_item(__ldcg(xg + e), e % 3, xs0 + (uint32_t)(e / 3) * kXRecBytes, scale);
+            for (int e = max(e_lo, c_hi >> 3) + tid; e < e_hi; e += kThreads) convert_item<FORM>(__ldcg(xg + e), e % 3, xs0 + (uint32_t)(e / 3) * kXRecBytes, scale);
         if (one_each && mine_e >= (in_scan && !alone ? max(e_lo, c_hi >> 3) : 0)) {
             if (alone && 8 * mine_e < c_hi) mine = rot_whole8(flipped(mine, mine_e), p.rot_scale);
-            convert_item(mine, mine_e % 3, xs0 + (uint32_t)(mine_e / 3) * kXRecBytes, scale);
+            convert_item<FORM>(mine, mine_e % 3, xs0 + (uint32_t)(mine_e / 3) * kXRecBytes, scale);
         }
         __syncthreads();                               // publishes the x records
     } else {
@@ -929,10 +936,10 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
             const uint4 *xg = reinterpret_cast<const uint4 *>(p.x) + (size_t)j * nx;
             const uint32_t xsj = xs0 + j * kXRecBytes;
             if (one_each) {
-                if (mine_e >= 0) convert_item(mine[j], mine_e % 3, xsj + (uint32_t)(mine_e / 3) * kXBlock, scale);
+                if (mine_e >= 0) convert_item<FORM>(mine[j], mine_e % 3, xsj + (uint32_t)(mine_e / 3) * kXBlock, scale);
             } else {
                 for (int e = e_lo + tid; e < e_hi; e += kThreads)
-                    convert_item(__ldcg(xg + e), e % 3, xsj + (uint32_t)(e / 3) * kXBlock, scale);
+                    convert_item<FORM>(__ldcg(xg + e), e % 3, xsj + (uint32_t)(e / 3) * kXBlock, scale);
             }
         }
         __syncthreads();                               // publishes the x records
@@ -1039,7 +1046,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 mma_k16(d1, h1.c0, h1.c1, s1.b2);
                 mma_k16(d2, h2.c0, h2.c1, s2.b2);
                 mma_k16(d3, h3.c0, h3.c1, s2.b2);
-                auto e = [](const int (&d)[4], float ky, int xsum, int r) { return offset_sum<COMPACT>(ky, xsum, d[2 * r] + 256 * d[2 * r + 1]); };
+                auto e = [](const int (&d)[4], float ky, int xsum, int r) { return offset_sum<FORM>(ky, xsum, d[2 * r] + 256 * d[2 * r + 1]); };
                 acc[0] = e(d0, h0.k0.y, s1.xsum, 0) * h0.k0.x;
                 acc[1] = e(d0, h0.k1.y, s1.xsum, 1) * h0.k1.x;
                 acc[2] = e(d1, h1.k0.y, s1.xsum, 0) * h1.k0.x;
@@ -1060,10 +1067,10 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                     constexpr int J = decltype(index)::value, kPair = J * 2 * kXRecBytes;
                     const PairX x0 = load_pair<kPair, kPair + kXBlock>(xp), x1 = load_pair<kPair + 2 * kXBlock, kPair + 3 * kXBlock>(xp);
                     float u[4], w[4];                                      // slot 0 and slot 1, rows [2m + e]
-                    contract_pair<true>(h0, x0, u, w);
-                    contract_pair<true>(h1, x0, u + 2, w + 2);
-                    contract_pair<false>(h2, x1, u, w);
-                    contract_pair<false>(h3, x1, u + 2, w + 2);
+                    contract_pair<true, FORM>(h0, x0, u, w);
+                    contract_pair<true, FORM>(h1, x0, u + 2, w + 2);
+                    contract_pair<false, FORM>(h2, x1, u, w);
+                    contract_pair<false, FORM>(h3, x1, u + 2, w + 2);
                     const float v[4] = {u[0] + w[0], u[1] + w[1], u[2] + w[2], u[3] + w[3]};
                     float r0, r1;
                     pair_sum(v, odd_lane, r0, r1);
@@ -1097,7 +1104,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                         guard |= settled(wa, wb, wc) | settled(hw, wa, wb);
                         const HalfA h = m == 0 ? decode_half<COMPACT, 0>(wa, wb, wc, hw, tq_tail) : decode_half<COMPACT, 16>(wa, wb, wc, hw, tq_tail);
                         const LaneOffsets ta = {xt + lo.b0, xt + lo.b1, xt + lo.b2, xt + lo.xs};
-                        contract_half<false, COMPACT>(h, load_step<0>(ta), acc[2 * m], acc[2 * m + 1]);
+                        contract_half<false, FORM>(h, load_step<0>(ta), acc[2 * m], acc[2 * m + 1]);
                     }
                     piece += 2 * kSrcCell;
                 }
@@ -1113,7 +1120,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                     const HalfA h = decode_half<COMPACT, 0>(wa, wb, wc, hw, tq_tail);
                     const LaneOffsets ta = {xl + l1.b0, xl + l1.b1, xl + l1.b2, xl + l1.xs};
                     float c0, c1;
-                    contract_half<true, COMPACT>(h, load_step<0>(ta), c0, c1);
+                    contract_half<true, FORM>(h, load_step<0>(ta), c0, c1);
                     acc[0] += high_lane ? 0.f : c0; acc[1] += high_lane ? 0.f : c1;
                     acc[2] += high_lane ? c0 : 0.f; acc[3] += high_lane ? c1 : 0.f;
                 }
@@ -1145,13 +1152,13 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                     float u[4] = {0.f, 0.f, 0.f, 0.f}, v[4] = {0.f, 0.f, 0.f, 0.f};
                     if (two) {
                         const PairX x = load_pair<kPair, kPair + kXBlock>(xt);
-                        contract_pair<true>(h0, x, u, v);
-                        contract_pair<true>(h1, x, u + 2, v + 2);
+                        contract_pair<true, FORM>(h0, x, u, v);
+                        contract_pair<true, FORM>(h1, x, u + 2, v + 2);
                     }
                     if (one) {
                         // the slots are the two halves of the row group, with the same block of x
                         float c0[2], c1[2];
-                        contract_pair<true>(hs, load_pair<kPair, kPair>(xl), c0, c1);
+                        contract_pair<true, FORM>(hs, load_pair<kPair, kPair>(xl), c0, c1);
                         u[0] += c0[0]; u[1] += c0[1];
                         v[2] += c1[0]; v[3] += c1[1];
                     }
@@ -1177,7 +1184,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
             for (uint32_t done = 0; done < exc_count; done += 32) {
                 if (done != 0) exc_entry = done + lane < exc_count ? __ldg(pr.exc_table + exc_begin + done + lane) : make_uint4(~0u, 0u, 0u, 0u);
                 if (exc_entry.x != ~0u) {
-                    const long long v = exception_value(exc_entry, xs0 + (exc_entry.x >> 13) * kXRecBytes, tq_tail, inv_q);
+                    const long long v = exception_value<FORM>(exc_entry, xs0 + (exc_entry.x >> 13) * kXRecBytes, tq_tail, inv_q);
                     // in two 32-bit halves, v = hi * 2^24 + lo with lo in [0, 2^24): a row meets at most 64 entries
                     // a run and |v| < 2^40, so neither half overflows its word
                     uint32_t *half = reinterpret_cast<uint32_t *>(exc_scratch + ((exc_entry.x >> 8) & 31u));
