@@ -244,7 +244,7 @@ int llvq_expand(llvq_ctx *ctx, int layout, const uint64_t *codes, int64_t rows, 
  * m_b the shell of block b's class.  gain is a HOST pointer to two floats; the larger of their magnitudes
  * must be zero or lie in [2^-60, 2^60) (LLVQ_EINVAL otherwise: the fixed-point quantum is a power of two
  * formed from its exponent).  x is fp16, 16-byte
- * aligned; y is f32; x must be finite.  LLVQ_PLANES: x is taken as fixed point on a scale set by
+ * aligned; y is f32; x must be finite, and where an entry is not, every entry of y is NaN.  LLVQ_PLANES: x is taken as fixed point on a scale set by
  * the largest |x| (X_i = rint(x_i 2^F), |X_i| < 2^29; exact for every x_i within 2^-18 of the
  * largest, rounded to within 2^-29 of the largest below that), the inner sums over a block are integer and
  * exact, the per-block scale is applied in f32.  LLVQ_ONEHOT: f32 products and sums.  Either way a
@@ -260,7 +260,7 @@ int llvq_gemv(llvq_ctx *ctx, int layout, const void *layout_buf, const void *row
  * one pass (the records are read and decoded once for them); five to eight take two passes where the
  * context's scratch holds the sums of four only, or on a device of few multiprocessors, whose shared memory may hold the
  * records of four, or of two, only.  Each vector has its own fixed-point scale and its own accumulators, and y[j] is bit-identical to what
- * llvq_gemv returns for x[j].  Needs min(batch, 4) times the scratch of llvq_gemv (LLVQ_ESIZE
+ * llvq_gemv returns for x[j] (all NaN, and the others as ever, where x[j] is not finite).  Needs min(batch, 4) times the scratch of llvq_gemv (LLVQ_ESIZE
  * otherwise). */
 int llvq_gemv_batch(llvq_ctx *ctx, const void *layout_buf, const void *row_scale, const float *gain,
                     const void *x, float *y, int64_t rows, int64_t k_padded, int batch, void *stream);

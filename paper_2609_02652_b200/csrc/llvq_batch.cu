@@ -175,11 +175,6 @@ __device__ __forceinline__ void contract(const Half &h, const StepB &b, float2 (
 // the unit's sum of a row from its two slots' shares, as quad_sum of llvq_gemv.cu adds them
 __device__ __forceinline__ float row_sum(float2 s0, float2 s1) { return fmaf(s0.y + s1.y, 65536.f, s0.x + s1.x); }
 
-// largest |fp16| of both halves of a word, as max_abs_pair, but a NaN stays one
-__device__ __forceinline__ uint32_t max_abs_or_nan(uint32_t m, uint32_t x2) {
-    const __half2 r = __hmax2_nan(*reinterpret_cast<const __half2 *>(&m), __habs2(*reinterpret_cast<const __half2 *>(&x2)));
-    return *reinterpret_cast<const uint32_t *>(&r);
-}
 // x (FP16, eight coordinates: a third of a block) -> its two chunks of the record, the first of them at `at`.  Returns the third's share of the block's
 // activation sum, {sum L, sum H} but for a unit between the two.  2 rint(x scale) and the nearest multiple of 65536 come from additions of
 // 1.5 * 2^23: x scale is a whole number of eleven significant bits, which such an addition leaves as it is, or below 2^11.  H is
@@ -402,7 +397,7 @@ __global__ void __launch_bounds__(32 * batch_warps(SETS), 1) gemv_batch_kernel(c
         load();
         for (;;) {
 #pragma unroll
-            for (int i = 0; i < kInFlight; i++) m = max_abs_or_nan(max_abs_or_nan(max_abs_or_nan(max_abs_or_nan(m, v[i].x), v[i].y), v[i].z), v[i].w);
+            for (int i = 0; i < kInFlight; i++) m = max_abs_pair(max_abs_pair(max_abs_pair(max_abs_pair(m, v[i].x), v[i].y), v[i].z), v[i].w);
             if (e - lane >= nx) break;
             load();
         }
@@ -416,7 +411,7 @@ __global__ void __launch_bounds__(32 * batch_warps(SETS), 1) gemv_batch_kernel(c
     for (int w = warp; w < work; w += kWarps) {
         const Share q = w == warp ? first_share : share_of(w);
         const uint32_t most = most_at[q.vector];
-        const float scale = pow2f(43 - max((int)(most >> 10), 1));
+        const float scale = pow2f(29 - x_exponent(most));
         int b = 10 * q.part + my_block;
         const uint32_t rec = xrec + (uint32_t)b * kXBlock + (SETS > 1 ? (q.vector >> 2) * kSetBytes : 0);
         uint32_t at = rec + ((q.vector >> 1) & 1) * kHalfBytes + (q.vector & 1) * 16 + 64 * third, sums = rec + kSumsAt + 8 * (q.vector & 3);
@@ -431,7 +426,7 @@ __global__ void __launch_bounds__(32 * batch_warps(SETS), 1) gemv_batch_kernel(c
             own0 = own1;
             own1 = load_piece(q, b + 20 * each);
             float2 s = make_float2(0.f, 0.f);
-            if (here) s = convert_third(now, at, scale, most < 0x7c00u, most_at + LLVQ_MAX_BATCH);
+            if (here) s = convert_third(now, at, scale, most < kInfinity16, most_at + LLVQ_MAX_BATCH);
             const float lo1 = __shfl_down_sync(0xffffffffu, s.x, 1), lo2 = __shfl_down_sync(0xffffffffu, s.x, 2);
             const float hi1 = __shfl_down_sync(0xffffffffu, s.y, 1), hi2 = __shfl_down_sync(0xffffffffu, s.y, 2);
             if (here && third == 0) {
@@ -448,9 +443,7 @@ __global__ void __launch_bounds__(32 * batch_warps(SETS), 1) gemv_batch_kernel(c
     const bool wide = most_at[LLVQ_MAX_BATCH] != 0u;
     // the last arrival of a row: `word` is the whole accumulator
     auto finish = [&](int v, int row, unsigned long long word, __half scale) {
-        const uint32_t most = most_at[v];
-        // a vector with an entry that is infinite or no number was taken as zeros: y must not look like a result
-        const float quantum = most < 0x7c00u ? pow2f(max((int)(most >> 10), 1) - 14 + pr.qexp_base) : __int_as_float(0x7fffffff);
+        const float quantum = x_factor(most_at[v]) * pow2f(pr.qexp_base);
         pr.y[(size_t)v * p.y_stride + row] = (float)((long long)(word & kSumMask) - (long long)p.units * kUnitBias) * (quantum * __half2float(scale));
         p.accum[(size_t)v * ((size_t)p.total_groups * 32) + row] = 0ull;           // ready for the next launch on this context
     };

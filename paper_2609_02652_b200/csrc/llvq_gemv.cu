@@ -93,7 +93,7 @@ __device__ __forceinline__ void warp_range(const GemvParams &p, int warp, int &u
 
 // Hands the warp's sum over `count` units of row group `group` to the row accumulators.
 __device__ __forceinline__ void deliver(const GemvParams &p, const GemvProblemDev &pr, int group, int lane,
-                                        long long sum, int count, int qexp, float row_scale) {
+                                        long long sum, int count, float quantum, float row_scale) {
     const int row = (group - pr.group_begin) * kRowsPerGroup + lane;
     if (row >= pr.rows) return;                      // padding rows of the last row group
     const unsigned long long addend = (unsigned long long)(sum + (long long)count * kUnitBias) + ((unsigned long long)count << kCountShift);
@@ -101,7 +101,7 @@ __device__ __forceinline__ void deliver(const GemvParams &p, const GemvProblemDe
     const unsigned long long old = atomicAdd(slot, addend);
     if ((int)(old >> kCountShift) + count == p.units) {
         const long long total = (long long)((old + addend) & kSumMask) - (long long)p.units * kUnitBias;
-        pr.y[row] = ((float)total * pow2f(qexp)) * row_scale;
+        pr.y[row] = ((float)total * quantum) * row_scale;
         *slot = 0ull;                                // ready for the next launch on this context
     }
 }
@@ -746,8 +746,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
     // pieces of x this CTA needs stay in registers meanwhile and then become fixed-point records on the scale
     // 2^(29 - xexp).
     bool failed = false;
-    int xexp[BATCH];
-    [[maybe_unused]] float x_scale;                    // ROTATE: 2^xexp
+    float x_scale[BATCH];                              // 2^xexp, or NaN (x_factor)
     if constexpr (ROTATE != kNoRotation) {
         // The rotated vector's largest magnitude is not known before it is rotated, but every rotated coordinate is
         // a unit-norm combination of its block, so |x'_k| <= ||x||_2: the scan sums the squares instead of taking
@@ -841,6 +840,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
         }
         if (!in_scan || rf.stride > last) __syncthreads();
         if (in_scan) fill_ring();
+        int xexp;
         {
             // every thread of every CTA adds the sixteen sums in the same order
             float total = __uint_as_float(warp_max[lane & (kWarps - 1)]);
@@ -849,12 +849,12 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
             // total * 1.0625 covers the rounding of the sum and of the FP16 results: it is below 2^e2, so
             // every |x'| is below 2^ceil(e2 / 2)
             const int e2 = (int)((__float_as_uint(total * 1.0625f) >> 23) & 255u) - 126;
-            xexp[0] = max((e2 + 1) >> 1, -13);
+            xexp = max((e2 + 1) >> 1, -13);
             // with an entry that is infinite or no number, all rotated entries are zero on the scale of their norm: y must not
             // look like a result, so its scale is NaN
-            x_scale = total - total == 0.f ? pow2f(xexp[0]) : __int_as_float(0x7fffffff);
+            x_scale[0] = total - total == 0.f ? pow2f(xexp) : __int_as_float(0x7fffffff);
         }
-        const float scale = pow2f(29 - xexp[0]);
+        const float scale = pow2f(29 - xexp);
         // rotated pieces: from the exact sums; pieces past the rotated length: as they are (the one this thread
         // met in the scan, or read again when the share is too wide for that)
         if (!alone)
@@ -930,9 +930,9 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
 #pragma unroll
         for (int j = 0; j < BATCH; j++) {
             if (BATCH > 2 && j >= p.batch) break;
-            const uint32_t most = warp_max[j * kWarps + (lane < kWarps ? lane : 0)];
-            xexp[j] = max((int)(__reduce_max_sync(0xffffffffu, most) >> 10), 1) - 14;
-            const float scale = pow2f(29 - xexp[j]);
+            const uint32_t most = __reduce_max_sync(0xffffffffu, warp_max[j * kWarps + (lane < kWarps ? lane : 0)]);
+            x_scale[j] = x_factor(most);
+            const float scale = pow2f(29 - x_exponent(most));
             const uint4 *xg = reinterpret_cast<const uint4 *>(p.x) + (size_t)j * nx;
             const uint32_t xsj = xs0 + j * kXRecBytes;
             if (one_each) {
@@ -1204,8 +1204,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
         // with no records read (the control launch) every unit contributes zero
         n += run;
         if (BATCH == 1) {
-            const float quantum = ROTATE != kNoRotation ? pow2f(pr.qexp_base) * x_scale : pow2f(xexp[0] + pr.qexp_base);
-            hand_over(p, pr, p.accum, pr.y, cc.group, my_row, sum[0], run, quantum, row_scale, handed);
+            hand_over(p, pr, p.accum, pr.y, cc.group, my_row, sum[0], run, x_scale[0] * pow2f(pr.qexp_base), row_scale, handed);
         } else {
             // this lane's rows are 16 * (lane & 1) + g and the one eight further on, its vector of a pair (lane & 3) >> 1; all the
             // atomics are on their way before the first answer is looked at
@@ -1227,8 +1226,8 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 const int v = (j & ~1) + of_pair, e = j & 1;
                 if (v < p.batch && row_in + 8 * e < pr.rows && (int)(old[j] >> kCountShift) + run == p.units) {
                     const long long total = (long long)((old[j] + ((unsigned long long)sum[j] + counted)) & kSumMask) - (long long)p.units * kUnitBias;
-                    const int xe = of_pair ? xexp[(j & ~1) + 1] : xexp[j & ~1];
-                    pr.y[(size_t)v * p.y_stride + row_in + 8 * e] = (float)total * (pow2f(xe + pr.qexp_base) * scale[e]);
+                    const float quantum = (of_pair ? x_scale[(j & ~1) + 1] : x_scale[j & ~1]) * pow2f(pr.qexp_base);
+                    pr.y[(size_t)v * p.y_stride + row_in + 8 * e] = (float)total * (quantum * scale[e]);
                     slot[v * stride + 8 * e] = 0ull;       // ready for the next launch on this context
                 }
             }
@@ -1277,7 +1276,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_onehot_kernel(const __grid_c
     m = __reduce_max_sync(0xffffffffu, max(m & 0xffffu, m >> 16));
     if (lane == 0 && m) atomicMax(&xor_word, m);
     __syncthreads();
-    const int xexp = max((int)(xor_word >> 10), 1) - 14;
+    const int xexp = x_exponent(xor_word);
+    const bool finite = xor_word < kInfinity16;        // where it is not, no product is either, and none may reach the accumulators
 
     int u0, n_units;
     warp_range(p, warp, u0, n_units);
@@ -1302,11 +1302,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_onehot_kernel(const __grid_c
             const float val[5] = {lv.x, lv.y, lv.z, lv.w, l4};
             s = fmaf(g, onehot_dot(v, val, xs + 24 * c), s);
         }
-        sum += __float2ll_rn(s * pow2f(-qexp));
+        if (finite) sum += __float2ll_rn(s * pow2f(-qexp));
         count++;
         if (++k == p.units || n + 1 == n_units) {
             const int row = (group - pr.group_begin) * kRowsPerGroup + lane;
-            deliver(p, pr, group, lane, sum, count, qexp, row < pr.rows ? __half2float(pr.row_scale[row]) : 0.f);
+            deliver(p, pr, group, lane, sum, count, x_factor(xor_word) * pow2f(pr.qexp_base), row < pr.rows ? __half2float(pr.row_scale[row]) : 0.f);
             sum = 0;
             count = 0;
             if (k == p.units) {

@@ -25,16 +25,22 @@ constexpr int kCountShift = 53;
 constexpr unsigned long long kSumMask = (1ull << kCountShift) - 1;
 constexpr long long kUnitBias = 1ll << 41;     // a unit's value is below 2^40 quanta in magnitude
 
-// running maximum of |fp16| over both halves of a word, kept as two 15-bit patterns.  The magnitude goes into the maximum's
+// running maximum of |fp16| over both halves of a word, kept as two 15-bit patterns; a NaN stays one.  The magnitude goes into the maximum's
 // instruction, which an AND of the bits did not: sixteen instructions less in the scan of x, which every launch waits for (us a launch in
 // a chain: 1024 x 2560 3.23 -> 3.19, 4096 x 4096 4.89 -> 4.84, 8192 x 8192 9.08 -> 9.01; two vectors on 4096 x 4096 6.37 -> 6.24)
 __device__ __forceinline__ uint32_t max_abs_pair(uint32_t m, uint32_t x2) {
-    const __half2 r = __hmax2(*reinterpret_cast<const __half2 *>(&m), __habs2(*reinterpret_cast<const __half2 *>(&x2)));
+    const __half2 r = __hmax2_nan(*reinterpret_cast<const __half2 *>(&m), __habs2(*reinterpret_cast<const __half2 *>(&x2)));
     return *reinterpret_cast<const uint32_t *>(&r);
 }
 
 // exact power of two as a float, |e| < 126
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }
+
+// 2^xexp, xexp the exponent that the largest |x| (FP16 bits) sets the fixed-point scale by: every |x| is below it.  NaN where an entry is infinite or no
+// number: such a vector's fixed-point activations mean nothing, and y, which has this factor, must not look like a result.
+constexpr uint32_t kInfinity16 = 0x7c00u;
+__device__ __forceinline__ int x_exponent(uint32_t most) { return max((int)(most >> 10), 1) - 14; }
+__device__ __forceinline__ float x_factor(uint32_t most) { return most < kInfinity16 ? pow2f(x_exponent(most)) : __int_as_float(0x7fffffff); }
 
 // ---- asynchronous copies: global -> shared, completion counted on an mbarrier in shared memory
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }

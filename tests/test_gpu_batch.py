@@ -91,3 +91,37 @@ def test_one_vector_that_is_not_finite(B, ctx, bad, batch):
     assert y[1].isnan().all() and torch.equal(y[[0, 2, batch - 1]], want[[0, 2, batch - 1]])
     assert torch.equal(B.gemv_batch(ctx, buf, case.d_scale, GAIN, X, case.rows, 24 * case.nb), want)
     B.status(ctx)
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("-inf"), float("nan")])
+@pytest.mark.parametrize("batch", [2, 3, 5, 6, 8])
+def test_not_finite_in_every_build(B, ctx, bad, batch):
+    """What is true of a vector that is not finite does not depend on how many go with it, nor on where among them it is."""
+    case = make_case(500, 24 * 53, seed=10)
+    buf = B.expand(ctx, 0, case.d_codes, case.rows, case.nb)
+    X = torch.stack([torch.roll(case.d_x, j) for j in range(batch)]).contiguous()
+    want = one_by_one(B, ctx, case, buf, X)
+    for at in (0, batch - 1):
+        broken = X.clone()
+        broken[at, 24 * 53 - 1 - at] = bad
+        y = B.gemv_batch(ctx, buf, case.d_scale, GAIN, broken, case.rows, 24 * case.nb)
+        others = [j for j in range(batch) if j != at]
+        assert y[at].isnan().all() and torch.equal(y[others], want[others])
+    assert torch.equal(B.gemv_batch(ctx, buf, case.d_scale, GAIN, X, case.rows, 24 * case.nb), want)
+    B.status(ctx)
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("-inf"), float("nan")])
+@pytest.mark.parametrize("layout", ["PLANES", "ONEHOT", "PLANES13", "PLANES10X"])
+def test_not_finite_in_every_layout(B, ctx, bad, layout):
+    """One vector alone: y is NaN, and the next launch finds the accumulators clean."""
+    case = make_case(200, 24 * 53, seed=11)
+    buf = B.expand(ctx, getattr(B, layout), case.d_codes, case.rows, case.nb)
+    call = lambda x: B.gemv(ctx, getattr(B, layout), buf, case.d_scale, GAIN, x, case.rows, 24 * case.nb)  # noqa: E731
+    want = call(case.d_x)
+    for at in (0, 700, 24 * 53 - 1):
+        broken = case.d_x.clone()
+        broken[at] = bad
+        assert call(broken).isnan().all()
+    assert want.isfinite().all() and torch.equal(call(case.d_x), want)
+    B.status(ctx)
