@@ -1678,9 +1678,14 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
     // meets two panels then has a piece of x for each of its twelve warps' threads, and none is read again, vector after vector
     // (five vectors, us with panels of 18 columns and of 15: 500 x 8192 12.3 and 10.0, two passes 10.7).  Vectors in sets of
     // four on a small matrix: of eight at most, for half the blocks of x to convert; the row groups' sums, twice as many, are added up by the CTA
-    // first (us with sixteen and eight: four vectors on 4096 x 4096 8.2 and 8.1, 1024 x 2560 5.7 and 5.2; eight 15.9 and 15.4, 10.2 and 8.7).
+    // first.  For three and four vectors as long as the first CTA's share, ten units above the mean (below), still goes to sixteen warps in
+    // halves of such panels; for seven and eight the conversion is twice the work and the line lies further out.  Us with
+    // sixteen columns and with eight, at so many units a multiprocessor: four vectors on 4096 x 4096 (37) 8.8 and 8.3, 4500 x 5120 (51) 10.1 and 9.1,
+    // 2560 x 9728 (55) 10.7 and 11.3, 5120 x 5120 (58) 10.4 and 11.0, 7000 x 4096 (64) 10.4 and 10.9, 8000 x 5120 (91) 12.2 and 12.6 (but 7000 x 5120 (80)
+    // 12.1 and 11.0); eight on 4096 x 4096 16.0 and 15.2, 5120 x 5120 17.7 and 16.8, 4096 x 8192 (74) 20.3 and 18.6, 7000 x 5120 (80) 19.7 and 18.8,
+    // 8000 x 5120 (91) 20.4 and 21.1, 8192 x 6144 (111) 22.4 and 24.3.
     constexpr int kPanelColumns = 16, kFewColumns = 8;
-    const bool few = batch_in_sets(p.batch) && p.total_units < 64 * sm_count;
+    const bool few = batch_in_sets(p.batch) && p.total_units < (batch_sets(p.batch) > 1 ? 84 : 54) * sm_count;
     const int columns = few ? kFewColumns : kPanelColumns, most = (p.units + (p.batch > 4 || few ? columns - 1 : columns / 2)) / columns, want = most > 1 ? most : 1;
     p.panel = (p.units + want - 1) / want;
     p.npanels = (p.units + p.panel - 1) / p.panel;

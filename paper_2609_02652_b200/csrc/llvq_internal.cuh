@@ -177,7 +177,8 @@ private:
 };
 
 // Three, four, seven and eight vectors have a kernel of their own, which takes them in sets of four (llvq_batch.cu).
-// Five and six would leave half of the second set idle (34816 x 5120, five: 51.7 us that way, 49.6 in pairs; 500 x 8192 10.9 and 9.9).
+// Five and six would leave half of the second set idle (us in sets and in pairs: five on 500 x 8192 10.8 and 8.3, 4096 x 4096 13.4 and 11.0,
+// 34816 x 5120 50.5 and 47.4; six on 1024 x 2560 7.2 and 6.1, 8192 x 8192 24.9 and 22.5).
 __host__ __device__ constexpr bool batch_in_sets(int batch) { return batch == 3 || batch == 4 || batch >= 7; }
 
 constexpr int kVectorsPerPass = 4;      // activation vectors a pass that llvq_gemv_plan describes carries at most
