@@ -36,13 +36,13 @@ from paper_2609_02652_b200 import datagen  # noqa: E402
 
 L2_BYTES = 126 * 1024 * 1024
 # DRAM bytes (read + write) per algorithmic byte of gemv_planes_kernel, from one ncu capture of the
-# 8192 x 8192 launch (profiles/gemv_planes_kernel_config4_8192x8192.txt); traffic grows in proportion
+# 8192 x 8192 launch (profiles/gemv_8192x8192.txt); traffic grows in proportion
 # to the records streamed, so a launch's traffic is its bytes times this.
 NCU_TRAFFIC_PER_ALGORITHMIC_BYTE = 39.362304 / 39.288864
 # from the same capture: warp instructions per block column (32 rows x 24 weights), and the share of issue
 # slots busy over the launch
-NCU_WARP_INSTR_PER_CELL = 5668779 / 87552
-NCU_ISSUE_BUSY_PCT = 54.4
+NCU_WARP_INSTR_PER_CELL = 5623111 / 87552
+NCU_ISSUE_BUSY_PCT = 57.0
 METRIC = "us_per_lattice_gemv"
 DISCARD_ROUNDS = 2
 
@@ -756,7 +756,7 @@ def main():
                          # the competing ceiling, from the ncu capture in profiles/ (8192 x 8192 launch): instruction issue
                          "secondary": {"bound": "issue", "warp_instructions_per_block_column": NCU_WARP_INSTR_PER_CELL,
                                        "issue_slots_busy_pct": NCU_ISSUE_BUSY_PCT,
-                                       "source": "profiles/gemv_planes_kernel_config4_8192x8192.txt"},
+                                       "source": "profiles/gemv_8192x8192.txt"},
                          "how": "algorithmic bytes of a step / median CUDA-event time of a step, averaged over its launches"},
             "cpu_baseline": cpu_baseline,
             "e2e": {"value": e2e_us, "unit": "us", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h, "us_min": e2e_min, "us_max": e2e_max,
