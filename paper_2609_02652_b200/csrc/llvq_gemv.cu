@@ -1678,15 +1678,17 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
     // meets two panels then has a piece of x for each of its twelve warps' threads, and none is read again, vector after vector
     // (five vectors, us with panels of 18 columns and of 15: 500 x 8192 12.3 and 10.0, two passes 10.7).  Vectors in sets of
     // four on a small matrix: of eight at most, for half the blocks of x to convert; the row groups' sums, twice as many, are added up by the CTA
-    // first.  For three and four vectors as long as the first CTA's share, ten units above the mean (below), still goes to sixteen warps in
-    // halves of such panels; for seven and eight the conversion is twice the work and the line lies further out.  Us with
-    // sixteen columns and with eight, at so many units a multiprocessor: four vectors on 4096 x 4096 (37) 8.8 and 8.3, 4500 x 5120 (51) 10.1 and 9.1,
-    // 2560 x 9728 (55) 10.7 and 11.3, 5120 x 5120 (58) 10.4 and 11.0, 7000 x 4096 (64) 10.4 and 10.9, 8000 x 5120 (91) 12.2 and 12.6 (but 7000 x 5120 (80)
-    // 12.1 and 11.0); eight on 4096 x 4096 16.0 and 15.2, 5120 x 5120 17.7 and 16.8, 4096 x 8192 (74) 20.3 and 18.6, 7000 x 5120 (80) 19.7 and 18.8,
-    // 8000 x 5120 (91) 20.4 and 21.1, 8192 x 6144 (111) 22.4 and 24.3.
+    // first.  For three and four vectors it stops short where the panels are of eight columns, not seven: from 54 units a multiprocessor on many a
+    // share no longer goes to sixteen warps in halves of a row group's stretch, which is when the sums are added up.  Us with sixteen columns and with eight,
+    // at so many units a multiprocessor: four vectors on 4096 x 4096 (37) 8.8 and 8.3, 4384 x 5120 (50) 9.9 and 9.1, 4896 x 5120 (56) 10.3 and 10.9, 2784 x
+    // 9728 (60) 11.4 and 11.5, 6624 x 4096 (60) 10.2 and 10.9, in sevens 13536 x 2000 (60) 11.2 and 9.7, 8608 x 3100 (60) 10.8 and 9.8; eight on
+    // 4096 x 4096 (37) 16.0 and 15.2, 5248 x 5120 (60) 18.1 and 16.8, 2208 x 12288 (60) 20.0 and 17.7, 7936 x 4096 (72) 18.5 and 19.3, 33568 x 1000 (78)
+    // 18.2 and 20.3.
     constexpr int kPanelColumns = 16, kFewColumns = 8;
-    const bool few = batch_in_sets(p.batch) && p.total_units < (batch_sets(p.batch) > 1 ? 84 : 54) * sm_count;
-    const int columns = few ? kFewColumns : kPanelColumns, most = (p.units + (p.batch > 4 || few ? columns - 1 : columns / 2)) / columns, want = most > 1 ? most : 1;
+    const int in_few = (p.units + kFewColumns - 1) / kFewColumns;                          // panels of eight at most, as equal as they come
+    const bool full = batch_sets(p.batch) == 1 && (p.units + in_few - 1) / in_few == kFewColumns;
+    const bool few = batch_in_sets(p.batch) && p.total_units < (full ? 54 : 64) * sm_count;
+    const int most = few ? in_few : (p.units + (p.batch > 4 ? kPanelColumns - 1 : kPanelColumns / 2)) / kPanelColumns, want = most > 1 ? most : 1;
     p.panel = (p.units + want - 1) / want;
     p.npanels = (p.units + p.panel - 1) / p.panel;
     p.div_panel = make_fastdiv((uint32_t)p.panel);
