@@ -144,15 +144,13 @@ LLVQ_HD uint32_t draw_position(uint32_t r, float ratio, uint32_t draws) {
     const uint32_t at = floor_product((float)r, ratio);
     return at < draws ? at : draws - 1u;
 }
-// The pair of rank r, from the entry at that position: the first rank of the pair there tells whether it was one too large.  Position 0 begins with
-// rank 0, so the loop ends; after one step, at that (a host test runs all the tables).  An `if` in its place: 17408 x 5120 into the
-// 10-byte layout 139.5 -> 140.2 us, 9728 x 2560 into the 14-byte layout 34.8 -> 34.6.
+// The pair of rank r, from the entry at that position: the first rank of the pair there tells whether it was one too large.  One step back is the
+// most there is (a host test runs all the tables), and the most that is taken, whatever a table holds: a loop that looked on until it
+// found the rank would not end on a table that does not hold it.  Against that loop, us: 9728 x 2560 34.8 -> 34.6, into the 13-byte layout 35.2 -> 34.7; 17408
+// x 5120 into the 10-byte layout 139.5 -> 140.2, 9728 x 2560 48.4 -> 48.2.
 LLVQ_HD uint64_t pair_drawn(const uint64_t *entry, uint32_t r) {
     uint64_t pair = *entry;
-#ifdef __CUDA_ARCH__
-#pragma unroll 1
-#endif
-    while (r < (uint32_t)pair) pair = *--entry;
+    if (r < (uint32_t)pair) pair = entry[-1];
     return pair;
 }
 

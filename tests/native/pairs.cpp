@@ -1,6 +1,7 @@
 // The expander's tables of pair draws, whole: for every multiset, every step and every ratio that leads there, the position estimated for the first and
-// the last rank of each pair.  Between those the estimate ascends, so the two hold it for all ranks.  Prints the pairs
-// looked at, the estimates that were one position too large, and those that were neither that nor right.
+// the last rank of each pair.  Between those the estimate ascends, so the two hold it for all ranks.  Then a table that names no rank, on which the
+// reader has to end all the same, one entry back.  Prints the pairs looked at, the estimates that were one position too
+// large, and those that were neither that nor right.
 #include <cstdio>
 #include <set>
 #include <vector>
@@ -53,6 +54,8 @@ int main() {
         first += (size_t)kOddSets * draws;
         ratios.swap(next);
     }
+    const uint64_t nowhere[3] = {7u, 0xffffffffu, 0xffffffffu};
+    wrong += pair_drawn(nowhere + 2, 5u) != nowhere[1];
     std::printf("%ld %ld %ld\n", pairs, above, wrong);
     return first == u.pairs.size() ? 0 : 1;
 }
