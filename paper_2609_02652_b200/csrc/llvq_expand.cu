@@ -12,7 +12,7 @@
 // 10-byte layout 171.  A lane a row with a 64-bit division a coordinate and candidate took 484 and 4700 (10-byte layout) us, one odd
 // coordinate at a time 45.  24 or 28 warps a CTA instead of 32: 47 and 50 us against 38.  A multiprocessor's memory that is not shared is the
 // L1 cache the lists are read through, so the shared tables are kept to 20 KB and a warp's scratch to 2 KB (with 51 and 3.6 KB
-// 33 % of the lists' sectors come from the cache, and 38 % now; with 104 KB of tables 53 us).  The gathers were 85 % of the
+// 33 % of the lists' sectors come from the cache, and 37 % now; with 104 KB of tables 53 us).  The gathers were 85 % of the
 // load unit's time: the parts of a class stand in tables of their own, where 32-byte records lay in one of four banks.
 #include "llvq_internal.cuh"
 #include "llvq_unrank.cuh"

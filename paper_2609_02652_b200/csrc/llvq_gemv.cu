@@ -314,8 +314,9 @@ __device__ __forceinline__ void contract_half(const HalfA &h, const StepX &sx, f
 // the other slot's positions zero in B.  Against one vector with block-diagonal B that is three instructions instead
 // of four for two vectors and two slots, and a row's sum lies in two lanes instead of four, so half the exchanges.
 // The price is that a lane looks up the headers of both slots; every vector shares that.  Two, five and six vectors go this way
-// (three, four, seven and eight: llvq_batch.cu).  Bound: latency, twelve warps for five and six.  Two vectors on 8192 x 8192: 11.9 us a launch, 12.5 a
-// vector at a time, its atomic waited for before the next vector's.
+// (three, four, seven and eight: llvq_batch.cu).  Bound: latency (4096 x 4096: issue slots 45 % busy
+// with two vectors, 44 % with five, whose twelve warps are three a scheduler).  Two vectors on 8192 x 8192: 11.8 us a launch, 12.5 a vector at a
+// time, its atomic waited for before the next vector's.
 struct PairA {
     uint32_t a0, a1, a2, a3, c0, c1;
     float2 k00, k01, k10, k11;                     // block constants: slot, then row g or g + 8
@@ -1755,7 +1756,7 @@ GemvLaunch gemv_plan(int layout, GemvParams &p, int sm_count) {
         return g;
     }
     // the kernel is built for 1, 2 and 6 (us, five vectors, against a build for eight whose fourth pair is skipped: 1024 x 2560 5.7 and 7.3,
-    // 8192 x 8192 22.3 and 24.9, 34816 x 5120 47.8 and 51.3); the room for x is asked for as for eight, and with it the line between one pass and two
+    // 8192 x 8192 22.2 and 24.9, 34816 x 5120 47.4 and 51.3); the room for x is asked for as for eight, and with it the line between one pass and two
     const int vectors = p.batch > 2 ? 8 : p.batch, warps = gemv_warps(vectors);
     const size_t records = ((size_t)p.xblocks * kXRecBytes * vectors + 127) / 128 * 128, raw = rot_first(p.rot_log2).stages ? ((size_t)p.rot_span * 2 + 127) / 128 * 128 : 0;
     g.smem = (size_t)warps * kSlots * kTileBytes + 8192 /* alignment of the tables */ + (size_t)p.nprob * 8192 + warps * kSlots * 8 + warps * 4 * vectors + 16;
@@ -1782,9 +1783,9 @@ int gemv_configure(const llvq_ctx *ctx) {
 }
 
 cudaError_t launch_gemv(int layout, const GemvParams &p, const GemvLaunch &g, bool no_weights, bool pdl, cudaStream_t s) {
-    // Us a launch in a chain, in pairs of vectors (8-bit limbs) and in sets of four: three vectors on 1024 x 2560 5.27 and 4.96, 4096 x 4096 8.41
-    // and 7.83, 500 x 8192 6.42 and 5.25, 34816 x 5120 35.7 and 32.1; four 5.57 and 5.24, 8.85 and 8.27, 6.93 and 5.96, 36.1 and 32.4; eight 9.65
-    // and 8.82, 16.5 and 15.1, 12.98 and 12.95, 62.1 and 53.9.  Two on 8192 x 8192 11.9 and 15.0; for five and six see batch_in_sets.
+    // Us a launch in a chain, in pairs of vectors (8-bit limbs, a build for four and one for eight) and in sets of four: three vectors on 1024 x 2560 5.28 and
+    // 4.96, four on 4096 x 4096 8.93 and 8.24, 34816 x 5120 36.2 and 32.0; eight on 1024 x 2560 9.62 and 8.67, 4096 x 4096 16.5 and 15.2, 34816 x 5120 62.2
+    // and 52.6.  Two on 8192 x 8192 11.8 and 15.0; for five and six see batch_in_sets.
     if (batch_in_sets(p.batch)) return launch_batch(p, g, pdl, s);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)g.grid);

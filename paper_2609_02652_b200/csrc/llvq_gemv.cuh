@@ -12,7 +12,7 @@ constexpr int kSlots = 2;                  // ring slots per warp
 constexpr int kEarlySlots = 1;             // slots filled before the wait for the previous kernel; the rest once x is being prepared
 
 // Vectors in sets of four (batch_in_sets): the bytes of a block's record of x a set, warps per CTA.  Two sets need more registers than
-// sixteen warps leave a thread (128): sixteen that spill take twice the time of twelve with 168.
+// sixteen warps leave a thread (128): sixteen that spill their sums take twice the time of twelve with 168, which spill 36 bytes.
 constexpr int kBatchSetBytes = 480;
 constexpr int kBatchSharedWords = sizeof(Cut) / 4 + LLVQ_MAX_BATCH + 1;        // what the CTA of such a launch shares besides: see gemv_batch_kernel
 __host__ __device__ constexpr int batch_sets(int batch) { return batch > 4 ? 2 : 1; }
