@@ -468,6 +468,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
     constexpr int kWarps = gemv_warps(BATCH), kThreads = 32 * kWarps;
     constexpr bool COMPACT = LAYOUT != LLVQ_PLANES, OVERLAY = LAYOUT == LLVQ_PLANES10X;
     constexpr Form FORM = BATCH > 2 ? kHalves : kWhole;
+    constexpr bool kTablesFirst = BATCH > 1 || OVERLAY;                  // the block constants are built before the wait for the previous kernel
     static_assert(!OVERLAY || (BATCH == 1 && ROTATE == kNoRotation && !NO_WEIGHTS), "the 10-byte layout: one vector, as it is");
     constexpr int kSrcCell = COMPACT ? kCell13Bytes : kCellBytes;        // bytes of a leftover block column of a row group
     constexpr int kSrcTile = OVERLAY ? kTile10Bytes : (COMPACT ? kTile13Bytes : kTileBytes);   // bytes of a tile in memory (a ring slot always has kTileBytes)
@@ -732,12 +733,16 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
             }
         }
     };
-    // The class constants are used here first, by a multiplication that the tables take back: a wait for them further on, where the tables are built,
-    // is a wait for the loads of x that are on their way by then (1024 x 2560 3.20 -> 3.11 us a launch, 4096 x 4096 5.17 -> 5.02).
+    // The class constants are first used here, in the previous kernel's shadow, by a multiplication that the tables take back: between the loads of x
+    // and their use, a wait for them is a wait for x.  Several vectors and the 10-byte layout build the whole tables here; one vector on the 14- or
+    // 13-byte layout is delayed by that by more than it saves.  Us a launch, without either, with the multiplication, with the tables too: one
+    // vector on 1024 x 2560 3.20, 3.10 and 3.16, 4096 x 4096 5.17, 5.01 and 5.08, rotated -, 6.64 and 6.71; two on 600 x 1000 -, 3.74 and 3.58, 6016 x
+    // 1088 -, 5.36 and 5.20; the 10-byte layout on 4096 x 4096 5.45, - and 5.31, the 13-byte one on 1024 x 2560 3.19, - and 3.29.
     if (!COMPACT) {
 #pragma unroll
         for (int i = 0; i < kClasses; i++) asm volatile("mul.rn.f32 %0, %0, 0f3F000000;" : "+f"(my_class[i].x));
     }
+    if (kTablesFirst) build_tables();
     // let the next kernel in the stream start its own prefetch, then wait for the previous one:
     // x, y and the reduction scratch may still be in use by it
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -904,7 +909,7 @@ __global__ void __launch_bounds__(32 * gemv_warps(BATCH), 1) gemv_planes_kernel(
                 // The zero word and the two sums of every x record this CTA will fill
                 for (int b = tid; b < BATCH * (blk_hi - blk_lo); b += kThreads)
                     asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(smem_addr(xrec) + b * kXRecBytes + 96), "r"(0) : "memory");
-                build_tables();
+                if (!kTablesFirst) build_tables();
             }
 #pragma unroll
             for (int j = 0; j < BATCH; j++)
