@@ -42,7 +42,7 @@ NCU_TRAFFIC_PER_ALGORITHMIC_BYTE = 39.362304 / 39.288864
 # from the same capture: warp instructions per block column (32 rows x 24 weights), and the share of issue
 # slots busy over the launch
 NCU_WARP_INSTR_PER_CELL = 5623111 / 87552
-NCU_ISSUE_BUSY_PCT = 57.0
+NCU_ISSUE_BUSY_PCT = 56.0
 METRIC = "us_per_lattice_gemv"
 DISCARD_ROUNDS = 2
 

@@ -16,9 +16,9 @@
 // through a second build of their code, which counts L' back: the contraction of the marks [L' >= 32640] takes 65536 times itself from L
 // and adds itself to H.
 //
-// Bound: instruction issue (four vectors on 8192 x 8192: 466 warp instructions a tile with the launch's start, issue slots 59 % busy, no stall above
-// 0.9 cycles an instruction; eight: 649 and 50 %, three warps a scheduler), and on small launches the preparation of x (4096 x 4096: issue slots
-// 49 and 39 % busy, barriers the longest stall).  Against the 8-bit limbs two vectors at a time that this replaces, us a launch in a chain: see
+// Bound: instruction issue (four vectors on 8192 x 8192: 466 warp instructions a tile with the launch's start, issue slots 59 % busy; eight: 649
+// and 50 %, three warps a scheduler), and on small launches the preparation of x (4096 x 4096: issue slots 48 and 37 % busy, barriers and reads of
+// global memory the longest stalls).  Against the 8-bit limbs two vectors at a time that this replaces, us a launch in a chain: see
 // launch_gemv (llvq_gemv.cu).
 #include <type_traits>
 

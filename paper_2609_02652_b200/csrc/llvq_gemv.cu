@@ -314,8 +314,8 @@ __device__ __forceinline__ void contract_half(const HalfA &h, const StepX &sx, f
 // the other slot's positions zero in B.  Against one vector with block-diagonal B that is three instructions instead
 // of four for two vectors and two slots, and a row's sum lies in two lanes instead of four, so half the exchanges.
 // The price is that a lane looks up the headers of both slots; every vector shares that.  Two, five and six vectors go this way
-// (three, four, seven and eight: llvq_batch.cu).  Bound: latency (4096 x 4096: issue slots 45 % busy
-// with two vectors, 44 % with five, whose twelve warps are three a scheduler).  Two vectors on 8192 x 8192: 11.8 us a launch, 12.5 a vector at a
+// (three, four, seven and eight: llvq_batch.cu).  Bound: latency (4096 x 4096: issue slots 44 % busy
+// with two vectors, 43 % with five, whose twelve warps are three a scheduler).  Two vectors on 8192 x 8192: 11.8 us a launch, 12.5 a vector at a
 // time, its atomic waited for before the next vector's.
 struct PairA {
     uint32_t a0, a1, a2, a3, c0, c1;
